@@ -240,38 +240,35 @@ static int md_dispatch(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled
 
 namespace he {
 
-// Whether the fused ModDown (or rescale) with nd dropped limbs runs, so that
-// its conversion kernel can finish the dropped limbs' inverse transform
-// (the caller then runs only its row pass).
-bool md_half_ok(const he_ctx* c, uint32_t nd) {
+// Whether the fused ModDown (or rescale) with nd dropped limbs and `targets`
+// remaining ones runs on `count` ciphertexts with a conversion kernel that
+// finishes the dropped limbs' inverse transform (the caller then runs only
+// its row pass).
+bool md_half_ok(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   if (!ks_fusable(c)) return false;
-  size_t smem = 0;
   switch (c->log_n) {
-    case 12: smem = md_col_smem_n12(c, nd); break;
-    case 13: smem = md_col_smem_n13(c, nd); break;
-    case 14: smem = md_col_smem_n14(c, nd); break;
-    case 15: smem = md_col_smem_n15(c, nd); break;
-    default: smem = md_col_smem_n16(c, nd); break;
+    case 12: return md_half_n12(c, nd, targets, count);
+    case 13: return md_half_n13(c, nd, targets, count);
+    case 14: return md_half_n14(c, nd, targets, count);
+    case 15: return md_half_n15(c, nd, targets, count);
+    default: return md_half_n16(c, nd, targets, count);
   }
-  return smem <= kModupAllSmem;
 }
 
-// Whether the fused key switch at this level converts each digit in one CTA
-// (then it can finish the inverse transform of its input itself).
-bool ks_converts_per_digit(const he_ctx* c, uint32_t level) {
+// Whether the fused key switch of `count` polynomials at this level finishes
+// the inverse transform of its input in its conversion kernel.
+bool ks_converts_per_digit(const he_ctx* c, uint32_t level, uint32_t count) {
   if (!ks_fusable(c)) return false;
   const uint32_t alpha = (uint32_t)c->alpha, beta = (level + alpha - 1) / alpha;
   uint32_t cnt[HE_MAX_PRIMES];
   for (uint32_t j = 0; j < beta; ++j) cnt[j] = c->modup[level][j].cnt;
-  size_t smem = 0;
   switch (c->log_n) {
-    case 12: smem = ks_all_smem_n12(c, beta, cnt); break;
-    case 13: smem = ks_all_smem_n13(c, beta, cnt); break;
-    case 14: smem = ks_all_smem_n14(c, beta, cnt); break;
-    case 15: smem = ks_all_smem_n15(c, beta, cnt); break;
-    default: smem = ks_all_smem_n16(c, beta, cnt); break;
+    case 12: return ks_half_n12(c, level, beta, cnt, count);
+    case 13: return ks_half_n13(c, level, beta, cnt, count);
+    case 14: return ks_half_n14(c, level, beta, cnt, count);
+    case 15: return ks_half_n15(c, level, beta, cnt, count);
+    default: return ks_half_n16(c, level, beta, cnt, count);
   }
-  return smem <= kModupAllSmem;
 }
 
 }  // namespace he

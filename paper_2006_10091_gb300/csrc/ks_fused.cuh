@@ -40,6 +40,7 @@ struct KsFusedArgs {
   const ulonglong2* tw;
   const ulonglong2* itw;   // inverse twiddles
   int half;                // d2c holds the inverse transform's row pass only (ks_modup_col_all finishes it)
+  uint32_t splits;         // CTAs of ks_modup_col_all that share one digit and tile's target limbs
   const uint64_t* consts;  // ModUp constant tables
   uint32_t lo[HE_MAX_PRIMES], cnt[HE_MAX_PRIMES];
   uint64_t off[HE_MAX_PRIMES];
@@ -135,11 +136,13 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
   }
 }
 
-// The same column pass for every target limb of one digit and tile in one
+// The same column pass for several target limbs of one digit and tile in one
 // CTA: the digit's limbs are read once and their products by
 // (Q_j/q_i)^-1 mod q_i (or, for a one-limb digit, the limb itself) are kept
-// in shared memory for all targets.  Grid: count * beta * TILES; dynamic
-// shared memory holds cnt_max * TILE more words.
+// in shared memory for those targets.  The nt targets are shared evenly by
+// a.splits CTAs (conv_splits: one CTA per digit and tile when the batch fills
+// the chip).  Grid: count * beta * splits * TILES; dynamic shared memory
+// holds cnt_max * TILE more words.
 template <int LOG_N, int LOG_M, int LOG_K>
 __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(KsFusedArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
@@ -151,8 +154,11 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
   uint32_t b = blockIdx.x;
   const uint32_t tile = b % S::TILES;
   b /= S::TILES;
+  const uint32_t part = b % a.splits;
+  b /= a.splits;
   const uint32_t j = b % a.beta, i = b / a.beta;
   const uint32_t lo = a.lo[j], cnt = a.cnt[j];
+  const uint32_t t_end = (part + 1) * a.nt / a.splits;
   const uint64_t* tab = a.consts + a.off[j];
   const uint64_t* mat = tab + 2 * cnt;
   const uint64_t* mat_sh = mat + (size_t)cnt * a.np;
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
     // the next limb's staging overwrites stw and sm: wait for every thread
     __syncthreads();
   }
-  for (uint32_t t = 0; t < a.nt; ++t) {
+  for (uint32_t t = part * a.nt / a.splits; t < t_end; ++t) {
     if (t >= lo && t < lo + cnt) continue;  // the digit's own limbs are used as they are
     const uint32_t prime = ks_prime(t, a.level, a.L);
     const PrimeDev pr = a.primes[prime];
@@ -588,12 +594,14 @@ struct MdArgs {
   const ulonglong2* tw;
   const ulonglong2* itw;  // inverse twiddles (half)
   int half;               // yP holds only the inverse transform's row pass: md_conv_col finishes it
+  uint32_t splits;        // CTAs of md_conv_col that share one tile's target limbs
   const uint64_t* md;   // ModDown tables (params.cu)
 };
 
-// Grid: count * 2 * TILES; the conversion's per-special-prime terms and the
-// multiple v of P are computed once per element and kept in shared memory
-// ([alpha][TILE] words and [TILE] counts) for all level target limbs.
+// Grid: count * 2 * splits * TILES; the conversion's per-special-prime terms
+// and the multiple v of P are computed once per element and kept in shared
+// memory ([alpha][TILE] words and [TILE] counts) for the CTA's share of the
+// level target limbs (all of them when the batch fills the chip, conv_splits).
 template <int LOG_N, int LOG_M, int LOG_K>
 __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
@@ -606,7 +614,10 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
   uint32_t b = blockIdx.x;
   const uint32_t tile = b % S::TILES;
   b /= S::TILES;
+  const uint32_t part = b % a.splits;
+  b /= a.splits;
   const uint32_t p = b % 2, i = b / 2;
+  const uint32_t t_end = (part + 1) * a.level / a.splits;
   const uint64_t* mat = a.md + 2 * a.alpha;
   const uint64_t* hP = mat + (size_t)a.alpha * a.L + 2 * a.L;
   const uint64_t* mat_sh = hP + a.alpha + a.L;
@@ -627,12 +638,18 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
       __syncthreads();
       run_rounds<true, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pp.q);
     }
-#pragma unroll 2
-    for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
-      const uint64_t y0 = a.half ? mul_shoup(sm[idx + (idx >> 3)], pp.n_inv, pp.n_inv_sh, pp.q)
-                                 : __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
-      const uint64_t y = add_mod(y0, hP[u], pp.q);
-      wv[(size_t)u * S::TILE + idx] = mul_shoup(y, a.md[2 * u], a.md[2 * u + 1], pp.q);
+    // the thread's words of the limb first (eight loads in flight), then their products
+    uint64_t y0[S::TILE / S::T];
+#pragma unroll
+    for (int v = 0; v < S::TILE / S::T; ++v) {
+      const uint32_t idx = threadIdx.x + v * S::T;
+      y0[v] = a.half ? sm[idx + (idx >> 3)] : __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
+    }
+    const uint64_t h = hP[u], w = a.md[2 * u], wsh = a.md[2 * u + 1];
+#pragma unroll
+    for (int v = 0; v < S::TILE / S::T; ++v) {
+      if (a.half) y0[v] = mul_shoup(y0[v], pp.n_inv, pp.n_inv_sh, pp.q);
+      wv[(size_t)u * S::TILE + threadIdx.x + v * S::T] = mul_shoup(add_mod(y0[v], h, pp.q), w, wsh, pp.q);
     }
     // the next limb's staging overwrites stw and sm: wait for every thread
     if (a.half) __syncthreads();
@@ -651,7 +668,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
     }
     vv[idx] = v;
   }
-  for (uint32_t t = 0; t < a.level; ++t) {
+  for (uint32_t t = part * a.level / a.splits; t < t_end; ++t) {
     const PrimeDev pr = a.primes[t];
     const uint64_t q2 = pr.q + pr.q, hQ = hP[a.alpha + t];
     const uint64_t* vP = wlo + a.alpha + a.L + (size_t)t * 8;  // v P mod q_t, v < 8
@@ -767,9 +784,63 @@ size_t md_col_smem(uint32_t nd) {
          (sizeof(uint64_t) * nd + sizeof(uint32_t)) * SC::TILE;
 }
 
-template <int LOG_N, int M1, int K1, int M2, int K2>
-int md_fused_run(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
+// How a conversion kernel's target limbs are shared: `blocks` groups of CTAs
+// (digits or parts times tiles), of which `slots` CTAs run at a time; a CTA
+// pays `setup` and then one unit per target.  A CTA's chain of targets is
+// bound by latency (a unit takes 4.4 us alone on its SM and 5.9 us beside two
+// others, N = 2^13 and 2^14), so a batch that leaves CTA slots free is split as
+// far as they reach, and the time is the number of waves times the chain.  (Splits
+// beyond one wave: inference of 21 ciphertexts at N = 2^13, 503 against 460 us.)
+// One rotation at N = 2^13, level 19: 20 and 8 CTAs walked 19 to 23 targets
+// each, 101 and 122 us.
+inline uint32_t conv_splits(size_t blocks, size_t slots, uint32_t targets, double setup, double* cost) {
+  uint32_t best = 1;
+  double bc = 0.0;
+  for (uint32_t s = 1; s <= targets && (s == 1 || blocks * s <= slots); ++s) {
+    const double c = (double)((blocks * s + slots - 1) / slots) * (setup + (double)((targets + s - 1) / s));
+    if (s == 1 || c < bc) {
+      bc = c;
+      best = s;
+    }
+  }
+  if (cost) *cost = bc;
+  return best;
+}
+
+// CTAs of `threads` threads and `smem` bytes that run at a time.
+inline size_t conv_slots(const he_ctx* c, size_t smem, int threads) {
+  return 152 * std::max<size_t>(1, std::min<size_t>(c->smem_per_sm / (smem + 1024), 1024 / threads));
+}
+
+// Units (one target's conversion and column pass) a conversion kernel pays
+// before its targets for one source limb: the inverse transform's column pass
+// on it when it finishes that transform itself, a load and a product if not.
+constexpr double kSetupHalf = 1.0, kSetupFull = 0.3;
+// ... and the units a column pass launched by itself costs instead.
+inline double col_pass_units(size_t polys, int tiles) {
+  return 1.5 + (double)((polys * tiles + 4 * 152 - 1) / (4 * 152));
+}
+
+template <int LOG_N, int M1, int K1>
+size_t md_col_smem(uint32_t nd);
+
+// Whether md_conv_col finishes the dropped limbs' inverse transform itself.
+template <int LOG_N, int M1, int K1>
+bool md_half(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   using SC = Shape<LOG_N, M1, K1, true>;
+  const size_t sm = md_col_smem<LOG_N, M1, K1>(nd), blocks = (size_t)count * 2 * SC::TILES;
+  if (sm > kModupAllSmem) return false;
+  const size_t slots = conv_slots(c, sm, SC::T);
+  double half, full;
+  conv_splits(blocks, slots, targets, kSetupHalf * nd, &half);
+  conv_splits(blocks, slots, targets, kSetupFull * nd, &full);
+  return half <= full + col_pass_units((size_t)count * 2 * nd, SC::TILES);
+}
+
+template <int LOG_N, int M1, int K1, int M2, int K2>
+int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
+  using SC = Shape<LOG_N, M1, K1, true>;
+  MdArgs a = a0;
   using SR = Shape<LOG_N, M2, K2, false>;
   const size_t smc = md_col_smem<LOG_N, M1, K1>(a.alpha);
   const size_t smr = sizeof(ulonglong2) * SR::NTW + sizeof(uint64_t) * (SR::TILE + SR::TILE / 8);
@@ -788,7 +859,10 @@ int md_fused_run(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
   const char* nm_row = a.kind == 1 ? "rescale_ntt_final" : a.kind == 2 ? "moddown_rescale_ntt_combine"
                                                                        : "moddown_ntt_combine";
   {
-    const size_t blocks = (size_t)count * 2 * SC::TILES;
+    size_t blocks = (size_t)count * 2 * SC::TILES;
+    a.splits = conv_splits(blocks, conv_slots(c, smc, SC::T), a.level, (a.half ? kSetupHalf : kSetupFull) * a.alpha,
+                           nullptr);
+    blocks *= a.splits;
     // with a half-transformed input, also the dropped limbs' inverse column pass
     const double bfly = polys * n / 2 * M1 + (a.half ? 2.0 * count * a.alpha * n / 2 * M1 : 0.0);
     ProfScope prof(c, nm_col, bfly + polys * n * a.alpha, n * 8 * (2.0 * count * a.alpha + polys), 0.0, bfly);
@@ -816,10 +890,25 @@ size_t ks_all_smem(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
          sizeof(uint64_t) * (size_t)cnt_max * SC::TILE;
 }
 
+// Whether ks_modup_col_all finishes the input's inverse transform itself.
+template <int LOG_N, int M1, int K1>
+bool ks_half(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
+  using SC = Shape<LOG_N, M1, K1, true>;
+  const size_t sm = ks_all_smem<LOG_N, M1, K1>(c, beta, cnt), blocks = (size_t)count * beta * SC::TILES;
+  if (sm > kModupAllSmem) return false;
+  const size_t slots = conv_slots(c, sm, SC::T);
+  const uint32_t nt = level + (uint32_t)c->alpha;
+  double half, full;
+  conv_splits(blocks, slots, nt, kSetupHalf * cnt[0], &half);
+  conv_splits(blocks, slots, nt, kSetupFull * cnt[0], &full);
+  return half <= full + col_pass_units((size_t)count * level, SC::TILES);
+}
+
 // The ModUp + column-pass launch shared by the key switch and the hoisted
 // rotate-and-sum.
 template <int LOG_N, int M1, int K1>
-int ks_modup_launch(he_ctx* c, const KsFusedArgs& a, uint32_t count) {
+int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
+  KsFusedArgs a = a0;
   using SC = Shape<LOG_N, M1, K1, true>;
   const size_t smc = sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8);
   static std::atomic<unsigned long long> attr_one{0}, attr_all{0};
@@ -841,8 +930,11 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a, uint32_t count) {
                    count * n * 8 * (a.level + conv), 0.0, bfly);
     const size_t sma = ks_all_smem<LOG_N, M1, K1>(c, a.beta, a.cnt);
     if (a.half && sma > kModupAllSmem) return fail(HE_EINVAL, "ks_fused: half-transformed input needs the all-targets kernel");
-    if (sma <= kModupAllSmem) {  // one CTA per digit and tile, all targets
-      const size_t blocks = (size_t)count * a.beta * SC::TILES;
+    if (sma <= kModupAllSmem) {  // the targets of one digit and tile in `splits` CTAs
+      size_t blocks = (size_t)count * a.beta * SC::TILES;
+      a.splits = conv_splits(blocks, conv_slots(c, sma, SC::T), a.nt, (a.half ? kSetupHalf : kSetupFull) * a.cnt[0],
+                             nullptr);
+      blocks *= a.splits;
       ks_modup_col_all<LOG_N, M1, K1><<<(unsigned)blocks, SC::T, sma, c->stream>>>(a);
     } else {
       const size_t blocks = (size_t)count * a.beta * a.nt * SC::TILES;
@@ -973,8 +1065,8 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, in
   int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, int* closed); \
   size_t ks_rot_smem_n##NN(const he_ctx* c, uint32_t beta);                          \
   int md_fused_n##NN(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled);     \
-  size_t md_col_smem_n##NN(const he_ctx* c, uint32_t nd);                            \
-  size_t ks_all_smem_n##NN(const he_ctx* c, uint32_t beta, const uint32_t* cnt);
+  bool md_half_n##NN(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count); \
+  bool ks_half_n##NN(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count);
 HE_KS_FUSED_DECL(12)
 HE_KS_FUSED_DECL(13)
 HE_KS_FUSED_DECL(14)

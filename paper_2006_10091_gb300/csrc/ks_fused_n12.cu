@@ -21,16 +21,16 @@ int md_fused_n12(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
        : sh == 2 ? md_fused_run<12, 3, 8, 9, 2>(c, a, count, handled) : md_fused_run<12, 6, 5, 6, 5>(c, a, count, handled);
 }
 
-size_t md_col_smem_n12(const he_ctx* c, uint32_t nd) {
+bool md_half_n12(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_col_smem<12, 5, 6>(nd)
-       : sh == 2 ? md_col_smem<12, 3, 8>(nd) : md_col_smem<12, 6, 5>(nd);
+  return sh == 1 ? md_half<12, 5, 6>(c, nd, targets, count)
+       : sh == 2 ? md_half<12, 3, 8>(c, nd, targets, count) : md_half<12, 6, 5>(c, nd, targets, count);
 }
 
-size_t ks_all_smem_n12(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
+bool ks_half_n12(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_all_smem<12, 5, 6>(c, beta, cnt)
-       : sh == 2 ? ks_all_smem<12, 3, 8>(c, beta, cnt) : ks_all_smem<12, 6, 5>(c, beta, cnt);
+  return sh == 1 ? ks_half<12, 5, 6>(c, level, beta, cnt, count)
+       : sh == 2 ? ks_half<12, 3, 8>(c, level, beta, cnt, count) : ks_half<12, 6, 5>(c, level, beta, cnt, count);
 }
 
 }  // namespace he

@@ -21,16 +21,16 @@ int md_fused_n13(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
        : sh == 2 ? md_fused_run<13, 4, 7, 9, 2>(c, a, count, handled) : md_fused_run<13, 7, 4, 6, 5>(c, a, count, handled);
 }
 
-size_t md_col_smem_n13(const he_ctx* c, uint32_t nd) {
+bool md_half_n13(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_col_smem<13, 6, 5>(nd)
-       : sh == 2 ? md_col_smem<13, 4, 7>(nd) : md_col_smem<13, 7, 4>(nd);
+  return sh == 1 ? md_half<13, 6, 5>(c, nd, targets, count)
+       : sh == 2 ? md_half<13, 4, 7>(c, nd, targets, count) : md_half<13, 7, 4>(c, nd, targets, count);
 }
 
-size_t ks_all_smem_n13(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
+bool ks_half_n13(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_all_smem<13, 6, 5>(c, beta, cnt)
-       : sh == 2 ? ks_all_smem<13, 4, 7>(c, beta, cnt) : ks_all_smem<13, 7, 4>(c, beta, cnt);
+  return sh == 1 ? ks_half<13, 6, 5>(c, level, beta, cnt, count)
+       : sh == 2 ? ks_half<13, 4, 7>(c, level, beta, cnt, count) : ks_half<13, 7, 4>(c, level, beta, cnt, count);
 }
 
 }  // namespace he

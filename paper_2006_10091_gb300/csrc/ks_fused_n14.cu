@@ -6,31 +6,31 @@ namespace he {
 
 int ks_rot_n14(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, int* closed) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_run<14, 8, 3, 6, 5>(c, a, count, handled, closed)
-       : sh == 2 ? ks_rot_run<14, 5, 6, 9, 2>(c, a, count, handled, closed) : ks_rot_run<14, 7, 4, 7, 4>(c, a, count, handled, closed);
+  return sh == 1 ? ks_rot_run<14, 7, 4, 7, 4>(c, a, count, handled, closed)
+       : sh == 2 ? ks_rot_run<14, 8, 3, 6, 5>(c, a, count, handled, closed) : ks_rot_run<14, 5, 6, 9, 2>(c, a, count, handled, closed);
 }
 
 size_t ks_rot_smem_n14(const he_ctx* c, uint32_t beta) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_smem<14, 6, 5>(beta) : sh == 2 ? ks_rot_smem<14, 9, 2>(beta) : ks_rot_smem<14, 7, 4>(beta);
+  return sh == 1 ? ks_rot_smem<14, 7, 4>(beta) : sh == 2 ? ks_rot_smem<14, 6, 5>(beta) : ks_rot_smem<14, 9, 2>(beta);
 }
 
 int md_fused_n14(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_fused_run<14, 8, 3, 6, 5>(c, a, count, handled)
-       : sh == 2 ? md_fused_run<14, 5, 6, 9, 2>(c, a, count, handled) : md_fused_run<14, 7, 4, 7, 4>(c, a, count, handled);
+  return sh == 1 ? md_fused_run<14, 7, 4, 7, 4>(c, a, count, handled)
+       : sh == 2 ? md_fused_run<14, 8, 3, 6, 5>(c, a, count, handled) : md_fused_run<14, 5, 6, 9, 2>(c, a, count, handled);
 }
 
-size_t md_col_smem_n14(const he_ctx* c, uint32_t nd) {
+bool md_half_n14(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_col_smem<14, 8, 3>(nd)
-       : sh == 2 ? md_col_smem<14, 5, 6>(nd) : md_col_smem<14, 7, 4>(nd);
+  return sh == 1 ? md_half<14, 7, 4>(c, nd, targets, count)
+       : sh == 2 ? md_half<14, 8, 3>(c, nd, targets, count) : md_half<14, 5, 6>(c, nd, targets, count);
 }
 
-size_t ks_all_smem_n14(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
+bool ks_half_n14(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_all_smem<14, 8, 3>(c, beta, cnt)
-       : sh == 2 ? ks_all_smem<14, 5, 6>(c, beta, cnt) : ks_all_smem<14, 7, 4>(c, beta, cnt);
+  return sh == 1 ? ks_half<14, 7, 4>(c, level, beta, cnt, count)
+       : sh == 2 ? ks_half<14, 8, 3>(c, level, beta, cnt, count) : ks_half<14, 5, 6>(c, level, beta, cnt, count);
 }
 
 }  // namespace he

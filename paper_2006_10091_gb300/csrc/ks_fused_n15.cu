@@ -6,31 +6,31 @@ namespace he {
 
 int ks_rot_n15(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, int* closed) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_run<15, 7, 4, 8, 3>(c, a, count, handled, closed)
-       : sh == 2 ? ks_rot_run<15, 6, 5, 9, 2>(c, a, count, handled, closed) : ks_rot_run<15, 8, 4, 7, 4>(c, a, count, handled, closed);
+  return sh == 1 ? ks_rot_run<15, 8, 4, 7, 4>(c, a, count, handled, closed)
+       : sh == 2 ? ks_rot_run<15, 6, 5, 9, 2>(c, a, count, handled, closed) : ks_rot_run<15, 7, 4, 8, 3>(c, a, count, handled, closed);
 }
 
 size_t ks_rot_smem_n15(const he_ctx* c, uint32_t beta) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_smem<15, 8, 3>(beta) : sh == 2 ? ks_rot_smem<15, 9, 2>(beta) : ks_rot_smem<15, 7, 4>(beta);
+  return sh == 1 ? ks_rot_smem<15, 7, 4>(beta) : sh == 2 ? ks_rot_smem<15, 9, 2>(beta) : ks_rot_smem<15, 8, 3>(beta);
 }
 
 int md_fused_n15(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_fused_run<15, 7, 4, 8, 3>(c, a, count, handled)
-       : sh == 2 ? md_fused_run<15, 6, 5, 9, 2>(c, a, count, handled) : md_fused_run<15, 8, 4, 7, 4>(c, a, count, handled);
+  return sh == 1 ? md_fused_run<15, 8, 4, 7, 4>(c, a, count, handled)
+       : sh == 2 ? md_fused_run<15, 6, 5, 9, 2>(c, a, count, handled) : md_fused_run<15, 7, 4, 8, 3>(c, a, count, handled);
 }
 
-size_t md_col_smem_n15(const he_ctx* c, uint32_t nd) {
+bool md_half_n15(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? md_col_smem<15, 7, 4>(nd)
-       : sh == 2 ? md_col_smem<15, 6, 5>(nd) : md_col_smem<15, 8, 4>(nd);
+  return sh == 1 ? md_half<15, 8, 4>(c, nd, targets, count)
+       : sh == 2 ? md_half<15, 6, 5>(c, nd, targets, count) : md_half<15, 7, 4>(c, nd, targets, count);
 }
 
-size_t ks_all_smem_n15(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
+bool ks_half_n15(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_all_smem<15, 7, 4>(c, beta, cnt)
-       : sh == 2 ? ks_all_smem<15, 6, 5>(c, beta, cnt) : ks_all_smem<15, 8, 4>(c, beta, cnt);
+  return sh == 1 ? ks_half<15, 8, 4>(c, level, beta, cnt, count)
+       : sh == 2 ? ks_half<15, 6, 5>(c, level, beta, cnt, count) : ks_half<15, 7, 4>(c, level, beta, cnt, count);
 }
 
 }  // namespace he

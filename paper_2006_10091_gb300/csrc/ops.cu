@@ -17,8 +17,8 @@
 #include "he_ops.h"
 
 namespace he {
-bool ks_converts_per_digit(const he_ctx* c, uint32_t level);
-bool md_half_ok(const he_ctx* c, uint32_t nd);
+bool ks_converts_per_digit(const he_ctx* c, uint32_t level, uint32_t count);
+bool md_half_ok(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count);
 int ntt2_inverse_rows(he_ctx* c, const PolyBatch& b);
 int md_fused(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t* conv, CtBatch add, int add_mode,
              uint64_t add_gal, CtBatch out, uint32_t level, uint32_t count, bool half, bool* handled);
@@ -179,7 +179,7 @@ int keyswitch_batch(he_ctx* c, const uint64_t* d, uint64_t d_stride, uint32_t le
   //    inverse transform's row pass here; the conversion kernel finishes it)
   const bool fits = ks_rot_fits(c, level, 1);
   if (gal && !fits) return fail(HE_EINVAL, "keyswitch_batch: automorphism needs the fused kernels");
-  const bool half = fits && ks_converts_per_digit(c, level);
+  const bool half = fits && ks_converts_per_digit(c, level, count);
   {
     PolyBatch b = pb(d, d2c, d_stride, (size_t)level * n, count, level, 0, level);
     b.gal = gal;
@@ -222,7 +222,7 @@ int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint
     HE_CUDA(cudaGetLastError());
     // the dropped limbs to coefficient form (only the row pass when the
     // fused conversion kernel finishes the transform)
-    const bool mh = md_half_ok(c, alpha + 1);
+    const bool mh = md_half_ok(c, alpha + 1, level - 1, count);
     const PolyBatch bd = pb(acc + (size_t)lo * n, acc + (size_t)lo * n, (size_t)nt * n, (size_t)nt * n, count * 2,
                             alpha + 1, lo, level);
     HE_TRY(mh ? ntt2_inverse_rows(c, bd) : ntt_inverse(c, bd));
@@ -231,7 +231,7 @@ int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint
     if (done) return HE_OK;
     return moddown_unfused(c, acc, conv, add, 2, out, level, count, true);
   }
-  const bool mh = md_half_ok(c, alpha);
+  const bool mh = md_half_ok(c, alpha, level, count);
   {
     const PolyBatch bd = pb(acc + (size_t)level * n, acc + (size_t)level * n, (size_t)nt * n, (size_t)nt * n,
                             count * 2, alpha, level, level);
@@ -257,7 +257,7 @@ int rescale_batch(he_ctx* c, CtBatch in, uint32_t level, uint32_t count, CtBatch
   uint64_t* last = ar.take<uint64_t>((size_t)count * 2 * n);
   uint64_t* corr = ar.take<uint64_t>((size_t)count * 2 * lt * n);
   if (!last || !corr) return fail(HE_ENOMEM, "rescale scratch too small");
-  const bool mh = md_half_ok(c, 1);  // the fused kernel finishes the inverse transform
+  const bool mh = md_half_ok(c, 1, lt, count);  // the fused kernel finishes the inverse transform
   for (uint32_t p = 0; p < 2; ++p) {
     const PolyBatch bd = pb(in.base + ((size_t)p * in.cap + lt) * n, last + (size_t)p * n, in.stride, 2ull * n,
                             count, 1, lt, c->L);
@@ -355,7 +355,7 @@ int rotsum_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, const uin
   if (!d2c || !ext || !acc || !conv) return fail(HE_ENOMEM, "rotate-and-sum scratch too small");
   const uint64_t* d = A.base + (size_t)A.cap * n;
   const bool fits = ks_rot_fits(c, level, nrot);
-  const bool half = fits && ks_converts_per_digit(c, level);
+  const bool half = fits && ks_converts_per_digit(c, level, count);
   {
     const PolyBatch b = pb(d, d2c, A.stride, (size_t)level * n, count, level, 0, level);
     HE_TRY(half ? ntt2_inverse_rows(c, b) : ntt_inverse(c, b));
@@ -385,7 +385,7 @@ int rotsum_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, const uin
     HE_CUDA(cudaGetLastError());
   }
   // ModDown of the summed inner products, plus A0 + sum_r kappa_r(A0) and A1
-  const bool mh = md_half_ok(c, alpha);
+  const bool mh = md_half_ok(c, alpha, level, count);
   {
     const PolyBatch bd = pb(acc + (size_t)level * n, acc + (size_t)level * n, (size_t)nt * n, (size_t)nt * n,
                             count * 2, alpha, level, level);

@@ -1,0 +1,47 @@
+"""A batch's residues do not depend on its size: the conversion kernels split
+target limbs over several CTAs when the batch leaves CTAs free, finish the
+inverse transform themselves or not, and the key-product kernel takes several
+ciphertexts per CTA; every route gives the residues of the others (small
+batches are compared with the oracle in the parity tests)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def uniform(ctx, torch, level, count, seed):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    cts = ctx.new_ct(level, count)
+    for c in cts:
+        for t in range(level):
+            c.tensor[:, t].random_(0, ctx.primes[t], generator=gen)
+        c.level, c.scale = level, 2.0 ** 40
+    return cts
+
+
+# (log_n, limbs, bits, special, special bits, level, batch): one limb per digit, a last digit that is not full,
+# digits of four limbs, wide special primes; batches on both sides of one wave of CTAs
+CASES = [(12, 4, 40, 1, 60, 4, 90), (12, 7, 45, 3, 59, 7, 70), (13, 9, 50, 4, 60, 6, 90), (14, 5, 40, 2, 59, 5, 61)]
+
+
+@pytest.mark.parametrize("log_n,limbs,bits,special,sbits,level,batch", CASES)
+def test_residues_do_not_depend_on_the_batch(log_n, limbs, bits, special, sbits, level, batch):
+    import torch
+    import paper_2006_10091_gb300 as he
+    ctx = he.Context(log_n, limbs, bits, special, sbits, 2.0 ** 40, seed=5, rot_steps=[3, 64])
+    A, B = uniform(ctx, torch, level, batch, 1), uniform(ctx, torch, level, batch, 2)
+    ops = {
+        "mul": lambda x, y, o: he.he_mul_relin_rescale_batch(ctx, x, y, o),
+        "rotate": lambda x, y, o: he.he_rotate_batch(ctx, x, 3, o),
+        "rotsum": lambda x, y, o: he.he_rotate_sum_batch(ctx, x, [3, 64], o),
+        "rotsum_closed": lambda x, y, o: he.he_rotate_sum_batch(ctx, x, [64], o),
+    }
+    for name, op in ops.items():
+        want = ctx.new_ct(level, batch)
+        op(A, B, want)
+        for first, count in ((0, 1), (batch - 1, 1), (7, 5), (3, 24)):
+            got = ctx.new_ct(level, count)
+            op(A[first:first + count], B[first:first + count], got)
+            for i in range(count):
+                assert np.array_equal(got[i].residues(), want[first + i].residues()), (name, first, count, i)
