@@ -167,23 +167,6 @@ __global__ void k_inner_product_rot(const uint64_t* ext, uint64_t ext_stride, co
   }
 }
 
-// Accumulators of both parts (limbs 0 .. nt-1, limb t over prime(t)) reduced
-// to [0, q) from sums of a few residues.
-__global__ void k_reduce_acc(uint64_t* acc, uint64_t acc_stride, uint32_t nt, uint32_t level, uint32_t L,
-                             uint32_t count, int log_n, const PrimeDev* primes) {
-  const uint32_t n = 1u << log_n;
-  const size_t total = (size_t)count * 2 * nt * n;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
-    const uint32_t e = (uint32_t)(g & (n - 1));
-    size_t r = g >> log_n;
-    const uint32_t t = rmod(r, nt);
-    size_t rq = r;
-    const uint32_t p = rmod(rq, 2), i = (uint32_t)rq;
-    uint64_t* a = acc + (size_t)i * acc_stride + ((size_t)p * nt + t) * n + e;
-    *a = reduce64(*a, primes[t < level ? t : L + t - level]);
-  }
-}
-
 // O = (A0 + sum_r kappa_r(A0), A1): the addend of a hoisted rotate-and-sum.
 __global__ void k_add_automorphs(CtBatch A, CtBatch O, RotSet rs, uint32_t level, uint32_t count, int log_n,
                                  const PrimeDev* primes) {

@@ -53,8 +53,6 @@ __global__ void k_inner_product_rot(const uint64_t* ext, uint64_t ext_stride, co
                                     uint64_t d_stride, RotSet rs, uint64_t* acc, uint64_t acc_stride,
                                     uint32_t level, uint32_t alpha, uint32_t beta, uint32_t L, uint32_t np,
                                     uint32_t count, int log_n, const PrimeDev* primes);
-__global__ void k_reduce_acc(uint64_t* acc, uint64_t acc_stride, uint32_t nt, uint32_t level, uint32_t L,
-                             uint32_t count, int log_n, const PrimeDev* primes);
 __global__ void k_add_automorphs(CtBatch A, CtBatch O, RotSet rs, uint32_t level, uint32_t count, int log_n,
                                  const PrimeDev* primes);
 // The dropped limbs of a ModDown: n limbs of acc starting at limb `first`,

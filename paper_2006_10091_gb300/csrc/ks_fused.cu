@@ -37,21 +37,8 @@ static KsFusedArgs ks_args(he_ctx* c, const uint64_t* d, uint64_t d_stride, cons
   return a;
 }
 
-// Inverse of an odd Galois element modulo 2N (Newton's iteration for the
-// inverse modulo 2^64, then reduced).
-static uint64_t gal_inverse(uint64_t gal, int log_n) {
-  uint64_t x = gal;  // correct to 3 bits
-  for (int i = 0; i < 5; ++i) x *= 2 - gal * x;
-  return x & ((2ull << log_n) - 1);
-}
-
-bool ks_rot_fits(const he_ctx* c, uint32_t level, uint32_t nrot) {
+bool ks_rot_fits(const he_ctx* c, uint32_t level) {
   if (!ks_fusable(c)) return false;
-  // rows moved between CTAs are summed as nrot unreduced residues in 64 bits
-  uint64_t qmax = 0;
-  for (uint32_t t = 0; t < level; ++t) qmax = std::max(qmax, c->q[t]);
-  for (uint32_t u = 0; u < (uint32_t)c->alpha; ++u) qmax = std::max(qmax, c->q[c->L + u]);
-  if (qmax > ~0ull / nrot) return false;
   const uint32_t beta = (level + (uint32_t)c->alpha - 1) / (uint32_t)c->alpha;
   size_t smem = 0;
   switch (c->log_n) {
@@ -65,43 +52,39 @@ bool ks_rot_fits(const he_ctx* c, uint32_t level, uint32_t nrot) {
 }
 
 // ModUp -> NTT -> the summed inner products of every rotation of a hoisted
-// rotate-and-sum, fused, into one accumulator; *unreduced when it holds sums
-// of rs.n residues (the rotations moved rows between CTAs).
+// rotate-and-sum into one accumulator; *c0_added when part 0 (c0) is in it.
 int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c, uint64_t* ext, uint64_t* acc,
-           const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled, bool* unreduced,
-           uint64_t in_gal, const uint64_t* c0, uint64_t c0_stride, bool* c0_added) {
+           const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled, uint64_t in_gal,
+           const uint64_t* c0, uint64_t c0_stride, bool* c0_added) {
   *handled = false;
-  *unreduced = false;
+  bool added = false;
   if (c0_added) *c0_added = false;
-  if (!ks_rot_fits(c, level, rs.n)) return HE_OK;
+  if (!ks_rot_fits(c, level)) return HE_OK;
   KsRotArgs ra;
   ra.k = ks_args(c, d, d_stride, d2c, ext, acc, nullptr, level, in_gal, half);
   ra.nrot = rs.n;
   ra.count = count;
   ra.c0 = c0;
   ra.c0_stride = c0_stride;
-  // the summed path adds nrot * beta products below q^2 in 128 bits (the
-  // other path beta of them)
+  // the kernels add nrot * beta products below q^2 in 128 bits
   uint32_t bits = 0;
   for (uint32_t t = 0; t < level; ++t) bits = std::max(bits, (uint32_t)(64 - __builtin_clzll(c->q[t])));
   for (uint32_t u = 0; u < (uint32_t)c->alpha; ++u) bits = std::max(bits, (uint32_t)(64 - __builtin_clzll(c->q[c->L + u])));
   const uint32_t nprod = rs.n * ((level + (uint32_t)c->alpha - 1) / (uint32_t)c->alpha);
-  ra.closed = 2 * bits + (32 - __builtin_clz(nprod)) <= 128 ? 1 : 0;
+  ra.reduce_each = 2 * bits + (32 - __builtin_clz(nprod)) <= 128 ? 0 : 1;
   for (uint32_t r = 0; r < rs.n; ++r) {
     ra.gal[r] = rs.gal[r];
-    ra.gal_inv[r] = gal_inverse(rs.gal[r], c->log_n);
     ra.evk[r] = rs.evk[r];
   }
-  int closed = 0, rc;
+  int rc;
   switch (c->log_n) {
-    case 12: rc = ks_rot_n12(c, ra, count, handled, &closed); break;
-    case 13: rc = ks_rot_n13(c, ra, count, handled, &closed); break;
-    case 14: rc = ks_rot_n14(c, ra, count, handled, &closed); break;
-    case 15: rc = ks_rot_n15(c, ra, count, handled, &closed); break;
-    default: rc = ks_rot_n16(c, ra, count, handled, &closed); break;
+    case 12: rc = ks_rot_n12(c, ra, count, handled, &added); break;
+    case 13: rc = ks_rot_n13(c, ra, count, handled, &added); break;
+    case 14: rc = ks_rot_n14(c, ra, count, handled, &added); break;
+    case 15: rc = ks_rot_n15(c, ra, count, handled, &added); break;
+    default: rc = ks_rot_n16(c, ra, count, handled, &added); break;
   }
-  *unreduced = *handled && !(closed & 1);
-  if (c0_added) *c0_added = *handled && (closed & 2);
+  if (c0_added) *c0_added = *handled && added;
   return rc;
 }
 

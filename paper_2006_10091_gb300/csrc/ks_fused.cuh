@@ -243,23 +243,21 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
 // with a permutation of the evaluation points that maps rows to rows: in
 // bit-reversed order a row of M points is a residue class of the natural
 // index modulo N/M, and X -> X^gal maps residue classes onto residue
-// classes.  So the CTA that holds input row c after the row pass can write
-// the whole of output row c' = src_{gal^-1}(c M) / M with coalesced stores and
-// key loads, reading its sources from shared memory.  When every rotation
-// maps each CTA's rows onto themselves, a thread sums all rotations for its
-// own positions; otherwise each rotation's row is added atomically to the
-// one accumulator (64-bit sums of at most 16 residues below 2^60).
+// classes.  When every rotation maps each CTA's rows onto themselves (a
+// closed stage), ks_row_rot runs the row pass and sums all rotations for its
+// own positions from the tiles it holds in shared memory; otherwise the row
+// pass runs by itself and ks_gather_rot fetches the rows each rotation reads.
 struct KsRotArgs {
   KsFusedArgs k;           // k.acc: the accumulator (summed over the rotations)
   uint32_t nrot, count;
-  int closed;              // every rotation maps each tile's rows onto themselves
-  uint64_t gal[HE_MAX_ROT], gal_inv[HE_MAX_ROT];
+  int reduce_each;         // nrot * beta products could exceed 128 bits: reduce after each rotation
+  uint64_t gal[HE_MAX_ROT];
   const uint64_t* evk[HE_MAX_ROT];
   // part 0 of the input (evaluation form, count x [level][N] at c0_stride):
   // when set, part 0 of the accumulator's limbs q_t also receives
   // (P mod q_t) * sum_r kappa_r(c0), which the ModDown turns into
-  // sum_r kappa_r(c0) exactly (nullptr: not added; closed stages whose
-  // target limbs q_t all take the split sums only)
+  // sum_r kappa_r(c0) exactly (nullptr: not added; in ks_row_rot only where
+  // the target limbs q_t all take the split sums)
   const uint64_t* c0;
   uint64_t c0_stride;
 };
@@ -375,7 +373,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   // key products as split sums (mac_split3) when the prime and the number of
   // summed terms allow it
   const uint32_t sb = (pr.k + 1) >> 1;
-  if (ra.closed && 2 * sb + 2 + (32 - __clz(ra.nrot * a.beta)) <= 64) {
+  if (2 * sb + 2 + (32 - __clz(ra.nrot * a.beta)) <= 64) {
     // one pair of neighbouring positions per pass, all CT ciphertexts with
     // each key load
     constexpr int PPT = PER / 2 / CT;
@@ -451,7 +449,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
     }
     return;
   }
-  if (ra.closed) {
+  {
     // each thread sums every rotation's products for its own positions, two
     // neighbouring positions at a time (16-byte key loads and stores), for
     // all CT ciphertexts with each key load
@@ -516,52 +514,187 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
         }
       }
     }
-    return;
   }
-  if constexpr (CT == 1) {  // rotations that move rows between CTAs (launched with one ciphertext per CTA)
-    constexpr int GRP = PER / 2;  // residues per thread and pass (bounds the registers)
-    for (uint32_t r = 0; r < ra.nrot; ++r) {
-      const uint64_t* ev = ra.evk[r];
-      uint64_t* o0 = a.acc + ((size_t)i * 2 * a.nt + t) * N;
-      uint64_t* o1 = o0 + (size_t)a.nt * N;
+}
+
+// Stages with rotations that move rows between tiles: the row pass runs
+// by itself (ntt2's, in place on the column pass's outputs) and this kernel
+// gathers.  A CTA of target limb t owns one tile of output positions and CT
+// ciphertexts.  Step (r, j) needs the rows of digit j that rotation r moves to
+// the tile (whole rows, see above) of each ciphertext and the key's two
+// polynomials at the tile; a ring of kGatherRing steps is kept in flight with
+// cp.async, since a step computes for about 0.3 us and its key words come from
+// HBM.  A thread sums one pair of neighbouring positions, like the closed
+// stages; each accumulator residue is reduced and written once.  Part 0 (ra.c0)
+// is one more step per rotation.  Bound by its instructions (FMA pipe 53 %,
+// issue slots half used, DRAM 28 %).  Fifteen unit steps at N = 2^16, 24 limbs,
+// four ciphertexts: 1.68 ms, and 0.34 ms for the row pass (every rotation's
+// reduced products added to the rows they move to with 64-bit atomics: 2.84 ms;
+// a rotation's digits per step and keys read by the products: 2.79 ms).
+// Grid: nt * ceil(count / CT) * TILES (as ks_row_rot).
+constexpr int kGatherThreads = 512, kGatherRing = 6;
+
+template <int LOG_N, int LOG_M, int LOG_K, int CT>
+__global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra) {
+  using S = Shape<LOG_N, LOG_M, LOG_K, false>;
+  constexpr uint32_t N = 1u << LOG_N, SLOT = (CT + 2) * S::TILE;
+  static_assert(S::TILE == 2 * kGatherThreads, "one pair of positions per thread");
+  const KsFusedArgs& a = ra.k;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);  // [ring][CT digit tiles, key b, key a][TILE]
+  uint32_t b = blockIdx.x;
+  const uint32_t tile = b % S::TILES;
+  b /= S::TILES;
+  const uint32_t ngrp = (ra.count + CT - 1) / CT;
+  const uint32_t i0 = (b % ngrp) * CT, t = b / ngrp;
+  const uint32_t prime = ks_prime(t, a.level, a.L);
+  const PrimeDev pr = a.primes[prime];
+  const bool add_c0 = ra.c0 && t < a.level;
+  const uint32_t ntile = a.beta + (add_c0 ? 1 : 0), nsteps = ra.nrot * ntile;
+  const uint32_t idx = 2 * threadIdx.x, kx = idx >> LOG_M;
+  const uint32_t eo = S::gidx(tile, kx, idx & (S::M - 1));
+  // where digit j's row starts: the digit's converted limb (one digit is nt
+  // limbs apart from the next), the input's own limb in digit jo, part 0
+  const uint64_t *ext[CT], *own[CT], *c0[CT];
+#pragma unroll
+  for (int c = 0; c < CT; ++c) {
+    const uint32_t i = min(i0 + c, ra.count - 1);
+    ext[c] = a.ext + ((size_t)i * a.beta * a.nt + t) * N;
+    own[c] = a.d + (size_t)i * a.d_stride + (size_t)t * N;
+    c0[c] = add_c0 ? ra.c0 + (size_t)i * ra.c0_stride + (size_t)t * N : nullptr;
+  }
+  const uint32_t to0 = (uint32_t)__cvta_generic_to_shared(buf + idx);
+  uint32_t jo = a.beta;  // (none)
+  for (uint32_t j = 0; j < a.beta; ++j)
+    if (t >= a.lo[j] && t < a.lo[j] + a.cnt[j]) jo = j;
+  const uint32_t ext_step = a.nt * N, key_step = a.np * N;  // 2 beta np N < 2^32
+  const uint32_t row = eo & ~(uint32_t)(S::M - 1), x = idx & (S::M - 1);
+  uint32_t cr = 0, cj = 0;  // the next step to copy
+  uint32_t off = 0, ko = 0, eoff = 0;
+  const uint64_t* key = nullptr;
+  auto next_rotation = [&]() {
+    off = (automorph_src(row, ra.gal[cr], LOG_N) & ~(uint32_t)(S::M - 1)) | x;
+    key = ra.evk[cr];
+    ko = prime * N + eo;
+    eoff = off;
+  };
+  next_rotation();
+  auto copy_step = [&](uint32_t slot) {
+    if (cr < ra.nrot) {
+      const uint32_t to = to0 + 8 * slot * SLOT;
+      if (cj < a.beta) {
+        if (cj == jo)
+#pragma unroll
+          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, own[c] + off);
+        else
+#pragma unroll
+          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, ext[c] + eoff);
+        cp_async16_s(to + 8 * CT * S::TILE, key + ko);
+        cp_async16_s(to + 8 * (CT + 1) * S::TILE, key + (ko + key_step));
+        ko += 2 * key_step;
+        eoff += ext_step;
+      } else {
+#pragma unroll
+        for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, c0[c] + off);
+      }
+      if (++cj == ntile) {
+        cj = 0;
+        if (++cr < ra.nrot) next_rotation();
+      }
+    }
+    cp_async_commit();  // (an empty group past the last step keeps the count)
+  };
+  const uint32_t sb = (pr.k + 1) >> 1, mask = (1u << (sb & 31)) - 1;
+  const bool split = 2 * sb + 2 + (32 - __clz(ra.nrot * a.beta)) <= 64;
+  // split sums (ll, hh, ss), or 128-bit sums (ll = low word, hh = high word)
+  uint64_t ll[CT][2][2], hh[CT][2][2], ss[CT][2][2], s0[CT][2];  // [ciphertext][part][position]
+#pragma unroll
+  for (int c = 0; c < CT; ++c) {
+    s0[c][0] = s0[c][1] = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int u = 0; u < 2; ++u) ll[c][p][u] = hh[c][p][u] = ss[c][p][u] = 0;
+  }
 #pragma unroll 1
-      for (int u0 = 0; u0 < PER; u0 += GRP) {
-        uint32_t so[GRP], eo[GRP];
+  for (uint32_t s = 0; s < kGatherRing - 1; ++s) copy_step(s);
+  uint32_t slot = 0;
+  for (uint32_t r = 0; r < ra.nrot; ++r) {
+    // the sources of two neighbouring positions are neighbours (their exponents
+    // differ by N, and gal is odd): one 16-byte load, its words swapped or not
+    const uint32_t sp0 = (kx << LOG_M) | (automorph_src(eo, ra.gal[r], LOG_N) & (S::M - 1));
+    const uint32_t sp = sp0 & ~1u;
+    const bool sw = sp0 & 1;
+    for (uint32_t j = 0; j < ntile; ++j) {
+      cp_async_wait<kGatherRing - 2>();  // this step's group has arrived
+      __syncthreads();                   // for every thread; and the slot before it is free
+      copy_step(slot == 0 ? kGatherRing - 1 : slot - 1);
+      const uint64_t* sm = buf + slot * SLOT;
+      slot = slot + 1 == kGatherRing ? 0 : slot + 1;
+      if (j == a.beta) {
 #pragma unroll
-        for (int u = 0; u < GRP; ++u) {
-          const uint32_t idx = threadIdx.x + (u0 + u) * S::T;
-          const uint32_t k = idx >> LOG_M, x = idx & (S::M - 1);
-          const uint32_t row = row0 + k;
-          const uint32_t orow = automorph_src(row << LOG_M, ra.gal_inv[r], LOG_N) >> LOG_M;
-          const uint32_t e = (orow << LOG_M) | x;
-          const uint32_t sl = (k << LOG_M) | (automorph_src(e, ra.gal[r], LOG_N) & (S::M - 1));
-          so[u] = sl + (sl >> 3);
-          eo[u] = e;
+        for (int c = 0; c < CT; ++c) {
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          s0[c][0] += sw ? xv.y : xv.x;
+          s0[c][1] += sw ? xv.x : xv.y;
         }
-        uint64_t a0l[GRP], a0h[GRP], a1l[GRP], a1h[GRP];  // 128-bit sums of full products
+        continue;
+      }
+      const ulonglong2 wb = *reinterpret_cast<const ulonglong2*>(sm + CT * S::TILE + idx);
+      const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(sm + (CT + 1) * S::TILE + idx);
+      if (split) {
+        const Split3 kb0 = split3(wb.x, sb, mask), kb1 = split3(wb.y, sb, mask);
+        const Split3 ka0 = split3(wa.x, sb, mask), ka1 = split3(wa.y, sb, mask);
 #pragma unroll
-        for (int u = 0; u < GRP; ++u) a0l[u] = a0h[u] = a1l[u] = a1h[u] = 0;
-        for (uint32_t j = 0; j < a.beta; ++j) {
-          const uint64_t* sm = dig + (size_t)j * TW;
-          const uint64_t* kb = ev + (((size_t)j * 2 + 0) * a.np + prime) * N;
-          const uint64_t* ka = ev + (((size_t)j * 2 + 1) * a.np + prime) * N;
-#pragma unroll
-          for (int u = 0; u < GRP; ++u) {
-            const uint64_t x = sm[so[u]];
-            mac128(a0l[u], a0h[u], x, __ldg(kb + eo[u]));
-            mac128(a1l[u], a1h[u], x, __ldg(ka + eo[u]));
-          }
+        for (int c = 0; c < CT; ++c) {
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          const Split3 x0 = split3(sw ? xv.y : xv.x, sb, mask), x1 = split3(sw ? xv.x : xv.y, sb, mask);
+          mac_split3(ll[c][0][0], hh[c][0][0], ss[c][0][0], x0, kb0);
+          mac_split3(ll[c][0][1], hh[c][0][1], ss[c][0][1], x1, kb1);
+          mac_split3(ll[c][1][0], hh[c][1][0], ss[c][1][0], x0, ka0);
+          mac_split3(ll[c][1][1], hh[c][1][1], ss[c][1][1], x1, ka1);
         }
-        // other CTAs add the other rotations' products to these rows: the
-        // accumulator (zeroed first) holds sums of nrot residues
+      } else {
 #pragma unroll
-        for (int u = 0; u < GRP; ++u) {
-          atomicAdd(reinterpret_cast<unsigned long long*>(o0 + eo[u]),
-                    (unsigned long long)reduce128_any(a0h[u], a0l[u], pr));
-          atomicAdd(reinterpret_cast<unsigned long long*>(o1 + eo[u]),
-                    (unsigned long long)reduce128_any(a1h[u], a1l[u], pr));
+        for (int c = 0; c < CT; ++c) {
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          const uint64_t x0 = sw ? xv.y : xv.x, x1 = sw ? xv.x : xv.y;
+          mac128(ll[c][0][0], hh[c][0][0], x0, wb.x);
+          mac128(ll[c][0][1], hh[c][0][1], x1, wb.y);
+          mac128(ll[c][1][0], hh[c][1][0], x0, wa.x);
+          mac128(ll[c][1][1], hh[c][1][1], x1, wa.y);
         }
       }
+    }
+    if (!split && ra.reduce_each)  // nrot * beta products could leave 128 bits: beta at a time
+#pragma unroll
+      for (int c = 0; c < CT; ++c)
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            ll[c][p][u] = reduce128_any(hh[c][p][u], ll[c][p][u], pr);
+            hh[c][p][u] = 0;
+          }
+  }
+  uint64_t pm = 1;  // P mod q_t
+  if (add_c0)
+    for (uint32_t u = 0; u < a.alpha; ++u) pm = mul_mod(pm, reduce64(a.primes[a.L + u].q, pr), pr);
+#pragma unroll
+  for (int c = 0; c < CT; ++c) {
+    if (i0 + c >= ra.count) break;
+    uint64_t* o = a.acc + ((size_t)(i0 + c) * 2 * a.nt + t) * N + eo;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      uint64_t r2[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        uint64_t lo = ll[c][p][u], hi = hh[c][p][u];
+        if (split) split3_total(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, lo, hi);
+        if (p == 0 && add_c0) mac128(lo, hi, reduce64(s0[c][u], pr), pm);
+        r2[u] = reduce128_any(hi, lo, pr);
+      }
+      *reinterpret_cast<ulonglong2*>(o + (size_t)p * a.nt * N) = make_ulonglong2(r2[0], r2[1]);
     }
   }
 }
@@ -956,9 +1089,6 @@ size_t ks_rot_smem(uint32_t beta, uint32_t ct = 1, bool c0 = false) {
 
 
 
-// The hoisted rotate-and-sum's ModUp, column pass and row pass with the
-// inner products of every rotation.  *handled = false (nothing launched)
-// when the digits' tiles do not fit in shared memory.
 inline uint32_t brev_host(uint32_t x, int bits) {
   uint32_t r = 0;
   for (int i = 0; i < bits; ++i) r |= ((x >> i) & 1u) << (bits - 1 - i);
@@ -968,92 +1098,120 @@ inline uint32_t brev_host(uint32_t x, int bits) {
 // Whether X -> X^gal maps every row tile of the hoisted row pass (2^LOG_K
 // rows of 2^LOG_M evaluation points) onto itself.
 template <int LOG_N, int LOG_M, int LOG_K>
-bool rot_closed(uint64_t gal_inv) {
+bool rot_closed(uint64_t gal) {
   for (uint32_t row = 0; row < (1u << (LOG_N - LOG_M)); ++row) {
     const uint32_t e = 2 * brev_host(row << LOG_M, LOG_N) + 1;
-    const uint32_t e2 = (uint32_t)(((uint64_t)e * gal_inv) & ((2ull << LOG_N) - 1));
-    const uint32_t orow = brev_host((e2 - 1) >> 1, LOG_N) >> LOG_M;
-    if ((orow >> LOG_K) != (row >> LOG_K)) return false;
+    const uint32_t e2 = (uint32_t)(((uint64_t)e * gal) & ((2ull << LOG_N) - 1));
+    const uint32_t srow = brev_host((e2 - 1) >> 1, LOG_N) >> LOG_M;
+    if ((srow >> LOG_K) != (row >> LOG_K)) return false;
   }
   return true;
 }
 
+int ntt2_forward_rows(he_ctx* c, const PolyBatch& b);
+
+// The hoisted rotate-and-sum's ModUp, column pass, row pass and the inner
+// products of every rotation.  *handled = false (nothing launched) when the
+// digits' tiles do not fit in shared memory; *c0_added: part 0 of the input
+// is in the accumulator.
 template <int LOG_N, int M1, int K1, int M2, int K2>
-int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, int* closed_out) {
+int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bool* c0_added) {
   using SR = Shape<LOG_N, M2, K2 - 1, false>;
   const KsFusedArgs& a = ra.k;
   const size_t smr = ks_rot_smem<LOG_N, M2, K2>(a.beta);
   *handled = smr <= kRotSmemMax;
   if (!*handled) return HE_OK;
-  static std::atomic<unsigned long long> attr1{0}, attr2{0}, attr4{0};
+  static std::atomic<unsigned long long> attr1{0}, attr2{0}, attr4{0}, attr_g1{0}, attr_g2{0};
   HE_TRY(set_smem_attr_once(attr1, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr2, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 2>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr4, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 4>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr_g1, c->device, (const void*)ks_gather_rot<LOG_N, M2, K2 - 1, 1>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr_g2, c->device, (const void*)ks_gather_rot<LOG_N, M2, K2 - 1, 2>, kRotSmemMax));
   HE_TRY((ks_modup_launch<LOG_N, M1, K1>(c, a, count)));
   const double n = (double)(1u << LOG_N);
   double own = 0;
   for (uint32_t j = 0; j < a.beta; ++j) own += a.cnt[j];
   const double conv = (double)a.beta * a.nt - own;
-  {
-    KsRotArgs rc = ra;
-    rc.count = count;
-    rc.closed = ra.closed;  // 0 when the summed products could exceed 128 bits
-    for (uint32_t r = 0; r < ra.nrot; ++r) rc.closed &= rot_closed<LOG_N, M2, K2 - 1>(ra.gal_inv[r]) ? 1 : 0;
-    // work: the converted limbs' row-pass butterflies, one reduction per
-    // accumulator residue, and the key products (split sums on the target
-    // limbs whose primes allow them in a closed stage, as the kernel decides;
-    // 128-bit multiply-accumulates on the others); bytes: the limbs read once,
-    // one accumulator written (the rotations' products are summed into it),
-    // each rotation's key read once per launch
-    const uint32_t terms_bits = 32 - __builtin_clz(ra.nrot * a.beta);
-    double split_limbs = 0, split_q = 0;
-    for (uint32_t t = 0; t < a.nt && rc.closed; ++t) {
-      const uint32_t k = 64 - __builtin_clzll(c->q[ks_prime(t, a.level, a.L)]), sb = (k + 1) / 2;
-      if (2 * sb + 2 + terms_bits <= 64) {
-        split_limbs += 1;
-        split_q += t < a.level ? 1 : 0;
-      }
-    }
-    // part 0 through the rotations: in closed stages whose limbs q_t all take
-    // the split sums, when its tile fits beside the digits'
-    if (!rc.closed || split_q < a.level || ks_rot_smem<LOG_N, M2, K2>(a.beta, 1, true) > kRotSmemMax)
-      rc.c0 = nullptr;
-    const bool c0 = rc.c0 != nullptr;
-    *closed_out = rc.closed | (c0 ? 2 : 0);
-    const double per_limb = count * 2.0 * ra.nrot * a.beta * n;
-    const double macs = per_limb * (a.nt - split_limbs), mac3 = per_limb * split_limbs;
-    // (with part 0: nrot additions and one 128-bit product per residue of its limbs, and those limbs read)
-    const double c0_work = c0 ? count * (double)a.level * n : 0.0;
-    ProfScope prof(c, "ks_ntt_rot_products", count * (conv * n / 2 * M2 + 2.0 * a.nt * n) + macs + mac3 + c0_work,
-                   count * n * 8 * (conv + own + 2.0 * a.nt + (c0 ? a.level : 0)) +
-                       8.0 * n * ra.nrot * a.beta * 2.0 * a.nt,
-                   macs + c0_work, count * conv * n / 2 * M2, mac3);
-    if (!rc.closed)
-      HE_CUDA(cudaMemsetAsync(ra.k.acc, 0, sizeof(uint64_t) * count * 2 * a.nt * (1u << LOG_N), c->stream));
-    // ciphertexts per CTA (closed stages only): the knob, else 2 when that
-    // keeps as many warps resident per SM as 1 does (a 15-rotation stage of
-    // 512 ciphertexts at N = 2^14, 16 warps either way: 9.3 ms against 10.1 ms
-    // for 1 and 10.0 ms for 4; six digits at N = 2^16 would fall from 12 to 8
-    // warps, slower)
-    uint32_t ct = 1;
-    if (rc.closed) {
-      auto warps = [&](uint32_t k) {  // resident warps per SM with k ciphertexts per CTA
-        const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, k, c0) + 1024;  // + the runtime's reserve per CTA
-        const size_t by_smem = c->smem_per_sm / sm, by_regs = 4 / k;
-        return std::min(by_smem, by_regs) * k * (size_t)SR::T / 32;
-      };
-      const uint32_t want = c->ks_ct ? (uint32_t)c->ks_ct : 2u;
-      for (uint32_t cand : {4u, 2u})
-        if (ct == 1 && cand <= want && cand <= count && ks_rot_smem<LOG_N, M2, K2>(a.beta, cand, c0) <= kRotSmemMax &&
-            (c->ks_ct || warps(cand) >= warps(1)))
-          ct = cand;
-    }
-    const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
-    const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, ct, c0);
-    if (ct == 4) ks_row_rot<LOG_N, M2, K2 - 1, 4><<<(unsigned)blocks, 4 * SR::T, sm, c->stream>>>(rc);
-    else if (ct == 2) ks_row_rot<LOG_N, M2, K2 - 1, 2><<<(unsigned)blocks, 2 * SR::T, sm, c->stream>>>(rc);
-    else ks_row_rot<LOG_N, M2, K2 - 1, 1><<<(unsigned)blocks, SR::T, sm, c->stream>>>(rc);
+  KsRotArgs rc = ra;
+  rc.count = count;
+  bool closed = !ra.reduce_each;
+  for (uint32_t r = 0; r < ra.nrot && closed; ++r) closed = rot_closed<LOG_N, M2, K2 - 1>(ra.gal[r]);
+  if (!closed) {  // the row pass by itself, in place (own limbs are read from the input)
+    PolyBatch e;
+    e.src = a.ext;
+    e.dst = a.ext;
+    e.src_stride = e.dst_stride = (uint64_t)a.nt << LOG_N;
+    e.npolys = count * a.beta;
+    e.nl = a.nt;
+    e.limb0 = 0;
+    e.level = a.level;
+    e.skip_alpha = a.alpha;
+    e.skip_beta = a.beta;
+    HE_TRY(ntt2_forward_rows(c, e));
   }
+  // work: the converted limbs' row-pass butterflies (closed stages), one
+  // reduction per accumulator residue, and the key products (split sums on the
+  // target limbs whose primes allow them, as the kernels decide; 128-bit
+  // multiply-accumulates on the others); bytes: the limbs read once, one
+  // accumulator written (the rotations' products are summed into it), each
+  // rotation's key read once per launch
+  const uint32_t terms_bits = 32 - __builtin_clz(ra.nrot * a.beta);
+  double split_limbs = 0;
+  uint32_t split_q = 0, qbits = 0;
+  for (uint32_t t = 0; t < a.nt; ++t) {
+    const uint32_t k = 64 - __builtin_clzll(c->q[ks_prime(t, a.level, a.L)]), sb = (k + 1) / 2;
+    if (t < a.level) qbits = std::max(qbits, k);
+    if (2 * sb + 2 + terms_bits <= 64) {
+      split_limbs += 1;
+      split_q += t < a.level ? 1 : 0;
+    }
+  }
+  // part 0 through the rotations: in closed stages whose limbs q_t all take
+  // the split sums, when its tile fits beside the digits'; in the others
+  // unless nrot residues could exceed 64 bits
+  if (closed ? split_q < a.level || ks_rot_smem<LOG_N, M2, K2>(a.beta, 1, true) > kRotSmemMax
+             : qbits + (32 - __builtin_clz(ra.nrot)) > 64)
+    rc.c0 = nullptr;
+  const bool c0 = rc.c0 != nullptr;
+  *c0_added = c0;
+  const double per_limb = count * 2.0 * ra.nrot * a.beta * n;
+  const double macs = per_limb * (a.nt - split_limbs), mac3 = per_limb * split_limbs;
+  // (with part 0: nrot additions and one 128-bit product per residue of its limbs, and those limbs read)
+  const double c0_work = c0 ? count * (double)a.level * n : 0.0;
+  const double bfly = closed ? count * conv * n / 2 * M2 : 0.0;
+  ProfScope prof(c, "ks_ntt_rot_products", bfly + count * 2.0 * a.nt * n + macs + mac3 + c0_work,
+                 count * n * 8 * (conv + own + 2.0 * a.nt + (c0 ? a.level : 0)) +
+                     8.0 * n * ra.nrot * a.beta * 2.0 * a.nt,
+                 macs + c0_work, bfly, mac3);
+  if (!closed) {
+    const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words
+    const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
+    const size_t sm = kGatherRing * (ct + 2) * sizeof(uint64_t) * SR::TILE;
+    if (ct == 2) ks_gather_rot<LOG_N, M2, K2 - 1, 2><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
+    else ks_gather_rot<LOG_N, M2, K2 - 1, 1><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
+    HE_CUDA(cudaGetLastError());
+    return HE_OK;
+  }
+  // ciphertexts per CTA: the knob, else 2 when that keeps as many warps
+  // resident per SM as 1 does (a 15-rotation stage of 512 ciphertexts at N =
+  // 2^14, 16 warps either way: 9.3 ms against 10.1 ms for 1 and 10.0 ms for
+  // 4; six digits at N = 2^16 would fall from 12 to 8 warps, slower)
+  uint32_t ct = 1;
+  auto warps = [&](uint32_t k) {  // resident warps per SM with k ciphertexts per CTA
+    const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, k, c0) + 1024;  // + the runtime's reserve per CTA
+    const size_t by_smem = c->smem_per_sm / sm, by_regs = 4 / k;
+    return std::min(by_smem, by_regs) * k * (size_t)SR::T / 32;
+  };
+  const uint32_t want = c->ks_ct ? (uint32_t)c->ks_ct : 2u;
+  for (uint32_t cand : {4u, 2u})
+    if (ct == 1 && cand <= want && cand <= count && ks_rot_smem<LOG_N, M2, K2>(a.beta, cand, c0) <= kRotSmemMax &&
+        (c->ks_ct || warps(cand) >= warps(1)))
+      ct = cand;
+  const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
+  const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, ct, c0);
+  if (ct == 4) ks_row_rot<LOG_N, M2, K2 - 1, 4><<<(unsigned)blocks, 4 * SR::T, sm, c->stream>>>(rc);
+  else if (ct == 2) ks_row_rot<LOG_N, M2, K2 - 1, 2><<<(unsigned)blocks, 2 * SR::T, sm, c->stream>>>(rc);
+  else ks_row_rot<LOG_N, M2, K2 - 1, 1><<<(unsigned)blocks, SR::T, sm, c->stream>>>(rc);
   HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
@@ -1062,7 +1220,7 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, in
 // each, so that the template instances compile in parallel): the launches
 // for the tile shape c->ntt_shape.
 #define HE_KS_FUSED_DECL(NN)                                                         \
-  int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, int* closed); \
+  int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added); \
   size_t ks_rot_smem_n##NN(const he_ctx* c, uint32_t beta);                          \
   int md_fused_n##NN(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled);     \
   bool md_half_n##NN(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count); \

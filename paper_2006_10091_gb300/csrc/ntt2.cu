@@ -24,6 +24,17 @@ int ntt2_inverse_rows(he_ctx* c, const PolyBatch& b) {
   }
 }
 
+int ntt2_forward_rows(he_ctx* c, const PolyBatch& b) {
+  switch (c->log_n) {
+    case 12: return ntt2_fwd_rows_n12(c, b);
+    case 13: return ntt2_fwd_rows_n13(c, b);
+    case 14: return ntt2_fwd_rows_n14(c, b);
+    case 15: return ntt2_fwd_rows_n15(c, b);
+    case 16: return ntt2_fwd_rows_n16(c, b);
+    default: return fail(HE_EINVAL, "ntt2_forward_rows: no compiled shape");
+  }
+}
+
 int ntt2(he_ctx* c, const PolyBatch& b, bool inv, bool* handled) {
   *handled = true;
   switch (c->log_n) {

@@ -174,11 +174,20 @@ int run2_inv_rows(he_ctx* c, const PolyBatch& b) {
   return launch2<true, LOG_N, M2, K2, false, LOG_V>(c, b, b.src, b.dst, b.src_stride, false, b.gal);
 }
 
+// Only the last pass (the row pass) of the forward transform, on a column
+// pass's outputs: the stages whose key products gather rows from memory.
+template <int LOG_N, int M1, int K1, int M2, int K2, int LOG_V = 3>
+int run2_fwd_rows(he_ctx* c, const PolyBatch& b) {
+  return launch2<false, LOG_N, M2, K2, false, LOG_V>(c, b, b.src, b.dst, b.src_stride, true);
+}
+
 // Per ring size (ntt2_n12.cu .. ntt2_n16.cu, compiled in parallel): both
-// passes, or the inverse's first pass only, for the tile shape c->ntt_shape.
+// passes, the inverse's first pass or the forward's last one only, for the
+// tile shape c->ntt_shape.
 #define HE_NTT2_DECL(NN)                                          \
   int ntt2_n##NN(he_ctx* c, const PolyBatch& b, bool inv);          \
-  int ntt2_inv_rows_n##NN(he_ctx* c, const PolyBatch& b);
+  int ntt2_inv_rows_n##NN(he_ctx* c, const PolyBatch& b);           \
+  int ntt2_fwd_rows_n##NN(he_ctx* c, const PolyBatch& b);
 HE_NTT2_DECL(12)
 HE_NTT2_DECL(13)
 HE_NTT2_DECL(14)

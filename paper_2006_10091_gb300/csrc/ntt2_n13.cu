@@ -14,4 +14,10 @@ int ntt2_inv_rows_n13(he_ctx* c, const PolyBatch& b) {
                                                    : run2_inv_rows<13, 7, 4, 6, 5>(c, b);
 }
 
+int ntt2_fwd_rows_n13(he_ctx* c, const PolyBatch& b) {
+  const int sh = c->ntt_shape;
+  return sh == 1 ? run2_fwd_rows<13, 6, 5, 7, 4>(c, b) : sh == 2 ? run2_fwd_rows<13, 4, 7, 9, 2>(c, b)
+                                                   : run2_fwd_rows<13, 7, 4, 6, 5>(c, b);
+}
+
 }  // namespace he

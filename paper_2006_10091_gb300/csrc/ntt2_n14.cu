@@ -14,4 +14,10 @@ int ntt2_inv_rows_n14(he_ctx* c, const PolyBatch& b) {
        : sh == 2 ? run2_inv_rows<14, 8, 3, 6, 5>(c, b) : run2_inv_rows<14, 5, 6, 9, 2>(c, b);
 }
 
+int ntt2_fwd_rows_n14(he_ctx* c, const PolyBatch& b) {
+  const int sh = c->ntt_shape;
+  return sh == 1 ? run2_fwd_rows<14, 7, 4, 7, 4>(c, b)
+       : sh == 2 ? run2_fwd_rows<14, 8, 3, 6, 5>(c, b) : run2_fwd_rows<14, 5, 6, 9, 2>(c, b);
+}
+
 }  // namespace he

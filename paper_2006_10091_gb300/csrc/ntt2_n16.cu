@@ -14,4 +14,10 @@ int ntt2_inv_rows_n16(he_ctx* c, const PolyBatch& b) {
        : sh == 2 ? run2_inv_rows<16, 7, 4, 9, 2>(c, b) : run2_inv_rows<16, 6, 5, 10, 1>(c, b);
 }
 
+int ntt2_fwd_rows_n16(he_ctx* c, const PolyBatch& b) {
+  const int sh = c->ntt_shape;
+  return sh == 1 ? run2_fwd_rows<16, 8, 4, 8, 3>(c, b)
+       : sh == 2 ? run2_fwd_rows<16, 7, 4, 9, 2>(c, b) : run2_fwd_rows<16, 6, 5, 10, 1>(c, b);
+}
+
 }  // namespace he

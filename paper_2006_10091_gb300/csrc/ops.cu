@@ -24,9 +24,9 @@ int md_fused(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t* conv
              uint64_t add_gal, CtBatch out, uint32_t level, uint32_t count, bool half, bool* handled);
 int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatch out, uint32_t level,
              uint32_t count, bool half, bool* handled);
-bool ks_rot_fits(const he_ctx* c, uint32_t level, uint32_t nrot);
+bool ks_rot_fits(const he_ctx* c, uint32_t level);
 int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c, uint64_t* ext, uint64_t* acc,
-           const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled, bool* unreduced,
+           const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled,
            uint64_t in_gal = 0, const uint64_t* c0 = nullptr, uint64_t c0_stride = 0, bool* c0_added = nullptr);
 int md_fused_gals(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t* conv, CtBatch add, int add_mode,
                   const uint64_t* gals, uint32_t n_gal, CtBatch out, uint32_t level, uint32_t count, bool half,
@@ -177,7 +177,7 @@ int keyswitch_batch(he_ctx* c, const uint64_t* d, uint64_t d_stride, uint32_t le
   if (!d2c || !ext || !acc || !conv) return fail(HE_ENOMEM, "key switch scratch too small");
   // 1. coefficient form (when each digit is converted in one CTA, only the
   //    inverse transform's row pass here; the conversion kernel finishes it)
-  const bool fits = ks_rot_fits(c, level, 1);
+  const bool fits = ks_rot_fits(c, level);
   if (gal && !fits) return fail(HE_EINVAL, "keyswitch_batch: automorphism needs the fused kernels");
   const bool half = fits && ks_converts_per_digit(c, level, count);
   {
@@ -194,8 +194,7 @@ int keyswitch_batch(he_ctx* c, const uint64_t* d, uint64_t d_stride, uint32_t le
     rs.n = 1;
     rs.gal[0] = 1;
     rs.evk[0] = evk;
-    bool unreduced = false;
-    HE_TRY(ks_rot(c, d, d_stride, d2c, ext, acc, rs, level, count, half, &fused, &unreduced, gal));
+    HE_TRY(ks_rot(c, d, d_stride, d2c, ext, acc, rs, level, count, half, &fused, gal));
   }
   if (!fused) {
     if (half || gal) return fail(HE_ECUDA, "keyswitch_batch: fused kernels declined");
@@ -310,7 +309,7 @@ int rotate_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, uint64_t 
   const char* a_hi = a_lo + sizeof(uint64_t) * ((size_t)(count - 1) * A.stride + (size_t)2 * A.cap * n);
   const char* o_lo = (const char*)out.base;
   const char* o_hi = o_lo + sizeof(uint64_t) * ((size_t)(count - 1) * out.stride + (size_t)2 * out.cap * n);
-  if (ks_rot_fits(c, level, 1) && (o_hi <= a_lo || a_hi <= o_lo))
+  if (ks_rot_fits(c, level) && (o_hi <= a_lo || a_hi <= o_lo))
     return keyswitch_batch(c, A.base + (size_t)A.cap * n, A.stride, level, count, key, A, 1, out, ar, gal);
   uint64_t* t = ar.take<uint64_t>((size_t)count * 2 * level * n);
   if (!t) return fail(HE_ENOMEM, "rotation scratch too small");
@@ -354,7 +353,7 @@ int rotsum_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, const uin
   uint64_t* conv = ar.take<uint64_t>((size_t)count * 2 * level * n);
   if (!d2c || !ext || !acc || !conv) return fail(HE_ENOMEM, "rotate-and-sum scratch too small");
   const uint64_t* d = A.base + (size_t)A.cap * n;
-  const bool fits = ks_rot_fits(c, level, nrot);
+  const bool fits = ks_rot_fits(c, level);
   const bool half = fits && ks_converts_per_digit(c, level, count);
   {
     const PolyBatch b = pb(d, d2c, A.stride, (size_t)level * n, count, level, 0, level);
@@ -362,9 +361,9 @@ int rotsum_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, const uin
   }
   // the fused kernel also adds P sum_r kappa_r(A0) to the accumulator where it
   // can (c0_added): the ModDown then adds A0 and A1 as they are
-  bool fused = false, unreduced = false, c0_added = false;
+  bool fused = false, c0_added = false;
   if (fits)
-    HE_TRY(ks_rot(c, d, A.stride, d2c, ext, acc, rs, level, count, half, &fused, &unreduced, 0, A.base, A.stride,
+    HE_TRY(ks_rot(c, d, A.stride, d2c, ext, acc, rs, level, count, half, &fused, 0, A.base, A.stride,
                   &c0_added));
   if (!fused) {
     if (half) return fail(HE_ECUDA, "rotate-and-sum: fused kernels declined a half-transformed input");
@@ -376,12 +375,6 @@ int rotsum_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, const uin
           ext, (size_t)beta * nt * n, d, A.stride, rs, acc, acc_stride, level, alpha, beta, L, np, count, c->log_n,
           c->d_primes);
     }
-    HE_CUDA(cudaGetLastError());
-  }
-  if (unreduced) {  // sums of nrot residues from the rows the rotations moved between CTAs
-    ProfScope prof(c, "elementwise", 0.0, (double)count * 2 * nt * n * 16);
-    k_reduce_acc<<<grid_for((size_t)count * 2 * nt * n), 256, 0, c->stream>>>(acc, acc_stride, nt, level, L, count,
-                                                                              c->log_n, c->d_primes);
     HE_CUDA(cudaGetLastError());
   }
   // ModDown of the summed inner products, plus A0 + sum_r kappa_r(A0) and A1

@@ -45,3 +45,26 @@ def test_residues_do_not_depend_on_the_batch(log_n, limbs, bits, special, sbits,
             op(A[first:first + count], B[first:first + count], got)
             for i in range(count):
                 assert np.array_equal(got[i].residues(), want[first + i].residues()), (name, first, count, i)
+
+
+# stages that move rows between tiles (unit steps) and closed ones; 40-bit limbs (split sums), 58-bit limbs with 61-bit
+# special primes and 75 products per residue (128-bit sums reduced after each rotation); one ciphertext and an odd count
+@pytest.mark.parametrize("bits,special,sbits", [(40, 2, 59), (50, 4, 60), (58, 1, 61)])
+@pytest.mark.parametrize("first,nrot", [(1, 15), (-1, 3), (64, 15)])
+def test_rotation_stages_match_the_separate_kernels(bits, special, sbits, first, nrot):
+    import torch
+    import paper_2006_10091_gb300 as he
+    steps = [first * m for m in range(1, nrot + 1)]
+    ctx = he.Context(12, 5, bits, special, sbits, 2.0 ** 40, seed=6, rot_steps=steps)
+    for count in (1, 3):
+        A = uniform(ctx, torch, 5, count, 9)
+        want, got = ctx.new_ct(5, count), ctx.new_ct(5, count)
+        he.he_set_tuning(ctx, "ntt_generic", 1)
+        he.he_rotate_sum_batch(ctx, A, steps, want)
+        he.he_set_tuning(ctx, "ntt_generic", 0)
+        for shape in (0, 1, 2):
+            he.he_set_tuning(ctx, "ntt_shape", shape)
+            he.he_rotate_sum_batch(ctx, A, steps, got)
+            for i in range(count):
+                assert np.array_equal(got[i].residues(), want[i].residues()), (shape, i)
+        he.he_set_tuning(ctx, "ntt_shape", 0)
