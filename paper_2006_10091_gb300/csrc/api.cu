@@ -114,6 +114,8 @@ he_ctx* ctx_view(he_ctx* base, cudaStream_t stream) {
   v->d_itw = base->d_itw;
   v->d_two64 = base->d_two64;
   v->d_gauss = base->d_gauss;
+  v->d_fft = base->d_fft;
+  v->d_slot_of = base->d_slot_of;
   v->gK = base->gK;
   v->modup = base->modup;
   v->d_modup = base->d_modup;
@@ -161,6 +163,8 @@ static void destroy(he_ctx* c) {
   cudaFree(c->d_itw);
   cudaFree(c->d_two64);
   cudaFree(c->d_gauss);
+  cudaFree(c->d_fft);
+  cudaFree(c->d_slot_of);
   cudaFree(c->d_modup);
   cudaFree(c->d_moddown);
   cudaFree(c->d_rescale);

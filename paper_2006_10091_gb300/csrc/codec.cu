@@ -18,88 +18,170 @@
 
 namespace he {
 
-// ---- radix-2 complex FFT in double, one launch per stage ---------------------
-__global__ void k_bitrev_copy(const double2* in, double2* out, int log_n) {
-  const uint32_t n = 1u << log_n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    out[brev_bits(i, log_n)] = in[i];
-}
+// ---- radix-2 complex FFT in double, two launches -------------------------------
+// Decimation in time on the bit-reversed input: stage with half-size h pairs
+// (p, p + h) in blocks of 2h with the twiddle exp(sign i pi (p mod h) / h).
+// The first launch runs the stages inside contiguous blocks of 2^m1 points
+// (m1 = ceil(log2(N)/2)) and reads its input where it lies (the encoder's
+// slots through slot_of, the decoder's coefficients with their twist), the
+// second runs the rest on kFftCols neighbouring columns and writes the result
+// (rounded coefficients, or the slots' values).  A CTA holds few points, one
+// butterfly per thread and stage: the double-precision rate of an SM is low, so
+// the work is spread wide.  Twiddles come from the context's table (the same
+// values, computed once): N = 2^12 forward 69 us in 12 launches of one stage
+// each with sincospi per butterfly.
+constexpr int kFftCols = 2;
 
-// Stage with half-size h: pairs (i, i + h) in blocks of 2h, twiddle
-// exp(sign * i pi * (i mod h) / h); sign -1 gives the e^- DFT, +1 the e^+ one.
-__global__ void k_fft_stage(double2* a, int log_n, uint32_t h, double sign) {
-  const uint32_t n = 1u << log_n;
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n / 2; g += gridDim.x * blockDim.x) {
-    const uint32_t pos = g % h, blk = g / h;
-    const uint32_t i0 = blk * 2 * h + pos, i1 = i0 + h;
+// tab[i] = (cos, sin)(pi i / N); slot_of[u] = j for the point w^(2u+1) of slot j
+// (2u + 1 = 5^j mod 2N), -1 - j for its conjugate's.
+__global__ void k_codec_tables(double2* tab, int32_t* slot_of, int log_n) {
+  const uint32_t n = 1u << log_n, m = 2 * n;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double sn, cs;
-    sincospi(sign * (double)pos / (double)h, &sn, &cs);
-    const double2 x = a[i0], y = a[i1];
-    const double2 ty = make_double2(y.x * cs - y.y * sn, y.x * sn + y.y * cs);
-    a[i0] = make_double2(x.x + ty.x, x.y + ty.y);
-    a[i1] = make_double2(x.x - ty.x, x.y - ty.y);
+    sincospi((double)i / (double)n, &sn, &cs);
+    tab[i] = make_double2(cs, sn);
+    if (i < n / 2) {
+      uint32_t e = 1, b = 5, x = i;  // 5^i mod 2N by square-and-multiply
+      while (x) {
+        if (x & 1) e = (uint32_t)(((uint64_t)e * b) & (m - 1));
+        b = (uint32_t)(((uint64_t)b * b) & (m - 1));
+        x >>= 1;
+      }
+      slot_of[(e - 1) / 2] = (int32_t)i;
+      slot_of[(m - e - 1) / 2] = -1 - (int32_t)i;
+    }
   }
 }
 
-// out = DFT(in) with kernel exp(sign * 2 pi i jk / n), sign = +-1.
-static int fft(he_ctx* c, double2* in, double2* out, double sign) {
-  const int log_n = c->log_n;
-  const uint32_t n = c->n;
-  k_bitrev_copy<<<grid_for(n), 256, 0, c->stream>>>(in, out, log_n);
-  for (uint32_t h = 1; h < n; h <<= 1)
-    k_fft_stage<<<grid_for(n / 2), 256, 0, c->stream>>>(out, log_n, h, sign);
+int codec_tables(he_ctx* c) {
+  const size_t n = c->n;
+  HE_CUDA(cudaMalloc(&c->d_fft, sizeof(double2) * n));
+  HE_CUDA(cudaMalloc(&c->d_slot_of, sizeof(int32_t) * n));
+  k_codec_tables<<<grid_for(n), 256>>>((double2*)c->d_fft, c->d_slot_of, c->log_n);
   HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
-// W[u(e_j)] = z_j, W[u(2N - e_j)] = z_j (real slots), zero elsewhere.
-__global__ void k_encode_scatter(const double* z, uint32_t nz, double2* W, int log_n) {
-  const uint32_t n = 1u << log_n, m = 2 * n, nh = n / 2;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < nh; j += gridDim.x * blockDim.x) {
-    // e_j = 5^j mod 2N by square-and-multiply
-    uint32_t e = 1, b = 5, x = j;
-    while (x) {
-      if (x & 1) e = (uint32_t)(((uint64_t)e * b) & (m - 1));
-      b = (uint32_t)(((uint64_t)b * b) & (m - 1));
-      x >>= 1;
+struct FftArgs {
+  const double* in;      // slots (encode: nz of them) or coefficients (decode)
+  double2* mid;          // between the passes, N points
+  const double2* tab;
+  const int32_t* slot_of;
+  int64_t* coeffs;       // encode: the result
+  int* overflow;         // encode: set when a coefficient leaves int64
+  double* re;            // decode: the result (nz slots)
+  uint32_t nz;
+  double scale;
+  int log_n, m1;
+};
+
+// sign of the exponent: -1 encode, +1 decode
+template <bool ENC>
+__device__ __forceinline__ void fft_butterfly(double2* sm, uint32_t i0, uint32_t i1, double2 w) {
+  const double cs = w.x, sn = ENC ? -w.y : w.y;
+  const double2 x = sm[i0], y = sm[i1];
+  const double2 ty = make_double2(y.x * cs - y.y * sn, y.x * sn + y.y * cs);
+  sm[i0] = make_double2(x.x + ty.x, x.y + ty.y);
+  sm[i1] = make_double2(x.x - ty.x, x.y - ty.y);
+}
+
+// Stages h = 1 .. 2^(m1-1) on the block of 2^m1 points blockIdx.x.
+template <bool ENC>
+__global__ void k_fft_first(FftArgs a) {
+  extern __shared__ double2 fsm[];
+  const uint32_t m = 1u << a.m1, base = blockIdx.x << a.m1;
+  for (uint32_t x = threadIdx.x; x < m; x += blockDim.x) {
+    const uint32_t i = brev_bits(base | x, a.log_n);
+    if (ENC) {
+      const int32_t sl = a.slot_of[i];
+      const uint32_t j = (uint32_t)(sl < 0 ? -1 - sl : sl);
+      fsm[x] = make_double2(j < a.nz ? a.in[j] : 0.0, 0.0);
+    } else {
+      const double2 w = a.tab[i];
+      const double v = a.in[i];
+      fsm[x] = make_double2(v * w.x, v * w.y);
     }
-    const double v = j < nz ? z[j] : 0.0;
-    W[(e - 1) / 2] = make_double2(v, 0.0);
-    W[(m - e - 1) / 2] = make_double2(v, 0.0);
+  }
+  __syncthreads();
+  for (int s = 0; s < a.m1; ++s) {
+    const uint32_t h = 1u << s;
+    for (uint32_t g = threadIdx.x; g < m / 2; g += blockDim.x) {
+      const uint32_t pos = g & (h - 1), i0 = ((g >> s) << (s + 1)) | pos;
+      fft_butterfly<ENC>(fsm, i0, i0 + h, a.tab[pos << (a.log_n - s)]);
+    }
+    __syncthreads();
+  }
+  for (uint32_t x = threadIdx.x; x < m; x += blockDim.x) a.mid[base | x] = fsm[x];
+}
+
+// The remaining stages on columns [kFftCols blockIdx.x, ...): points x 2^m1 + f.
+template <bool ENC>
+__global__ void k_fft_second(FftArgs a) {
+  extern __shared__ double2 fsm[];
+  const uint32_t n = 1u << a.log_n;
+  const int m2 = a.log_n - a.m1;
+  const uint32_t pts = (uint32_t)kFftCols << m2, f0 = blockIdx.x * kFftCols;
+  for (uint32_t q = threadIdx.x; q < pts; q += blockDim.x)
+    fsm[q] = a.mid[((q / kFftCols) << a.m1) | (f0 + q % kFftCols)];
+  __syncthreads();
+  for (int s = 0; s < m2; ++s) {
+    const uint32_t h = 1u << s;
+    for (uint32_t g = threadIdx.x; g < pts / 2; g += blockDim.x) {
+      const uint32_t f = g % kFftCols, x = g / kFftCols, pos = x & (h - 1);
+      const uint32_t i0 = ((((x >> s) << (s + 1)) | pos) * kFftCols) + f;
+      const uint32_t gp = (pos << a.m1) | (f0 + f);  // position within the stage's block of 2^(m1+s+1)
+      fft_butterfly<ENC>(fsm, i0, i0 + h * kFftCols, a.tab[gp << (m2 - s)]);
+    }
+    __syncthreads();
+  }
+  for (uint32_t q = threadIdx.x; q < pts; q += blockDim.x) {
+    const uint32_t i = ((q / kFftCols) << a.m1) | (f0 + q % kFftCols);
+    const double2 v = fsm[q];
+    if (ENC) {
+      const double cs = a.tab[i].x, sn = -a.tab[i].y;  // w^-i
+      const double re = v.x * cs - v.y * sn;
+      const double raw = (a.scale / (double)n) * re;
+      if (!(fabs(raw) < 9.2e18)) {
+        *a.overflow = 1;
+        a.coeffs[i] = 0;
+      } else {
+        a.coeffs[i] = llround(raw);
+      }
+    } else {
+      const int32_t j = a.slot_of[i];
+      if (j >= 0 && (uint32_t)j < a.nz) a.re[j] = v.x / a.scale;
+    }
   }
 }
 
-__global__ void k_encode_finish(const double2* F, int64_t* out, double scale, int log_n, int* overflow) {
-  const uint32_t n = 1u << log_n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double sn, cs;
-    sincospi(-(double)i / (double)n, &sn, &cs);  // w^-i
-    const double re = F[i].x * cs - F[i].y * sn;
-    const double raw = (scale / (double)n) * re;
-    if (!(fabs(raw) < 9.2e18)) {
-      *overflow = 1;
-      out[i] = 0;
-    } else {
-      out[i] = llround(raw);
-    }
-  }
+template <bool ENC>
+static int fft_run(he_ctx* c, FftArgs a) {
+  a.log_n = c->log_n;
+  a.m1 = (c->log_n + 1) / 2;
+  a.tab = (const double2*)c->d_fft;
+  a.slot_of = c->d_slot_of;
+  const uint32_t p1 = 1u << a.m1, p2 = (uint32_t)kFftCols << (c->log_n - a.m1);
+  k_fft_first<ENC><<<c->n / p1, p1 / 2, sizeof(double2) * p1, c->stream>>>(a);
+  HE_CUDA(cudaGetLastError());
+  k_fft_second<ENC><<<c->n / p2, p2 / 2, sizeof(double2) * p2, c->stream>>>(a);
+  HE_CUDA(cudaGetLastError());
+  return HE_OK;
 }
 
 // Encode device slots d_z (n_slots doubles) into device int64 coefficients
-// d_out.  scratch: 2N double2; d_ovf: one int (set when a coefficient leaves int64).
+// d_out.  scratch: N double2; d_ovf: one int (set when a coefficient leaves int64).
 int encode_dev(he_ctx* c, const double* d_z, size_t n_slots, double scale, int64_t* d_out,
                double2* scratch, int* d_ovf) {
-  const uint32_t n = c->n;
-  if (n_slots > n / 2) return fail(HE_EINVAL, "more slots than N/2");
+  if (n_slots > (size_t)c->n / 2) return fail(HE_EINVAL, "more slots than N/2");
   if (!(scale > 0.0)) return fail(HE_EINVAL, "scale must be positive");
-  double2* W = scratch;
-  double2* F = scratch + n;
-  HE_CUDA(cudaMemsetAsync(W, 0, sizeof(double2) * n, c->stream));
-  k_encode_scatter<<<grid_for(n / 2), 256, 0, c->stream>>>(d_z, (uint32_t)n_slots, W, c->log_n);
-  HE_TRY(fft(c, W, F, -1.0));
-  k_encode_finish<<<grid_for(n), 256, 0, c->stream>>>(F, d_out, scale, c->log_n, d_ovf);
-  HE_CUDA(cudaGetLastError());
-  return HE_OK;
+  FftArgs a{};
+  a.in = d_z;
+  a.mid = scratch;
+  a.coeffs = d_out;
+  a.overflow = d_ovf;
+  a.nz = (uint32_t)n_slots;
+  a.scale = scale;
+  return fft_run<true>(c, a);
 }
 
 // ---- decryption -----------------------------------------------------------------
@@ -185,46 +267,18 @@ int decrypt_dev(he_ctx* c, const he_ct* ct, uint64_t* m, double* d_coeffs) {
   return HE_OK;
 }
 
-// W_i = m_i w^i (m as centered doubles), then G = e^+ DFT; slot j = G[u(e_j)] / scale.
-__global__ void k_decode_twist(const double* m, double2* W, int log_n) {
-  const uint32_t n = 1u << log_n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double sn, cs;
-    sincospi((double)i / (double)n, &sn, &cs);
-    W[i] = make_double2(m[i] * cs, m[i] * sn);
-  }
-}
-
-__global__ void k_decode_gather(const double2* G, double* re, double* im, uint32_t nz, double scale,
-                                int log_n) {
-  const uint32_t n = 1u << log_n, m = 2 * n;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < nz; j += gridDim.x * blockDim.x) {
-    uint32_t e = 1, b = 5, x = j;
-    while (x) {
-      if (x & 1) e = (uint32_t)(((uint64_t)e * b) & (m - 1));
-      b = (uint32_t)(((uint64_t)b * b) & (m - 1));
-      x >>= 1;
-    }
-    const double2 v = G[(e - 1) / 2];
-    re[j] = v.x / scale;
-    if (im) im[j] = v.y / scale;
-  }
-}
-
 // Decode centered coefficients (device doubles d_m) into n_slots device
-// values d_re.  scratch: 2N double2.
+// values d_re.  scratch: N double2.
 int decode_dev(he_ctx* c, const double* d_m, double scale, double* d_re, size_t n_slots,
                double2* scratch) {
-  const uint32_t n = c->n;
-  if (n_slots > n / 2) return fail(HE_EINVAL, "more slots than N/2");
-  double2* W = scratch;
-  double2* G = scratch + n;
-  k_decode_twist<<<grid_for(n), 256, 0, c->stream>>>(d_m, W, c->log_n);
-  HE_TRY(fft(c, W, G, 1.0));
-  k_decode_gather<<<grid_for(n_slots), 256, 0, c->stream>>>(G, d_re, nullptr, (uint32_t)n_slots, scale,
-                                                            c->log_n);
-  HE_CUDA(cudaGetLastError());
-  return HE_OK;
+  if (n_slots > (size_t)c->n / 2) return fail(HE_EINVAL, "more slots than N/2");
+  FftArgs a{};
+  a.in = d_m;
+  a.mid = scratch;
+  a.re = d_re;
+  a.nz = (uint32_t)n_slots;
+  a.scale = scale;
+  return fft_run<false>(c, a);
 }
 
 }  // namespace he

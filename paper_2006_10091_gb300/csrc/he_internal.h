@@ -95,6 +95,8 @@ struct he_ctx {
   uint64_t* d_two64 = nullptr;   // [np] 2^64 mod q
   uint64_t* d_gauss = nullptr;   // Gaussian CDT
   int gK = 0;
+  void* d_fft = nullptr;         // [N] (cos, sin)(pi i / N), doubles (codec.cu)
+  int32_t* d_slot_of = nullptr;  // [N] slot of each evaluation point (codec.cu)
 
   // ModUp constants per (level, digit): host index + device words
   std::vector<std::vector<he::ModUpConst>> modup;  // [level][digit]

@@ -23,6 +23,15 @@ __device__ __forceinline__ uint32_t map_prime(uint32_t t, uint32_t level, uint32
   return t < level ? t : L + t - level;
 }
 
+__device__ __forceinline__ int64_t ternary(uint4 w) { return (int64_t)(((uint64_t)w.x * 3) >> 32) - 1; }
+
+__device__ __forceinline__ int64_t gaussian(uint4 w, const uint64_t* gauss, int gK) {
+  const uint64_t u = ((uint64_t)w.y << 32) | w.x;
+  int m = 0;
+  while (m < gK && u >= gauss[m]) ++m;
+  return (w.z & 1) ? -m : m;
+}
+
 // kind 0 ternary, 1 Gaussian (both written to every limb), 2 uniform per limb.
 __global__ void k_sample(uint64_t* out, uint64_t out_stride, uint32_t kind, uint32_t nl,
                          uint32_t limb0, uint32_t level, uint32_t L, uint64_t seed, uint32_t sid,
@@ -45,15 +54,7 @@ __global__ void k_sample(uint64_t* out, uint64_t out_stride, uint32_t kind, uint
       continue;
     }
     const uint4 w = philox4x32_10(make_uint4(k, 0, s, dom), k0, k1);
-    int64_t v;
-    if (kind == 0) {
-      v = (int64_t)(((uint64_t)w.x * 3) >> 32) - 1;
-    } else {
-      const uint64_t u = ((uint64_t)w.y << 32) | w.x;
-      int m = 0;
-      while (m < gK && u >= gauss[m]) ++m;
-      v = (w.z & 1) ? -m : m;
-    }
+    const int64_t v = kind == 0 ? ternary(w) : gaussian(w, gauss, gK);
     for (uint32_t tl = 0; tl < nl; ++tl) {
       const uint32_t p = map_prime(limb0 + tl, level, L);
       o[(size_t)tl * n] = from_signed(v, primes[p]);
@@ -116,12 +117,28 @@ __global__ void k_enc_combine(CtBatch out, const uint64_t* v, const uint64_t* em
   }
 }
 
-__global__ void k_add_raw(const uint64_t* a, const uint64_t* b, uint64_t* o, uint32_t nl, int log_n,
-                          const PrimeDev* primes) {
+// The polynomials of one public-key encryption (np = 3: e0 + m, v, e1; np = 1
+// for a secret-key one: e0 + m), coefficient form on every limb: the same
+// streams and samplers as k_sample, one launch, the message added to e0.
+__global__ void k_enc_sample(uint64_t* out, uint64_t out_stride, uint32_t np, const int64_t* msg, uint32_t level,
+                             uint64_t seed, uint32_t cid, const uint64_t* gauss, int gK, int log_n,
+                             const PrimeDev* primes) {
   const uint32_t n = 1u << log_n;
-  const size_t total = (size_t)nl * n;
-  for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x)
-    o[g] = add_mod(a[g], b[g], primes[g / n].q);
+  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < np * n; g += gridDim.x * blockDim.x) {
+    const uint32_t k = g & (n - 1), c = g >> log_n;
+    const uint32_t dom = c == 0 ? DOM_ENC_E0 : c == 1 ? DOM_ENC_V : DOM_ENC_E1;
+    const uint4 w = philox4x32_10(make_uint4(k, 0, cid, dom), k0, k1);
+    const int64_t v = c == 1 ? ternary(w) : gaussian(w, gauss, gK);
+    const int64_t m = c == 0 ? msg[k] : 0;
+    uint64_t* o = out + (size_t)c * out_stride + k;
+    for (uint32_t t = 0; t < level; ++t) {
+      const PrimeDev pr = primes[t];
+      uint64_t r = from_signed(v, pr);
+      if (c == 0) r = add_mod(r, from_signed(m, pr), pr.q);
+      o[(size_t)t * n] = r;
+    }
+  }
 }
 
 static int sample(he_ctx* c, uint64_t* out, uint64_t out_stride, uint32_t kind, uint32_t nl,
@@ -226,25 +243,16 @@ int encrypt_dev(he_ctx* c, const int64_t* d_m, uint32_t level, int use_sk, uint3
                 uint64_t* scratch) {
   const uint32_t n = c->n, L = c->L;
   const size_t lw = (size_t)level * n;
-  uint64_t* M = scratch;
-  uint64_t* E0 = M + lw;
+  uint64_t* E0 = scratch;  // e0 + m, then v and e1 (public-key encryption)
   uint64_t* V = E0 + lw;
   uint64_t* E1 = V + lw;
-  k_signed_to_residues<<<grid_for(lw), 256, 0, c->stream>>>(d_m, M, level, c->log_n, c->d_primes);
-  HE_CUDA(cudaGetLastError());
-  HE_TRY(sample(c, E0, 0, 1, level, 0, L, cid, DOM_ENC_E0, 1, 0));
-  k_add_raw<<<grid_for(lw), 256, 0, c->stream>>>(E0, M, E0, level, c->log_n, c->d_primes);
-  HE_CUDA(cudaGetLastError());
-  HE_TRY(ntt_forward(c, one_batch(E0, E0, 0, 1, level, L)));
   CtBatch o{out->data, 0, out->cap, 0};
-  if (use_sk) {
-    HE_TRY(sample(c, out->data + (size_t)out->cap * n, 0, 2, level, 0, L, cid, DOM_ENC_A, 1, 0));
-  } else {
-    HE_TRY(sample(c, V, 0, 0, level, 0, L, cid, DOM_ENC_V, 1, 0));
-    HE_TRY(sample(c, E1, 0, 1, level, 0, L, cid, DOM_ENC_E1, 1, 0));
-    HE_TRY(ntt_forward(c, one_batch(V, V, 0, 1, level, L)));
-    HE_TRY(ntt_forward(c, one_batch(E1, E1, 0, 1, level, L)));
-  }
+  const uint32_t np = use_sk ? 1 : 3;
+  k_enc_sample<<<grid_for((size_t)np * n), 256, 0, c->stream>>>(E0, lw, np, d_m, level, c->prm.seed, cid, c->d_gauss,
+                                                                c->gK, c->log_n, c->d_primes);
+  HE_CUDA(cudaGetLastError());
+  HE_TRY(ntt_forward(c, one_batch(E0, E0, lw, np, level, L)));
+  if (use_sk) HE_TRY(sample(c, out->data + (size_t)out->cap * n, 0, 2, level, 0, L, cid, DOM_ENC_A, 1, 0));
   k_enc_combine<<<grid_for(lw), 256, 0, c->stream>>>(o, V, E0, E1, c->d_pk, c->d_s, use_sk, level, L,
                                                      c->log_n, c->d_primes);
   HE_CUDA(cudaGetLastError());

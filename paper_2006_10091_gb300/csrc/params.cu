@@ -133,6 +133,8 @@ static int bitlen(uint64_t q) {
   return k;
 }
 
+int codec_tables(he_ctx* c);
+
 // Build every table and upload it.  Returns an HE_* code.
 int build_tables(he_ctx* c) {
   const int n = c->n, np = c->np, L = c->L, alpha = c->alpha;
@@ -411,6 +413,7 @@ int build_tables(he_ctx* c) {
     HE_CUDA(cudaMalloc(&c->d_garner, sizeof(uint64_t) * words.size()));
     HE_CUDA(cudaMemcpy(c->d_garner, words.data(), sizeof(uint64_t) * words.size(), cudaMemcpyHostToDevice));
   }
+  HE_TRY(codec_tables(c));
   // copies from pageable memory may still be in flight when cudaMemcpy
   // returns; kernels on a non-blocking stream would not wait for them
   HE_CUDA(cudaDeviceSynchronize());
