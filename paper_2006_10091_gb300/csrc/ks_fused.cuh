@@ -519,40 +519,40 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
 
 // Stages with rotations that move rows between tiles: the row pass runs
 // by itself (ntt2's, in place on the column pass's outputs) and this kernel
-// gathers.  A CTA of target limb t owns one tile of output positions and CT
-// ciphertexts.  Step (r, j) needs the rows of digit j that rotation r moves to
-// the tile (whole rows, see above) of each ciphertext and the key's two
-// polynomials at the tile; a ring of kGatherRing steps is kept in flight with
+// gathers.  A CTA of target limb t owns one block of output positions and CT
+// ciphertexts.  Step (r, j) needs the words of digit j that rotation r moves to
+// the block (any aligned block of 2^k positions is a residue class like a row,
+// so they are one block too) of each ciphertext and the key's two
+// polynomials at the block; a ring of kGatherRing steps is kept in flight with
 // cp.async, since a step computes for about 0.3 us and its key words come from
 // HBM.  A thread sums one pair of neighbouring positions, like the closed
 // stages; each accumulator residue is reduced and written once.  Part 0 (ra.c0)
 // is one more step per rotation.  Bound by its instructions (FMA pipe 53 %,
 // issue slots half used, DRAM 28 %).  Fifteen unit steps at N = 2^16, 24 limbs,
-// four ciphertexts: 1.68 ms, and 0.34 ms for the row pass (every rotation's
+// four ciphertexts: 1.44 ms (1.68 with one CTA of 1024 positions per SM instead
+// of two of 512), and 0.34 ms for the row pass (every rotation's
 // reduced products added to the rows they move to with 64-bit atomics: 2.84 ms;
 // a rotation's digits per step and keys read by the products: 2.79 ms).
-// Grid: nt * ceil(count / CT) * TILES (as ks_row_rot).
-constexpr int kGatherThreads = 512, kGatherRing = 6;
+// Grid: nt * ceil(count / CT) * N / BLK, blocks of one limb's neighbouring CTAs
+// sharing its key words in L2.
+constexpr int kGatherThreads = 256, kGatherRing = 6;
 
-template <int LOG_N, int LOG_M, int LOG_K, int CT>
-__global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra) {
-  using S = Shape<LOG_N, LOG_M, LOG_K, false>;
-  constexpr uint32_t N = 1u << LOG_N, SLOT = (CT + 2) * S::TILE;
-  static_assert(S::TILE == 2 * kGatherThreads, "one pair of positions per thread");
+template <int LOG_N, int CT>
+__global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra) {
+  constexpr uint32_t N = 1u << LOG_N, BLK = 2 * kGatherThreads, SLOT = (CT + 2) * BLK;
   const KsFusedArgs& a = ra.k;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);  // [ring][CT digit tiles, key b, key a][TILE]
+  uint64_t* buf = reinterpret_cast<uint64_t*>(smem_raw);  // [ring][CT digit blocks, key b, key a][BLK]
   uint32_t b = blockIdx.x;
-  const uint32_t tile = b % S::TILES;
-  b /= S::TILES;
+  const uint32_t blk = b % (N / BLK);
+  b /= N / BLK;
   const uint32_t ngrp = (ra.count + CT - 1) / CT;
   const uint32_t i0 = (b % ngrp) * CT, t = b / ngrp;
   const uint32_t prime = ks_prime(t, a.level, a.L);
   const PrimeDev pr = a.primes[prime];
   const bool add_c0 = ra.c0 && t < a.level;
   const uint32_t ntile = a.beta + (add_c0 ? 1 : 0), nsteps = ra.nrot * ntile;
-  const uint32_t idx = 2 * threadIdx.x, kx = idx >> LOG_M;
-  const uint32_t eo = S::gidx(tile, kx, idx & (S::M - 1));
+  const uint32_t idx = 2 * threadIdx.x, eo = blk * BLK + idx;
   // where digit j's row starts: the digit's converted limb (one digit is nt
   // limbs apart from the next), the input's own limb in digit jo, part 0
   const uint64_t *ext[CT], *own[CT], *c0[CT];
@@ -568,12 +568,11 @@ __global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra)
   for (uint32_t j = 0; j < a.beta; ++j)
     if (t >= a.lo[j] && t < a.lo[j] + a.cnt[j]) jo = j;
   const uint32_t ext_step = a.nt * N, key_step = a.np * N;  // 2 beta np N < 2^32
-  const uint32_t row = eo & ~(uint32_t)(S::M - 1), x = idx & (S::M - 1);
   uint32_t cr = 0, cj = 0;  // the next step to copy
   uint32_t off = 0, ko = 0, eoff = 0;
   const uint64_t* key = nullptr;
   auto next_rotation = [&]() {
-    off = (automorph_src(row, ra.gal[cr], LOG_N) & ~(uint32_t)(S::M - 1)) | x;
+    off = (automorph_src(blk * BLK, ra.gal[cr], LOG_N) & ~(BLK - 1)) | idx;
     key = ra.evk[cr];
     ko = prime * N + eo;
     eoff = off;
@@ -585,17 +584,17 @@ __global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra)
       if (cj < a.beta) {
         if (cj == jo)
 #pragma unroll
-          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, own[c] + off);
+          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * BLK, own[c] + off);
         else
 #pragma unroll
-          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, ext[c] + eoff);
-        cp_async16_s(to + 8 * CT * S::TILE, key + ko);
-        cp_async16_s(to + 8 * (CT + 1) * S::TILE, key + (ko + key_step));
+          for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * BLK, ext[c] + eoff);
+        cp_async16_s(to + 8 * CT * BLK, key + ko);
+        cp_async16_s(to + 8 * (CT + 1) * BLK, key + (ko + key_step));
         ko += 2 * key_step;
         eoff += ext_step;
       } else {
 #pragma unroll
-        for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * S::TILE, c0[c] + off);
+        for (int c = 0; c < CT; ++c) cp_async16_s(to + 8 * c * BLK, c0[c] + off);
       }
       if (++cj == ntile) {
         cj = 0;
@@ -622,7 +621,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra)
   for (uint32_t r = 0; r < ra.nrot; ++r) {
     // the sources of two neighbouring positions are neighbours (their exponents
     // differ by N, and gal is odd): one 16-byte load, its words swapped or not
-    const uint32_t sp0 = (kx << LOG_M) | (automorph_src(eo, ra.gal[r], LOG_N) & (S::M - 1));
+    const uint32_t sp0 = automorph_src(eo, ra.gal[r], LOG_N) & (BLK - 1);
     const uint32_t sp = sp0 & ~1u;
     const bool sw = sp0 & 1;
     for (uint32_t j = 0; j < ntile; ++j) {
@@ -634,20 +633,20 @@ __global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra)
       if (j == a.beta) {
 #pragma unroll
         for (int c = 0; c < CT; ++c) {
-          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * BLK + sp);
           s0[c][0] += sw ? xv.y : xv.x;
           s0[c][1] += sw ? xv.x : xv.y;
         }
         continue;
       }
-      const ulonglong2 wb = *reinterpret_cast<const ulonglong2*>(sm + CT * S::TILE + idx);
-      const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(sm + (CT + 1) * S::TILE + idx);
+      const ulonglong2 wb = *reinterpret_cast<const ulonglong2*>(sm + CT * BLK + idx);
+      const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(sm + (CT + 1) * BLK + idx);
       if (split) {
         const Split3 kb0 = split3(wb.x, sb, mask), kb1 = split3(wb.y, sb, mask);
         const Split3 ka0 = split3(wa.x, sb, mask), ka1 = split3(wa.y, sb, mask);
 #pragma unroll
         for (int c = 0; c < CT; ++c) {
-          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * BLK + sp);
           const Split3 x0 = split3(sw ? xv.y : xv.x, sb, mask), x1 = split3(sw ? xv.x : xv.y, sb, mask);
           mac_split3(ll[c][0][0], hh[c][0][0], ss[c][0][0], x0, kb0);
           mac_split3(ll[c][0][1], hh[c][0][1], ss[c][0][1], x1, kb1);
@@ -657,7 +656,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) ks_gather_rot(KsRotArgs ra)
       } else {
 #pragma unroll
         for (int c = 0; c < CT; ++c) {
-          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * S::TILE + sp);
+          const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm + c * BLK + sp);
           const uint64_t x0 = sw ? xv.y : xv.x, x1 = sw ? xv.x : xv.y;
           mac128(ll[c][0][0], hh[c][0][0], x0, wb.x);
           mac128(ll[c][0][1], hh[c][0][1], x1, wb.y);
@@ -919,18 +918,20 @@ size_t md_col_smem(uint32_t nd) {
 
 // How a conversion kernel's target limbs are shared: `blocks` groups of CTAs
 // (digits or parts times tiles), of which `slots` CTAs run at a time; a CTA
-// pays `setup` and then one unit per target.  A CTA's chain of targets is
-// bound by latency (a unit takes 4.4 us alone on its SM and 5.9 us beside two
-// others, N = 2^13 and 2^14), so a batch that leaves CTA slots free is split as
-// far as they reach, and the time is the number of waves times the chain.  (Splits
-// beyond one wave: inference of 21 ciphertexts at N = 2^13, 503 against 460 us.)
+// pays `setup` and then one unit per target.  Alone on its SM a CTA is bound by
+// latency (a unit takes 4.4 us at N = 2^13), so a batch that leaves CTA slots
+// free is split as far as they reach; together the CTAs of an SM finish a unit
+// every 2.1 us, so the repeated setup must not cost more than the shorter
+// chains give: the time is the larger of the chain and 0.48 of the SM's units.
 // One rotation at N = 2^13, level 19: 20 and 8 CTAs walked 19 to 23 targets
-// each, 101 and 122 us.
+// each, 101 and 122 us, split 25 and 23.  288 CTAs of 9 units at N = 2^12 stay
+// as they are: 36 us, split in two 48.
 inline uint32_t conv_splits(size_t blocks, size_t slots, uint32_t targets, double setup, double* cost) {
   uint32_t best = 1;
   double bc = 0.0;
   for (uint32_t s = 1; s <= targets && (s == 1 || blocks * s <= slots); ++s) {
-    const double c = (double)((blocks * s + slots - 1) / slots) * (setup + (double)((targets + s - 1) / s));
+    const double chain = (double)((blocks * s + slots - 1) / slots) * (setup + (double)((targets + s - 1) / s));
+    const double c = std::max(chain, 0.48 / 152 * (double)blocks * (s * setup + targets));
     if (s == 1 || c < bc) {
       bc = c;
       best = s;
@@ -951,7 +952,7 @@ inline size_t conv_slots(const he_ctx* c, size_t smem, int threads) {
 constexpr double kSetupHalf = 1.0, kSetupFull = 0.3;
 // ... and the units a column pass launched by itself costs instead.
 inline double col_pass_units(size_t polys, int tiles) {
-  return 1.5 + (double)((polys * tiles + 4 * 152 - 1) / (4 * 152));
+  return 1.5 + std::max(1.0, 0.48 / 152 * (double)(polys * tiles));
 }
 
 template <int LOG_N, int M1, int K1>
@@ -1125,8 +1126,8 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   HE_TRY(set_smem_attr_once(attr1, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr2, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 2>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr4, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 4>, kRotSmemMax));
-  HE_TRY(set_smem_attr_once(attr_g1, c->device, (const void*)ks_gather_rot<LOG_N, M2, K2 - 1, 1>, kRotSmemMax));
-  HE_TRY(set_smem_attr_once(attr_g2, c->device, (const void*)ks_gather_rot<LOG_N, M2, K2 - 1, 2>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr_g1, c->device, (const void*)ks_gather_rot<LOG_N, 1>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr_g2, c->device, (const void*)ks_gather_rot<LOG_N, 2>, kRotSmemMax));
   HE_TRY((ks_modup_launch<LOG_N, M1, K1>(c, a, count)));
   const double n = (double)(1u << LOG_N);
   double own = 0;
@@ -1185,10 +1186,10 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
                  macs + c0_work, bfly, mac3);
   if (!closed) {
     const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words
-    const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
-    const size_t sm = kGatherRing * (ct + 2) * sizeof(uint64_t) * SR::TILE;
-    if (ct == 2) ks_gather_rot<LOG_N, M2, K2 - 1, 2><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
-    else ks_gather_rot<LOG_N, M2, K2 - 1, 1><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
+    const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * ((1u << LOG_N) / (2 * kGatherThreads));
+    const size_t sm = kGatherRing * (ct + 2) * sizeof(uint64_t) * 2 * kGatherThreads;
+    if (ct == 2) ks_gather_rot<LOG_N, 2><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
+    else ks_gather_rot<LOG_N, 1><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
     HE_CUDA(cudaGetLastError());
     return HE_OK;
   }
