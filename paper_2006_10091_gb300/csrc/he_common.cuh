@@ -9,6 +9,10 @@
 //  * Barrett (1986) for a product of two variable residues: k = bitlen(q),
 //    mu = floor(2^(2k) / q); for x < 2^(2k), t = x >> (k-1),
 //    qe = (t*mu) >> (k+1) undershoots floor(x/q) by at most 2.
+// The primes are scanned downward from a power of two, so q = 2^k - delta with a
+// small delta: 2^k = delta mod q folds the high part of a value into its low
+// part with one 32 x 32 -> 64-bit multiply-add (fold), where it applies
+// (PrimeDev::delta != 0).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -19,7 +23,7 @@ struct PrimeDev {
   uint64_t q;
   uint64_t mu;        // Barrett constant floor(2^(2k)/q)
   uint32_t k;         // bit length of q
-  uint32_t pad;
+  uint32_t delta;     // 2^k - q when 33 <= k <= 60 and it is below 2^28, 2^(k-11) and 2^((2k-4)/3), else 0
   uint64_t n_inv;     // N^-1 mod q
   uint64_t n_inv_sh;  // its Shoup companion
   uint64_t one_sh;    // Shoup companion of 1: floor(2^64 / q)
@@ -40,6 +44,27 @@ __device__ __forceinline__ uint64_t mul_shoup_lazy(uint64_t a, uint64_t w, uint6
 __device__ __forceinline__ uint64_t mul_shoup(uint64_t a, uint64_t w, uint64_t wsh, uint64_t q) {
   uint64_t r = mul_shoup_lazy(a, w, wsh, q);
   return r >= q ? r - q : r;
+}
+
+// c + a*b, 32 x 32 -> 64 bits (one instruction).
+__device__ __forceinline__ uint64_t madw(uint32_t a, uint32_t b, uint64_t c) {
+  uint64_t r;
+  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t pack64(uint32_t lo, uint32_t hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ uint32_t lo32(uint64_t x) { return (uint32_t)x; }
+__device__ __forceinline__ uint32_t hi32(uint64_t x) { return (uint32_t)(x >> 32); }
+
+// x mod q up to a few q: (x mod 2^k) + (x >> k) delta, for any 64-bit x and a
+// prime with delta != 0.  For x < 2^k 2^7 the result is below 2q.
+__device__ __forceinline__ uint64_t fold(uint64_t x, const PrimeDev& p) {
+  const uint32_t sh = p.k - 32, h = hi32(x);
+  return madw(h >> sh, p.delta, pack64(lo32(x), h & ((1u << sh) - 1)));
 }
 
 // (hi:lo) mod q for hi:lo < 2^(2k).
@@ -95,12 +120,15 @@ __device__ __forceinline__ bool frac_in_window(uint64_t fs, uint32_t a) { return
 
 // Exact v for an element in that window: v = vc + 1 iff
 // sum_k u_k (P/p_k) >= (vc + 1) P, compared as 8-word integers.  u_k at
-// u[k * ustride]; phat = [a][8] words of P/p_k, pw = [8] words of P.
+// u[k * ustride] (as 30-bit halves (low, high) in a word's halves when `halves`);
+// phat = [a][8] words of P/p_k, pw = [8] words of P.
 static __device__ __noinline__ uint32_t exact_lift_multiple(const uint64_t* u, size_t ustride, uint32_t a,
-                                                            const uint64_t* phat, const uint64_t* pw, uint32_t vc) {
+                                                            const uint64_t* phat, const uint64_t* pw, uint32_t vc,
+                                                            bool halves = false) {
   uint64_t s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (uint32_t k = 0; k < a; ++k) {
-    const uint64_t x = u[(size_t)k * ustride];
+    uint64_t x = u[(size_t)k * ustride];
+    if (halves) x = (x >> 32 << 30) | (uint32_t)x;
     uint64_t carry = 0;
     for (int w = 0; w < 8; ++w) {
       const uint64_t ph = phat[(size_t)k * 8 + w];
@@ -177,7 +205,8 @@ __device__ __forceinline__ void mac128(uint64_t& lo, uint64_t& hi, uint64_t a, u
 // (any 64-bit hi, result in [0, 2q)) plus lo mod q, corrected once.
 __device__ __forceinline__ uint64_t reduce128_any(uint64_t hi, uint64_t lo, const PrimeDev& p) {
   const uint64_t q = p.q;
-  uint64_t r = mul_shoup_lazy(hi, p.r64, p.r64_sh, q) + reduce64(lo, p);
+  // lo by a fold where it leaves less than 2q (any 64-bit lo: 2^(64-k) delta < 2^k - 2 delta)
+  uint64_t r = mul_shoup_lazy(hi, p.r64, p.r64_sh, q) + (p.delta && p.k >= 50 ? fold(lo, p) : reduce64(lo, p));
   r = r >= q + q ? r - q - q : r;
   return r >= q ? r - q : r;
 }
@@ -213,6 +242,24 @@ __device__ __forceinline__ void split3_total(uint64_t ll, uint64_t hh, uint64_t 
   const uint64_t h_lo = hh << (2 * sb), h_hi = hh >> (64 - 2 * sb);
   asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(m_lo), "l"(m_hi));
   asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(h_lo), "l"(h_hi));
+}
+
+// The residue of the sum held by ll, hh, ss (2 sb = k or k + 1, prime with
+// delta != 0, at most 2^7 terms below 2^(k+1)): the sum is ll + mid 2^sb + hh 2^(2 sb) and 2^(2 sb)
+// = rho mod q (delta, or 2 delta for odd k), so with mid = mh 2^sb + ml it is
+// ll + ml 2^sb + (hh + mh) rho; hh + mh is folded below 1.25 2^k first, its
+// product by rho (up to 89 bits) folded like the value, which leaves it below
+// 1.3 rho delta + 2^k; the last fold leaves less than 2q because 3 delta^3 < 2^(2k-2).
+__device__ __forceinline__ uint64_t split3_residue(uint64_t ll, uint64_t hh, uint64_t ss, uint32_t sb,
+                                                   const PrimeDev& p) {
+  const uint64_t mid = ss - ll - hh;  // sum (xl wh + xh wl), exact
+  const uint32_t sh = p.k - 32, mask = (1u << sh) - 1, rho = p.delta << (2 * sb - p.k);
+  const uint64_t h = fold(hh + (mid >> sb), p);
+  const uint64_t a = madw(lo32(h), rho, 0), t = madw(hi32(h), rho, hi32(a));  // h rho = t 2^32 + lo32(a)
+  uint64_t r = madw((uint32_t)(t >> sh), p.delta, pack64(lo32(a), lo32(t) & mask));
+  r += madw((uint32_t)mid & ((1u << sb) - 1), 1u << sb, ll);
+  r = fold(r, p);
+  return r >= p.q ? r - p.q : r;
 }
 
 // 128-bit word (w3:w2:w1:w0) mod q, by Horner on 64-bit halves:

@@ -41,6 +41,7 @@ struct KsFusedArgs {
   const ulonglong2* itw;   // inverse twiddles
   int half;                // d2c holds the inverse transform's row pass only (ks_modup_col_all finishes it)
   uint32_t splits;         // CTAs of ks_modup_col_all that share one digit and tile's target limbs
+  int split_conv;          // the conversions run as conv_split_tile (every target allows it)
   const uint64_t* consts;  // ModUp constant tables
   uint32_t lo[HE_MAX_PRIMES], cnt[HE_MAX_PRIMES];
   uint64_t off[HE_MAX_PRIMES];
@@ -50,32 +51,117 @@ __host__ __device__ __forceinline__ uint32_t ks_prime(uint32_t t, uint32_t level
   return t < level ? t : L + t - level;
 }
 
-// The basis conversion of one tile into shared memory: for the T threads'
-// elements idx of the tile, sum over u < CNT of wv[u][idx] times the constant
-// (w[u * stride], its Shoup companion), reduced to [0, q); the CNT constants
-// sit in registers for the whole tile.  With vv (ModDown's exact lift), the
-// element's multiple of P and h are then subtracted in the same pass:
-// - vP[vv[idx]] - h mod q.
+// The basis conversion of one tile into shared memory, y = sum over u < CNT of
+// v_u c_u mod q for the T threads' elements of the tile (a few q, not reduced to
+// [0, q): the lazy transform that follows takes any 64-bit input, the corrected
+// one less than 2q).  Sources come as two 30-bit halves (split_source), v = v0
+// + v1 2^30, constants as two half-width limbs at 2^e, e = ceil(k/2), of c and
+// c2 = 2^30 c mod q, so that the sum is A + B 2^e with two 64-bit sums of 32 x 32
+// -> 64-bit products, four multiply-adds per term and no carries, and one
+// reduction for all terms: 2^(2e) = rho mod q (delta or 2 delta) folds B's upper
+// part, then a fold.  (A Shoup product and a correction per term, 23 instructions
+// against 4, plus 9 per element.)  CNT = 1: c = 1, the source itself.  With vv
+// (ModDown's exact lift), minus vP[vv[idx]] and h.  conv_split_ok has the bounds.
+__device__ __forceinline__ uint64_t split_source(uint64_t v) {
+  return (v & ((1u << 30) - 1)) | ((v >> 30) << 32);
+}
+__device__ __forceinline__ uint64_t join_source(uint64_t x) { return (x >> 32 << 30) | (uint32_t)x; }
+
 template <int TILE, int T, int CNT>
-__device__ __forceinline__ void conv_sum_tile(uint64_t* sm, const uint64_t* wv, const uint64_t* w, const uint64_t* wsh,
-                                              uint32_t stride, uint64_t q, const uint32_t* vv = nullptr,
-                                              const uint64_t* vP = nullptr, uint64_t h = 0) {
-  uint64_t cw[CNT], cs[CNT];
+__device__ __forceinline__ void conv_split_tile(uint64_t* sm, const uint64_t* wv, const uint64_t* w, const uint64_t* w2,
+                                                uint32_t stride, const PrimeDev& pr, const uint32_t* vv = nullptr,
+                                                const uint64_t* vP = nullptr, uint64_t h = 0) {
+  const uint32_t e = (pr.k + 1) >> 1, mask = (1u << e) - 1, rho = pr.delta << (2 * e - pr.k);
+  const uint64_t minus = 2 * pr.q - h;
+  uint32_t c0[CNT], c1[CNT], d0[CNT], d1[CNT];
 #pragma unroll
-  for (int u = 0; u < CNT; ++u) {
-    cw[u] = w[(size_t)u * stride];
-    cs[u] = wsh[(size_t)u * stride];
+  for (int u = 0; u < CNT && CNT > 1; ++u) {
+    const uint64_t x = w[(size_t)u * stride], y = w2[(size_t)u * stride];
+    c0[u] = lo32(x) & mask;
+    c1[u] = (uint32_t)(x >> e);
+    d0[u] = lo32(y) & mask;
+    d1[u] = (uint32_t)(y >> e);
   }
-  const uint64_t q2 = q + q;
+#pragma unroll 4
+  for (uint32_t idx = threadIdx.x; idx < (uint32_t)TILE; idx += T) {
+    uint64_t a = 0, b = 0;
+    if (CNT == 1) {
+      a = wv[idx];
+    } else {
+#pragma unroll
+      for (int u = 0; u < CNT; ++u) {
+        const uint2 x = *reinterpret_cast<const uint2*>(wv + (size_t)u * TILE + idx);
+        a = madw(x.x, c0[u], a);
+        b = madw(x.x, c1[u], b);
+        a = madw(x.y, d0[u], a);
+        b = madw(x.y, d1[u], b);
+      }
+      a = madw(lo32(b) & mask, 1u << e, a);
+      const uint64_t q = b >> e;  // below 2^35
+      a = madw(lo32(q), rho, a);
+      a = pack64(lo32(a), hi32(a) + hi32(q) * rho);
+    }
+    if (vv) a += minus - (CNT == 1 ? 0 : vP[vv[idx]]);
+    sm[idx + (idx >> 3)] = fold(a, pr);
+  }
+}
+
+// The same on T threads for a runtime count of 1 to 5 sources.
+template <int TILE, int T>
+__device__ __forceinline__ void conv_split(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
+                                           const uint64_t* w2, uint32_t stride, const PrimeDev& pr,
+                                           const uint32_t* vv = nullptr, const uint64_t* vP = nullptr, uint64_t h = 0) {
+  if (cnt == 1) conv_split_tile<TILE, T, 1>(sm, wv, w, w2, stride, pr, vv, vP, h);
+  else if (cnt == 2) conv_split_tile<TILE, T, 2>(sm, wv, w, w2, stride, pr, vv, vP, h);
+  else if (cnt == 3) conv_split_tile<TILE, T, 3>(sm, wv, w, w2, stride, pr, vv, vP, h);
+  else if (cnt == 4) conv_split_tile<TILE, T, 4>(sm, wv, w, w2, stride, pr, vv, vP, h);
+  else conv_split_tile<TILE, T, 5>(sm, wv, w, w2, stride, pr, vv, vP, h);
+}
+
+// Whether the conversion of cnt sources below 2^src_bits to q runs as
+// conv_split_tile: the sum (plus 3q for ModDown's lift) stays below 2^64 and its
+// fold below 2^(k+5) (below 2q for the corrected transforms' primes), so that
+// the lazy transform's values stay below 66 2^k.
+inline bool conv_split_ok(uint64_t q, uint32_t cnt, uint32_t src_bits) {
+  const uint32_t k = 64 - __builtin_clzll(q), e = (k + 1) / 2;
+  if (k < 33 || k > 60 || cnt < 1 || cnt > 5 || src_bits > 60) return false;
+  const uint64_t delta = (1ull << k) - q;
+  if (delta >= (1ull << std::min({28u, k - 11, (2 * k - 4) / 3}))) return false;
+  typedef unsigned __int128 u128;
+  const u128 rho = (u128)delta << (2 * e - k);
+  u128 most = (u128)1 << src_bits;
+  if (cnt > 1) {
+    const u128 a = (u128)(2 * cnt) << (30 + e), b = (u128)(2 * cnt) << (30 + k - e);
+    if (b >> 64) return false;
+    most = a + ((u128)1 << (2 * e)) + ((b >> e) + 1) * rho;
+  }
+  most += 3 * (u128)q;
+  if (most >> 64) return false;
+  const u128 folded = ((u128)1 << k) + (most >> k) * delta;
+  return folded <= (q < (1ull << 58) ? (u128)1 << (k + 5) : 2 * (u128)q);
+}
+
+// The conversion of one tile for primes conv_split_ok turns down: Shoup
+// products by the constants (w[u * stride], companions wsh), kept in [0, 2q),
+// then to [0, q) and minus vP[vv[idx]] and h.
+template <int TILE, int T>
+__device__ __forceinline__ void conv_sum_tile(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
+                                              const uint64_t* wsh, uint32_t stride, const PrimeDev& pr,
+                                              const uint32_t* vv = nullptr, const uint64_t* vP = nullptr,
+                                              uint64_t h = 0) {
+  const uint64_t q = pr.q, q2 = q + q;
 #pragma unroll 2
   for (uint32_t idx = threadIdx.x; idx < (uint32_t)TILE; idx += T) {
     uint64_t y = 0;
-#pragma unroll
-    for (int u = 0; u < CNT; ++u) {
-      y += mul_shoup_lazy(wv[(size_t)u * TILE + idx], cw[u], cs[u], q);
-      y = y >= q2 ? y - q2 : y;
+    if (cnt == 1 && !vv) {
+      y = reduce64(wv[idx], pr);  // the constant is 1
+    } else {
+      for (uint32_t u = 0; u < cnt; ++u) {
+        y += mul_shoup_lazy(wv[(size_t)u * TILE + idx], w[(size_t)u * stride], wsh[(size_t)u * stride], q);
+        y = y >= q2 ? y - q2 : y;
+      }
+      y = y >= q ? y - q : y;
     }
-    y = y >= q ? y - q : y;
     if (vv) y = sub_mod(sub_mod(y, vP[vv[idx]], q), h, q);
     sm[idx + (idx >> 3)] = y;
   }
@@ -162,6 +248,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
   const uint64_t* tab = a.consts + a.off[j];
   const uint64_t* mat = tab + 2 * cnt;
   const uint64_t* mat_sh = mat + (size_t)cnt * a.np;
+  const uint64_t* mat_2 = mat_sh + (size_t)cnt * a.np + 2 * cnt;
   const uint64_t* x = a.d2c + (size_t)i * a.level * N;
   for (uint32_t u = 0; u < cnt; ++u) {
     const PrimeDev pa = a.primes[lo + u];
@@ -181,13 +268,17 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
       const uint64_t w = tabn[2 * u], wsh = tabn[2 * u + 1];
 #pragma unroll 8
       for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T)
-        wv[(size_t)u * S::TILE + idx] = mul_shoup(sm[idx + (idx >> 3)], w, wsh, pa.q);
+      {
+        const uint64_t v = mul_shoup(sm[idx + (idx >> 3)], w, wsh, pa.q);
+        wv[(size_t)u * S::TILE + idx] = a.split_conv && cnt > 1 ? split_source(v) : v;
+      }
     } else {
 #pragma unroll 8
       for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint32_t e = S::gidx(tile, idx & (S::K - 1), idx >> LOG_K);
         const uint64_t xv = __ldg(x + (size_t)(lo + u) * N + e);
-        wv[(size_t)u * S::TILE + idx] = cnt == 1 ? xv : mul_shoup(xv, tab[2 * u], tab[2 * u + 1], pa.q);
+        const uint64_t v = cnt == 1 ? xv : mul_shoup(xv, tab[2 * u], tab[2 * u + 1], pa.q);
+        wv[(size_t)u * S::TILE + idx] = a.split_conv && cnt > 1 ? split_source(v) : v;
       }
     }
     // the next limb's staging overwrites stw and sm: wait for every thread
@@ -197,32 +288,11 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
     if (t >= lo && t < lo + cnt) continue;  // the digit's own limbs are used as they are
     const uint32_t prime = ks_prime(t, a.level, a.L);
     const PrimeDev pr = a.primes[prime];
-    const uint64_t q2 = pr.q + pr.q;
     // the previous target's rounds ended with a barrier, and its write-out
     // reads only the words each thread rewrites below
     stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)prime * N, tile);
-    // Shoup products by (Q_j/q_i) mod q_t, the digit's limb count a compile-time
-    // constant for the usual digit sizes
-    if (cnt == 2) conv_sum_tile<S::TILE, S::T, 2>(sm, wv, mat + prime, mat_sh + prime, a.np, pr.q);
-    else if (cnt == 3) conv_sum_tile<S::TILE, S::T, 3>(sm, wv, mat + prime, mat_sh + prime, a.np, pr.q);
-    else if (cnt == 4) conv_sum_tile<S::TILE, S::T, 4>(sm, wv, mat + prime, mat_sh + prime, a.np, pr.q);
-    else
-#pragma unroll 2
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
-        uint64_t y;
-        if (cnt == 1) {
-          y = reduce64(wv[idx], pr);  // Q_j / q_lo = 1
-        } else {  // kept in [0, 2q)
-          y = 0;
-          for (uint32_t u = 0; u < cnt; ++u) {
-            y += mul_shoup_lazy(wv[(size_t)u * S::TILE + idx], mat[(size_t)u * a.np + prime],
-                                mat_sh[(size_t)u * a.np + prime], pr.q);
-            y = y >= q2 ? y - q2 : y;
-          }
-          y = y >= pr.q ? y - pr.q : y;
-        }
-        sm[idx + (idx >> 3)] = y;
-      }
+    if (a.split_conv) conv_split<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_2 + prime, a.np, pr);
+    else conv_sum_tile<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr);
     __syncthreads();
     uint64_t* out = a.ext + (((size_t)i * a.beta + j) * a.nt + t) * N;
     if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
@@ -261,6 +331,31 @@ struct KsRotArgs {
   const uint64_t* c0;
   uint64_t c0_stride;
 };
+
+// The residue of a split sum, with part 0's term s0 pm (s0 a sum of up to 16
+// residues, pm = P mod q) when add.
+__device__ __forceinline__ uint64_t split3_final(uint64_t ll, uint64_t hh, uint64_t ss, uint32_t sb, const PrimeDev& pr,
+                                                 bool add, uint64_t s0, uint64_t pm) {
+  if (pr.delta) {
+    if (add) {
+      const uint32_t mask = (1u << sb) - 1;
+      mac_split3(ll, hh, ss, split3(fold(s0, pr), sb, mask), split3(pm, sb, mask));
+    }
+    return split3_residue(ll, hh, ss, sb, pr);
+  }
+  uint64_t lo, hi;
+  split3_total(ll, hh, ss, sb, lo, hi);
+  if (add) mac128(lo, hi, s0, pm);
+  return reduce128_any(hi, lo, pr);
+}
+
+// Whether nterms key products of residues below 2^k (and part 0's term, below
+// 1.01 times as much) can be summed as split sums.
+__host__ __device__ __forceinline__ bool split3_fits(uint32_t k, uint32_t nterms) {
+  uint32_t bits = 0;
+  for (uint32_t x = nterms + 2; x; x >>= 1) ++bits;
+  return 2 * ((k + 1) / 2) + 2 + bits <= 64;
+}
 
 // Grid: nt * ceil(count / CT) * TILES, target limb slowest and row tile
 // fastest, so that the CTAs resident at one time share their keys (one limb
@@ -373,7 +468,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   // key products as split sums (mac_split3) when the prime and the number of
   // summed terms allow it
   const uint32_t sb = (pr.k + 1) >> 1;
-  if (2 * sb + 2 + (32 - __clz(ra.nrot * a.beta)) <= 64) {
+  if (split3_fits(pr.k, ra.nrot * a.beta)) {
     // one pair of neighbouring positions per pass, all CT ciphertexts with
     // each key load
     constexpr int PPT = PER / 2 / CT;
@@ -438,10 +533,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
           uint64_t r2[2];
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            uint64_t lo, hi;
-            split3_total(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, lo, hi);
-            if (p == 0 && add_c0) mac128(lo, hi, s0[c][u], pm);
-            r2[u] = reduce128_any(hi, lo, pr);
+            r2[u] = split3_final(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, pr, p == 0 && add_c0, s0[c][u], pm);
           }
           *reinterpret_cast<ulonglong2*>(o0 + (size_t)p * a.nt * N + eo) = make_ulonglong2(r2[0], r2[1]);
         }
@@ -604,7 +696,7 @@ __global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra)
     cp_async_commit();  // (an empty group past the last step keeps the count)
   };
   const uint32_t sb = (pr.k + 1) >> 1, mask = (1u << (sb & 31)) - 1;
-  const bool split = 2 * sb + 2 + (32 - __clz(ra.nrot * a.beta)) <= 64;
+  const bool split = split3_fits(pr.k, ra.nrot * a.beta);
   // split sums (ll, hh, ss), or 128-bit sums (ll = low word, hh = high word)
   uint64_t ll[CT][2][2], hh[CT][2][2], ss[CT][2][2], s0[CT][2];  // [ciphertext][part][position]
 #pragma unroll
@@ -688,10 +780,13 @@ __global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra)
       uint64_t r2[2];
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        uint64_t lo = ll[c][p][u], hi = hh[c][p][u];
-        if (split) split3_total(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, lo, hi);
-        if (p == 0 && add_c0) mac128(lo, hi, reduce64(s0[c][u], pr), pm);
-        r2[u] = reduce128_any(hi, lo, pr);
+        if (split) {
+          r2[u] = split3_final(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, pr, p == 0 && add_c0, s0[c][u], pm);
+        } else {
+          uint64_t lo = ll[c][p][u], hi = hh[c][p][u];
+          if (p == 0 && add_c0) mac128(lo, hi, reduce64(s0[c][u], pr), pm);
+          r2[u] = reduce128_any(hi, lo, pr);
+        }
       }
       *reinterpret_cast<ulonglong2*>(o + (size_t)p * a.nt * N) = make_ulonglong2(r2[0], r2[1]);
     }
@@ -727,6 +822,7 @@ struct MdArgs {
   const ulonglong2* itw;  // inverse twiddles (half)
   int half;               // yP holds only the inverse transform's row pass: md_conv_col finishes it
   uint32_t splits;        // CTAs of md_conv_col that share one tile's target limbs
+  int split_conv;         // the conversions run as conv_split_tile (every target allows it)
   const uint64_t* md;   // ModDown tables (params.cu)
 };
 
@@ -754,6 +850,8 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
   const uint64_t* hP = mat + (size_t)a.alpha * a.L + 2 * a.L;
   const uint64_t* mat_sh = hP + a.alpha + a.L;
   const uint64_t* wlo = mat_sh + (size_t)a.alpha * a.L;
+  const uint64_t* phat = wlo + a.alpha + 9 * (size_t)a.L;         // [alpha][8] words of P/p_u, then [8] of P
+  const uint64_t* mat_2 = phat + 8 * (size_t)a.alpha + 8;         // (alpha > 1)
   const uint64_t* yP = a.yP + (size_t)i * a.yp_stride + (size_t)p * a.yp_pstride;
   // exact conversion: sum_u w_u (P/p_u) - v P, w_u = [y_u (P/p_u)^-1]_{p_u},
   // v = floor(sum_u w_u / p_u) (64.64 fixed point, resolved exactly near an
@@ -781,7 +879,8 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
 #pragma unroll
     for (int v = 0; v < S::TILE / S::T; ++v) {
       if (a.half) y0[v] = mul_shoup(y0[v], pp.n_inv, pp.n_inv_sh, pp.q);
-      wv[(size_t)u * S::TILE + threadIdx.x + v * S::T] = mul_shoup(add_mod(y0[v], h, pp.q), w, wsh, pp.q);
+      const uint64_t x = mul_shoup(add_mod(y0[v], h, pp.q), w, wsh, pp.q);
+      wv[(size_t)u * S::TILE + threadIdx.x + v * S::T] = a.split_conv && a.alpha > 1 ? split_source(x) : x;
     }
     // the next limb's staging overwrites stw and sm: wait for every thread
     if (a.half) __syncthreads();
@@ -792,40 +891,24 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
     uint32_t v = 0;
     if (a.alpha > 1) {
       for (uint32_t u = 0; u < a.alpha; ++u)
-        frac_acc(wv[(size_t)u * S::TILE + idx], a.primes[a.spr[u]].one_sh, wlo[u], &fs, &v);
-      if (frac_in_window(fs, a.alpha)) {
-        const uint64_t* phat = wlo + a.alpha + 9 * (size_t)a.L;  // [alpha][8] words of P/p_u, then [8] of P
-        v = exact_lift_multiple(wv + idx, S::TILE, a.alpha, phat, phat + 8 * (size_t)a.alpha, v);
+      {
+        const uint64_t x = wv[(size_t)u * S::TILE + idx];
+        frac_acc(a.split_conv ? join_source(x) : x, a.primes[a.spr[u]].one_sh, wlo[u], &fs, &v);
       }
+      if (frac_in_window(fs, a.alpha))
+        v = exact_lift_multiple(wv + idx, S::TILE, a.alpha, phat, phat + 8 * (size_t)a.alpha, v, a.split_conv);
     }
     vv[idx] = v;
   }
   for (uint32_t t = part * a.level / a.splits; t < t_end; ++t) {
     const PrimeDev pr = a.primes[t];
-    const uint64_t q2 = pr.q + pr.q, hQ = hP[a.alpha + t];
+    const uint64_t hQ = hP[a.alpha + t];
     const uint64_t* vP = wlo + a.alpha + a.L + (size_t)t * 8;  // v P mod q_t, v < 8
     stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)t * N, tile);
-    // Shoup products by (P/p_u) mod q_t (the dropped-prime count a
-    // compile-time constant for the usual counts), then - v P - h
-    if (a.alpha >= 2 && a.alpha <= 5) {
-      if (a.alpha == 2) conv_sum_tile<S::TILE, S::T, 2>(sm, wv, mat + t, mat_sh + t, a.L, pr.q, vv, vP, hQ);
-      else if (a.alpha == 3) conv_sum_tile<S::TILE, S::T, 3>(sm, wv, mat + t, mat_sh + t, a.L, pr.q, vv, vP, hQ);
-      else if (a.alpha == 4) conv_sum_tile<S::TILE, S::T, 4>(sm, wv, mat + t, mat_sh + t, a.L, pr.q, vv, vP, hQ);
-      else conv_sum_tile<S::TILE, S::T, 5>(sm, wv, mat + t, mat_sh + t, a.L, pr.q, vv, vP, hQ);
-    } else {
-#pragma unroll 2
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
-        uint64_t acc = 0;  // kept in [0, 2q)
-        for (uint32_t u = 0; u < a.alpha; ++u) {
-          acc += mul_shoup_lazy(wv[(size_t)u * S::TILE + idx], mat[(size_t)u * a.L + t], mat_sh[(size_t)u * a.L + t],
-                                pr.q);
-          acc = acc >= q2 ? acc - q2 : acc;
-        }
-        acc = acc >= pr.q ? acc - pr.q : acc;
-        acc = sub_mod(acc, vP[vv[idx]], pr.q);
-        sm[idx + (idx >> 3)] = sub_mod(acc, hQ, pr.q);
-      }
-    }
+    if (a.split_conv)
+      conv_split<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_2 + t, a.L, pr, vv, vP, hQ);
+    else
+      conv_sum_tile<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, vv, vP, hQ);
     __syncthreads();
     if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
     else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
@@ -975,6 +1058,11 @@ template <int LOG_N, int M1, int K1, int M2, int K2>
 int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   using SC = Shape<LOG_N, M1, K1, true>;
   MdArgs a = a0;
+  uint32_t src_bits = 0;
+  for (uint32_t u = 0; u < a.alpha; ++u)
+    src_bits = std::max(src_bits, (uint32_t)(64 - __builtin_clzll(c->q[a.spr[u]])));
+  a.split_conv = 1;
+  for (uint32_t t = 0; t < a.level; ++t) a.split_conv &= conv_split_ok(c->q[t], a.alpha, src_bits) ? 1 : 0;
   using SR = Shape<LOG_N, M2, K2, false>;
   const size_t smc = md_col_smem<LOG_N, M1, K1>(a.alpha);
   const size_t smr = sizeof(ulonglong2) * SR::NTW + sizeof(uint64_t) * (SR::TILE + SR::TILE / 8);
@@ -1043,6 +1131,12 @@ bool ks_half(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt
 template <int LOG_N, int M1, int K1>
 int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
   KsFusedArgs a = a0;
+  uint32_t src_bits = 0;
+  for (uint32_t t = 0; t < a.level; ++t) src_bits = std::max(src_bits, (uint32_t)(64 - __builtin_clzll(c->q[t])));
+  a.split_conv = 1;
+  for (uint32_t t = 0; t < a.nt; ++t)
+    for (uint32_t j : {0u, a.beta - 1})  // (only the last digit may be shorter)
+      a.split_conv &= conv_split_ok(c->q[ks_prime(t, a.level, a.L)], a.cnt[j], src_bits) ? 1 : 0;
   using SC = Shape<LOG_N, M1, K1, true>;
   const size_t smc = sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8);
   static std::atomic<unsigned long long> attr_one{0}, attr_all{0};
@@ -1156,13 +1250,12 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   // multiply-accumulates on the others); bytes: the limbs read once, one
   // accumulator written (the rotations' products are summed into it), each
   // rotation's key read once per launch
-  const uint32_t terms_bits = 32 - __builtin_clz(ra.nrot * a.beta);
   double split_limbs = 0;
   uint32_t split_q = 0, qbits = 0;
   for (uint32_t t = 0; t < a.nt; ++t) {
-    const uint32_t k = 64 - __builtin_clzll(c->q[ks_prime(t, a.level, a.L)]), sb = (k + 1) / 2;
+    const uint32_t k = 64 - __builtin_clzll(c->q[ks_prime(t, a.level, a.L)]);
     if (t < a.level) qbits = std::max(qbits, k);
-    if (2 * sb + 2 + terms_bits <= 64) {
+    if (split3_fits(k, ra.nrot * a.beta)) {
       split_limbs += 1;
       split_q += t < a.level ? 1 : 0;
     }

@@ -257,12 +257,13 @@ __device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, 
   run_rounds<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, LOG_V>(sm, stw, q, threadIdx.x);
 }
 
-// Canonical residue of a forward-pass output: lazy values (< 33q) by one
-// Shoup product by 1, corrected ones ([0, 4q)) by subtractions.
+// Canonical residue of a forward-pass output: lazy values (below 66 2^k) by a
+// fold, or a Shoup product by 1 where the prime has none, corrected ones
+// ([0, 4q)) by subtractions.
 template <bool LAZY>
 __device__ __forceinline__ uint64_t fwd_final(uint64_t v, const PrimeDev& pr) {
   const uint64_t q = pr.q, q2 = q + q;
-  if (LAZY) v = mul_shoup_lazy(v, 1, pr.one_sh, q);
+  if (LAZY) v = pr.delta ? fold(v, pr) : mul_shoup_lazy(v, 1, pr.one_sh, q);
   else v = v >= q2 ? v - q2 : v;
   return v >= q ? v - q : v;
 }

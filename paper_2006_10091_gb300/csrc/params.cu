@@ -12,6 +12,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -157,6 +158,9 @@ int build_tables(he_ctx* c) {
     p.q = q;
     p.k = (uint32_t)bitlen(q);
     p.mu = (uint64_t)(((u128)1 << (2 * p.k)) / q);
+    const uint64_t d = ((uint64_t)1 << p.k) - q;
+    // (the bounds the folds of he_common.cuh rely on)
+    if (p.k >= 33 && p.k <= 60 && d < (1ull << std::min({28u, p.k - 11, (2 * p.k - 4) / 3}))) p.delta = (uint32_t)d;
     p.n_inv = h_invmod((uint64_t)n % q, q);
     p.n_inv_sh = h_shoup(p.n_inv, q);
     p.one_sh = h_shoup(1, q);
@@ -208,7 +212,8 @@ int build_tables(he_ctx* c) {
   // Table: [cnt] Shoup pairs (inv_i = (Q_j/q_i)^-1 mod q_i), then [cnt][np] values
   // (Q_j/q_i) mod p for every prime index p, then their [cnt][np] Shoup companions,
   // then [cnt] Shoup pairs of inv_i * N^-1 mod q_i (the conversion's first product
-  // folded with the scaling that ends an inverse transform).
+  // folded with the scaling that ends an inverse transform), then [cnt][np] values
+  // 2^30 (Q_j/q_i) mod p (the constants of the sources' upper halves, conv_split_tile).
   {
     std::vector<uint64_t> words;
     c->modup.assign(L + 1, {});
@@ -246,6 +251,9 @@ int build_tables(he_ctx* c) {
           words.push_back(v);
           words.push_back(h_shoup(v, qi));
         }
+        for (uint32_t a = 0; a < mc.cnt; ++a)
+          for (int p = 0; p < np; ++p)
+            words.push_back(h_mulmod(words[mat0 + (size_t)a * np + p], (1ull << 30) % c->q[p], c->q[p]));
         c->modup[lv].push_back(mc);
       }
     }
@@ -265,8 +273,8 @@ int build_tables(he_ctx* c) {
   // subtracted.  Then, for the rare elements whose fixed-point sum lies
   // within its error of an integer, the integers themselves: [a][8] words of
   // P/p_k and [8] words of P (little-endian 64-bit words; a <= 8 primes below
-  // 2^61 keep sum_k u_k P/p_k and 8 P below 2^512).  4a + 2aL + 12L + 8a + 8
-  // words.
+  // 2^61 keep sum_k u_k P/p_k and 8 P below 2^512).  Last, [a][L] values
+  // 2^30 (P/p_k) mod q_t (conv_split_tile).  4a + 2aL + 12L + 8a + 8 + aL words.
   auto md_words = [&](const std::vector<int>& drop) {
     const int a = (int)drop.size();
     std::vector<uint64_t> words;
@@ -320,6 +328,9 @@ int build_tables(he_ctx* c) {
     for (int k = 0; k < a; ++k)
       for (uint64_t w : prod_words(k)) words.push_back(w);
     for (uint64_t w : prod_words(-1)) words.push_back(w);
+    for (int k = 0; k < a; ++k)
+      for (int t = 0; t < L; ++t)
+        words.push_back(h_mulmod(words[2 * a + (size_t)k * L + t], (1ull << 30) % c->q[t], c->q[t]));
     return words;
   };
   {
@@ -334,9 +345,9 @@ int build_tables(he_ctx* c) {
   }
   // The same for dividing by P q_{l-1} (ModDown merged with the rescale of a
   // multiplication at level l, 2 <= l <= L): dropped primes q_{l-1}, then the
-  // special primes; one table of 12(alpha+1) + 2(alpha+1)L + 12L + 8 words per l.
+  // special primes; one table of 12(alpha+1) + 3(alpha+1)L + 12L + 8 words per l.
   if (alpha + 1 <= 8) {
-    const size_t W = 12 * (size_t)(alpha + 1) + 2 * (size_t)(alpha + 1) * L + 12 * (size_t)L + 8;
+    const size_t W = 12 * (size_t)(alpha + 1) + 3 * (size_t)(alpha + 1) * L + 12 * (size_t)L + 8;
     std::vector<uint64_t> all(W * (L + 1), 0);
     for (int l = 2; l <= L; ++l) {
       std::vector<int> drop{l - 1};

@@ -68,3 +68,28 @@ def test_rotation_stages_match_the_separate_kernels(bits, special, sbits, first,
             for i in range(count):
                 assert np.array_equal(got[i].residues(), want[i].residues()), (shape, i)
         he.he_set_tuning(ctx, "ntt_shape", 0)
+
+
+# the conversions' sums for one to five sources, prime sizes on both sides of what they take (30-bit limbs and 61-bit
+# special primes keep the Shoup products), a last digit that is not full, inputs random and all q - 1
+@pytest.mark.parametrize("limbs,bits,special,sbits", [(5, 30, 2, 45), (4, 34, 1, 40), (7, 40, 3, 59), (9, 45, 4, 60),
+                                                      (6, 50, 5, 60), (5, 57, 2, 60), (5, 58, 2, 61), (4, 60, 3, 60)])
+def test_conversions_match_the_separate_kernels(limbs, bits, special, sbits):
+    import torch
+    import paper_2006_10091_gb300 as he
+    ctx = he.Context(12, limbs, bits, special, sbits, 2.0 ** 25, seed=7, rot_steps=[1])
+    A, B = uniform(ctx, torch, limbs, 3, 3), uniform(ctx, torch, limbs, 3, 4)
+    for t in range(limbs):
+        A[2].tensor[:, t] = ctx.primes[t] - 1
+        B[2].tensor[:, t] = ctx.primes[t] - 1
+    res = {}
+    for generic in (1, 0):
+        he.he_set_tuning(ctx, "ntt_generic", generic)
+        mul, rot, low = ctx.new_ct(limbs, 3), ctx.new_ct(limbs, 3), ctx.new_ct(limbs, 3)
+        he.he_mul_relin_rescale_batch(ctx, A, B, mul)
+        he.he_rotate_batch(ctx, A, 1, rot)
+        for a, o in zip(A, low):
+            he.he_rescale(ctx, a, o)
+        res[generic] = [c.residues() for c in mul + rot + low]
+    for got, want in zip(res[0], res[1]):
+        assert np.array_equal(got, want)
