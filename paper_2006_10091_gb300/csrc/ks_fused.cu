@@ -243,8 +243,7 @@ bool md_half_ok(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) 
 bool ks_converts_per_digit(const he_ctx* c, uint32_t level, uint32_t count) {
   if (!ks_fusable(c)) return false;
   const uint32_t alpha = (uint32_t)c->alpha, beta = (level + alpha - 1) / alpha;
-  uint32_t cnt[HE_MAX_PRIMES];
-  for (uint32_t j = 0; j < beta; ++j) cnt[j] = c->modup[level][j].cnt;
+  const uint32_t cnt = c->modup[level][0].cnt;  // (the first digit has the most limbs)
   switch (c->log_n) {
     case 12: return ks_half_n12(c, level, beta, cnt, count);
     case 13: return ks_half_n13(c, level, beta, cnt, count);

@@ -22,8 +22,8 @@
 
 namespace he {
 
-// Dynamic shared memory the all-targets conversion kernels may take.
-constexpr size_t kModupAllSmem = 160 * 1024;
+// Dynamic shared memory the conversion kernels may take.
+constexpr size_t kConvSmemMax = 200 * 1024;
 // ... and the hoisted rotate-and-sum's row pass (every digit's tile).
 constexpr size_t kRotSmemMax = 200 * 1024;
 
@@ -69,8 +69,9 @@ __device__ __forceinline__ uint64_t join_source(uint64_t x) { return (x >> 32 <<
 
 template <int TILE, int T, int CNT>
 __device__ __forceinline__ void conv_split_tile(uint64_t* sm, const uint64_t* wv, const uint64_t* w, const uint64_t* w2,
-                                                uint32_t stride, const PrimeDev& pr, const uint32_t* vv = nullptr,
-                                                const uint64_t* vP = nullptr, uint64_t h = 0) {
+                                                uint32_t stride, const PrimeDev& pr, uint32_t tid,
+                                                const uint32_t* vv = nullptr, const uint64_t* vP = nullptr,
+                                                uint64_t h = 0) {
   const uint32_t e = (pr.k + 1) >> 1, mask = (1u << e) - 1, rho = pr.delta << (2 * e - pr.k);
   const uint64_t minus = 2 * pr.q - h;
   uint32_t c0[CNT], c1[CNT], d0[CNT], d1[CNT];
@@ -83,7 +84,7 @@ __device__ __forceinline__ void conv_split_tile(uint64_t* sm, const uint64_t* wv
     d1[u] = (uint32_t)(y >> e);
   }
 #pragma unroll 4
-  for (uint32_t idx = threadIdx.x; idx < (uint32_t)TILE; idx += T) {
+  for (uint32_t idx = tid; idx < (uint32_t)TILE; idx += T) {
     uint64_t a = 0, b = 0;
     if (CNT == 1) {
       a = wv[idx];
@@ -109,13 +110,13 @@ __device__ __forceinline__ void conv_split_tile(uint64_t* sm, const uint64_t* wv
 // The same on T threads for a runtime count of 1 to 5 sources.
 template <int TILE, int T>
 __device__ __forceinline__ void conv_split(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
-                                           const uint64_t* w2, uint32_t stride, const PrimeDev& pr,
+                                           const uint64_t* w2, uint32_t stride, const PrimeDev& pr, uint32_t tid,
                                            const uint32_t* vv = nullptr, const uint64_t* vP = nullptr, uint64_t h = 0) {
-  if (cnt == 1) conv_split_tile<TILE, T, 1>(sm, wv, w, w2, stride, pr, vv, vP, h);
-  else if (cnt == 2) conv_split_tile<TILE, T, 2>(sm, wv, w, w2, stride, pr, vv, vP, h);
-  else if (cnt == 3) conv_split_tile<TILE, T, 3>(sm, wv, w, w2, stride, pr, vv, vP, h);
-  else if (cnt == 4) conv_split_tile<TILE, T, 4>(sm, wv, w, w2, stride, pr, vv, vP, h);
-  else conv_split_tile<TILE, T, 5>(sm, wv, w, w2, stride, pr, vv, vP, h);
+  if (cnt == 1) conv_split_tile<TILE, T, 1>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
+  else if (cnt == 2) conv_split_tile<TILE, T, 2>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
+  else if (cnt == 3) conv_split_tile<TILE, T, 3>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
+  else if (cnt == 4) conv_split_tile<TILE, T, 4>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
+  else conv_split_tile<TILE, T, 5>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
 }
 
 // Whether the conversion of cnt sources below 2^src_bits to q runs as
@@ -146,12 +147,12 @@ inline bool conv_split_ok(uint64_t q, uint32_t cnt, uint32_t src_bits) {
 // then to [0, q) and minus vP[vv[idx]] and h.
 template <int TILE, int T>
 __device__ __forceinline__ void conv_sum_tile(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
-                                              const uint64_t* wsh, uint32_t stride, const PrimeDev& pr,
+                                              const uint64_t* wsh, uint32_t stride, const PrimeDev& pr, uint32_t tid,
                                               const uint32_t* vv = nullptr, const uint64_t* vP = nullptr,
                                               uint64_t h = 0) {
   const uint64_t q = pr.q, q2 = q + q;
 #pragma unroll 2
-  for (uint32_t idx = threadIdx.x; idx < (uint32_t)TILE; idx += T) {
+  for (uint32_t idx = tid; idx < (uint32_t)TILE; idx += T) {
     uint64_t y = 0;
     if (cnt == 1 && !vv) {
       y = reduce64(wv[idx], pr);  // the constant is 1
@@ -226,17 +227,21 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
 // CTA: the digit's limbs are read once and their products by
 // (Q_j/q_i)^-1 mod q_i (or, for a one-limb digit, the limb itself) are kept
 // in shared memory for those targets.  The nt targets are shared evenly by
-// a.splits CTAs (conv_splits: one CTA per digit and tile when the batch fills
-// the chip).  Grid: count * beta * splits * TILES; dynamic shared memory
-// holds cnt_max * TILE more words.
-template <int LOG_N, int LOG_M, int LOG_K>
-__global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(KsFusedArgs a) {
+// a.splits CTAs, and by the G groups of T threads of a CTA, each with its own
+// tile and twiddles (the sources' tiles are what limits the CTAs of an SM, so
+// groups are how its warps are filled; conv_plan).  Grid: count * beta * splits
+// * TILES; dynamic shared memory: [G] twiddles, [G] tiles, cnt_max * TILE words.
+template <int LOG_N, int LOG_M, int LOG_K, int G>
+__global__ void __launch_bounds__(G * ((1 << (LOG_M + LOG_K)) / 8), 1024 / (G * ((1 << (LOG_M + LOG_K)) / 8)))
+ks_modup_col_all(KsFusedArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
-  constexpr uint32_t N = 1u << LOG_N;
+  constexpr uint32_t N = 1u << LOG_N, TW = S::TILE + S::TILE / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  ulonglong2* stw = reinterpret_cast<ulonglong2*>(smem_raw);
-  uint64_t* sm = reinterpret_cast<uint64_t*>(smem_raw + sizeof(ulonglong2) * S::NTW);
-  uint64_t* wv = sm + S::TILE + S::TILE / 8;  // [cnt][TILE]
+  const uint32_t grp = G == 1 ? 0u : threadIdx.x / S::T, tid = G == 1 ? threadIdx.x : threadIdx.x % S::T;
+  ulonglong2* stw = reinterpret_cast<ulonglong2*>(smem_raw) + grp * S::NTW;
+  uint64_t* sm0 = reinterpret_cast<uint64_t*>(smem_raw + sizeof(ulonglong2) * S::NTW * G);
+  uint64_t* sm = sm0 + grp * TW;
+  uint64_t* wv = sm0 + G * TW;  // [cnt][TILE]
   uint32_t b = blockIdx.x;
   const uint32_t tile = b % S::TILES;
   b /= S::TILES;
@@ -250,55 +255,55 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col_all(K
   const uint64_t* mat_sh = mat + (size_t)cnt * a.np;
   const uint64_t* mat_2 = mat_sh + (size_t)cnt * a.np + 2 * cnt;
   const uint64_t* x = a.d2c + (size_t)i * a.level * N;
-  for (uint32_t u = 0; u < cnt; ++u) {
+  const bool halves = a.split_conv && cnt > 1;
+  for (uint32_t u = grp; u < cnt; u += G) {
     const PrimeDev pa = a.primes[lo + u];
     if (a.half) {
-      // the inverse transform's column pass on this tile, then the scaling by N^-1
-      stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)(lo + u) * N, tile);
+      // the inverse transform's column pass on this tile, then the scaling by
+      // N^-1 and the product by (Q_j/q_i)^-1 as one constant
+      stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)(lo + u) * N, tile, tid, S::T);
 #pragma unroll 8
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
+      for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint32_t e = S::gidx(tile, idx & (S::K - 1), idx >> LOG_K);
         sm[idx + (idx >> 3)] = __ldg(x + (size_t)(lo + u) * N + e);
       }
-      __syncthreads();
-      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pa.q);
-    }
-    if (a.half) {  // the scaling by N^-1 and the product by (Q_j/q_i)^-1 as one constant
+      group_sync<G, S::T>(grp);
+      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pa.q, tid, grp);
       const uint64_t* tabn = mat_sh + (size_t)cnt * a.np;
       const uint64_t w = tabn[2 * u], wsh = tabn[2 * u + 1];
 #pragma unroll 8
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T)
-      {
+      for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint64_t v = mul_shoup(sm[idx + (idx >> 3)], w, wsh, pa.q);
-        wv[(size_t)u * S::TILE + idx] = a.split_conv && cnt > 1 ? split_source(v) : v;
+        wv[(size_t)u * S::TILE + idx] = halves ? split_source(v) : v;
       }
     } else {
 #pragma unroll 8
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
+      for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint32_t e = S::gidx(tile, idx & (S::K - 1), idx >> LOG_K);
         const uint64_t xv = __ldg(x + (size_t)(lo + u) * N + e);
         const uint64_t v = cnt == 1 ? xv : mul_shoup(xv, tab[2 * u], tab[2 * u + 1], pa.q);
-        wv[(size_t)u * S::TILE + idx] = a.split_conv && cnt > 1 ? split_source(v) : v;
+        wv[(size_t)u * S::TILE + idx] = halves ? split_source(v) : v;
       }
     }
     // the next limb's staging overwrites stw and sm: wait for every thread
-    __syncthreads();
+    group_sync<G, S::T>(grp);
   }
-  for (uint32_t t = part * a.nt / a.splits; t < t_end; ++t) {
+  if (G > 1) __syncthreads();  // every group's sources
+  for (uint32_t t = part * a.nt / a.splits + grp; t < t_end; t += G) {
     if (t >= lo && t < lo + cnt) continue;  // the digit's own limbs are used as they are
     const uint32_t prime = ks_prime(t, a.level, a.L);
     const PrimeDev pr = a.primes[prime];
     // the previous target's rounds ended with a barrier, and its write-out
     // reads only the words each thread rewrites below
-    stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)prime * N, tile);
-    if (a.split_conv) conv_split<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_2 + prime, a.np, pr);
-    else conv_sum_tile<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr);
-    __syncthreads();
+    stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)prime * N, tile, tid, S::T);
+    if (a.split_conv) conv_split<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_2 + prime, a.np, pr, tid);
+    else conv_sum_tile<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr, tid);
+    group_sync<G, S::T>(grp);
     uint64_t* out = a.ext + (((size_t)i * a.beta + j) * a.nt + t) * N;
-    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
+    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
+    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
 #pragma unroll 8
-    for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
+    for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
       const uint32_t xx = idx >> LOG_K, k = idx & (S::K - 1);
       out[S::gidx(tile, k, xx)] = sm[idx + (idx >> 3)];
     }
@@ -829,15 +834,19 @@ struct MdArgs {
 // Grid: count * 2 * splits * TILES; the conversion's per-special-prime terms
 // and the multiple v of P are computed once per element and kept in shared
 // memory ([alpha][TILE] words and [TILE] counts) for the CTA's share of the
-// level target limbs (all of them when the batch fills the chip, conv_splits).
-template <int LOG_N, int LOG_M, int LOG_K>
-__global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs a) {
+// level target limbs, which its G groups of T threads take in turn (as in
+// ks_modup_col_all).
+template <int LOG_N, int LOG_M, int LOG_K, int G>
+__global__ void __launch_bounds__(G * ((1 << (LOG_M + LOG_K)) / 8), 1024 / (G * ((1 << (LOG_M + LOG_K)) / 8)))
+md_conv_col(MdArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
-  constexpr uint32_t N = 1u << LOG_N;
+  constexpr uint32_t N = 1u << LOG_N, TW = S::TILE + S::TILE / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  ulonglong2* stw = reinterpret_cast<ulonglong2*>(smem_raw);
-  uint64_t* sm = reinterpret_cast<uint64_t*>(smem_raw + sizeof(ulonglong2) * S::NTW);
-  uint64_t* wv = sm + S::TILE + S::TILE / 8;                          // [alpha][TILE]
+  const uint32_t grp = G == 1 ? 0u : threadIdx.x / S::T, tid = G == 1 ? threadIdx.x : threadIdx.x % S::T;
+  ulonglong2* stw = reinterpret_cast<ulonglong2*>(smem_raw) + grp * S::NTW;
+  uint64_t* sm0 = reinterpret_cast<uint64_t*>(smem_raw + sizeof(ulonglong2) * S::NTW * G);
+  uint64_t* sm = sm0 + grp * TW;
+  uint64_t* wv = sm0 + G * TW;                                                  // [alpha][TILE]
   uint32_t* vv = reinterpret_cast<uint32_t*>(wv + (size_t)a.alpha * S::TILE);  // [TILE]
   uint32_t b = blockIdx.x;
   const uint32_t tile = b % S::TILES;
@@ -853,26 +862,27 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
   const uint64_t* phat = wlo + a.alpha + 9 * (size_t)a.L;         // [alpha][8] words of P/p_u, then [8] of P
   const uint64_t* mat_2 = phat + 8 * (size_t)a.alpha + 8;         // (alpha > 1)
   const uint64_t* yP = a.yP + (size_t)i * a.yp_stride + (size_t)p * a.yp_pstride;
+  const bool halves = a.split_conv && a.alpha > 1;
   // exact conversion: sum_u w_u (P/p_u) - v P, w_u = [y_u (P/p_u)^-1]_{p_u},
   // v = floor(sum_u w_u / p_u) (64.64 fixed point, resolved exactly near an
   // integer)
-  for (uint32_t u = 0; u < a.alpha; ++u) {
+  for (uint32_t u = grp; u < a.alpha; u += G) {
     const PrimeDev pp = a.primes[a.spr[u]];
     const uint64_t* src = yP + (size_t)u * N;
     if (a.half) {
       // the inverse transform's column pass on this tile, then the scaling by N^-1
-      stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)a.spr[u] * N, tile);
+      stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)a.spr[u] * N, tile, tid, S::T);
 #pragma unroll 8
-      for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T)
+      for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T)
         sm[idx + (idx >> 3)] = __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
-      __syncthreads();
-      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pp.q);
+      group_sync<G, S::T>(grp);
+      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pp.q, tid, grp);
     }
     // the thread's words of the limb first (eight loads in flight), then their products
     uint64_t y0[S::TILE / S::T];
 #pragma unroll
     for (int v = 0; v < S::TILE / S::T; ++v) {
-      const uint32_t idx = threadIdx.x + v * S::T;
+      const uint32_t idx = tid + v * S::T;
       y0[v] = a.half ? sm[idx + (idx >> 3)] : __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
     }
     const uint64_t h = hP[u], w = a.md[2 * u], wsh = a.md[2 * u + 1];
@@ -880,41 +890,42 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) md_conv_col(MdArgs
     for (int v = 0; v < S::TILE / S::T; ++v) {
       if (a.half) y0[v] = mul_shoup(y0[v], pp.n_inv, pp.n_inv_sh, pp.q);
       const uint64_t x = mul_shoup(add_mod(y0[v], h, pp.q), w, wsh, pp.q);
-      wv[(size_t)u * S::TILE + threadIdx.x + v * S::T] = a.split_conv && a.alpha > 1 ? split_source(x) : x;
+      wv[(size_t)u * S::TILE + tid + v * S::T] = halves ? split_source(x) : x;
     }
     // the next limb's staging overwrites stw and sm: wait for every thread
-    if (a.half) __syncthreads();
+    if (a.half) group_sync<G, S::T>(grp);
   }
+  if (G > 1) __syncthreads();  // every group's sources
 #pragma unroll 2
-  for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
+  for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += G * S::T) {
     uint64_t fs = 0;
     uint32_t v = 0;
     if (a.alpha > 1) {
-      for (uint32_t u = 0; u < a.alpha; ++u)
-      {
+      for (uint32_t u = 0; u < a.alpha; ++u) {
         const uint64_t x = wv[(size_t)u * S::TILE + idx];
-        frac_acc(a.split_conv ? join_source(x) : x, a.primes[a.spr[u]].one_sh, wlo[u], &fs, &v);
+        frac_acc(halves ? join_source(x) : x, a.primes[a.spr[u]].one_sh, wlo[u], &fs, &v);
       }
       if (frac_in_window(fs, a.alpha))
-        v = exact_lift_multiple(wv + idx, S::TILE, a.alpha, phat, phat + 8 * (size_t)a.alpha, v, a.split_conv);
+        v = exact_lift_multiple(wv + idx, S::TILE, a.alpha, phat, phat + 8 * (size_t)a.alpha, v, halves);
     }
     vv[idx] = v;
   }
-  for (uint32_t t = part * a.level / a.splits; t < t_end; ++t) {
+  if (G > 1) __syncthreads();
+  for (uint32_t t = part * a.level / a.splits + grp; t < t_end; t += G) {
     const PrimeDev pr = a.primes[t];
     const uint64_t hQ = hP[a.alpha + t];
     const uint64_t* vP = wlo + a.alpha + a.L + (size_t)t * 8;  // v P mod q_t, v < 8
-    stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)t * N, tile);
+    stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)t * N, tile, tid, S::T);
     if (a.split_conv)
-      conv_split<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_2 + t, a.L, pr, vv, vP, hQ);
+      conv_split<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_2 + t, a.L, pr, tid, vv, vP, hQ);
     else
-      conv_sum_tile<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, vv, vP, hQ);
-    __syncthreads();
-    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
+      conv_sum_tile<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, tid, vv, vP, hQ);
+    group_sync<G, S::T>(grp);
+    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
+    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
     uint64_t* out = a.conv + (((size_t)i * 2 + p) * a.level + t) * N;
 #pragma unroll 8
-    for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
+    for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
       const uint32_t xx = idx >> LOG_K, k = idx & (S::K - 1);
       out[S::gidx(tile, k, xx)] = sm[idx + (idx >> 3)];
     }
@@ -991,67 +1002,78 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
   }
 }
 
-// Shared memory of md_conv_col with nd dropped limbs.
+// Dynamic shared memory of the conversion kernels with ns source limbs (md:
+// and the lift's counts) and g groups.
 template <int LOG_N, int M1, int K1>
-size_t md_col_smem(uint32_t nd) {
+size_t conv_smem(uint32_t ns, bool md, int g) {
   using SC = Shape<LOG_N, M1, K1, true>;
-  return sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8) +
-         (sizeof(uint64_t) * nd + sizeof(uint32_t)) * SC::TILE;
+  return (sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8)) * g +
+         (sizeof(uint64_t) * ns + (md ? sizeof(uint32_t) : 0)) * SC::TILE;
 }
 
-// How a conversion kernel's target limbs are shared: `blocks` groups of CTAs
-// (digits or parts times tiles), of which `slots` CTAs run at a time; a CTA
-// pays `setup` and then one unit per target.  Alone on its SM a CTA is bound by
-// latency (a unit takes 4.4 us at N = 2^13), so a batch that leaves CTA slots
-// free is split as far as they reach; together the CTAs of an SM finish a unit
-// every 2.1 us, so the repeated setup must not cost more than the shorter
-// chains give: the time is the larger of the chain and 0.48 of the SM's units.
-// One rotation at N = 2^13, level 19: 20 and 8 CTAs walked 19 to 23 targets
-// each, 101 and 122 us, split 25 and 23.  288 CTAs of 9 units at N = 2^12 stay
-// as they are: 36 us, split in two 48.
-inline uint32_t conv_splits(size_t blocks, size_t slots, uint32_t targets, double setup, double* cost) {
-  uint32_t best = 1;
-  double bc = 0.0;
-  for (uint32_t s = 1; s <= targets && (s == 1 || blocks * s <= slots); ++s) {
-    const double chain = (double)((blocks * s + slots - 1) / slots) * (setup + (double)((targets + s - 1) / s));
-    const double c = std::max(chain, 0.48 / 152 * (double)blocks * (s * setup + targets));
-    if (s == 1 || c < bc) {
-      bc = c;
-      best = s;
+// How a conversion kernel's target limbs are shared: `blocks` CTAs (digits or
+// parts times tiles), each split in `splits`, of `groups` groups of threads.  A
+// CTA pays a setup of `setup` units per source limb and then one unit per
+// target (a target's conversion and column pass), its groups side by side.  A
+// group's chain is bound by latency (a unit takes 4.4 us alone on its SM, 5.9
+// beside two others, N = 2^13), so a batch that leaves CTA slots free is split
+// as far as they reach; together an SM's groups finish a unit every 2.1 us, so
+// the repeated setup must not cost more than the shorter chains give: the time
+// is the larger of the chain and 0.48 of the SM's units.  One rotation at N = 2^13, level 19: 20 and
+// 8 CTAs walked 19 to 23 targets each, 101 and 122 us, split 25 and 23.
+// 288 CTAs of 9 units at N = 2^12 stay as they are: 36 us, split in two 48.
+// Groups instead of splits or where the sources leave an SM few CTAs: five
+// ciphertexts' step at N = 2^13 1072 us with one group, 999 with two; ModUp of
+// eight ciphertexts at N = 2^16 740 and 667.
+struct ConvPlan {
+  uint32_t splits = 1;
+  int groups = 1;
+  double cost = 0.0;
+  size_t smem = 0;  // 0: no number of groups fits
+};
+constexpr double kSetupHalf = 1.0, kSetupFull = 0.3;  // (with the inverse column pass; a load and a product)
+
+template <int LOG_N, int M1, int K1>
+ConvPlan conv_plan(const he_ctx* c, size_t blocks, uint32_t ns, bool md, uint32_t targets, bool half) {
+  using SC = Shape<LOG_N, M1, K1, true>;
+  const double per = half ? kSetupHalf : kSetupFull;
+  ConvPlan best;
+  size_t best_warps = 0;
+  for (int g : {1, 2, 4}) {
+    const size_t sm = conv_smem<LOG_N, M1, K1>(ns, md, g);
+    if (g * SC::T > 1024 || sm > kConvSmemMax || (uint32_t)g > targets) continue;
+    const size_t ctas = std::max<size_t>(1, std::min<size_t>(c->smem_per_sm / (sm + 1024), 1024 / (g * SC::T)));
+    const size_t warps = ctas * g * SC::T / 32, slots = 152 * ctas;
+    for (uint32_t s = 1; s <= targets && (s == 1 || blocks * s <= slots); ++s) {
+      const uint32_t chain_t = ((targets + s - 1) / s + g - 1) / g;
+      // (groups beside each other slow a chain by 0.35 each: rotation at N = 2^13 97 us with 0.17, 93 with 0.35)
+      const double beside = 0.35 * (double)(std::min(ctas, (blocks * s + 151) / 152) * g - 1);
+      const double chain =
+          (double)((blocks * s + slots - 1) / slots) * (per * ((ns + g - 1) / g) + chain_t) * (1.0 + beside);
+      const double cost = std::max(chain, 0.48 / 152 * (double)blocks * (s * per * ns + targets));
+      // equal times: more resident warps, then fewer CTAs and groups
+      if (!best.smem || cost < best.cost || (cost == best.cost && warps > best_warps)) {
+        best = ConvPlan{s, g, cost, sm};
+        best_warps = warps;
+      }
     }
   }
-  if (cost) *cost = bc;
   return best;
 }
 
-// CTAs of `threads` threads and `smem` bytes that run at a time.
-inline size_t conv_slots(const he_ctx* c, size_t smem, int threads) {
-  return 152 * std::max<size_t>(1, std::min<size_t>(c->smem_per_sm / (smem + 1024), 1024 / threads));
-}
-
-// Units (one target's conversion and column pass) a conversion kernel pays
-// before its targets for one source limb: the inverse transform's column pass
-// on it when it finishes that transform itself, a load and a product if not.
-constexpr double kSetupHalf = 1.0, kSetupFull = 0.3;
-// ... and the units a column pass launched by itself costs instead.
+// Units a column pass launched by itself costs.
 inline double col_pass_units(size_t polys, int tiles) {
   return 1.5 + std::max(1.0, 0.48 / 152 * (double)(polys * tiles));
 }
-
-template <int LOG_N, int M1, int K1>
-size_t md_col_smem(uint32_t nd);
 
 // Whether md_conv_col finishes the dropped limbs' inverse transform itself.
 template <int LOG_N, int M1, int K1>
 bool md_half(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
   using SC = Shape<LOG_N, M1, K1, true>;
-  const size_t sm = md_col_smem<LOG_N, M1, K1>(nd), blocks = (size_t)count * 2 * SC::TILES;
-  if (sm > kModupAllSmem) return false;
-  const size_t slots = conv_slots(c, sm, SC::T);
-  double half, full;
-  conv_splits(blocks, slots, targets, kSetupHalf * nd, &half);
-  conv_splits(blocks, slots, targets, kSetupFull * nd, &full);
-  return half <= full + col_pass_units((size_t)count * 2 * nd, SC::TILES);
+  const size_t blocks = (size_t)count * 2 * SC::TILES;
+  const ConvPlan half = conv_plan<LOG_N, M1, K1>(c, blocks, nd, true, targets, true);
+  const ConvPlan full = conv_plan<LOG_N, M1, K1>(c, blocks, nd, true, targets, false);
+  return half.smem && half.cost <= full.cost + col_pass_units((size_t)count * 2 * nd, SC::TILES);
 }
 
 template <int LOG_N, int M1, int K1, int M2, int K2>
@@ -1064,16 +1086,23 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   a.split_conv = 1;
   for (uint32_t t = 0; t < a.level; ++t) a.split_conv &= conv_split_ok(c->q[t], a.alpha, src_bits) ? 1 : 0;
   using SR = Shape<LOG_N, M2, K2, false>;
-  const size_t smc = md_col_smem<LOG_N, M1, K1>(a.alpha);
+  const ConvPlan plan =
+      conv_plan<LOG_N, M1, K1>(c, (size_t)count * 2 * SC::TILES, a.alpha, true, a.level, a.half != 0);
   const size_t smr = sizeof(ulonglong2) * SR::NTW + sizeof(uint64_t) * (SR::TILE + SR::TILE / 8);
-  if (smc > kModupAllSmem) {  // too many special primes for this tile: the caller runs the unfused sequence
+  if (!plan.smem) {  // too many special primes for this tile: the caller runs the unfused sequence
     *handled = false;
     if (a.half) return fail(HE_EINVAL, "md_fused: half-transformed input needs the fused kernels");
     return HE_OK;
   }
   *handled = true;
-  static std::atomic<unsigned long long> attr_col{0}, attr_row{0};
-  HE_TRY(set_smem_attr_once(attr_col, c->device, (const void*)md_conv_col<LOG_N, M1, K1>, kModupAllSmem));
+  static std::atomic<unsigned long long> attr_row{0};
+  const auto conv_kernel = [&]() -> void (*)(MdArgs) {
+    if constexpr (4 * SC::T <= 1024)
+      if (plan.groups == 4) return md_conv_col<LOG_N, M1, K1, 4>;
+    return plan.groups == 2 ? md_conv_col<LOG_N, M1, K1, 2> : md_conv_col<LOG_N, M1, K1, 1>;
+  }();
+  static std::atomic<unsigned long long> attr_g[3]{};
+  HE_TRY(set_smem_attr_once(attr_g[plan.groups >> 1], c->device, (const void*)conv_kernel, kConvSmemMax));
   HE_TRY(set_smem_attr_once(attr_row, c->device, (const void*)md_row_combine<LOG_N, M2, K2>, smr));
   const double n = (double)(1u << LOG_N);
   const double polys = 2.0 * count * a.level;  // transformed limbs
@@ -1081,14 +1110,12 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   const char* nm_row = a.kind == 1 ? "rescale_ntt_final" : a.kind == 2 ? "moddown_rescale_ntt_combine"
                                                                        : "moddown_ntt_combine";
   {
-    size_t blocks = (size_t)count * 2 * SC::TILES;
-    a.splits = conv_splits(blocks, conv_slots(c, smc, SC::T), a.level, (a.half ? kSetupHalf : kSetupFull) * a.alpha,
-                           nullptr);
-    blocks *= a.splits;
+    a.splits = plan.splits;
+    const size_t blocks = (size_t)count * 2 * SC::TILES * a.splits;
     // with a half-transformed input, also the dropped limbs' inverse column pass
     const double bfly = polys * n / 2 * M1 + (a.half ? 2.0 * count * a.alpha * n / 2 * M1 : 0.0);
     ProfScope prof(c, nm_col, bfly + polys * n * a.alpha, n * 8 * (2.0 * count * a.alpha + polys), 0.0, bfly);
-    md_conv_col<LOG_N, M1, K1><<<(unsigned)blocks, SC::T, smc, c->stream>>>(a);
+    conv_kernel<<<(unsigned)blocks, plan.groups * SC::T, plan.smem, c->stream>>>(a);
   }
   HE_CUDA(cudaGetLastError());
   {
@@ -1101,29 +1128,15 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   return HE_OK;
 }
 
-// Dynamic shared memory of ks_modup_col_all for these digits.
-template <int LOG_N, int M1, int K1>
-size_t ks_all_smem(const he_ctx* c, uint32_t beta, const uint32_t* cnt) {
-  using SC = Shape<LOG_N, M1, K1, true>;
-  uint32_t cnt_max = 0;
-  for (uint32_t j = 0; j < beta; ++j) cnt_max = std::max(cnt_max, cnt[j]);
-  (void)c;
-  return sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8) +
-         sizeof(uint64_t) * (size_t)cnt_max * SC::TILE;
-}
-
 // Whether ks_modup_col_all finishes the input's inverse transform itself.
 template <int LOG_N, int M1, int K1>
-bool ks_half(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
+bool ks_half(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint32_t count) {
   using SC = Shape<LOG_N, M1, K1, true>;
-  const size_t sm = ks_all_smem<LOG_N, M1, K1>(c, beta, cnt), blocks = (size_t)count * beta * SC::TILES;
-  if (sm > kModupAllSmem) return false;
-  const size_t slots = conv_slots(c, sm, SC::T);
+  const size_t blocks = (size_t)count * beta * SC::TILES;
   const uint32_t nt = level + (uint32_t)c->alpha;
-  double half, full;
-  conv_splits(blocks, slots, nt, kSetupHalf * cnt[0], &half);
-  conv_splits(blocks, slots, nt, kSetupFull * cnt[0], &full);
-  return half <= full + col_pass_units((size_t)count * level, SC::TILES);
+  const ConvPlan half = conv_plan<LOG_N, M1, K1>(c, blocks, cnt, false, nt, true);
+  const ConvPlan full = conv_plan<LOG_N, M1, K1>(c, blocks, cnt, false, nt, false);
+  return half.smem && half.cost <= full.cost + col_pass_units((size_t)count * level, SC::TILES);
 }
 
 // The ModUp + column-pass launch shared by the key switch and the hoisted
@@ -1139,9 +1152,8 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
       a.split_conv &= conv_split_ok(c->q[ks_prime(t, a.level, a.L)], a.cnt[j], src_bits) ? 1 : 0;
   using SC = Shape<LOG_N, M1, K1, true>;
   const size_t smc = sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8);
-  static std::atomic<unsigned long long> attr_one{0}, attr_all{0};
+  static std::atomic<unsigned long long> attr_one{0}, attr_g[3]{};
   HE_TRY(set_smem_attr_once(attr_one, c->device, (const void*)ks_modup_col<LOG_N, M1, K1>, smc));
-  HE_TRY(set_smem_attr_once(attr_all, c->device, (const void*)ks_modup_col_all<LOG_N, M1, K1>, kModupAllSmem));
   const double n = (double)(1u << LOG_N);
   double own = 0;  // limbs each ciphertext takes as they are
   for (uint32_t j = 0; j < a.beta; ++j) own += a.cnt[j];
@@ -1156,14 +1168,20 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
     const double bfly = count * (conv * n / 2 * M1 + (a.half ? (double)a.level * n / 2 * M1 : 0.0));
     ProfScope prof(c, "ks_modup_ntt", count * (conv * n / 2 * M1 + conv_products * n + inv_bfly),
                    count * n * 8 * (a.level + conv), 0.0, bfly);
-    const size_t sma = ks_all_smem<LOG_N, M1, K1>(c, a.beta, a.cnt);
-    if (a.half && sma > kModupAllSmem) return fail(HE_EINVAL, "ks_fused: half-transformed input needs the all-targets kernel");
-    if (sma <= kModupAllSmem) {  // the targets of one digit and tile in `splits` CTAs
-      size_t blocks = (size_t)count * a.beta * SC::TILES;
-      a.splits = conv_splits(blocks, conv_slots(c, sma, SC::T), a.nt, (a.half ? kSetupHalf : kSetupFull) * a.cnt[0],
-                             nullptr);
-      blocks *= a.splits;
-      ks_modup_col_all<LOG_N, M1, K1><<<(unsigned)blocks, SC::T, sma, c->stream>>>(a);
+    // (the first digit has the most limbs)
+    const ConvPlan plan =
+        conv_plan<LOG_N, M1, K1>(c, (size_t)count * a.beta * SC::TILES, a.cnt[0], false, a.nt, a.half != 0);
+    if (a.half && !plan.smem) return fail(HE_EINVAL, "ks_fused: half-transformed input needs the all-targets kernel");
+    if (plan.smem) {  // the targets of one digit and tile in `splits` CTAs
+      const auto kernel = [&]() -> void (*)(KsFusedArgs) {
+        if constexpr (4 * SC::T <= 1024)
+          if (plan.groups == 4) return ks_modup_col_all<LOG_N, M1, K1, 4>;
+        return plan.groups == 2 ? ks_modup_col_all<LOG_N, M1, K1, 2> : ks_modup_col_all<LOG_N, M1, K1, 1>;
+      }();
+      HE_TRY(set_smem_attr_once(attr_g[plan.groups >> 1], c->device, (const void*)kernel, kConvSmemMax));
+      a.splits = plan.splits;
+      const size_t blocks = (size_t)count * a.beta * SC::TILES * a.splits;
+      kernel<<<(unsigned)blocks, plan.groups * SC::T, plan.smem, c->stream>>>(a);
     } else {
       const size_t blocks = (size_t)count * a.beta * a.nt * SC::TILES;
       ks_modup_col<LOG_N, M1, K1><<<(unsigned)blocks, SC::T, smc, c->stream>>>(a);
@@ -1318,7 +1336,7 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   size_t ks_rot_smem_n##NN(const he_ctx* c, uint32_t beta);                          \
   int md_fused_n##NN(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled);     \
   bool md_half_n##NN(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count); \
-  bool ks_half_n##NN(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count);
+  bool ks_half_n##NN(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint32_t count);
 HE_KS_FUSED_DECL(12)
 HE_KS_FUSED_DECL(13)
 HE_KS_FUSED_DECL(14)

@@ -27,7 +27,7 @@ bool md_half_n14(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count)
        : sh == 2 ? md_half<14, 8, 3>(c, nd, targets, count) : md_half<14, 5, 6>(c, nd, targets, count);
 }
 
-bool ks_half_n14(const he_ctx* c, uint32_t level, uint32_t beta, const uint32_t* cnt, uint32_t count) {
+bool ks_half_n14(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint32_t count) {
   const int sh = c->ntt_shape;
   return sh == 1 ? ks_half<14, 7, 4>(c, level, beta, cnt, count)
        : sh == 2 ? ks_half<14, 8, 3>(c, level, beta, cnt, count) : ks_half<14, 5, 6>(c, level, beta, cnt, count);

@@ -235,9 +235,19 @@ __device__ __forceinline__ void stage_twiddles(ulonglong2* stw, const ulonglong2
                                                   (uint32_t)Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>::T);
 }
 
-// All rounds of one pass on the tile in shared memory (ends with a barrier).
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3>
-__device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, uint64_t q, uint32_t tid) {
+// Barrier of the T threads that share a tile: the CTA's, or, when G groups of T
+// threads (T a multiple of 32) each have a tile, named barrier grp + 1.
+template <int G, int T>
+__device__ __forceinline__ void group_sync(uint32_t grp) {
+  if (G == 1) __syncthreads();
+  else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(T) : "memory");
+}
+
+// All rounds of one pass on the tile in shared memory (ends with a barrier of
+// the tile's group).
+template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3, int G = 1>
+__device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, uint64_t q, uint32_t tid,
+                                           uint32_t grp = 0) {
   constexpr int NR = (LOG_M + LOG_V - 1) / LOG_V;
 #pragma unroll
   for (int rr = 0; rr < NR; ++rr) {
@@ -248,7 +258,7 @@ __device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, 
     else if (R == 3) round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 3, LOG_V>(sm, stw, sig0, q, tid);
     else if (R == 2) round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 2, LOG_V>(sm, stw, sig0, q, tid);
     else round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 1, LOG_V>(sm, stw, sig0, q, tid);
-    __syncthreads();
+    group_sync<G, Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>::T>(grp);
   }
 }
 
