@@ -191,9 +191,8 @@ int mul_plain_dev(he_ctx* c, CtBatch A, const int64_t* d_coeffs, CtBatch O, uint
   if (!pt) return fail(HE_ENOMEM, "plaintext scratch too small");
   {
     ProfScope prof(c, "elementwise", 0.0, (double)level * n * 16);
-    k_signed_to_residues<<<grid_for((size_t)level * n), 256, 0, c->stream>>>(d_coeffs, pt, level, c->log_n,
-                                                                             c->d_primes);
-    HE_CUDA(cudaGetLastError());
+    HE_TRY(launch_pdl(k_signed_to_residues, grid_for((size_t)level * n), 256, 0, c->stream,
+                      d_coeffs, pt, level, c->log_n, c->d_primes));
   }
   PolyBatch b;
   b.src = pt;
@@ -207,9 +206,8 @@ int mul_plain_dev(he_ctx* c, CtBatch A, const int64_t* d_coeffs, CtBatch O, uint
   b.skip_beta = 1;
   HE_TRY(ntt_forward(c, b));
   ProfScope prof(c, "elementwise", 0.0, (double)(4 * count + 1) * level * n * 8);
-  k_mul_plain<<<grid_for((size_t)count * level * n), 256, 0, c->stream>>>(A, pt, O, level, count, c->log_n,
-                                                                          c->d_primes);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_mul_plain, grid_for((size_t)count * level * n), 256, 0, c->stream,
+                    A, pt, O, level, count, c->log_n, c->d_primes));
   return HE_OK;
 }
 

@@ -27,6 +27,7 @@ __device__ __forceinline__ uint32_t rmod(size_t& r, uint32_t d) {
 // ---- tensor product: (a0 b0, a0 b1 + a1 b0, a1 b1) ---------------------------
 __global__ void k_tensor(CtBatch A, CtBatch B, CtBatch D, uint64_t* d2, uint64_t d2_stride,
                          uint32_t level, uint32_t count, int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -273,6 +274,7 @@ __global__ void k_ks_combine(const uint64_t* acc, uint64_t acc_stride, uint32_t 
 // q_l holds V = acc + P d (P d vanishes on the special primes).
 __global__ void k_add_pd(uint64_t* acc, uint64_t acc_stride, uint32_t nt, CtBatch d, uint32_t l, uint64_t Pl,
                          uint64_t Pl_sh, uint32_t count, int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   const size_t total = (size_t)count * 2 * n;
   const uint64_t q = primes[l].q;
@@ -352,6 +354,7 @@ __global__ void k_automorph(CtBatch in, CtBatch out, uint32_t nparts, uint32_t l
 // op 0: a + b, 1: a - b
 __global__ void k_addsub(CtBatch A, CtBatch B, CtBatch O, int op, uint32_t level, uint32_t count,
                          int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * 2 * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -373,6 +376,7 @@ __global__ void k_addsub(CtBatch A, CtBatch B, CtBatch O, int op, uint32_t level
 // Multiply both parts by per-limb constants (Shoup pairs in kc).
 __global__ void k_mul_const(CtBatch A, CtBatch O, LimbConsts kc, uint32_t level, uint32_t count,
                             int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * 2 * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -393,6 +397,7 @@ __global__ void k_mul_const(CtBatch A, CtBatch O, LimbConsts kc, uint32_t level,
 // Add per-limb constants to every evaluation of part 0; copy part 1.
 __global__ void k_add_const(CtBatch A, CtBatch O, LimbConsts kc, uint32_t level, uint32_t count,
                             int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * 2 * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -411,6 +416,7 @@ __global__ void k_add_const(CtBatch A, CtBatch O, LimbConsts kc, uint32_t level,
 // Multiply both parts by a plaintext in evaluation form pt[level][N].
 __global__ void k_mul_plain(CtBatch A, const uint64_t* pt, CtBatch O, uint32_t level, uint32_t count,
                             int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * 2 * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -431,6 +437,7 @@ __global__ void k_mul_plain(CtBatch A, const uint64_t* pt, CtBatch O, uint32_t l
 
 // Copy limbs [0, level) of both parts (level drop / re-layout).
 __global__ void k_copy_limbs(CtBatch A, CtBatch O, uint32_t level, uint32_t count, int log_n) {
+  pdl_wait();
   const uint32_t n = 1u << log_n, half = n >> 1;
   const size_t total = (size_t)count * 2 * level * half;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {

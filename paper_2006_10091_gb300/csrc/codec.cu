@@ -88,6 +88,7 @@ __device__ __forceinline__ void fft_butterfly(double2* sm, uint32_t i0, uint32_t
 // Stages h = 1 .. 2^(m1-1) on the block of 2^m1 points blockIdx.x.
 template <bool ENC>
 __global__ void k_fft_first(FftArgs a) {
+  pdl_wait();
   extern __shared__ double2 fsm[];
   const uint32_t m = 1u << a.m1, base = blockIdx.x << a.m1;
   for (uint32_t x = threadIdx.x; x < m; x += blockDim.x) {
@@ -117,6 +118,7 @@ __global__ void k_fft_first(FftArgs a) {
 // The remaining stages on columns [kFftCols blockIdx.x, ...): points x 2^m1 + f.
 template <bool ENC>
 __global__ void k_fft_second(FftArgs a) {
+  pdl_wait();
   extern __shared__ double2 fsm[];
   const uint32_t n = 1u << a.log_n;
   const int m2 = a.log_n - a.m1;
@@ -161,10 +163,10 @@ static int fft_run(he_ctx* c, FftArgs a) {
   a.tab = (const double2*)c->d_fft;
   a.slot_of = c->d_slot_of;
   const uint32_t p1 = 1u << a.m1, p2 = (uint32_t)kFftCols << (c->log_n - a.m1);
-  k_fft_first<ENC><<<c->n / p1, p1 / 2, sizeof(double2) * p1, c->stream>>>(a);
-  HE_CUDA(cudaGetLastError());
-  k_fft_second<ENC><<<c->n / p2, p2 / 2, sizeof(double2) * p2, c->stream>>>(a);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_fft_first<ENC>, c->n / p1, p1 / 2, sizeof(double2) * p1, c->stream,
+                    a));
+  HE_TRY(launch_pdl(k_fft_second<ENC>, c->n / p2, p2 / 2, sizeof(double2) * p2, c->stream,
+                    a));
   return HE_OK;
 }
 
@@ -187,6 +189,7 @@ int encode_dev(he_ctx* c, const double* d_z, size_t n_slots, double scale, int64
 // ---- decryption -----------------------------------------------------------------
 __global__ void k_decrypt_dot(CtBatch A, const uint64_t* s, uint64_t* m, uint32_t level, int log_n,
                               const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   const size_t total = (size_t)level * n;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -205,6 +208,7 @@ struct GarnerArgs {
 // (q_0..q_{i'-1}) mod q_i at [i][i'].
 __global__ void k_crt_double(const uint64_t* m, double* out, uint32_t level, int log_n,
                              const PrimeDev* primes, const uint64_t* gar, uint32_t L, GarnerArgs ga) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
     uint64_t d[HE_MAX_PRIMES];
@@ -240,8 +244,8 @@ int decrypt_dev(he_ctx* c, const he_ct* ct, uint64_t* m, double* d_coeffs) {
   const uint32_t n = c->n, level = ct->level;
   const size_t lw = (size_t)level * n;
   CtBatch A{ct->data, 0, ct->cap, 0};
-  k_decrypt_dot<<<grid_for(lw), 256, 0, c->stream>>>(A, c->d_s, m, level, c->log_n, c->d_primes);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_decrypt_dot, grid_for(lw), 256, 0, c->stream,
+                    A, c->d_s, m, level, c->log_n, c->d_primes));
   PolyBatch b;
   b.src = m;
   b.dst = m;
@@ -261,9 +265,8 @@ int decrypt_dev(he_ctx* c, const he_ct* ct, uint64_t* m, double* d_coeffs) {
     ga.half[i] = (uint64_t)(cur / 2);
     carry = cur % 2;
   }
-  k_crt_double<<<grid_for(n), 256, 0, c->stream>>>(m, d_coeffs, level, c->log_n, c->d_primes,
-                                                   c->d_garner, (uint32_t)c->L, ga);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_crt_double, grid_for(n), 256, 0, c->stream,
+                    m, d_coeffs, level, c->log_n, c->d_primes, c->d_garner, (uint32_t)c->L, ga));
   return HE_OK;
 }
 

@@ -46,6 +46,19 @@ __device__ __forceinline__ uint64_t mul_shoup(uint64_t a, uint64_t w, uint64_t w
   return r >= q ? r - q : r;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl may start
+// before its predecessor in the stream has finished, so it reads and writes
+// nothing that another kernel or copy writes before pdl_wait (which returns when
+// the predecessor has finished and its writes are visible); only the context's
+// constants (primes, twiddles, conversion tables, keys) may be read earlier, and
+// only they through the read-only path (__ldg): other words change during such
+// a kernel's life.  No kernel triggers its successor early
+// (griddepcontrol.launch_dependents), so it starts as the predecessor's CTAs
+// exit: CTAs placed while a grid still covers part of the chip crowd on the rest
+// of it (16 multiplications at N = 2^12 82 us without the attribute, 68 with it,
+// 91 with an early trigger; the five-ciphertext step at N = 2^13 998, 831 and 1126).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // c + a*b, 32 x 32 -> 64 bits (one instruction).
 __device__ __forceinline__ uint64_t madw(uint32_t a, uint32_t b, uint64_t c) {
   uint64_t r;

@@ -43,6 +43,25 @@ inline int set_smem_attr_once(std::atomic<unsigned long long>& bits, int device,
   return HE_OK;
 }
 
+// Launches a kernel that may start before its predecessor in the stream has
+// finished (it calls pdl_wait before it touches what others write): its launch
+// latency and its twiddles' loads overlap the predecessor's tail.
+template <class... K, class... A>
+int launch_pdl(void (*kernel)(K...), size_t blocks, unsigned threads, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  HE_CUDA(cudaLaunchKernelEx(&cfg, kernel, K(args)...));
+  return HE_OK;
+}
+
 // ---- host number theory (params.cpp) ---------------------------------------
 uint64_t h_mulmod(uint64_t a, uint64_t b, uint64_t q);
 uint64_t h_powmod(uint64_t a, uint64_t e, uint64_t q);

@@ -64,6 +64,7 @@ __global__ void k_sample(uint64_t* out, uint64_t out_stride, uint32_t kind, uint
 
 __global__ void k_signed_to_residues(const int64_t* src, uint64_t* out, uint32_t nl, int log_n,
                                      const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   const size_t total = (size_t)nl * n;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -100,6 +101,7 @@ __global__ void k_evk_combine(uint64_t* key, const uint64_t* e, const uint64_t* 
 __global__ void k_enc_combine(CtBatch out, const uint64_t* v, const uint64_t* em, const uint64_t* e1,
                               const uint64_t* pk, const uint64_t* s, int use_sk, uint32_t level,
                               uint32_t L, int log_n, const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   const size_t total = (size_t)level * n;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total; g += (size_t)gridDim.x * blockDim.x) {
@@ -123,6 +125,7 @@ __global__ void k_enc_combine(CtBatch out, const uint64_t* v, const uint64_t* em
 __global__ void k_enc_sample(uint64_t* out, uint64_t out_stride, uint32_t np, const int64_t* msg, uint32_t level,
                              uint64_t seed, uint32_t cid, const uint64_t* gauss, int gK, int log_n,
                              const PrimeDev* primes) {
+  pdl_wait();
   const uint32_t n = 1u << log_n;
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < np * n; g += gridDim.x * blockDim.x) {
@@ -248,14 +251,12 @@ int encrypt_dev(he_ctx* c, const int64_t* d_m, uint32_t level, int use_sk, uint3
   uint64_t* E1 = V + lw;
   CtBatch o{out->data, 0, out->cap, 0};
   const uint32_t np = use_sk ? 1 : 3;
-  k_enc_sample<<<grid_for((size_t)np * n), 256, 0, c->stream>>>(E0, lw, np, d_m, level, c->prm.seed, cid, c->d_gauss,
-                                                                c->gK, c->log_n, c->d_primes);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_enc_sample, grid_for((size_t)np * n), 256, 0, c->stream,
+                    E0, lw, np, d_m, level, c->prm.seed, cid, c->d_gauss, c->gK, c->log_n, c->d_primes));
   HE_TRY(ntt_forward(c, one_batch(E0, E0, lw, np, level, L)));
   if (use_sk) HE_TRY(sample(c, out->data + (size_t)out->cap * n, 0, 2, level, 0, L, cid, DOM_ENC_A, 1, 0));
-  k_enc_combine<<<grid_for(lw), 256, 0, c->stream>>>(o, V, E0, E1, c->d_pk, c->d_s, use_sk, level, L,
-                                                     c->log_n, c->d_primes);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl(k_enc_combine, grid_for(lw), 256, 0, c->stream,
+                    o, V, E0, E1, c->d_pk, c->d_s, use_sk, level, L, c->log_n, c->d_primes));
   out->level = level;
   return HE_OK;
 }

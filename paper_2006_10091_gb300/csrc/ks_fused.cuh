@@ -183,10 +183,14 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
   b /= a.nt;
   const uint32_t j = b % a.beta, i = b / a.beta;
   const uint32_t lo = a.lo[j], cnt = a.cnt[j];
-  if (t >= lo && t < lo + cnt) return;  // the digit's own limbs are used as they are
+  if (t >= lo && t < lo + cnt) {  // the digit's own limbs are used as they are
+    pdl_wait();
+    return;
+  }
   const uint32_t prime = ks_prime(t, a.level, a.L);
   const PrimeDev pr = a.primes[prime];
   stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)prime * N, tile);
+  pdl_wait();
   const uint64_t* tab = a.consts + a.off[j];
   const uint64_t* mat = tab + 2 * cnt;
   const uint64_t* mat_sh = mat + (size_t)cnt * a.np;
@@ -198,13 +202,13 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
     const uint32_t e = S::gidx(tile, k, xx);
     uint64_t y;
     if (cnt == 1) {
-      y = reduce64(__ldg(x + (size_t)lo * N + e), pr);  // Q_j / q_lo = 1
+      y = reduce64(x[(size_t)lo * N + e], pr);  // Q_j / q_lo = 1
     } else {
       // products by the constant (Q_j/q_i) mod q_t are Shoup products in [0, 2q), kept in [0, 2q)
       y = 0;
       for (uint32_t u = 0; u < cnt; ++u) {
         const uint64_t qa = a.primes[lo + u].q;
-        const uint64_t v = mul_shoup(__ldg(x + (size_t)(lo + u) * N + e), tab[2 * u], tab[2 * u + 1], qa);
+        const uint64_t v = mul_shoup(x[(size_t)(lo + u) * N + e], tab[2 * u], tab[2 * u + 1], qa);
         y += mul_shoup_lazy(v, mat[(size_t)u * a.np + prime], mat_sh[(size_t)u * a.np + prime], pr.q);
         y = y >= q2 ? y - q2 : y;
       }
@@ -262,10 +266,11 @@ ks_modup_col_all(KsFusedArgs a) {
       // the inverse transform's column pass on this tile, then the scaling by
       // N^-1 and the product by (Q_j/q_i)^-1 as one constant
       stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)(lo + u) * N, tile, tid, S::T);
+      pdl_wait();
 #pragma unroll 8
       for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint32_t e = S::gidx(tile, idx & (S::K - 1), idx >> LOG_K);
-        sm[idx + (idx >> 3)] = __ldg(x + (size_t)(lo + u) * N + e);
+        sm[idx + (idx >> 3)] = x[(size_t)(lo + u) * N + e];
       }
       group_sync<G, S::T>(grp);
       run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pa.q, tid, grp);
@@ -277,10 +282,11 @@ ks_modup_col_all(KsFusedArgs a) {
         wv[(size_t)u * S::TILE + idx] = halves ? split_source(v) : v;
       }
     } else {
+      pdl_wait();
 #pragma unroll 8
       for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
         const uint32_t e = S::gidx(tile, idx & (S::K - 1), idx >> LOG_K);
-        const uint64_t xv = __ldg(x + (size_t)(lo + u) * N + e);
+        const uint64_t xv = x[(size_t)(lo + u) * N + e];
         const uint64_t v = cnt == 1 ? xv : mul_shoup(xv, tab[2 * u], tab[2 * u + 1], pa.q);
         wv[(size_t)u * S::TILE + idx] = halves ? split_source(v) : v;
       }
@@ -288,6 +294,7 @@ ks_modup_col_all(KsFusedArgs a) {
     // the next limb's staging overwrites stw and sm: wait for every thread
     group_sync<G, S::T>(grp);
   }
+  pdl_wait();  // (groups without a source)
   if (G > 1) __syncthreads();  // every group's sources
   for (uint32_t t = part * a.nt / a.splits + grp; t < t_end; t += G) {
     if (t >= lo && t < lo + cnt) continue;  // the digit's own limbs are used as they are
@@ -406,6 +413,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   // while earlier ones transform
   stage_twiddles_async<LOG_N, LOG_M, LOG_K, false>(stw, a.tw + (size_t)prime * N, tile, threadIdx.x, CT * S::T);
   cp_async_commit();
+  pdl_wait();
   for (uint32_t j = 0; j < a.beta; ++j) {
     uint64_t* sm = dig + ((size_t)grp * a.beta + j) * TW;
     const bool own = t >= a.lo[j] && t < a.lo[j] + a.cnt[j];
@@ -712,6 +720,7 @@ __global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra)
 #pragma unroll
       for (int u = 0; u < 2; ++u) ll[c][p][u] = hh[c][p][u] = ss[c][p][u] = 0;
   }
+  pdl_wait();
 #pragma unroll 1
   for (uint32_t s = 0; s < kGatherRing - 1; ++s) copy_step(s);
   uint32_t slot = 0;
@@ -872,18 +881,20 @@ md_conv_col(MdArgs a) {
     if (a.half) {
       // the inverse transform's column pass on this tile, then the scaling by N^-1
       stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.itw + (size_t)a.spr[u] * N, tile, tid, S::T);
+      pdl_wait();
 #pragma unroll 8
       for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T)
-        sm[idx + (idx >> 3)] = __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
+        sm[idx + (idx >> 3)] = src[S::gidx(tile, idx & (S::K - 1), idx >> LOG_K)];
       group_sync<G, S::T>(grp);
       run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pp.q, tid, grp);
     }
+    pdl_wait();
     // the thread's words of the limb first (eight loads in flight), then their products
     uint64_t y0[S::TILE / S::T];
 #pragma unroll
     for (int v = 0; v < S::TILE / S::T; ++v) {
       const uint32_t idx = tid + v * S::T;
-      y0[v] = a.half ? sm[idx + (idx >> 3)] : __ldg(src + S::gidx(tile, idx & (S::K - 1), idx >> LOG_K));
+      y0[v] = a.half ? sm[idx + (idx >> 3)] : src[S::gidx(tile, idx & (S::K - 1), idx >> LOG_K)];
     }
     const uint64_t h = hP[u], w = a.md[2 * u], wsh = a.md[2 * u + 1];
 #pragma unroll
@@ -895,6 +906,7 @@ md_conv_col(MdArgs a) {
     // the next limb's staging overwrites stw and sm: wait for every thread
     if (a.half) group_sync<G, S::T>(grp);
   }
+  pdl_wait();  // (groups without a source)
   if (G > 1) __syncthreads();  // every group's sources
 #pragma unroll 2
   for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += G * S::T) {
@@ -950,13 +962,14 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
   const uint64_t w = pinv[2 * t], wsh = pinv[2 * t + 1];
   const uint64_t dw = a.addw ? a.addw[2 * t] : 1, dwsh = a.addw ? a.addw[2 * t + 1] : 0;
   stage_twiddles<LOG_N, LOG_M, LOG_K, false>(stw, a.tw + (size_t)t * N, tile);
+  pdl_wait();
   constexpr int PER = S::TILE / S::T;
   for (uint32_t p = 0; p < 2; ++p) {
     const uint64_t* src = a.conv + (((size_t)i * 2 + p) * a.level + t) * N;
 #pragma unroll 8
     for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
       const uint32_t k = idx >> LOG_M, x = idx & (S::M - 1);
-      sm[idx + (idx >> 3)] = __ldg(src + S::gidx(tile, k, x));
+      sm[idx + (idx >> 3)] = src[S::gidx(tile, k, x)];
     }
     // the epilogue's operands are loaded before the transform so that their
     // latency overlaps its rounds
@@ -970,8 +983,8 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
     for (int u = 0; u < PER; ++u) {
       const uint32_t idx = threadIdx.x + u * S::T;
       const uint32_t e = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
-      av[u] = __ldg(accq + e);
-      dv[u] = add_plain ? __ldg(ad + e) : 0;
+      av[u] = accq[e];
+      dv[u] = add_plain ? ad[e] : 0;
     }
     if (add_perm)  // one automorphism at a time: the thread's PER gathers are independent loads
       for (uint32_t g = 0; g < a.n_gal; ++g) {
@@ -980,7 +993,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
         for (int u = 0; u < PER; ++u) {
           const uint32_t idx = threadIdx.x + u * S::T;
           const uint32_t e = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
-          gv[u] = __ldg(ad + automorph_src(e, a.gal[g], LOG_N));
+          gv[u] = ad[automorph_src(e, a.gal[g], LOG_N)];
         }
 #pragma unroll
         for (int u = 0; u < PER; ++u) dv[u] = add_mod(dv[u], gv[u], q);
@@ -1115,16 +1128,16 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
     // with a half-transformed input, also the dropped limbs' inverse column pass
     const double bfly = polys * n / 2 * M1 + (a.half ? 2.0 * count * a.alpha * n / 2 * M1 : 0.0);
     ProfScope prof(c, nm_col, bfly + polys * n * a.alpha, n * 8 * (2.0 * count * a.alpha + polys), 0.0, bfly);
-    conv_kernel<<<(unsigned)blocks, plan.groups * SC::T, plan.smem, c->stream>>>(a);
+    HE_TRY(launch_pdl(conv_kernel, blocks, plan.groups * SC::T, plan.smem, c->stream,
+                      a));
   }
-  HE_CUDA(cudaGetLastError());
   {
     const size_t blocks = (size_t)count * a.level * SR::TILES;
     const double addw = a.has_add == 3 ? 1.5 * polys : a.has_add == 2 ? polys : a.has_add == 1 ? polys / 2 : 0.0;
     ProfScope prof(c, nm_row, polys * (n / 2 * M2 + 2 * n), n * 8 * (3.0 * polys + addw), 0.0, polys * n / 2 * M2);
-    md_row_combine<LOG_N, M2, K2><<<(unsigned)blocks, SR::T, smr, c->stream>>>(a);
+    HE_TRY(launch_pdl((md_row_combine<LOG_N, M2, K2>), blocks, SR::T, smr, c->stream,
+                      a));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
@@ -1181,10 +1194,12 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
       HE_TRY(set_smem_attr_once(attr_g[plan.groups >> 1], c->device, (const void*)kernel, kConvSmemMax));
       a.splits = plan.splits;
       const size_t blocks = (size_t)count * a.beta * SC::TILES * a.splits;
-      kernel<<<(unsigned)blocks, plan.groups * SC::T, plan.smem, c->stream>>>(a);
+      HE_TRY(launch_pdl(kernel, blocks, plan.groups * SC::T, plan.smem, c->stream,
+                        a));
     } else {
       const size_t blocks = (size_t)count * a.beta * a.nt * SC::TILES;
-      ks_modup_col<LOG_N, M1, K1><<<(unsigned)blocks, SC::T, smc, c->stream>>>(a);
+      HE_TRY(launch_pdl((ks_modup_col<LOG_N, M1, K1>), blocks, SC::T, smc, c->stream,
+                        a));
     }
   }
   HE_CUDA(cudaGetLastError());
@@ -1299,9 +1314,10 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
     const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words
     const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * ((1u << LOG_N) / (2 * kGatherThreads));
     const size_t sm = kGatherRing * (ct + 2) * sizeof(uint64_t) * 2 * kGatherThreads;
-    if (ct == 2) ks_gather_rot<LOG_N, 2><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
-    else ks_gather_rot<LOG_N, 1><<<(unsigned)blocks, kGatherThreads, sm, c->stream>>>(rc);
-    HE_CUDA(cudaGetLastError());
+    if (ct == 2) HE_TRY(launch_pdl((ks_gather_rot<LOG_N, 2>), blocks, kGatherThreads, sm, c->stream,
+                      rc));
+    else HE_TRY(launch_pdl((ks_gather_rot<LOG_N, 1>), blocks, kGatherThreads, sm, c->stream,
+                      rc));
     return HE_OK;
   }
   // ciphertexts per CTA: the knob, else 2 when that keeps as many warps
@@ -1321,10 +1337,12 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
       ct = cand;
   const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
   const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, ct, c0);
-  if (ct == 4) ks_row_rot<LOG_N, M2, K2 - 1, 4><<<(unsigned)blocks, 4 * SR::T, sm, c->stream>>>(rc);
-  else if (ct == 2) ks_row_rot<LOG_N, M2, K2 - 1, 2><<<(unsigned)blocks, 2 * SR::T, sm, c->stream>>>(rc);
-  else ks_row_rot<LOG_N, M2, K2 - 1, 1><<<(unsigned)blocks, SR::T, sm, c->stream>>>(rc);
-  HE_CUDA(cudaGetLastError());
+  if (ct == 4) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 4>), blocks, 4 * SR::T, sm, c->stream,
+                    rc));
+  else if (ct == 2) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 2>), blocks, 2 * SR::T, sm, c->stream,
+                   rc));
+  else HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 1>), blocks, SR::T, sm, c->stream,
+                    rc));
   return HE_OK;
 }
 

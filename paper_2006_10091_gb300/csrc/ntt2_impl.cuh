@@ -72,6 +72,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) >> LOG_V) ntt2_kernel(N
   const PrimeDev pr = a.primes[prime];
   const ulonglong2* tw = a.tw + (size_t)prime * (1u << LOG_N);
   stage_twiddles<LOG_N, LOG_M, LOG_K, COL, LOG_V>(stw, tw, tile);
+  pdl_wait();
   const uint32_t p1 = min(pg * a.pb + a.pb, a.np);
   for (uint32_t p = pg * a.pb; p < p1; ++p) {
     if (a.skip_alpha) {
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) >> LOG_V) ntt2_kernel(N
       if (COL) { x = idx >> LOG_K; k = idx & (S::K - 1); }
       else { k = idx >> LOG_M; x = idx & (S::M - 1); }
       const uint32_t e = S::gidx(tile, k, x);
-      sm[idx + (idx >> 3)] = __ldg(src + (a.gal ? automorph_src(e, a.gal, LOG_N) : e));
+      sm[idx + (idx >> 3)] = src[a.gal ? automorph_src(e, a.gal, LOG_N) : e];
     }
     __syncthreads();
     if (!INV && pr.q < (1ull << 58))
@@ -145,8 +146,8 @@ int launch2(he_ctx* c, const PolyBatch& b, const uint64_t* src, uint64_t* dst, u
   const double scale = INV && last ? transforms * nn : 0.0;
   ProfScope prof(c, INV ? "intt" : "ntt", transforms * nn / 2 * LOG_M + scale, transforms * nn * 16, 0.0,
                  transforms * nn / 2 * LOG_M);
-  ntt2_kernel<INV, LOG_N, LOG_M, LOG_K, COL, LOG_V><<<(unsigned)blocks, S::T, smem, c->stream>>>(a);
-  HE_CUDA(cudaGetLastError());
+  HE_TRY(launch_pdl((ntt2_kernel<INV, LOG_N, LOG_M, LOG_K, COL, LOG_V>), blocks, S::T, smem, c->stream,
+                    a));
   return HE_OK;
 }
 

@@ -214,11 +214,9 @@ int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint
     const uint32_t lo = level - 1;
     {
       ProfScope prof(c, "elementwise", (double)count * 2 * n, (double)count * 2 * n * 24);
-      k_add_pd<<<grid_for((size_t)count * 2 * n), 256, 0, c->stream>>>(
-          acc, (size_t)2 * nt * n, nt, add, lo, c->P_mod_q[lo], h_shoup(c->P_mod_q[lo], c->q[lo]), count, c->log_n,
-          c->d_primes);
+      HE_TRY(launch_pdl(k_add_pd, grid_for((size_t)count * 2 * n), 256, 0, c->stream,
+                        acc, (size_t)2 * nt * n, nt, add, lo, c->P_mod_q[lo], h_shoup(c->P_mod_q[lo], c->q[lo]), count, c->log_n, c->d_primes));
     }
-    HE_CUDA(cudaGetLastError());
     // the dropped limbs to coefficient form (only the row pass when the
     // fused conversion kernel finishes the transform)
     const bool mh = md_half_ok(c, alpha + 1, level - 1, count);
@@ -290,10 +288,9 @@ int mul_relin_batch(he_ctx* c, CtBatch A, CtBatch B, uint32_t level, uint32_t co
   CtBatch D{d01, (size_t)2 * level * n, level, 0};
   {
     ProfScope prof(c, "tensor", 4.0 * count * level * n, (double)count * level * n * 8 * 7);
-    k_tensor<<<grid_for((size_t)count * level * n / 2), 256, 0, c->stream>>>(
-        A, B, D, d2, (size_t)level * n, level, count, c->log_n, c->d_primes);
+    HE_TRY(launch_pdl(k_tensor, grid_for((size_t)count * level * n / 2), 256, 0, c->stream,
+                      A, B, D, d2, (size_t)level * n, level, count, c->log_n, c->d_primes));
   }
-  HE_CUDA(cudaGetLastError());
   // with the rescale: the key switch's ModDown and the rescale as one division by P q_{level-1}
   return keyswitch_batch(c, d2, (size_t)level * n, level, count, c->d_rlk, D, 2, out, ar, 0, rescale);
 }
@@ -406,10 +403,9 @@ size_t rotsum_words(const he_ctx* c, uint32_t level, uint32_t count) {
 int addsub_batch(he_ctx* c, CtBatch A, CtBatch B, CtBatch O, int op, uint32_t level, uint32_t count) {
   {
     ProfScope prof(c, "elementwise", 0.0, (double)count * 2 * level * c->n * 24);
-    k_addsub<<<grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream>>>(A, B, O, op, level, count,
-                                                                                    c->log_n, c->d_primes);
+    HE_TRY(launch_pdl(k_addsub, grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream,
+                      A, B, O, op, level, count, c->log_n, c->d_primes));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
@@ -428,30 +424,27 @@ static LimbConsts int_consts(const he_ctx* c, int64_t k, uint32_t level) {
 int mul_int_batch(he_ctx* c, CtBatch A, CtBatch O, int64_t k, uint32_t level, uint32_t count) {
   {
     ProfScope prof(c, "elementwise", 0.0, (double)count * 2 * level * c->n * 16);
-    k_mul_const<<<grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream>>>(
-        A, O, int_consts(c, k, level), level, count, c->log_n, c->d_primes);
+    HE_TRY(launch_pdl(k_mul_const, grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream,
+                      A, O, int_consts(c, k, level), level, count, c->log_n, c->d_primes));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
 int add_int_batch(he_ctx* c, CtBatch A, CtBatch O, int64_t k, uint32_t level, uint32_t count) {
   {
     ProfScope prof(c, "elementwise", 0.0, (double)count * 2 * level * c->n * 16);
-    k_add_const<<<grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream>>>(
-        A, O, int_consts(c, k, level), level, count, c->log_n, c->d_primes);
+    HE_TRY(launch_pdl(k_add_const, grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream,
+                      A, O, int_consts(c, k, level), level, count, c->log_n, c->d_primes));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
 int copy_batch(he_ctx* c, CtBatch A, CtBatch O, uint32_t level, uint32_t count) {
   {
     ProfScope prof(c, "elementwise", 0.0, (double)count * 2 * level * c->n * 16);
-    k_copy_limbs<<<grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream>>>(A, O, level, count,
-                                                                                        c->log_n);
+    HE_TRY(launch_pdl(k_copy_limbs, grid_for((size_t)count * 2 * level * c->n / 2), 256, 0, c->stream,
+                      A, O, level, count, c->log_n));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
@@ -493,6 +486,7 @@ constexpr int kTaSlices = 8;
 
 __global__ void __launch_bounds__(32 * kTaSlices) k_tensor_acc(CtBatch A, CtBatch B, uint32_t count, uint64_t* acc,
                                                              uint32_t level, int log_n, const PrimeDev* primes) {
+  pdl_wait();
   __shared__ uint64_t part[3][kTaSlices][32];
   const uint32_t n = 1u << log_n;
   const uint32_t lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
@@ -508,8 +502,8 @@ __global__ void __launch_bounds__(32 * kTaSlices) k_tensor_acc(CtBatch A, CtBatc
       t = (uint32_t)(g >> log_n);
       pr = primes[t];
       for (uint32_t i = slice; i < count; i += kTaSlices) {
-        const uint64_t x0 = __ldg(cpoly(A, i, 0, t, n) + k), x1 = __ldg(cpoly(A, i, 1, t, n) + k);
-        const uint64_t y0 = __ldg(cpoly(B, i, 0, t, n) + k), y1 = __ldg(cpoly(B, i, 1, t, n) + k);
+        const uint64_t x0 = cpoly(A, i, 0, t, n)[k], x1 = cpoly(A, i, 1, t, n)[k];
+        const uint64_t y0 = cpoly(B, i, 0, t, n)[k], y1 = cpoly(B, i, 1, t, n)[k];
         s0 = add_mod(s0, mul_mod(x0, y0, pr), pr.q);
         s1 = add_mod(s1, add_mod(mul_mod(x0, y1, pr), mul_mod(x1, y0, pr), pr.q), pr.q);
         s2 = add_mod(s2, mul_mod(x1, y1, pr), pr.q);
@@ -534,10 +528,9 @@ int tensor_acc_batch(he_ctx* c, CtBatch A, CtBatch B, uint32_t count, uint64_t* 
   {
     ProfScope prof(c, "tensor", 4.0 * count * level * c->n, (double)(4 * count + 6) * level * c->n * 8);
     const size_t groups = ((size_t)level * c->n + 31) / 32;  // CTAs of 32 coefficients
-    k_tensor_acc<<<(unsigned)std::min<size_t>(groups, 152 * 32), 32 * kTaSlices, 0, c->stream>>>(
-        A, B, count, acc, level, c->log_n, c->d_primes);
+    HE_TRY(launch_pdl(k_tensor_acc, std::min<size_t>(groups, 152 * 32), 32 * kTaSlices, 0, c->stream,
+                      A, B, count, acc, level, c->log_n, c->d_primes));
   }
-  HE_CUDA(cudaGetLastError());
   return HE_OK;
 }
 
