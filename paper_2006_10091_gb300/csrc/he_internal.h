@@ -109,8 +109,8 @@ struct he_ctx {
 
   // device tables
   PrimeDev* d_primes = nullptr;  // [np]
-  uint64_t* d_tw = nullptr;      // [np][N] pairs (psi^brv(m), its Shoup companion)
-  uint64_t* d_itw = nullptr;     // [np][N] pairs (psi^-brv(m), its Shoup companion)
+  uint64_t* d_tw = nullptr;      // [np][N] pairs (psi^brv(m), its companion, params.cu)
+  uint64_t* d_itw = nullptr;     // [np][N] pairs (psi^-brv(m), its companion)
   uint64_t* d_two64 = nullptr;   // [np] 2^64 mod q
   uint64_t* d_gauss = nullptr;   // Gaussian CDT
   int gK = 0;

@@ -121,8 +121,8 @@ __device__ __forceinline__ void conv_split(uint32_t cnt, uint64_t* sm, const uin
 
 // Whether the conversion of cnt sources below 2^src_bits to q runs as
 // conv_split_tile: the sum (plus 3q for ModDown's lift) stays below 2^64 and its
-// fold below 2^(k+5) (below 2q for the corrected transforms' primes), so that
-// the lazy transform's values stay below 66 2^k.
+// fold below 2^(k+5) (2^(k+3) for the split products' primes, 2q for the corrected
+// transforms'), so that the transform's values stay in range.
 inline bool conv_split_ok(uint64_t q, uint32_t cnt, uint32_t src_bits) {
   const uint32_t k = 64 - __builtin_clzll(q), e = (k + 1) / 2;
   if (k < 33 || k > 60 || cnt < 1 || cnt > 5 || src_bits > 60) return false;
@@ -139,7 +139,7 @@ inline bool conv_split_ok(uint64_t q, uint32_t cnt, uint32_t src_bits) {
   most += 3 * (u128)q;
   if (most >> 64) return false;
   const u128 folded = ((u128)1 << k) + (most >> k) * delta;
-  return folded <= (q < (1ull << 58) ? (u128)1 << (k + 5) : 2 * (u128)q);
+  return folded <= (k <= 40 ? (u128)1 << (k + 3) : q < (1ull << 58) ? (u128)1 << (k + 5) : 2 * (u128)q);
 }
 
 // The conversion of one tile for primes conv_split_ok turns down: Shoup
@@ -218,8 +218,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
   }
   __syncthreads();
   uint64_t* out = a.ext + (((size_t)i * a.beta + j) * a.nt + t) * N;
-  if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
-  else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr.q);
+  run_rounds<false, LOG_N, LOG_M, LOG_K, true>(sm, stw, pr, threadIdx.x);
 #pragma unroll 8
   for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
     const uint32_t xx = idx >> LOG_K, k = idx & (S::K - 1);
@@ -273,7 +272,7 @@ ks_modup_col_all(KsFusedArgs a) {
         sm[idx + (idx >> 3)] = x[(size_t)(lo + u) * N + e];
       }
       group_sync<G, S::T>(grp);
-      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pa.q, tid, grp);
+      run_rounds<true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pa, tid, grp);
       const uint64_t* tabn = mat_sh + (size_t)cnt * a.np;
       const uint64_t w = tabn[2 * u], wsh = tabn[2 * u + 1];
 #pragma unroll 8
@@ -307,8 +306,7 @@ ks_modup_col_all(KsFusedArgs a) {
     else conv_sum_tile<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr, tid);
     group_sync<G, S::T>(grp);
     uint64_t* out = a.ext + (((size_t)i * a.beta + j) * a.nt + t) * N;
-    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
+    run_rounds<false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr, tid, grp);
 #pragma unroll 8
     for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
       const uint32_t xx = idx >> LOG_K, k = idx & (S::K - 1);
@@ -403,7 +401,6 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   const uint32_t prime = ks_prime(t, a.level, a.L);
   const PrimeDev pr = a.primes[prime];
   const uint64_t q = pr.q;
-  const bool lazy = q < (1ull << 58);
   // the input's part 0, added through each rotation on the limbs q_t
   const bool add_c0 = ra.c0 && t < a.level;
   uint64_t* c0s = dig + (size_t)CT * a.beta * TW;  // its tiles, [CT][TW] after every digit tile
@@ -445,7 +442,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
     for (int u = 0; u < PER; ++u) {
       const uint32_t idx = ltid + u * S::T;
       const uint64_t v = sm[idx + (idx >> 3)];
-      sm[idx + (idx >> 3)] = lazy ? fwd_final<true>(v, pr) : fwd_final<false>(v, pr);
+      sm[idx + (idx >> 3)] = fwd_final(v, pr);
     }
   };
   int pend = -1;  // a converted digit waiting for a partner
@@ -459,8 +456,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
     cp_async_wait_dyn(a.beta - 1 - j);  // the twiddles and tiles 0 .. j have arrived
     __syncthreads();
     uint64_t* sms[2] = {dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW, dig + ((size_t)grp * a.beta + j) * TW};
-    if (lazy) run_rounds_n<false, true, LOG_N, LOG_M, LOG_K, false, 2>(sms, stw, q, ltid);
-    else run_rounds_n<false, false, LOG_N, LOG_M, LOG_K, false, 2>(sms, stw, q, ltid);
+    run_rounds_n<false, LOG_N, LOG_M, LOG_K, false, 2>(sms, stw, pr, ltid);
     finish_tile(sms[0]);
     finish_tile(sms[1]);
     pend = -1;
@@ -469,8 +465,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
     uint64_t* sm = dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW;
     cp_async_wait_dyn(a.beta - 1 - (uint32_t)pend);
     __syncthreads();
-    if (lazy) run_rounds<false, true, LOG_N, LOG_M, LOG_K, false>(sm, stw, q, ltid);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, false>(sm, stw, q, ltid);
+    run_rounds<false, LOG_N, LOG_M, LOG_K, false>(sm, stw, pr, ltid);
     finish_tile(sm);
   }
   cp_async_wait<0>();  // the own limb's tile
@@ -886,7 +881,7 @@ md_conv_col(MdArgs a) {
       for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T)
         sm[idx + (idx >> 3)] = src[S::gidx(tile, idx & (S::K - 1), idx >> LOG_K)];
       group_sync<G, S::T>(grp);
-      run_rounds<true, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pp.q, tid, grp);
+      run_rounds<true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pp, tid, grp);
     }
     pdl_wait();
     // the thread's words of the limb first (eight loads in flight), then their products
@@ -933,8 +928,7 @@ md_conv_col(MdArgs a) {
     else
       conv_sum_tile<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, tid, vv, vP, hQ);
     group_sync<G, S::T>(grp);
-    if (pr.q < (1ull << 58)) run_rounds<false, true, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr.q, tid, grp);
+    run_rounds<false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr, tid, grp);
     uint64_t* out = a.conv + (((size_t)i * 2 + p) * a.level + t) * N;
 #pragma unroll 8
     for (uint32_t idx = tid; idx < (uint32_t)S::TILE; idx += S::T) {
@@ -957,7 +951,6 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
   const uint32_t t = b % a.level, i = b / a.level;
   const PrimeDev pr = a.primes[t];
   const uint64_t q = pr.q;
-  const bool lazy = q < (1ull << 58);
   const uint64_t* pinv = a.md + 2 * a.alpha + (size_t)a.alpha * a.L;
   const uint64_t w = pinv[2 * t], wsh = pinv[2 * t + 1];
   const uint64_t dw = a.addw ? a.addw[2 * t] : 1, dwsh = a.addw ? a.addw[2 * t + 1] : 0;
@@ -999,15 +992,14 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
         for (int u = 0; u < PER; ++u) dv[u] = add_mod(dv[u], gv[u], q);
       }
     __syncthreads();
-    if (lazy) run_rounds<false, true, LOG_N, LOG_M, LOG_K, false>(sm, stw, q);
-    else run_rounds<false, false, LOG_N, LOG_M, LOG_K, false>(sm, stw, q);
+    run_rounds<false, LOG_N, LOG_M, LOG_K, false>(sm, stw, pr, threadIdx.x);
     uint64_t* o = cpoly(a.out, i, p, t, N);
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const uint32_t idx = threadIdx.x + u * S::T;
       const uint32_t e = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
       const uint64_t v = sm[idx + (idx >> 3)];
-      const uint64_t cv = lazy ? fwd_final<true>(v, pr) : fwd_final<false>(v, pr);
+      const uint64_t cv = fwd_final(v, pr);
       uint64_t r = mul_shoup(sub_mod(av[u], cv, q), w, wsh, q);
       if (add) r = add_mod(r, a.addw ? mul_shoup(dv[u], dw, dwsh, q) : dv[u], q);
       o[e] = r;
@@ -1061,8 +1053,8 @@ ConvPlan conv_plan(const he_ctx* c, size_t blocks, uint32_t ns, bool md, uint32_
       const uint32_t chain_t = ((targets + s - 1) / s + g - 1) / g;
       // (groups beside each other slow a chain by 0.35 each: rotation at N = 2^13 97 us with 0.17, 93 with 0.35)
       const double beside = 0.35 * (double)(std::min(ctas, (blocks * s + 151) / 152) * g - 1);
-      const double chain =
-          (double)((blocks * s + slots - 1) / slots) * (per * ((ns + g - 1) / g) + chain_t) * (1.0 + beside);
+      const size_t waves = (blocks * s + slots - 1) / slots;
+      const double chain = (double)waves * (per * ((ns + g - 1) / g) + chain_t) * (waves <= 2 ? 1.0 + beside : 1.0);
       const double cost = std::max(chain, 0.48 / 152 * (double)blocks * (s * per * ns + targets));
       // equal times: more resident warps, then fewer CTAs and groups
       if (!best.smem || cost < best.cost || (cost == best.cost && warps > best_warps)) {

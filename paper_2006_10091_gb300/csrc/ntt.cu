@@ -13,11 +13,13 @@
 // transforms into shared memory with coalesced loads, runs radix-8 rounds
 // (three stages per round, eight residues in registers per thread), and
 // writes the tile back.  Butterflies are Harvey's lazy ones (forward values
-// in [0, 4q), inverse in [0, 2q), Shoup products); the last pass returns
-// canonical residues.
+// in [0, 4q), inverse in [0, 2q), Shoup products), or split products on the
+// primes that take them (NttMode in ntt2.cuh); the last pass returns canonical
+// residues.
 #include <algorithm>
 
 #include "he_internal.h"
+#include "ntt2.cuh"
 
 namespace he {
 
@@ -27,7 +29,7 @@ struct NttPassArgs {
   uint64_t src_stride, dst_stride;
   uint32_t nl, limb0, level, L;
   uint32_t skip_alpha, skip_beta;
-  const ulonglong2* tw;  // twiddle pairs (value, Shoup companion), [np][N]
+  const ulonglong2* tw;  // twiddle pairs (value, companion), [np][N]
   const PrimeDev* primes;
   int log_n, log_m, bit_lo, K, log_k, tiles_per_limb;
   int last;  // final pass: canonical output (and N^-1 for the inverse)
@@ -49,12 +51,13 @@ __device__ __forceinline__ uint32_t smem_index(const NttPassArgs& a, uint32_t k,
 }
 
 // One round of R stages on every group of 2^R residues.
-template <bool INV, bool COL, int R>
+template <bool INV, bool COL, int R, int MODE>
 __device__ __forceinline__ void ntt_round(const NttPassArgs& a, uint64_t* sm, uint32_t tile, int sig0,
-                                          const ulonglong2* tw, uint64_t q) {
+                                          const ulonglong2* tw, const PrimeDev& pr) {
   constexpr int G = 1 << R;       // residues per group
   constexpr int GPT = 8 >> R;     // groups per thread
-  const uint64_t q2 = q + q;
+  const uint64_t q = pr.q;
+  const SplitQ sq = split_q(pr);
   const int lo_bits = a.log_m - sig0 - R;
   const uint32_t lo_mask = (1u << lo_bits) - 1;
   const int stage0 = a.log_n - a.bit_lo - a.log_m + sig0;  // global stage of local stage sig0
@@ -84,43 +87,40 @@ __device__ __forceinline__ void ntt_round(const NttPassArgs& a, uint64_t* sm, ui
       v[j] = sm[si[j]];
     }
     const uint32_t i0 = elem_index<COL>(a, tile, k, xbase);
-    if (!INV) {
 #pragma unroll
-      for (int st = 0; st < R; ++st) {
-        const int s = stage0 + st;
-        const int half = G >> (st + 1);
+    for (int k2 = 0; k2 < R; ++k2) {
+      const int st = INV ? R - 1 - k2 : k2;
+      const int s = stage0 + st;
+      const int half = G >> (st + 1);
 #pragma unroll
-        for (int j = 0; j < G; ++j) {
-          if (j & half) continue;
-          const uint32_t i = i0 | ((uint32_t)j << (lo_bits + a.bit_lo));
-          const ulonglong2 w = tw[(1u << s) + (i >> (a.log_n - s))];
-          uint64_t X = v[j];
-          X = X >= q2 ? X - q2 : X;
-          const uint64_t t = mul_shoup_lazy(v[j + half], w.x, w.y, q);
-          v[j] = X + t;
-          v[j + half] = X + q2 - t;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int st = R - 1; st >= 0; --st) {
-        const int s = stage0 + st;
-        const int half = G >> (st + 1);
-#pragma unroll
-        for (int j = 0; j < G; ++j) {
-          if (j & half) continue;
-          const uint32_t i = i0 | ((uint32_t)j << (lo_bits + a.bit_lo));
-          const ulonglong2 w = tw[(1u << s) + (i >> (a.log_n - s))];
-          const uint64_t X = v[j], Y = v[j + half];
-          uint64_t sum = X + Y;
-          sum = sum >= q2 ? sum - q2 : sum;
-          v[j + half] = mul_shoup_lazy(X + q2 - Y, w.x, w.y, q);
-          v[j] = sum;
-        }
+      for (int j = 0; j < G; ++j) {
+        if (j & half) continue;
+        const uint32_t i = i0 | ((uint32_t)j << (lo_bits + a.bit_lo));
+        const ulonglong2 w = tw[(1u << s) + (i >> (a.log_n - s))];
+        butterfly<INV, MODE>(v[j], v[j + half], w, k2, q, sq);
       }
     }
+    if (INV && MODE == kSplit)  // the round's sums; its products are below 3q
+#pragma unroll
+      for (int j = 0; j < G / 2; ++j) v[j] = fold(v[j], pr);
 #pragma unroll
     for (int j = 0; j < G; ++j) sm[si[j]] = v[j];
+  }
+}
+
+// All rounds of a pass in one mode.
+template <bool INV, bool COL, int MODE>
+__device__ __forceinline__ void ntt_rounds(const NttPassArgs& a, uint64_t* sm, uint32_t tile, const ulonglong2* tw,
+                                           const PrimeDev& pr) {
+  const int nr = (a.log_m + 2) / 3;
+  for (int rr = 0; rr < nr; ++rr) {
+    const int r = INV ? nr - 1 - rr : rr;
+    const int sig0 = 3 * r;
+    const int R = min(3, a.log_m - sig0);
+    if (R == 3) ntt_round<INV, COL, 3, MODE>(a, sm, tile, sig0, tw, pr);
+    else if (R == 2) ntt_round<INV, COL, 2, MODE>(a, sm, tile, sig0, tw, pr);
+    else ntt_round<INV, COL, 1, MODE>(a, sm, tile, sig0, tw, pr);
+    __syncthreads();
   }
 }
 
@@ -153,16 +153,8 @@ __global__ void __launch_bounds__(512) ntt_pass_kernel(NttPassArgs a) {
   }
   __syncthreads();
 
-  const int nr = (a.log_m + 2) / 3;
-  for (int rr = 0; rr < nr; ++rr) {
-    const int r = INV ? nr - 1 - rr : rr;
-    const int sig0 = 3 * r;
-    const int R = min(3, a.log_m - sig0);
-    if (R == 3) ntt_round<INV, COL, 3>(a, sm, tile, sig0, tw, q);
-    else if (R == 2) ntt_round<INV, COL, 2>(a, sm, tile, sig0, tw, q);
-    else ntt_round<INV, COL, 1>(a, sm, tile, sig0, tw, q);
-    __syncthreads();
-  }
+  if (split_prime(pr)) ntt_rounds<INV, COL, kSplit>(a, sm, tile, tw, pr);
+  else ntt_rounds<INV, COL, kCorrected>(a, sm, tile, tw, pr);
 
   for (uint32_t idx = threadIdx.x; idx < tilesz; idx += blockDim.x) {
     uint32_t k, x;
@@ -171,6 +163,7 @@ __global__ void __launch_bounds__(512) ntt_pass_kernel(NttPassArgs a) {
     uint64_t v = sm[pad8(idx)];
     if (a.last) {
       if (INV) v = mul_shoup_lazy(v, pr.n_inv, pr.n_inv_sh, q);
+      else if (split_prime(pr)) v = fold(v, pr);
       else v = v >= q2 ? v - q2 : v;
       v = v >= q ? v - q : v;
     }

@@ -31,6 +31,48 @@ struct Shape {
   }
 };
 
+// How a prime's butterflies run (compile-time in the rounds, chosen per CTA):
+// kCorrected: Shoup products, Harvey's corrections (forward values in [0, 4q),
+//   inverse in [0, 2q)); primes of 58 bits and more, and every inverse
+//   transform but kSplit's;
+// kLazy: Shoup products without the forward corrections (a value grows by at
+//   most 2q per stage);
+// kSplit: split products below 3q (mul_split).  Forward values start below
+//   8 2^k and grow by at most 3q per stage, below 2^46 after 16; inverse values
+//   start a round below 3q, double per stage, and the round's sums are folded.
+enum NttMode { kCorrected = 0, kLazy = 1, kSplit = 2 };
+__device__ __forceinline__ NttMode ntt_mode(const PrimeDev& p) {
+  return split_prime(p) ? kSplit : p.q < (1ull << 58) ? kLazy : kCorrected;
+}
+
+// One butterfly of executed stage i of a round: forward (X, Y) -> X + wY, X - wY;
+// inverse (X, Y) -> X + Y, w (X - Y).
+template <bool INV, int MODE>
+__device__ __forceinline__ void butterfly(uint64_t& x, uint64_t& y, const ulonglong2& w, int i, uint64_t q,
+                                          const SplitQ& sq) {
+  const uint64_t q2 = q + q;
+  if (!INV) {
+    if (MODE == kSplit) {
+      const uint64_t t = mul_split(y, w.x, w.y, sq);
+      y = x + sq.q3 - t;
+      x += t;
+    } else {
+      const uint64_t X = MODE == kCorrected && x >= q2 ? x - q2 : x;
+      const uint64_t t = mul_shoup_lazy(y, w.x, w.y, q);
+      x = X + t;
+      y = X + q2 - t;
+    }
+  } else if (MODE == kSplit) {
+    const uint64_t d = x + (sq.q3 << i) - y;
+    x += y;
+    y = mul_split(d, w.x, w.y, sq);
+  } else {
+    const uint64_t X = x, Y = y, sum = X + Y;
+    x = sum >= q2 ? sum - q2 : sum;
+    y = mul_shoup_lazy(X + q2 - Y, w.x, w.y, q);
+  }
+}
+
 // One round: R consecutive local stages (radix 2^R) on groups of G = 2^R
 // elements held in registers.  Within a group the elements sit at shared
 // memory offsets j*s + (j*s >> 3) from the first (s the group's stride, a
@@ -40,11 +82,13 @@ struct Shape {
 // is loaded once.
 // `tid` is the thread's index among the T threads that share the tile (a CTA
 // may hold several tiles, one per group of T threads).
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int R, int LOG_V = 3>
-__device__ __forceinline__ void round2(uint64_t* sm, const ulonglong2* stw, int sig0, uint64_t q, uint32_t tid) {
+template <bool INV, int MODE, int LOG_N, int LOG_M, int LOG_K, bool COL, int R, int LOG_V = 3>
+__device__ __forceinline__ void round2(uint64_t* sm, const ulonglong2* stw, int sig0, const PrimeDev& pr,
+                                       uint32_t tid) {
   using S = Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>;
   constexpr int G = 1 << R, GPT = (1 << LOG_V) >> R;
-  const uint64_t q2 = q + q;
+  const uint64_t q = pr.q;
+  const SplitQ sq = split_q(pr);
   const int lo_bits = LOG_M - sig0 - R;
   const uint32_t lo_mask = (1u << lo_bits) - 1;
   const uint32_t s = COL ? (1u << (lo_bits + LOG_K)) : (1u << lo_bits);
@@ -79,22 +123,13 @@ __device__ __forceinline__ void round2(uint64_t* sm, const ulonglong2* stw, int 
 #pragma unroll
         for (int jj = 0; jj < half; ++jj) {
           const int j = (b << (R - st)) + jj;
-          if (!INV) {
-            uint64_t X = v[j];
-            if (!LAZY) X = X >= q2 ? X - q2 : X;
-            const uint64_t t = mul_shoup_lazy(v[j + half], w.x, w.y, q);
-            v[j] = X + t;
-            v[j + half] = X + q2 - t;
-          } else {
-            const uint64_t X = v[j], Y = v[j + half];
-            uint64_t sum = X + Y;
-            sum = sum >= q2 ? sum - q2 : sum;
-            v[j + half] = mul_shoup_lazy(X + q2 - Y, w.x, w.y, q);
-            v[j] = sum;
-          }
+          butterfly<INV, MODE>(v[j], v[j + half], w, i, q, sq);
         }
       }
     }
+    if (INV && MODE == kSplit)  // the round's sums; its products are below 3q
+#pragma unroll
+      for (int j = 0; j < G / 2; ++j) v[j] = fold(v[j], pr);
 #pragma unroll
     for (int j = 0; j < G; ++j) sm[s0 + j * s + ((j * s) >> 3)] = v[j];
   }
@@ -102,12 +137,13 @@ __device__ __forceinline__ void round2(uint64_t* sm, const ulonglong2* stw, int 
 
 // The same round on NT tiles of the same prime and positions at once (each
 // twiddle loaded once for all of them; NT independent groups in registers).
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int R, int NT, int LOG_V = 3>
-__device__ __forceinline__ void round2_n(uint64_t* const* sms, const ulonglong2* stw, int sig0, uint64_t q,
+template <bool INV, int MODE, int LOG_N, int LOG_M, int LOG_K, bool COL, int R, int NT, int LOG_V = 3>
+__device__ __forceinline__ void round2_n(uint64_t* const* sms, const ulonglong2* stw, int sig0, const PrimeDev& pr,
                                          uint32_t tid) {
   using S = Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>;
   constexpr int G = 1 << R, GPT = (1 << LOG_V) >> R;
-  const uint64_t q2 = q + q;
+  const uint64_t q = pr.q;
+  const SplitQ sq = split_q(pr);
   const int lo_bits = LOG_M - sig0 - R;
   const uint32_t lo_mask = (1u << lo_bits) - 1;
   const uint32_t s = COL ? (1u << (lo_bits + LOG_K)) : (1u << lo_bits);
@@ -145,24 +181,15 @@ __device__ __forceinline__ void round2_n(uint64_t* const* sms, const ulonglong2*
         for (int jj = 0; jj < half; ++jj) {
           const int j = (b << (R - st)) + jj;
 #pragma unroll
-          for (int t = 0; t < NT; ++t) {
-            if (!INV) {
-              uint64_t X = v[t][j];
-              if (!LAZY) X = X >= q2 ? X - q2 : X;
-              const uint64_t tt = mul_shoup_lazy(v[t][j + half], w.x, w.y, q);
-              v[t][j] = X + tt;
-              v[t][j + half] = X + q2 - tt;
-            } else {
-              const uint64_t X = v[t][j], Y = v[t][j + half];
-              uint64_t sum = X + Y;
-              sum = sum >= q2 ? sum - q2 : sum;
-              v[t][j + half] = mul_shoup_lazy(X + q2 - Y, w.x, w.y, q);
-              v[t][j] = sum;
-            }
-          }
+          for (int t = 0; t < NT; ++t) butterfly<INV, MODE>(v[t][j], v[t][j + half], w, i, q, sq);
         }
       }
     }
+    if (INV && MODE == kSplit)
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+#pragma unroll
+        for (int j = 0; j < G / 2; ++j) v[t][j] = fold(v[t][j], pr);
 #pragma unroll
     for (int t = 0; t < NT; ++t)
 #pragma unroll
@@ -171,19 +198,29 @@ __device__ __forceinline__ void round2_n(uint64_t* const* sms, const ulonglong2*
 }
 
 // All rounds of one pass on NT tiles at once (ends with a barrier).
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int NT, int LOG_V = 3>
-__device__ __forceinline__ void run_rounds_n(uint64_t* const* sms, const ulonglong2* stw, uint64_t q, uint32_t tid) {
+template <bool INV, int MODE, int LOG_N, int LOG_M, int LOG_K, bool COL, int NT, int LOG_V = 3>
+__device__ __forceinline__ void run_rounds_mode_n(uint64_t* const* sms, const ulonglong2* stw, const PrimeDev& pr,
+                                                  uint32_t tid) {
+  // (unrolled, but the lazy rounds a loop: their code, doubled for two tiles and
+  // beside the corrected rounds of the special primes, crowded the instruction
+  // cache: eight multiplications at N = 2^16 2.57 -> 2.47 ms)
   constexpr int NR = (LOG_M + LOG_V - 1) / LOG_V;
-#pragma unroll
-  for (int rr = 0; rr < NR; ++rr) {
+  auto one = [&](int rr) {
     const int r = INV ? NR - 1 - rr : rr;
     const int sig0 = LOG_V * r;
     const int R = LOG_M - sig0 < LOG_V ? LOG_M - sig0 : LOG_V;
-    if (R == 4) round2_n<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, (LOG_V >= 4 ? 4 : 1), NT, LOG_V>(sms, stw, sig0, q, tid);
-    else if (R == 3) round2_n<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 3, NT, LOG_V>(sms, stw, sig0, q, tid);
-    else if (R == 2) round2_n<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 2, NT, LOG_V>(sms, stw, sig0, q, tid);
-    else round2_n<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 1, NT, LOG_V>(sms, stw, sig0, q, tid);
+    if (R == 4) round2_n<INV, MODE, LOG_N, LOG_M, LOG_K, COL, (LOG_V >= 4 ? 4 : 1), NT, LOG_V>(sms, stw, sig0, pr, tid);
+    else if (R == 3) round2_n<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 3, NT, LOG_V>(sms, stw, sig0, pr, tid);
+    else if (R == 2) round2_n<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 2, NT, LOG_V>(sms, stw, sig0, pr, tid);
+    else round2_n<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 1, NT, LOG_V>(sms, stw, sig0, pr, tid);
     __syncthreads();
+  };
+  if (MODE != kLazy) {
+#pragma unroll
+    for (int rr = 0; rr < NR; ++rr) one(rr);
+  } else {
+#pragma unroll 1
+    for (int rr = 0; rr < NR; ++rr) one(rr);
   }
 }
 
@@ -245,35 +282,47 @@ __device__ __forceinline__ void group_sync(uint32_t grp) {
 
 // All rounds of one pass on the tile in shared memory (ends with a barrier of
 // the tile's group).
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3, int G = 1>
-__device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, uint64_t q, uint32_t tid,
-                                           uint32_t grp = 0) {
+template <bool INV, int MODE, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3, int G = 1>
+__device__ __forceinline__ void run_rounds_mode(uint64_t* sm, const ulonglong2* stw, const PrimeDev& pr, uint32_t tid,
+                                                uint32_t grp = 0) {
   constexpr int NR = (LOG_M + LOG_V - 1) / LOG_V;
 #pragma unroll
   for (int rr = 0; rr < NR; ++rr) {
     const int r = INV ? NR - 1 - rr : rr;
     const int sig0 = LOG_V * r;
     const int R = LOG_M - sig0 < LOG_V ? LOG_M - sig0 : LOG_V;
-    if (R == 4) round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, (LOG_V >= 4 ? 4 : 1), LOG_V>(sm, stw, sig0, q, tid);
-    else if (R == 3) round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 3, LOG_V>(sm, stw, sig0, q, tid);
-    else if (R == 2) round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 2, LOG_V>(sm, stw, sig0, q, tid);
-    else round2<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, 1, LOG_V>(sm, stw, sig0, q, tid);
+    if (R == 4) round2<INV, MODE, LOG_N, LOG_M, LOG_K, COL, (LOG_V >= 4 ? 4 : 1), LOG_V>(sm, stw, sig0, pr, tid);
+    else if (R == 3) round2<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 3, LOG_V>(sm, stw, sig0, pr, tid);
+    else if (R == 2) round2<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 2, LOG_V>(sm, stw, sig0, pr, tid);
+    else round2<INV, MODE, LOG_N, LOG_M, LOG_K, COL, 1, LOG_V>(sm, stw, sig0, pr, tid);
     group_sync<G, Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>::T>(grp);
   }
 }
 
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3>
-__device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, uint64_t q) {
-  run_rounds<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, LOG_V>(sm, stw, q, threadIdx.x);
+// The rounds in the prime's mode (the same branch for the whole CTA).
+template <bool INV, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V = 3, int G = 1>
+__device__ __forceinline__ void run_rounds(uint64_t* sm, const ulonglong2* stw, const PrimeDev& pr, uint32_t tid,
+                                           uint32_t grp = 0) {
+  const NttMode m = ntt_mode(pr);
+  if (m == kSplit) run_rounds_mode<INV, kSplit, LOG_N, LOG_M, LOG_K, COL, LOG_V, G>(sm, stw, pr, tid, grp);
+  else if (!INV && m == kLazy) run_rounds_mode<INV, kLazy, LOG_N, LOG_M, LOG_K, COL, LOG_V, G>(sm, stw, pr, tid, grp);
+  else run_rounds_mode<INV, kCorrected, LOG_N, LOG_M, LOG_K, COL, LOG_V, G>(sm, stw, pr, tid, grp);
+}
+template <bool INV, int LOG_N, int LOG_M, int LOG_K, bool COL, int NT, int LOG_V = 3>
+__device__ __forceinline__ void run_rounds_n(uint64_t* const* sms, const ulonglong2* stw, const PrimeDev& pr,
+                                             uint32_t tid) {
+  const NttMode m = ntt_mode(pr);
+  if (m == kSplit) run_rounds_mode_n<INV, kSplit, LOG_N, LOG_M, LOG_K, COL, NT, LOG_V>(sms, stw, pr, tid);
+  else if (!INV && m == kLazy) run_rounds_mode_n<INV, kLazy, LOG_N, LOG_M, LOG_K, COL, NT, LOG_V>(sms, stw, pr, tid);
+  else run_rounds_mode_n<INV, kCorrected, LOG_N, LOG_M, LOG_K, COL, NT, LOG_V>(sms, stw, pr, tid);
 }
 
-// Canonical residue of a forward-pass output: lazy values (below 66 2^k) by a
-// fold, or a Shoup product by 1 where the prime has none, corrected ones
+// Canonical residue of a forward-pass output: lazy and split values (below 66
+// 2^k) by a fold, or a Shoup product by 1 where the prime has none, corrected ones
 // ([0, 4q)) by subtractions.
-template <bool LAZY>
 __device__ __forceinline__ uint64_t fwd_final(uint64_t v, const PrimeDev& pr) {
   const uint64_t q = pr.q, q2 = q + q;
-  if (LAZY) v = pr.delta ? fold(v, pr) : mul_shoup_lazy(v, 1, pr.one_sh, q);
+  if (q < (1ull << 58)) v = pr.delta ? fold(v, pr) : mul_shoup_lazy(v, 1, pr.one_sh, q);
   else v = v >= q2 ? v - q2 : v;
   return v >= q ? v - q : v;
 }

@@ -1,18 +1,16 @@
 // ntt2_impl.cuh -- the two-pass NTT for N = 2^12 .. 2^16 with compile-time tile
 // shapes.  Same transform, same output as ntt.cu (slot j = value at
 // psi^(2*brv(j)+1)); what differs is how a pass runs:
-//  * each CTA first copies the twiddle pairs (value, Shoup companion) its
+//  * each CTA first copies the twiddle pairs (value, companion) its
 //    stages will use into shared memory with coalesced loads -- a column
 //    pass (the top index bits) needs tw[1 .. 2^m), a row pass for its K
 //    consecutive rows needs K*2^sigma consecutive entries per local stage
 //    sigma -- so every butterfly reads its twiddle from shared memory;
 //  * tile shapes are template parameters, so index arithmetic is shifts by
 //    constants;
-//  * forward transforms over primes below 2^58 skip Harvey's per-stage
-//    correction: with Shoup products in [0, 2q) a value grows by at most 2q
-//    per stage, so after the n <= 16 stages it stays below 33q < 2^64; the
-//    last pass reduces once (a Shoup product by 1, then one subtraction).
-//    Larger primes keep the corrected butterfly ([0, 4q)).
+//  * butterflies run in the prime's mode (NttMode in ntt2.cuh): split products
+//    up to 40 bits; forward transforms over primes below 2^58 without Harvey's
+//    per-stage correction, reduced once by the last pass; larger primes with it.
 #pragma once
 #include <algorithm>
 
@@ -34,12 +32,12 @@ struct Ntt2Args {
   int last;
 };
 
-template <bool INV, bool LAZY, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V>
+template <bool INV, int LOG_N, int LOG_M, int LOG_K, bool COL, int LOG_V>
 __device__ __forceinline__ void pass_body(const Ntt2Args& a, uint64_t* sm, ulonglong2* stw, uint32_t tile,
                                           const uint64_t* src, uint64_t* dst, const PrimeDev& pr) {
   using S = Shape<LOG_N, LOG_M, LOG_K, COL, LOG_V>;
   const uint64_t q = pr.q;
-  run_rounds<INV, LAZY, LOG_N, LOG_M, LOG_K, COL, LOG_V>(sm, stw, q);
+  run_rounds<INV, LOG_N, LOG_M, LOG_K, COL, LOG_V>(sm, stw, pr, threadIdx.x);
 #pragma unroll 4
   for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
     uint32_t k, x;
@@ -51,7 +49,7 @@ __device__ __forceinline__ void pass_body(const Ntt2Args& a, uint64_t* sm, ulong
         v = mul_shoup_lazy(v, pr.n_inv, pr.n_inv_sh, q);
         v = v >= q ? v - q : v;
       } else {
-        v = fwd_final<LAZY>(v, pr);
+        v = fwd_final(v, pr);
       }
     }
     dst[S::gidx(tile, k, x)] = v;
@@ -93,10 +91,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) >> LOG_V) ntt2_kernel(N
       sm[idx + (idx >> 3)] = src[a.gal ? automorph_src(e, a.gal, LOG_N) : e];
     }
     __syncthreads();
-    if (!INV && pr.q < (1ull << 58))
-      pass_body<INV, true, LOG_N, LOG_M, LOG_K, COL, LOG_V>(a, sm, stw, tile, src, dst, pr);
-    else
-      pass_body<INV, false, LOG_N, LOG_M, LOG_K, COL, LOG_V>(a, sm, stw, tile, src, dst, pr);
+    pass_body<INV, LOG_N, LOG_M, LOG_K, COL, LOG_V>(a, sm, stw, tile, src, dst, pr);
   }
 }
 

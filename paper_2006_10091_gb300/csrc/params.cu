@@ -173,7 +173,9 @@ int build_tables(he_ctx* c) {
   HE_CUDA(cudaMalloc(&c->d_two64, sizeof(uint64_t) * np));
   HE_CUDA(cudaMemcpy(c->d_two64, two64.data(), sizeof(uint64_t) * np, cudaMemcpyHostToDevice));
 
-  // twiddles: tw[m] = psi^brv(m), itw[m] = psi^-brv(m), interleaved with Shoup companions
+  // twiddles: tw[m] = psi^brv(m), itw[m] = psi^-brv(m), each followed by its
+  // companion: 2^23 times it mod q for the primes whose butterflies take split
+  // products (mul_split), else Shoup's
   {
     std::vector<uint64_t> tw((size_t)np * n * 2), itw((size_t)np * n * 2), pw(n), ipw(n);
     for (int t = 0; t < np; ++t) {
@@ -188,9 +190,14 @@ int build_tables(he_ctx* c) {
         const uint32_t r = brv_host((uint32_t)m, c->log_n);
         size_t o = ((size_t)t * n + m) * 2;
         tw[o] = pw[r];
-        tw[o + 1] = h_shoup(pw[r], q);
         itw[o] = ipw[r];
-        itw[o + 1] = h_shoup(ipw[r], q);
+        if (split_prime(pd[t])) {
+          tw[o + 1] = h_mulmod(pw[r], 1ull << kSplitBits, q);
+          itw[o + 1] = h_mulmod(ipw[r], 1ull << kSplitBits, q);
+        } else {
+          tw[o + 1] = h_shoup(pw[r], q);
+          itw[o + 1] = h_shoup(ipw[r], q);
+        }
       }
     }
     HE_CUDA(cudaMalloc(&c->d_tw, sizeof(uint64_t) * tw.size()));
