@@ -70,6 +70,10 @@ bool h_is_prime(uint64_t n);
 std::vector<uint64_t> h_ntt_primes(int bits, int log_n, int count, const std::vector<uint64_t>& skip);
 uint64_t h_min_root(uint64_t q, int log_n);
 uint64_t h_shoup(uint64_t w, uint64_t q);
+inline uint64_t h_mod(int64_t k, uint64_t q) {  // k mod q in [0, q)
+  const __int128 r = (__int128)k % (__int128)q;
+  return (uint64_t)(r < 0 ? r + q : r);
+}
 int h_gauss_table(double sigma, uint64_t* T);
 uint64_t h_galois_elt(int log_n, int32_t r);
 

@@ -60,6 +60,17 @@ int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint
 // Whether N has compiled shapes for the fused key-switching kernels.
 inline bool ks_fusable(const he_ctx* c) { return !c->ntt_generic && c->log_n >= 12 && c->log_n <= 16; }
 int rescale_batch(he_ctx* c, CtBatch in, uint32_t level, uint32_t count, CtBatch out, Arena& ar);
+// out = rescale(k in) (+ add, + the constant k0 on part 0) on the first
+// `targets` <= level - 1 limbs, as rescale_batch of mul_int_batch's result and
+// the additions would give; tmp holds the product where the fused kernels do not
+// run.  add may be out.
+struct RescaleScale {
+  int64_t k;
+  const CtBatch* add;
+  const int64_t* k0;
+};
+int rescale_scaled_batch(he_ctx* c, CtBatch in, const RescaleScale& sc, uint32_t level, uint32_t targets,
+                         uint32_t count, CtBatch tmp, CtBatch out, Arena& ar);
 int mul_relin_batch(he_ctx* c, CtBatch A, CtBatch B, uint32_t level, uint32_t count, CtBatch out,
                     bool rescale, Arena& ar);
 int rotate_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, uint64_t gal, CtBatch out,

@@ -108,6 +108,7 @@ int md_fused_gals(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t*
   const uint32_t nt = level + (uint32_t)c->alpha;
   MdArgs a;
   a.n_gal = n_gal;
+  a.scaled = a.with_k0 = 0;
   for (uint32_t g = 0; g < n_gal; ++g) a.gal[g] = gals[g];
   a.yP = acc + (size_t)level * c->n;
   a.yp_stride = acc_stride;
@@ -152,6 +153,7 @@ int md_fused_rescale(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64
   const uint32_t nt = level + (uint32_t)c->alpha, lo = level - 1;
   MdArgs a;
   a.n_gal = 0;
+  a.scaled = a.with_k0 = 0;
   a.yP = acc + (size_t)lo * c->n;
   a.yp_stride = acc_stride;
   a.yp_pstride = (uint64_t)nt * c->n;
@@ -177,8 +179,10 @@ int md_fused_rescale(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64
 
 // Rescale by q_{l-1} as a ModDown by that one prime, fused the same way.
 // last: the dropped limb of both parts in coefficient form, count x [2][N].
+// With sc (RescaleScale): out = rescale(k in) + add + k0, on the first `targets`
+// of the level - 1 limbs.
 int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatch out, uint32_t level,
-             uint32_t count, bool half, bool* handled) {
+             uint32_t count, bool half, bool* handled, uint32_t targets, const RescaleScale* sc) {
   *handled = false;
   if (!ks_fusable(c) || level < 2) {
     if (half) return fail(HE_EINVAL, "md_fused: half-transformed input needs the fused kernels");
@@ -187,6 +191,7 @@ int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatc
   const uint32_t lt = level - 1;
   MdArgs a;
   a.n_gal = 0;
+  a.scaled = a.with_k0 = 0;
   a.yP = last;
   a.yp_stride = 2ull * c->n;
   a.yp_pstride = c->n;
@@ -198,7 +203,25 @@ int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatc
   a.add = out;
   a.out = out;
   a.has_add = 0;
-  a.level = lt;
+  if (sc) {
+    a.scaled = 1;
+    const uint64_t ql = c->q[lt], kl = h_mod(sc->k, ql);
+    a.src_w = half ? h_mulmod(kl, h_invmod((uint64_t)c->n % ql, ql), ql) : kl;
+    a.src_wsh = h_shoup(a.src_w, ql);
+    for (uint32_t t = 0; t < targets; ++t) {
+      a.kw[t] = h_mod(sc->k, c->q[t]);
+      a.kwsh[t] = h_shoup(a.kw[t], c->q[t]);
+    }
+    if (sc->add) {
+      a.add = *sc->add;
+      a.has_add = 2;
+    }
+    if (sc->k0) {
+      a.with_k0 = 1;
+      for (uint32_t t = 0; t < targets; ++t) a.k0[t] = h_mod(*sc->k0, c->q[t]);
+    }
+  }
+  a.level = targets;
   a.alpha = 1;
   a.L = (uint32_t)c->L;
   a.primes = c->d_primes;

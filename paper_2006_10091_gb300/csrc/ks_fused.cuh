@@ -824,6 +824,12 @@ struct MdArgs {
   uint32_t level, alpha, L;
   uint32_t spr[HE_MAX_DIGIT];  // prime indices of the alpha dropped limbs (the special primes; q_l for a
                                // rescale by q_l; q_{l-1} and the special primes for a ModDown merged with it)
+  // a rescale of k times the input (kind 1 with scaled set): k modulo the target
+  // limbs (Shoup pairs) and, times N^-1 where the inverse transform is finished
+  // here, modulo the dropped one; k0 (with_k0) is added to part 0
+  int scaled, with_k0;
+  uint64_t src_w, src_wsh;
+  uint64_t kw[HE_MAX_PRIMES], kwsh[HE_MAX_PRIMES], k0[HE_MAX_PRIMES];
   int kind;                    // 0 ModDown, 1 rescale, 2 ModDown merged with the rescale (profile names)
   const uint64_t* addw;        // the addend is multiplied by these Shoup pairs per target limb (nullptr: not)
   const PrimeDev* primes;
@@ -894,7 +900,8 @@ md_conv_col(MdArgs a) {
     const uint64_t h = hP[u], w = a.md[2 * u], wsh = a.md[2 * u + 1];
 #pragma unroll
     for (int v = 0; v < S::TILE / S::T; ++v) {
-      if (a.half) y0[v] = mul_shoup(y0[v], pp.n_inv, pp.n_inv_sh, pp.q);
+      if (a.scaled) y0[v] = mul_shoup(y0[v], a.src_w, a.src_wsh, pp.q);
+      else if (a.half) y0[v] = mul_shoup(y0[v], pp.n_inv, pp.n_inv_sh, pp.q);
       const uint64_t x = mul_shoup(add_mod(y0[v], h, pp.q), w, wsh, pp.q);
       wv[(size_t)u * S::TILE + tid + v * S::T] = halves ? split_source(x) : x;
     }
@@ -1000,8 +1007,10 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
       const uint32_t e = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
       const uint64_t v = sm[idx + (idx >> 3)];
       const uint64_t cv = fwd_final(v, pr);
-      uint64_t r = mul_shoup(sub_mod(av[u], cv, q), w, wsh, q);
+      const uint64_t x = a.scaled ? mul_shoup(av[u], a.kw[t], a.kwsh[t], q) : av[u];
+      uint64_t r = mul_shoup(sub_mod(x, cv, q), w, wsh, q);
       if (add) r = add_mod(r, a.addw ? mul_shoup(dv[u], dw, dwsh, q) : dv[u], q);
+      if (a.with_k0 && p == 0) r = add_mod(r, a.k0[t], q);
       o[e] = r;
     }
   }

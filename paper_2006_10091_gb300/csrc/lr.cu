@@ -141,10 +141,10 @@ static int lr_plan(const he_ctx* c, uint32_t l0, double sZ, double sW, const he_
 }
 
 // Per-ciphertext words of the circuit's intermediates at input level l0:
-// U, T, A, C, B, Q, Tmp, and the gathered copies of Z and W.
+// U, T, A, C, Tmp, and the gathered copies of Z and W.
 static size_t lr_ct_words(const he_ctx* c, uint32_t l0) {
   const size_t n = c->n;
-  return n * 2 * ((l0 - 1) + (l0 - 2) + (l0 - 2) + (l0 - 3) + (l0 - 2) + (l0 - 3) + (l0 - 1) + 2 * l0) + 9 * 32;
+  return n * 2 * ((l0 - 1) + (l0 - 2) + (l0 - 2) + (l0 - 3) + (l0 - 1) + 2 * l0) + 7 * 32;
 }
 
 // Scratch words of one operation of the step: those of the per-ciphertext
@@ -201,7 +201,7 @@ static int lr_gal(he_ctx* c, const LrPlan& P, LrGal* gl) {
 }
 
 struct LrBufs {
-  CtBatch U, T, A, Cc, B, Q, Tmp, Zcopy, Wrep;
+  CtBatch U, T, A, Cc, Tmp, Zcopy, Wrep;
 };
 
 static CtBatch carve(Arena& a, size_t count, uint32_t cap, uint32_t n) {
@@ -226,19 +226,12 @@ static int lr_chunk(he_ctx* c, const LrPlan& P, const LrGal& gl, CtBatch Zc, CtB
   }
   // T = M^2; A = c3 M; C = T A
   HE_TRY(mul_relin_batch(c, b.U, b.U, l0 - 1, m, b.T, true, fresh()));
-  HE_TRY(mul_int_batch(c, b.U, b.Tmp, P.kA, l0 - 1, m));
-  HE_TRY(rescale_batch(c, b.Tmp, l0 - 1, m, b.A, fresh()));
+  HE_TRY(rescale_scaled_batch(c, b.U, RescaleScale{P.kA, nullptr, nullptr}, l0 - 1, l0 - 2, m, b.Tmp, b.A, fresh()));
   HE_TRY(mul_relin_batch(c, b.T, b.A, l0 - 2, m, b.Cc, true, fresh()));
-  // B = c1 M (dropped to l0-3); Q = c2 M^2
-  HE_TRY(mul_int_batch(c, b.U, b.Tmp, P.kB, l0 - 1, m));
-  HE_TRY(rescale_batch(c, b.Tmp, l0 - 1, m, b.B, fresh()));
-  HE_TRY(addsub_batch(c, b.Cc, b.B, b.Cc, 0, l0 - 3, m));
-  if (P.has_c2) {
-    HE_TRY(mul_int_batch(c, b.T, b.Tmp, P.kQ, l0 - 2, m));
-    HE_TRY(rescale_batch(c, b.Tmp, l0 - 2, m, b.Q, fresh()));
-    HE_TRY(addsub_batch(c, b.Cc, b.Q, b.Cc, 0, l0 - 3, m));
-  }
-  HE_TRY(add_int_batch(c, b.Cc, b.Cc, P.k0, l0 - 3, m));
+  // C + B (B = c1 M, dropped to l0-3) + c0, + Q (Q = c2 M^2)
+  HE_TRY(rescale_scaled_batch(c, b.U, RescaleScale{P.kB, &b.Cc, &P.k0}, l0 - 1, l0 - 3, m, b.Tmp, b.Cc, fresh()));
+  if (P.has_c2)
+    HE_TRY(rescale_scaled_batch(c, b.T, RescaleScale{P.kQ, &b.Cc, nullptr}, l0 - 2, l0 - 3, m, b.Tmp, b.Cc, fresh()));
   (void)infer;  // S_k = p(M_k) is in b.Cc
   return HE_OK;
 }
@@ -341,8 +334,6 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
     b.T = carve(a, chunk, l0 - 2, n);
     b.A = carve(a, chunk, l0 - 2, n);
     b.Cc = carve(a, chunk, l0 - 3, n);
-    b.B = carve(a, chunk, l0 - 2, n);
-    b.Q = carve(a, chunk, l0 - 3, n);
     b.Tmp = carve(a, chunk, l0 - 1, n);
     b.Zcopy = carve(a, chunk, l0, n);
     b.Wrep = carve(a, chunk, l0, n);
@@ -422,6 +413,15 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
       if (infer) {  // copy S_k of each segment's ciphertexts to their outputs
         for (auto& sg : seg) {
           const Shard& s = sh[grp[sg.first]];
+          CtBatch ou;
+          if (uniform_view(s.S_out + sg.second.first, sg.second.second, &ou) &&
+              (sg.second.second == 1 || ou.stride >= 2ull * ou.cap * n)) {  // (apart: one launch)
+            CtBatch src = b.Cc;
+            src.base += off * b.Cc.stride;
+            HE_TRY(copy_batch(c, src, ou, l0 - 3, (uint32_t)sg.second.second));
+            off += sg.second.second;
+            continue;
+          }
           for (size_t i = 0; i < sg.second.second; ++i) {
             CtBatch src = b.Cc;
             src.base += (off + i) * b.Cc.stride;

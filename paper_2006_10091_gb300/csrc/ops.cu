@@ -23,7 +23,7 @@ int ntt2_inverse_rows(he_ctx* c, const PolyBatch& b);
 int md_fused(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t* conv, CtBatch add, int add_mode,
              uint64_t add_gal, CtBatch out, uint32_t level, uint32_t count, bool half, bool* handled);
 int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatch out, uint32_t level,
-             uint32_t count, bool half, bool* handled);
+             uint32_t count, bool half, bool* handled, uint32_t targets, const RescaleScale* sc);
 bool ks_rot_fits(const he_ctx* c, uint32_t level);
 int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c, uint64_t* ext, uint64_t* acc,
            const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled,
@@ -248,20 +248,56 @@ int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint
   return moddown_unfused(c, acc, conv, add, add_mode, out, level, count);
 }
 
+// The rescale's fused part: the dropped limb of both parts to coefficient form
+// (corr: scratch of the conversion) and the fused kernels; *fused = false when
+// N has none (last then holds the coefficient form).
+static int rescale_fused(he_ctx* c, CtBatch in, uint32_t level, uint32_t targets, uint32_t count, CtBatch out,
+                         uint64_t* last, uint64_t* corr, const RescaleScale* sc, bool* fused) {
+  const uint32_t n = c->n, lt = level - 1;
+  const bool mh = md_half_ok(c, 1, targets, count);  // the fused kernel finishes the inverse transform
+  // both parts in one launch where their limbs lie at one stride
+  const bool even = count == 1 || in.stride == 2ull * in.cap * n;
+  for (uint32_t p = 0; p < (even ? 1u : 2u); ++p) {
+    const PolyBatch bd = even ? pb(in.base + (size_t)lt * n, last, (uint64_t)in.cap * n, n, 2 * count, 1, lt, c->L)
+                              : pb(in.base + ((size_t)p * in.cap + lt) * n, last + (size_t)p * n, in.stride, 2ull * n,
+                                   count, 1, lt, c->L);
+    HE_TRY(mh ? ntt2_inverse_rows(c, bd) : ntt_inverse(c, bd));
+  }
+  *fused = false;  // correction, NTT and division fused like ModDown's
+  return rs_fused(c, in, last, corr, out, level, count, mh, fused, targets, sc);
+}
+
+int rescale_scaled_batch(he_ctx* c, CtBatch in, const RescaleScale& sc, uint32_t level, uint32_t targets,
+                         uint32_t count, CtBatch tmp, CtBatch out, Arena& ar) {
+  const uint32_t n = c->n, lt = level - 1;
+  if (level < 2 || targets < 1 || targets > lt) return fail(HE_ELEVEL, "rescale needs two limbs");
+  if (ks_fusable(c)) {
+    uint64_t* last = ar.take<uint64_t>((size_t)count * 2 * n);
+    uint64_t* corr = ar.take<uint64_t>((size_t)count * 2 * lt * n);
+    if (!last || !corr) return fail(HE_ENOMEM, "rescale scratch too small");
+    bool fused = false;
+    HE_TRY(rescale_fused(c, in, level, targets, count, out, last, corr, &sc, &fused));
+    if (fused) return HE_OK;
+    ar.off = 0;
+  }
+  HE_TRY(mul_int_batch(c, in, tmp, sc.k, level, count));
+  if (!sc.add) {
+    HE_TRY(rescale_batch(c, tmp, level, count, out, ar));
+  } else {  // (tmp's own storage holds the rescaled product: rescale reads a limb before it writes it)
+    HE_TRY(rescale_batch(c, tmp, level, count, tmp, ar));
+    HE_TRY(addsub_batch(c, *sc.add, tmp, out, 0, targets, count));
+  }
+  return sc.k0 ? add_int_batch(c, out, out, *sc.k0, targets, count) : HE_OK;
+}
+
 int rescale_batch(he_ctx* c, CtBatch in, uint32_t level, uint32_t count, CtBatch out, Arena& ar) {
   const uint32_t n = c->n, lt = level - 1;
   if (level < 2) return fail(HE_ELEVEL, "rescale needs two limbs");
   uint64_t* last = ar.take<uint64_t>((size_t)count * 2 * n);
   uint64_t* corr = ar.take<uint64_t>((size_t)count * 2 * lt * n);
   if (!last || !corr) return fail(HE_ENOMEM, "rescale scratch too small");
-  const bool mh = md_half_ok(c, 1, lt, count);  // the fused kernel finishes the inverse transform
-  for (uint32_t p = 0; p < 2; ++p) {
-    const PolyBatch bd = pb(in.base + ((size_t)p * in.cap + lt) * n, last + (size_t)p * n, in.stride, 2ull * n,
-                            count, 1, lt, c->L);
-    HE_TRY(mh ? ntt2_inverse_rows(c, bd) : ntt_inverse(c, bd));
-  }
-  bool fused = false;  // correction, NTT and division fused like ModDown's
-  HE_TRY(rs_fused(c, in, last, corr, out, level, count, mh, &fused));
+  bool fused = false;
+  HE_TRY(rescale_fused(c, in, level, lt, count, out, last, corr, nullptr, &fused));
   if (fused) return HE_OK;
   {
     ProfScope prof(c, "rescale", (double)count * 2 * n * lt, (double)count * 2 * n * 8 * (1 + lt));
@@ -412,11 +448,8 @@ int addsub_batch(he_ctx* c, CtBatch A, CtBatch B, CtBatch O, int op, uint32_t le
 static LimbConsts int_consts(const he_ctx* c, int64_t k, uint32_t level) {
   LimbConsts kc;
   for (uint32_t t = 0; t < level; ++t) {
-    const uint64_t q = c->q[t];
-    const __int128 r = (__int128)k % (__int128)q;
-    const uint64_t v = (uint64_t)(r < 0 ? r + q : r);
-    kc.w[t] = v;
-    kc.wsh[t] = h_shoup(v, q);
+    kc.w[t] = h_mod(k, c->q[t]);
+    kc.wsh[t] = h_shoup(kc.w[t], c->q[t]);
   }
   return kc;
 }
