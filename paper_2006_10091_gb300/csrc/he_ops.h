@@ -55,8 +55,9 @@ int keyswitch_batch(he_ctx* c, const uint64_t* d, uint64_t d_stride, uint32_t le
 // evaluation form over Q_level and P; its dropped limbs are overwritten)
 // divided by P with rounding (merged: P add + acc divided by P q_{level-1}),
 // conv (count x [2][level][N]) as scratch; add_mode and gal as above.
+// pd_added: acc's limb level - 1 already holds acc + P add (merged).
 int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint32_t count, CtBatch add,
-                  int add_mode, CtBatch out, Arena& ar, uint64_t gal, bool merged);
+                  int add_mode, CtBatch out, Arena& ar, uint64_t gal, bool merged, bool pd_added = false);
 // Whether N has compiled shapes for the fused key-switching kernels.
 inline bool ks_fusable(const he_ctx* c) { return !c->ntt_generic && c->log_n >= 12 && c->log_n <= 16; }
 int rescale_batch(he_ctx* c, CtBatch in, uint32_t level, uint32_t count, CtBatch out, Arena& ar);

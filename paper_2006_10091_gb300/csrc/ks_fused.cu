@@ -52,12 +52,14 @@ bool ks_rot_fits(const he_ctx* c, uint32_t level) {
 }
 
 // ModUp -> NTT -> the summed inner products of every rotation of a hoisted
-// rotate-and-sum into one accumulator; *c0_added when part 0 (c0) is in it.
+// rotate-and-sum into one accumulator; *c0_added when part 0 (c0) is in it.  pd
+// (a key switch's merged ModDown): P times its limb level - 1 is added to acc's
+// where the kernel that runs does that (*pd_added).
 int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c, uint64_t* ext, uint64_t* acc,
            const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled, uint64_t in_gal,
-           const uint64_t* c0, uint64_t c0_stride, bool* c0_added) {
+           const uint64_t* c0, uint64_t c0_stride, bool* c0_added, const CtBatch* pd, bool* pd_added) {
   *handled = false;
-  bool added = false;
+  bool added = false, pd_in = false;
   if (c0_added) *c0_added = false;
   if (!ks_rot_fits(c, level)) return HE_OK;
   KsRotArgs ra;
@@ -66,6 +68,10 @@ int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c,
   ra.count = count;
   ra.c0 = c0;
   ra.c0_stride = c0_stride;
+  ra.pd = pd ? *pd : CtBatch{nullptr, 0, 0, 0};
+  ra.pd_limb = pd ? level - 1 : ~0u;
+  ra.pd_w = pd ? c->P_mod_q[level - 1] : 0;
+  ra.pd_wsh = pd ? h_shoup(ra.pd_w, c->q[level - 1]) : 0;
   // the kernels add nrot * beta products below q^2 in 128 bits
   uint32_t bits = 0;
   for (uint32_t t = 0; t < level; ++t) bits = std::max(bits, (uint32_t)(64 - __builtin_clzll(c->q[t])));
@@ -78,13 +84,14 @@ int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c,
   }
   int rc;
   switch (c->log_n) {
-    case 12: rc = ks_rot_n12(c, ra, count, handled, &added); break;
-    case 13: rc = ks_rot_n13(c, ra, count, handled, &added); break;
-    case 14: rc = ks_rot_n14(c, ra, count, handled, &added); break;
-    case 15: rc = ks_rot_n15(c, ra, count, handled, &added); break;
-    default: rc = ks_rot_n16(c, ra, count, handled, &added); break;
+    case 12: rc = ks_rot_n12(c, ra, count, handled, &added, &pd_in); break;
+    case 13: rc = ks_rot_n13(c, ra, count, handled, &added, &pd_in); break;
+    case 14: rc = ks_rot_n14(c, ra, count, handled, &added, &pd_in); break;
+    case 15: rc = ks_rot_n15(c, ra, count, handled, &added, &pd_in); break;
+    default: rc = ks_rot_n16(c, ra, count, handled, &added, &pd_in); break;
   }
   if (c0_added) *c0_added = *handled && added;
+  if (pd_added) *pd_added = *handled && pd && pd_in;
   return rc;
 }
 

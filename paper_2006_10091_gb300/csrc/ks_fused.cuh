@@ -24,7 +24,10 @@ namespace he {
 
 // Dynamic shared memory the conversion kernels may take.
 constexpr size_t kConvSmemMax = 200 * 1024;
-// ... and the hoisted rotate-and-sum's row pass (every digit's tile).
+// Largest grid of the row pass that gives each ciphertext four digit groups.
+// (One multiplication at N = 2^12 54 -> 47 us, sixteen 66 -> 61, whose grid is 256.)
+constexpr size_t kDigitGroupCtas = 304;
+// Shared memory of the hoisted rotate-and-sum's row pass (every digit's tile).
 constexpr size_t kRotSmemMax = 200 * 1024;
 
 struct KsFusedArgs {
@@ -340,6 +343,13 @@ struct KsRotArgs {
   // the target limbs q_t all take the split sums)
   const uint64_t* c0;
   uint64_t c0_stride;
+  // the merged ModDown's dropped limb (pd_limb: that limb, or beyond the targets):
+  // acc there also receives P d, both parts (pd_w: P mod q, Shoup pair).  In the
+  // kernels of small grids, whose launches count; the registers it takes cost
+  // ks_row_rot's others 3 %, more than the separate kernel.
+  CtBatch pd;
+  uint32_t pd_limb;
+  uint64_t pd_w, pd_wsh;
 };
 
 // The residue of a split sum, with part 0's term s0 pm (s0 a sum of up to 16
@@ -376,16 +386,19 @@ __host__ __device__ __forceinline__ bool split3_fits(uint32_t k, uint32_t nterms
 // key word it loads serves CT ciphertexts (8/CT bytes of key per key
 // product).  CT > 1 only for closed stages; a tail CTA repeats its last
 // ciphertext in the groups beyond the count and stores nothing for them.
+// In small grids (DG > 1, CT = 1) DG groups share one ciphertext's digits: each
+// runs the row pass of every DG-th digit, so the passes run side by side instead
+// of in pairs one after the other, and all threads sum the products.
 // Shared memory: the tile's twiddles, every digit's transformed tile of each
 // ciphertext ([CT][beta][TILE + TILE/8] words) and, with ra.c0, each
 // ciphertext's part-0 tile ([CT][TILE + TILE/8]).
-template <int LOG_N, int LOG_M, int LOG_K, int CT>
-__global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_row_rot(KsRotArgs ra) {
+template <int LOG_N, int LOG_M, int LOG_K, int CT, int DG>
+__global__ void __launch_bounds__(CT * DG * ((1 << (LOG_M + LOG_K)) / 8), DG > 1 ? 1 : 4 / CT) ks_row_rot(KsRotArgs ra) {
   using S = Shape<LOG_N, LOG_M, LOG_K, false>;
   constexpr uint32_t N = 1u << LOG_N;
   constexpr int PER = S::TILE / S::T;  // 8
   constexpr uint32_t TW = S::TILE + S::TILE / 8;
-  static_assert(CT == 1 || CT == 2 || CT == 4, "ciphertexts per CTA");
+  static_assert((CT == 1 || CT == 2 || CT == 4) && (DG == 1 || CT == 1), "ciphertexts and digit groups per CTA");
   const KsFusedArgs& a = ra.k;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* stw = reinterpret_cast<ulonglong2*>(smem_raw);
@@ -395,8 +408,10 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   b /= S::TILES;
   const uint32_t ngrp = (ra.count + CT - 1) / CT;
   const uint32_t i0 = (b % ngrp) * CT, t = b / ngrp;
-  const uint32_t grp = CT == 1 ? 0u : threadIdx.x / S::T;  // warp-uniform: T is a multiple of 32
-  const uint32_t ltid = CT == 1 ? threadIdx.x : threadIdx.x % S::T;
+  constexpr uint32_t NG = CT * DG;                                   // groups of T threads
+  const uint32_t gid = NG == 1 ? 0u : threadIdx.x / S::T;            // warp-uniform: T is a multiple of 32
+  const uint32_t ltid = NG == 1 ? threadIdx.x : threadIdx.x % S::T;
+  const uint32_t grp = gid / DG, dg = gid % DG;                      // ciphertext, digit group
   const uint32_t i = min(i0 + grp, ra.count - 1);
   const uint32_t prime = ks_prime(t, a.level, a.L);
   const PrimeDev pr = a.primes[prime];
@@ -408,10 +423,10 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
   // twiddles and all digit tiles are copied asynchronously up front (one
   // group each, part 0's tile with the last), so that later tiles arrive
   // while earlier ones transform
-  stage_twiddles_async<LOG_N, LOG_M, LOG_K, false>(stw, a.tw + (size_t)prime * N, tile, threadIdx.x, CT * S::T);
+  stage_twiddles_async<LOG_N, LOG_M, LOG_K, false>(stw, a.tw + (size_t)prime * N, tile, threadIdx.x, NG * S::T);
   cp_async_commit();
   pdl_wait();
-  for (uint32_t j = 0; j < a.beta; ++j) {
+  for (uint32_t j = dg; j < a.beta; j += DG) {
     uint64_t* sm = dig + ((size_t)grp * a.beta + j) * TW;
     const bool own = t >= a.lo[j] && t < a.lo[j] + a.cnt[j];
     const uint64_t* src = own ? a.d + (size_t)i * a.d_stride + (size_t)t * N
@@ -445,48 +460,62 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
       sm[idx + (idx >> 3)] = fwd_final(v, pr);
     }
   };
-  int pend = -1;  // a converted digit waiting for a partner
-  for (uint32_t j = 0; j < a.beta; ++j) {
-    const bool own = t >= a.lo[j] && t < a.lo[j] + a.cnt[j];
-    if (own) continue;
-    if (pend < 0) {
-      pend = (int)j;
-      continue;
+  if constexpr (DG > 1) {
+    cp_async_wait<0>();
+    __syncthreads();  // the twiddles, which all threads copied
+    for (uint32_t j = dg; j < a.beta; j += DG) {
+      if (t >= a.lo[j] && t < a.lo[j] + a.cnt[j]) continue;
+      uint64_t* sm = dig + (size_t)j * TW;
+      run_rounds<false, LOG_N, LOG_M, LOG_K, false, 3, DG>(sm, stw, pr, ltid, dg);
+      finish_tile(sm);
     }
-    cp_async_wait_dyn(a.beta - 1 - j);  // the twiddles and tiles 0 .. j have arrived
-    __syncthreads();
-    uint64_t* sms[2] = {dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW, dig + ((size_t)grp * a.beta + j) * TW};
-    run_rounds_n<false, LOG_N, LOG_M, LOG_K, false, 2>(sms, stw, pr, ltid);
-    finish_tile(sms[0]);
-    finish_tile(sms[1]);
-    pend = -1;
-  }
-  if (pend >= 0) {
-    uint64_t* sm = dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW;
-    cp_async_wait_dyn(a.beta - 1 - (uint32_t)pend);
-    __syncthreads();
-    run_rounds<false, LOG_N, LOG_M, LOG_K, false>(sm, stw, pr, ltid);
-    finish_tile(sm);
+  } else {
+    int pend = -1;  // a converted digit waiting for a partner
+    for (uint32_t j = 0; j < a.beta; ++j) {
+      const bool own = t >= a.lo[j] && t < a.lo[j] + a.cnt[j];
+      if (own) continue;
+      if (pend < 0) {
+        pend = (int)j;
+        continue;
+      }
+      cp_async_wait_dyn(a.beta - 1 - j);  // the twiddles and tiles 0 .. j have arrived
+      __syncthreads();
+      uint64_t* sms[2] = {dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW, dig + ((size_t)grp * a.beta + j) * TW};
+      run_rounds_n<false, LOG_N, LOG_M, LOG_K, false, 2>(sms, stw, pr, ltid);
+      finish_tile(sms[0]);
+      finish_tile(sms[1]);
+      pend = -1;
+    }
+    if (pend >= 0) {
+      uint64_t* sm = dig + ((size_t)grp * a.beta + (uint32_t)pend) * TW;
+      cp_async_wait_dyn(a.beta - 1 - (uint32_t)pend);
+      __syncthreads();
+      run_rounds<false, LOG_N, LOG_M, LOG_K, false>(sm, stw, pr, ltid);
+      finish_tile(sm);
+    }
   }
   cp_async_wait<0>();  // the own limb's tile
   __syncthreads();
   // 2. the products of the permuted digits with each rotation's key, summed
   // exactly (split sums or 128-bit sums) and reduced once per residue
   const uint32_t row0 = (uint32_t)tile << LOG_K;
+  auto add_pd = [&](uint32_t ct, uint32_t p, uint32_t e, uint64_t v) {
+    return add_mod(v, mul_shoup(cpoly(ra.pd, ct, p, t, N)[e], ra.pd_w, ra.pd_wsh, q), q);
+  };
   // key products as split sums (mac_split3) when the prime and the number of
   // summed terms allow it
   const uint32_t sb = (pr.k + 1) >> 1;
   if (split3_fits(pr.k, ra.nrot * a.beta)) {
     // one pair of neighbouring positions per pass, all CT ciphertexts with
     // each key load
-    constexpr int PPT = PER / 2 / CT;
+    constexpr int PPT = PER / 2 / NG;
     const uint32_t mask = (1u << sb) - 1;
     uint64_t pm = 1;  // P mod q_t
     if (add_c0)
       for (uint32_t u = 0; u < a.alpha; ++u) pm = mul_mod(pm, reduce64(a.primes[a.L + u].q, pr), pr);
 #pragma unroll 1
     for (int v0 = 0; v0 < PPT; ++v0) {
-      const uint32_t idx = 2 * (threadIdx.x + v0 * CT * S::T);
+      const uint32_t idx = 2 * (threadIdx.x + v0 * NG * S::T);
       const uint32_t eo = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
       uint64_t ll[CT][2][2], hh[CT][2][2], ss[CT][2][2];  // [ciphertext][part][position]
       uint64_t s0[CT][2];                                  // sum_r kappa_r(c0) (below nrot q)
@@ -542,6 +571,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             r2[u] = split3_final(ll[c][p][u], hh[c][p][u], ss[c][p][u], sb, pr, p == 0 && add_c0, s0[c][u], pm);
+            if (DG > 1 && t == ra.pd_limb) r2[u] = add_pd(i0 + c, p, eo + u, r2[u]);
           }
           *reinterpret_cast<ulonglong2*>(o0 + (size_t)p * a.nt * N + eo) = make_ulonglong2(r2[0], r2[1]);
         }
@@ -553,7 +583,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
     // each thread sums every rotation's products for its own positions, two
     // neighbouring positions at a time (16-byte key loads and stores), for
     // all CT ciphertexts with each key load
-    constexpr int PPT = PER / 2 / CT;          // position pairs per thread
+    constexpr int PPT = PER / 2 / NG;          // position pairs per thread
     constexpr int PAIRS = PPT < 2 ? PPT : 2;   // pairs per pass (bounds the registers)
     constexpr int NP = 2 * PAIRS;              // positions per pass
 #pragma unroll 1
@@ -562,7 +592,7 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
       uint64_t a0l[CT][NP], a0h[CT][NP], a1l[CT][NP], a1h[CT][NP];  // 128-bit sums of full products
 #pragma unroll
       for (int v = 0; v < PAIRS; ++v) {
-        const uint32_t idx = 2 * (threadIdx.x + (v0 + v) * CT * S::T);
+        const uint32_t idx = 2 * (threadIdx.x + (v0 + v) * NG * S::T);
         eo[v] = S::gidx(tile, idx >> LOG_M, idx & (S::M - 1));
       }
 #pragma unroll
@@ -605,12 +635,16 @@ __global__ void __launch_bounds__(CT * ((1 << (LOG_M + LOG_K)) / 8), 4 / CT) ks_
         uint64_t* o1 = o0 + (size_t)a.nt * N;
 #pragma unroll
         for (int v = 0; v < PAIRS; ++v) {
-          *reinterpret_cast<ulonglong2*>(o0 + eo[v]) =
-              make_ulonglong2(reduce128_any(a0h[c][2 * v], a0l[c][2 * v], pr),
-                              reduce128_any(a0h[c][2 * v + 1], a0l[c][2 * v + 1], pr));
-          *reinterpret_cast<ulonglong2*>(o1 + eo[v]) =
-              make_ulonglong2(reduce128_any(a1h[c][2 * v], a1l[c][2 * v], pr),
-                              reduce128_any(a1h[c][2 * v + 1], a1l[c][2 * v + 1], pr));
+          uint64_t r2[2][2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            r2[0][u] = reduce128_any(a0h[c][2 * v + u], a0l[c][2 * v + u], pr);
+            r2[1][u] = reduce128_any(a1h[c][2 * v + u], a1l[c][2 * v + u], pr);
+            if (DG > 1 && t == ra.pd_limb)
+              for (uint32_t p = 0; p < 2; ++p) r2[p][u] = add_pd(i0 + c, p, eo[v] + u, r2[p][u]);
+          }
+          *reinterpret_cast<ulonglong2*>(o0 + eo[v]) = make_ulonglong2(r2[0][0], r2[0][1]);
+          *reinterpret_cast<ulonglong2*>(o1 + eo[v]) = make_ulonglong2(r2[1][0], r2[1][1]);
         }
       }
     }
@@ -796,6 +830,8 @@ __global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra)
           if (p == 0 && add_c0) mac128(lo, hi, reduce64(s0[c][u], pr), pm);
           r2[u] = reduce128_any(hi, lo, pr);
         }
+        if (t == ra.pd_limb)
+          r2[u] = add_mod(r2[u], mul_shoup(cpoly(ra.pd, i0 + c, p, t, N)[eo + u], ra.pd_w, ra.pd_wsh, pr.q), pr.q);
       }
       *reinterpret_cast<ulonglong2*>(o + (size_t)p * a.nt * N) = make_ulonglong2(r2[0], r2[1]);
     }
@@ -837,6 +873,7 @@ struct MdArgs {
   const ulonglong2* itw;  // inverse twiddles (half)
   int half;               // yP holds only the inverse transform's row pass: md_conv_col finishes it
   uint32_t splits;        // CTAs of md_conv_col that share one tile's target limbs
+  int part_ctas;          // md_row_combine: a CTA per part instead of both parts in turn
   int split_conv;         // the conversions run as conv_split_tile (every target allows it)
   const uint64_t* md;   // ModDown tables (params.cu)
 };
@@ -955,7 +992,9 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
   uint32_t b = blockIdx.x;
   const uint32_t tile = b % S::TILES;
   b /= S::TILES;
-  const uint32_t t = b % a.level, i = b / a.level;
+  const uint32_t t = b % a.level;
+  b /= a.level;
+  const uint32_t i = a.part_ctas ? b >> 1 : b;
   const PrimeDev pr = a.primes[t];
   const uint64_t q = pr.q;
   const uint64_t* pinv = a.md + 2 * a.alpha + (size_t)a.alpha * a.L;
@@ -965,6 +1004,7 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8, 3) md_row_combine(
   pdl_wait();
   constexpr int PER = S::TILE / S::T;
   for (uint32_t p = 0; p < 2; ++p) {
+    if (a.part_ctas && p != (b & 1)) continue;  // (the other part has its own CTA)
     const uint64_t* src = a.conv + (((size_t)i * 2 + p) * a.level + t) * N;
 #pragma unroll 8
     for (uint32_t idx = threadIdx.x; idx < (uint32_t)S::TILE; idx += S::T) {
@@ -1133,7 +1173,10 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
                       a));
   }
   {
-    const size_t blocks = (size_t)count * a.level * SR::TILES;
+    // both parts in one CTA share its twiddles; in a grid that leaves the chip
+    // idle each has its own CTA, half the chain
+    a.part_ctas = (size_t)count * a.level * SR::TILES <= 304;
+    const size_t blocks = (size_t)count * a.level * SR::TILES * (a.part_ctas ? 2 : 1);
     const double addw = a.has_add == 3 ? 1.5 * polys : a.has_add == 2 ? polys : a.has_add == 1 ? polys / 2 : 0.0;
     ProfScope prof(c, nm_row, polys * (n / 2 * M2 + 2 * n), n * 8 * (3.0 * polys + addw), 0.0, polys * n / 2 * M2);
     HE_TRY(launch_pdl((md_row_combine<LOG_N, M2, K2>), blocks, SR::T, smr, c->stream,
@@ -1242,18 +1285,19 @@ int ntt2_forward_rows(he_ctx* c, const PolyBatch& b);
 // The hoisted rotate-and-sum's ModUp, column pass, row pass and the inner
 // products of every rotation.  *handled = false (nothing launched) when the
 // digits' tiles do not fit in shared memory; *c0_added: part 0 of the input
-// is in the accumulator.
+// is in the accumulator; *pd_added: so is P d on the merged ModDown's limb.
 template <int LOG_N, int M1, int K1, int M2, int K2>
-int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bool* c0_added) {
+int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bool* c0_added, bool* pd_added) {
   using SR = Shape<LOG_N, M2, K2 - 1, false>;
   const KsFusedArgs& a = ra.k;
   const size_t smr = ks_rot_smem<LOG_N, M2, K2>(a.beta);
   *handled = smr <= kRotSmemMax;
   if (!*handled) return HE_OK;
-  static std::atomic<unsigned long long> attr1{0}, attr2{0}, attr4{0}, attr_g1{0}, attr_g2{0};
-  HE_TRY(set_smem_attr_once(attr1, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 1>, kRotSmemMax));
-  HE_TRY(set_smem_attr_once(attr2, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 2>, kRotSmemMax));
-  HE_TRY(set_smem_attr_once(attr4, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 4>, kRotSmemMax));
+  static std::atomic<unsigned long long> attr1{0}, attr2{0}, attr4{0}, attr_d{0}, attr_g1{0}, attr_g2{0};
+  HE_TRY(set_smem_attr_once(attr1, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 1, 1>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr2, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 2, 1>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr_d, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 1, 4>, kRotSmemMax));
+  HE_TRY(set_smem_attr_once(attr4, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 4, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr_g1, c->device, (const void*)ks_gather_rot<LOG_N, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr_g2, c->device, (const void*)ks_gather_rot<LOG_N, 2>, kRotSmemMax));
   HE_TRY((ks_modup_launch<LOG_N, M1, K1>(c, a, count)));
@@ -1311,6 +1355,7 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
                  count * n * 8 * (conv + own + 2.0 * a.nt + (c0 ? a.level : 0)) +
                      8.0 * n * ra.nrot * a.beta * 2.0 * a.nt,
                  macs + c0_work, bfly, mac3);
+  *pd_added = !closed;
   if (!closed) {
     const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words
     const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * ((1u << LOG_N) / (2 * kGatherThreads));
@@ -1338,11 +1383,17 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
       ct = cand;
   const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * SR::TILES;
   const size_t sm = ks_rot_smem<LOG_N, M2, K2>(a.beta, ct, c0);
-  if (ct == 4) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 4>), blocks, 4 * SR::T, sm, c->stream,
+  // four digit groups where the grid leaves most of the chip idle
+  if (!c->ks_ct && a.beta > 1 && (size_t)a.nt * count * SR::TILES <= kDigitGroupCtas) {
+    *pd_added = true;
+    const size_t one_ct = (size_t)a.nt * count * SR::TILES, sm1 = ks_rot_smem<LOG_N, M2, K2>(a.beta, 1, c0);
+    return launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 1, 4>), one_ct, 4 * SR::T, sm1, c->stream, rc);
+  }
+  if (ct == 4) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 4, 1>), blocks, 4 * SR::T, sm, c->stream,
                     rc));
-  else if (ct == 2) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 2>), blocks, 2 * SR::T, sm, c->stream,
+  else if (ct == 2) HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 2, 1>), blocks, 2 * SR::T, sm, c->stream,
                    rc));
-  else HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 1>), blocks, SR::T, sm, c->stream,
+  else HE_TRY(launch_pdl((ks_row_rot<LOG_N, M2, K2 - 1, 1, 1>), blocks, SR::T, sm, c->stream,
                     rc));
   return HE_OK;
 }
@@ -1351,7 +1402,8 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
 // each, so that the template instances compile in parallel): the launches
 // for the tile shape c->ntt_shape.
 #define HE_KS_FUSED_DECL(NN)                                                         \
-  int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added); \
+  int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added, \
+                 bool* pd_added);                                                      \
   size_t ks_rot_smem_n##NN(const he_ctx* c, uint32_t beta);                          \
   int md_fused_n##NN(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled);     \
   bool md_half_n##NN(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count); \

@@ -4,10 +4,10 @@
 
 namespace he {
 
-int ks_rot_n12(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added) {
+int ks_rot_n12(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added, bool* pd_added) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_run<12, 5, 6, 7, 4>(c, a, count, handled, c0_added)
-       : sh == 2 ? ks_rot_run<12, 3, 8, 9, 2>(c, a, count, handled, c0_added) : ks_rot_run<12, 6, 5, 6, 5>(c, a, count, handled, c0_added);
+  return sh == 1 ? ks_rot_run<12, 5, 6, 7, 4>(c, a, count, handled, c0_added, pd_added)
+       : sh == 2 ? ks_rot_run<12, 3, 8, 9, 2>(c, a, count, handled, c0_added, pd_added) : ks_rot_run<12, 6, 5, 6, 5>(c, a, count, handled, c0_added, pd_added);
 }
 
 size_t ks_rot_smem_n12(const he_ctx* c, uint32_t beta) {

@@ -4,10 +4,10 @@
 
 namespace he {
 
-int ks_rot_n15(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added) {
+int ks_rot_n15(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added, bool* pd_added) {
   const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_run<15, 8, 4, 7, 4>(c, a, count, handled, c0_added)
-       : sh == 2 ? ks_rot_run<15, 6, 5, 9, 2>(c, a, count, handled, c0_added) : ks_rot_run<15, 7, 4, 8, 3>(c, a, count, handled, c0_added);
+  return sh == 1 ? ks_rot_run<15, 8, 4, 7, 4>(c, a, count, handled, c0_added, pd_added)
+       : sh == 2 ? ks_rot_run<15, 6, 5, 9, 2>(c, a, count, handled, c0_added, pd_added) : ks_rot_run<15, 7, 4, 8, 3>(c, a, count, handled, c0_added, pd_added);
 }
 
 size_t ks_rot_smem_n15(const he_ctx* c, uint32_t beta) {

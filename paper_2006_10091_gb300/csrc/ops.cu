@@ -27,7 +27,8 @@ int rs_fused(he_ctx* c, CtBatch in, const uint64_t* last, uint64_t* conv, CtBatc
 bool ks_rot_fits(const he_ctx* c, uint32_t level);
 int ks_rot(he_ctx* c, const uint64_t* d, uint64_t d_stride, const uint64_t* d2c, uint64_t* ext, uint64_t* acc,
            const RotSet& rs, uint32_t level, uint32_t count, bool half, bool* handled,
-           uint64_t in_gal = 0, const uint64_t* c0 = nullptr, uint64_t c0_stride = 0, bool* c0_added = nullptr);
+           uint64_t in_gal = 0, const uint64_t* c0 = nullptr, uint64_t c0_stride = 0, bool* c0_added = nullptr,
+           const CtBatch* pd = nullptr, bool* pd_added = nullptr);
 int md_fused_gals(he_ctx* c, const uint64_t* acc, uint64_t acc_stride, uint64_t* conv, CtBatch add, int add_mode,
                   const uint64_t* gals, uint32_t n_gal, CtBatch out, uint32_t level, uint32_t count, bool half,
                   bool* handled);
@@ -188,31 +189,32 @@ int keyswitch_batch(he_ctx* c, const uint64_t* d, uint64_t d_stride, uint32_t le
   // 2-3. ModUp + NTT + inner product, fused where N has compiled shapes and
   //      the digits' tiles fit in shared memory (the hoisted row kernel with
   //      one rotation by the identity; d read through X -> X^gal)
-  bool fused = false;
+  bool fused = false, pd_added = false;
   if (fits) {
     RotSet rs;
     rs.n = 1;
     rs.gal[0] = 1;
     rs.evk[0] = evk;
-    HE_TRY(ks_rot(c, d, d_stride, d2c, ext, acc, rs, level, count, half, &fused, gal));
+    HE_TRY(ks_rot(c, d, d_stride, d2c, ext, acc, rs, level, count, half, &fused, gal, nullptr, 0, nullptr,
+                  merged ? &add : nullptr, &pd_added));
   }
   if (!fused) {
     if (half || gal) return fail(HE_ECUDA, "keyswitch_batch: fused kernels declined");
     HE_TRY(ks_unfused_middle(c, d, d_stride, d2c, ext, acc, evk, level, count));
   }
   // 4. ModDown
-  return moddown_batch(c, acc, conv, level, count, add, add_mode, out, ar, gal, merged);
+  return moddown_batch(c, acc, conv, level, count, add, add_mode, out, ar, gal, merged, pd_added);
 }
 
 // Step 4 of the key switch on acc (count x [2][level + alpha][N], evaluation
 // form; its dropped limbs are overwritten), with conv (count x [2][level][N])
 // as scratch.
 int moddown_batch(he_ctx* c, uint64_t* acc, uint64_t* conv, uint32_t level, uint32_t count, CtBatch add,
-                  int add_mode, CtBatch out, Arena& ar, uint64_t gal, bool merged) {
+                  int add_mode, CtBatch out, Arena& ar, uint64_t gal, bool merged, bool pd_added) {
   const uint32_t n = c->n, alpha = c->alpha, nt = level + alpha;
   if (merged) {  // divide P (d0, d1) + acc by P q_{level-1}: its dropped limbs are acc's last alpha + 1
     const uint32_t lo = level - 1;
-    {
+    if (!pd_added) {
       ProfScope prof(c, "elementwise", (double)count * 2 * n, (double)count * 2 * n * 24);
       HE_TRY(launch_pdl(k_add_pd, grid_for((size_t)count * 2 * n), 256, 0, c->stream,
                         acc, (size_t)2 * nt * n, nt, add, lo, c->P_mod_q[lo], h_shoup(c->P_mod_q[lo], c->q[lo]), count, c->log_n, c->d_primes));
