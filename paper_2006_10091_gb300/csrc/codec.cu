@@ -75,10 +75,18 @@ struct FftArgs {
   int log_n, m1;
 };
 
-// sign of the exponent: -1 encode, +1 decode
+// sign of the exponent: -1 encode, +1 decode.  The negated sine is kept opaque to
+// the compiler: folded into the products it changes which of the two a fused
+// multiply-add rounds, and with it last bits and, rarely, a rounded coefficient.
+template <bool ENC>
+__device__ __forceinline__ double signed_sine(double2 w) {
+  double sn = ENC ? -w.y : w.y;
+  if (ENC) asm("" : "+d"(sn));
+  return sn;
+}
 template <bool ENC>
 __device__ __forceinline__ void fft_butterfly(double2* sm, uint32_t i0, uint32_t i1, double2 w) {
-  const double cs = w.x, sn = ENC ? -w.y : w.y;
+  const double cs = w.x, sn = signed_sine<ENC>(w);
   const double2 x = sm[i0], y = sm[i1];
   const double2 ty = make_double2(y.x * cs - y.y * sn, y.x * sn + y.y * cs);
   sm[i0] = make_double2(x.x + ty.x, x.y + ty.y);
@@ -140,7 +148,7 @@ __global__ void k_fft_second(FftArgs a) {
     const uint32_t i = ((q / kFftCols) << a.m1) | (f0 + q % kFftCols);
     const double2 v = fsm[q];
     if (ENC) {
-      const double cs = a.tab[i].x, sn = -a.tab[i].y;  // w^-i
+      const double cs = a.tab[i].x, sn = signed_sine<true>(a.tab[i]);  // w^-i
       const double re = v.x * cs - v.y * sn;
       const double raw = (a.scale / (double)n) * re;
       if (!(fabs(raw) < 9.2e18)) {
