@@ -25,6 +25,33 @@ __device__ __forceinline__ uint32_t rmod(size_t& r, uint32_t d) {
 }
 
 // ---- tensor product: (a0 b0, a0 b1 + a1 b0, a1 b1) ---------------------------
+// As split sums with one reduction per part where the prime allows it (the
+// middle part's two products in one sum), by Barrett products otherwise (279
+// instructions per coefficient, which bound the kernel, not its bytes).
+__device__ __forceinline__ void tensor3(uint64_t a0, uint64_t a1, uint64_t b0, uint64_t b1, const PrimeDev& pr,
+                                        bool split, unsigned long long& o0, unsigned long long& o1,
+                                        unsigned long long& o2) {
+  if (split) {
+    const uint32_t sb = (pr.k + 1) >> 1, mask = (1u << sb) - 1;
+    const Split3 x0 = split3(a0, sb, mask), x1 = split3(a1, sb, mask);
+    const Split3 y0 = split3(b0, sb, mask), y1 = split3(b1, sb, mask);
+    uint64_t ll = 0, hh = 0, ss = 0;
+    mac_split3(ll, hh, ss, x0, y0);
+    o0 = split3_residue(ll, hh, ss, sb, pr);
+    ll = hh = ss = 0;
+    mac_split3(ll, hh, ss, x0, y1);
+    mac_split3(ll, hh, ss, x1, y0);
+    o1 = split3_residue(ll, hh, ss, sb, pr);
+    ll = hh = ss = 0;
+    mac_split3(ll, hh, ss, x1, y1);
+    o2 = split3_residue(ll, hh, ss, sb, pr);
+  } else {
+    o0 = mul_mod(a0, b0, pr);
+    o1 = add_mod(mul_mod(a0, b1, pr), mul_mod(a1, b0, pr), pr.q);
+    o2 = mul_mod(a1, b1, pr);
+  }
+}
+
 __global__ void k_tensor(CtBatch A, CtBatch B, CtBatch D, uint64_t* d2, uint64_t d2_stride,
                          uint32_t level, uint32_t count, int log_n, const PrimeDev* primes) {
   pdl_wait();
@@ -41,12 +68,9 @@ __global__ void k_tensor(CtBatch A, CtBatch B, CtBatch D, uint64_t* d2, uint64_t
     const ulonglong2 b0 = *(const ulonglong2*)(cpoly(B, i, 0, t, n) + k);
     const ulonglong2 b1 = *(const ulonglong2*)(cpoly(B, i, 1, t, n) + k);
     ulonglong2 o0, o1, o2;
-    o0.x = mul_mod(a0.x, b0.x, pr);
-    o0.y = mul_mod(a0.y, b0.y, pr);
-    o1.x = add_mod(mul_mod(a0.x, b1.x, pr), mul_mod(a1.x, b0.x, pr), pr.q);
-    o1.y = add_mod(mul_mod(a0.y, b1.y, pr), mul_mod(a1.y, b0.y, pr), pr.q);
-    o2.x = mul_mod(a1.x, b1.x, pr);
-    o2.y = mul_mod(a1.y, b1.y, pr);
+    const bool split = pr.delta && split3_fits(pr.k, 2);
+    tensor3(a0.x, a1.x, b0.x, b1.x, pr, split, o0.x, o1.x, o2.x);
+    tensor3(a0.y, a1.y, b0.y, b1.y, pr, split, o0.y, o1.y, o2.y);
     *(ulonglong2*)(cpoly(D, i, 0, t, n) + k) = o0;
     *(ulonglong2*)(cpoly(D, i, 1, t, n) + k) = o1;
     *(ulonglong2*)(d2 + (size_t)i * d2_stride + (size_t)t * n + k) = o2;

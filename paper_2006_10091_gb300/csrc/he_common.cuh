@@ -272,6 +272,14 @@ __device__ __forceinline__ void mac_split3(uint64_t& ll, uint64_t& hh, uint64_t&
   hh += (uint64_t)x.h * w.h;
   ss += (uint64_t)x.s * w.s;
 }
+// Whether nterms products of residues below 2^k (and part 0's term, below
+// 1.01 times as much) can be summed as split sums.
+__host__ __device__ __forceinline__ bool split3_fits(uint32_t k, uint32_t nterms) {
+  uint32_t bits = 0;
+  for (uint32_t x = nterms + 2; x; x >>= 1) ++bits;
+  return 2 * ((k + 1) / 2) + 2 + bits <= 64;
+}
+
 // The sum as a 128-bit value (hi:lo).
 __device__ __forceinline__ void split3_total(uint64_t ll, uint64_t hh, uint64_t ss, uint32_t sb, uint64_t& lo,
                                              uint64_t& hi) {

@@ -369,14 +369,6 @@ __device__ __forceinline__ uint64_t split3_final(uint64_t ll, uint64_t hh, uint6
   return reduce128_any(hi, lo, pr);
 }
 
-// Whether nterms key products of residues below 2^k (and part 0's term, below
-// 1.01 times as much) can be summed as split sums.
-__host__ __device__ __forceinline__ bool split3_fits(uint32_t k, uint32_t nterms) {
-  uint32_t bits = 0;
-  for (uint32_t x = nterms + 2; x; x >>= 1) ++bits;
-  return 2 * ((k + 1) / 2) + 2 + bits <= 64;
-}
-
 // Grid: nt * ceil(count / CT) * TILES, target limb slowest and row tile
 // fastest, so that the CTAs resident at one time share their keys (one limb
 // of each rotation's key) in L2 and finish each ciphertext's limb together.

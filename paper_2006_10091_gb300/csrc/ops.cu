@@ -514,10 +514,11 @@ int accumulate_batch(he_ctx* c, CtBatch in, uint32_t count, CtBatch acc, uint32_
 // (a0 b0, a0 b1 + a1 b0, a1 b1) of each product summed into the three-part
 // accumulator acc [3][level][N] (limbs below level of A and B).  A CTA of
 // kTaSlices warps takes 32 consecutive coefficients (one per lane, coalesced
-// loads); warp w sums the products of ciphertexts w, w + kTaSlices, ..., and
-// the slices' sums are added in shared memory (modular sums are exact, so
-// the order does not change a residue).
-constexpr int kTaSlices = 8;
+// loads); warp w sums the products of ciphertexts w, w + kTaSlices, ... (as
+// split sums reduced once where the prime and their number allow it, else as
+// Barrett products), and the slices' sums are added in shared memory (modular
+// sums are exact, so the order does not change a residue).
+constexpr uint32_t kTaSlices = 8, kTaTerms = 64;  // ciphertexts a split sum takes (two products each, 2^7 at most)
 
 __global__ void __launch_bounds__(32 * kTaSlices) k_tensor_acc(CtBatch A, CtBatch B, uint32_t count, uint64_t* acc,
                                                              uint32_t level, int log_n, const PrimeDev* primes) {
@@ -536,12 +537,32 @@ __global__ void __launch_bounds__(32 * kTaSlices) k_tensor_acc(CtBatch A, CtBatc
       k = (uint32_t)(g & (n - 1));
       t = (uint32_t)(g >> log_n);
       pr = primes[t];
-      for (uint32_t i = slice; i < count; i += kTaSlices) {
-        const uint64_t x0 = cpoly(A, i, 0, t, n)[k], x1 = cpoly(A, i, 1, t, n)[k];
-        const uint64_t y0 = cpoly(B, i, 0, t, n)[k], y1 = cpoly(B, i, 1, t, n)[k];
-        s0 = add_mod(s0, mul_mod(x0, y0, pr), pr.q);
-        s1 = add_mod(s1, add_mod(mul_mod(x0, y1, pr), mul_mod(x1, y0, pr), pr.q), pr.q);
-        s2 = add_mod(s2, mul_mod(x1, y1, pr), pr.q);
+      const uint32_t sb = (pr.k + 1) >> 1, mask = (1u << (sb & 31)) - 1;
+      if (pr.delta && split3_fits(pr.k, 2 * kTaTerms)) {
+        for (uint32_t i0 = slice; i0 < count; i0 += kTaSlices * kTaTerms) {
+          uint64_t l[3] = {0, 0, 0}, h[3] = {0, 0, 0}, m[3] = {0, 0, 0};
+          const uint32_t i1 = min(count, i0 + kTaSlices * kTaTerms);
+#pragma unroll 2
+          for (uint32_t i = i0; i < i1; i += kTaSlices) {
+            const Split3 x0 = split3(cpoly(A, i, 0, t, n)[k], sb, mask), x1 = split3(cpoly(A, i, 1, t, n)[k], sb, mask);
+            const Split3 y0 = split3(cpoly(B, i, 0, t, n)[k], sb, mask), y1 = split3(cpoly(B, i, 1, t, n)[k], sb, mask);
+            mac_split3(l[0], h[0], m[0], x0, y0);
+            mac_split3(l[1], h[1], m[1], x0, y1);
+            mac_split3(l[1], h[1], m[1], x1, y0);
+            mac_split3(l[2], h[2], m[2], x1, y1);
+          }
+          s0 = add_mod(s0, split3_residue(l[0], h[0], m[0], sb, pr), pr.q);
+          s1 = add_mod(s1, split3_residue(l[1], h[1], m[1], sb, pr), pr.q);
+          s2 = add_mod(s2, split3_residue(l[2], h[2], m[2], sb, pr), pr.q);
+        }
+      } else {
+        for (uint32_t i = slice; i < count; i += kTaSlices) {
+          const uint64_t x0 = cpoly(A, i, 0, t, n)[k], x1 = cpoly(A, i, 1, t, n)[k];
+          const uint64_t y0 = cpoly(B, i, 0, t, n)[k], y1 = cpoly(B, i, 1, t, n)[k];
+          s0 = add_mod(s0, mul_mod(x0, y0, pr), pr.q);
+          s1 = add_mod(s1, add_mod(mul_mod(x0, y1, pr), mul_mod(x1, y0, pr), pr.q), pr.q);
+          s2 = add_mod(s2, mul_mod(x1, y1, pr), pr.q);
+        }
       }
     }
     part[0][slice][lane] = s0;

@@ -126,7 +126,7 @@ def test_split_sum_residue(bits):
                 continue
             k = q.bit_length()
             sb = (k + 1) // 2
-            terms = 96
+            terms = 128
             while 2 * sb + 2 + (terms + 2).bit_length() > 64:
                 terms //= 2
             for trial in range(4):

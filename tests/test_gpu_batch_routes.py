@@ -93,3 +93,21 @@ def test_conversions_match_the_separate_kernels(limbs, bits, special, sbits):
         res[generic] = [c.residues() for c in mul + rot + low]
     for got, want in zip(res[0], res[1]):
         assert np.array_equal(got, want)
+
+
+def test_gradient_sum_over_more_ciphertexts_than_a_split_sum_takes():
+    """600 data ciphertexts in one tensor accumulation (split sums of 512 at
+    most) give the residues of accumulations of 100."""
+    import torch
+    import paper_2006_10091_gb300 as he
+    g = 64
+    ctx = he.Context(12, 6, 40, 2, 59, 2.0 ** 40, seed=8, rot_steps=he.lr_rot_steps(1 << 11, g))
+    Z, W = uniform(ctx, torch, 6, 600, 5), uniform(ctx, torch, 6, 1, 6)[0]
+    cfg = he.lr_config((0.5, -0.0843, 0.0, 0.0002), 1.0 / 4096, g, 2.0 ** 27)
+    res = []
+    for chunk in (0, 100):
+        he.he_set_tuning(ctx, "lr_chunk", chunk)
+        out = ctx.new_ct(1)
+        he.he_lr_gradient_step(ctx, Z, W, cfg, out)
+        res.append(out.residues())
+    assert np.array_equal(res[0], res[1])
