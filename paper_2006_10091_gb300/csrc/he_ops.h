@@ -74,6 +74,14 @@ int rescale_scaled_batch(he_ctx* c, CtBatch in, const RescaleScale& sc, uint32_t
                          uint32_t count, CtBatch tmp, CtBatch out, Arena& ar);
 int mul_relin_batch(he_ctx* c, CtBatch A, CtBatch B, uint32_t level, uint32_t count, CtBatch out,
                     bool rescale, Arena& ar);
+// The same for factors that lie in several uniform pieces (one after the other
+// in out): a tensor product launch per piece instead of copies side by side.
+struct MulPiece {
+  CtBatch A, B;
+  uint32_t count;
+};
+int mul_relin_pieces(he_ctx* c, const std::vector<MulPiece>& pieces, uint32_t level, CtBatch out, bool rescale,
+                     Arena& ar);
 int rotate_batch(he_ctx* c, CtBatch A, uint32_t level, uint32_t count, uint64_t gal, CtBatch out,
                  Arena& ar);
 int addsub_batch(he_ctx* c, CtBatch A, CtBatch B, CtBatch O, int op, uint32_t level, uint32_t count);

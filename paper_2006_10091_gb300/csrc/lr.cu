@@ -141,10 +141,10 @@ static int lr_plan(const he_ctx* c, uint32_t l0, double sZ, double sW, const he_
 }
 
 // Per-ciphertext words of the circuit's intermediates at input level l0:
-// U, T, A, C, Tmp, and the gathered copies of Z and W.
+// U, T, A, C, Tmp, and the gathered copy of Z.
 static size_t lr_ct_words(const he_ctx* c, uint32_t l0) {
   const size_t n = c->n;
-  return n * 2 * ((l0 - 1) + (l0 - 2) + (l0 - 2) + (l0 - 3) + (l0 - 1) + 2 * l0) + 7 * 32;
+  return n * 2 * ((l0 - 1) + (l0 - 2) + (l0 - 2) + (l0 - 3) + (l0 - 1) + l0) + 6 * 32;
 }
 
 // Scratch words of one operation of the step: those of the per-ciphertext
@@ -201,7 +201,7 @@ static int lr_gal(he_ctx* c, const LrPlan& P, LrGal* gl) {
 }
 
 struct LrBufs {
-  CtBatch U, T, A, Cc, Tmp, Zcopy, Wrep;
+  CtBatch U, T, A, Cc, Tmp, Zcopy;
 };
 
 static CtBatch carve(Arena& a, size_t count, uint32_t cap, uint32_t n) {
@@ -209,9 +209,9 @@ static CtBatch carve(Arena& a, size_t count, uint32_t cap, uint32_t n) {
   return CtBatch{p, (uint64_t)2 * cap * n, cap, 0};
 }
 
-// The per-ciphertext part of the step for m data ciphertexts Zc with weights
-// Wc (stride 0: one W for all): S_k = p(M_k) in b.Cc.
-static int lr_chunk(he_ctx* c, const LrPlan& P, const LrGal& gl, CtBatch Zc, CtBatch Wc, uint32_t m, LrBufs& b,
+// The per-ciphertext part of the step for m data ciphertexts in uniform pieces,
+// each with its weights (stride 0: one W for the piece): S_k = p(M_k) in b.Cc.
+static int lr_chunk(he_ctx* c, const LrPlan& P, const LrGal& gl, const std::vector<MulPiece>& zw, uint32_t m, LrBufs& b,
                     Arena& ops, bool infer) {
   const uint32_t l0 = P.l0;
   auto fresh = [&]() -> Arena& {
@@ -219,7 +219,7 @@ static int lr_chunk(he_ctx* c, const LrPlan& P, const LrGal& gl, CtBatch Zc, CtB
     return ops;
   };
   // U = Z_k * W, then the rotate-and-sum over the F feature positions
-  HE_TRY(mul_relin_batch(c, Zc, Wc, l0, m, b.U, true, fresh()));
+  HE_TRY(mul_relin_pieces(c, zw, l0, b.U, true, fresh()));
   for (const auto& st : gl.in) {  // U <- U + its rotations, alternating buffers
     HE_TRY(rotsum_batch(c, b.U, l0 - 1, m, st.data(), (uint32_t)st.size(), b.Tmp, fresh()));
     std::swap(b.U, b.Tmp);
@@ -336,11 +336,10 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
     b.Cc = carve(a, chunk, l0 - 3, n);
     b.Tmp = carve(a, chunk, l0 - 1, n);
     b.Zcopy = carve(a, chunk, l0, n);
-    b.Wrep = carve(a, chunk, l0, n);
     Arena ops;
     ops.base = a.base + a.off;
     ops.size = a.size > a.off ? a.size - a.off : 0;
-    if (!b.Wrep.base || ops.size < lr_op_words(c, l0, (uint32_t)chunk, ns) * sizeof(uint64_t))
+    if (!b.Zcopy.base || ops.size < lr_op_words(c, l0, (uint32_t)chunk, ns) * sizeof(uint64_t))
       return fail(HE_ENOMEM, "step scratch too small");
     if (!D3) return fail(HE_ENOMEM, "step scratch too small");
     HE_CUDA(cudaMemsetAsync(D3, 0, sizeof(uint64_t) * d3_stride * ns, c->stream));
@@ -364,34 +363,28 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
           idx = 0;
         }
       }
-      CtBatch Zc, Wc;
-      CtBatch zu;
-      const Shard& s0 = sh[grp[seg[0].first]];
-      if (seg.size() == 1 && uniform_view(s0.Z + seg[0].second.first, seg[0].second.second, &zu)) {
-        Zc = zu;
-        Wc = CtBatch{s0.W.data, 0, s0.W.cap, 0};
-      } else {
-        size_t off = 0;
-        for (auto& sg : seg) {
-          const Shard& s = sh[grp[sg.first]];
-          const size_t first = sg.second.first, cnt = sg.second.second;
-          CtBatch dz = b.Zcopy, dw = b.Wrep;
-          dz.base += off * b.Zcopy.stride;
-          dw.base += off * b.Wrep.stride;
-          if (uniform_view(s.Z + first, cnt, &zu)) {
-            HE_TRY(copy_batch(c, zu, dz, l0, (uint32_t)cnt));
-          } else {
-            for (size_t i = 0; i < cnt; ++i) {
-              CtBatch one{s.Z[first + i].data, 0, s.Z[first + i].cap, 0}, d1 = dz;
-              d1.base += i * b.Zcopy.stride;
-              HE_TRY(copy_batch(c, one, d1, l0, 1));
-            }
+      // Each segment's data where it lies, or gathered when not at one stride:
+      // the first product is a tensor launch per segment. Copying Z and the
+      // replicated W side by side for one launch moved three times the bytes
+      // (inference of 21 ciphertexts in three shards, N = 2^13, level 9: 1856
+      // against 1841 us; one shard: the same launches either way).
+      std::vector<MulPiece> zw;
+      for (auto& sg : seg) {
+        const Shard& s = sh[grp[sg.first]];
+        const size_t first = sg.second.first, cnt = sg.second.second;
+        CtBatch z;
+        if (!uniform_view(s.Z + first, cnt, &z)) {
+          size_t off = 0;
+          for (const MulPiece& p : zw) off += p.count;
+          z = b.Zcopy;
+          z.base += off * b.Zcopy.stride;
+          for (size_t i = 0; i < cnt; ++i) {
+            CtBatch one{s.Z[first + i].data, 0, s.Z[first + i].cap, 0}, d1 = z;
+            d1.base += i * b.Zcopy.stride;
+            HE_TRY(copy_batch(c, one, d1, l0, 1));
           }
-          HE_TRY(copy_batch(c, CtBatch{s.W.data, 0, s.W.cap, 0}, dw, l0, (uint32_t)cnt));
-          off += cnt;
         }
-        Zc = b.Zcopy;
-        Wc = b.Wrep;
+        zw.push_back(MulPiece{z, CtBatch{s.W.data, 0, s.W.cap, 0}, (uint32_t)cnt});
       }
       if (c->io_piece) {  // pipelined host input (one shard): wait for the pieces this chunk reads
         const size_t last = seg.back().second.first + seg.back().second.second;  // ciphertexts [0, last) needed
@@ -402,7 +395,7 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
         }
       }
       if (time_first) HE_CUDA(cudaEventRecord(c->io_time[2], c->stream));
-      HE_TRY(lr_chunk(c, P, gl, Zc, Wc, (uint32_t)m, b, ops, infer));
+      HE_TRY(lr_chunk(c, P, gl, zw, (uint32_t)m, b, ops, infer));
       if (time_first) {
         HE_CUDA(cudaEventRecord(c->io_time[3], c->stream));
         c->io_timed_first = m;
@@ -432,10 +425,10 @@ static int lr_run(he_ctx* c, std::vector<Shard>& sh, const he_lr_config* cfg, ui
         }
         continue;
       }
-      for (auto& sg : seg) {  // D += tensor(S_k, Z_k) of each segment's ciphertexts
-        CtBatch sk = b.Cc, zk = Zc;
+      for (size_t k = 0; k < seg.size(); ++k) {  // D += tensor(S_k, Z_k) of each segment's ciphertexts
+        const auto& sg = seg[k];
+        CtBatch sk = b.Cc, zk = zw[k].A;
         sk.base += off * b.Cc.stride;
-        zk.base += off * Zc.stride;
         HE_TRY(tensor_acc_batch(c, sk, zk, (uint32_t)sg.second.second, D3 + sg.first * d3_stride, l0 - 3));
         off += sg.second.second;
       }

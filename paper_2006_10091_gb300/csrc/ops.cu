@@ -319,15 +319,25 @@ int rescale_batch(he_ctx* c, CtBatch in, uint32_t level, uint32_t count, CtBatch
 
 int mul_relin_batch(he_ctx* c, CtBatch A, CtBatch B, uint32_t level, uint32_t count, CtBatch out,
                     bool rescale, Arena& ar) {
+  return mul_relin_pieces(c, {MulPiece{A, B, count}}, level, out, rescale, ar);
+}
+
+int mul_relin_pieces(he_ctx* c, const std::vector<MulPiece>& pieces, uint32_t level, CtBatch out, bool rescale,
+                     Arena& ar) {
   const uint32_t n = c->n;
+  uint32_t count = 0;
+  for (const MulPiece& p : pieces) count += p.count;
   uint64_t* d01 = ar.take<uint64_t>((size_t)count * 2 * level * n);
   uint64_t* d2 = ar.take<uint64_t>((size_t)count * level * n);
   if (!d01 || !d2) return fail(HE_ENOMEM, "multiplication scratch too small");
   CtBatch D{d01, (size_t)2 * level * n, level, 0};
-  {
-    ProfScope prof(c, "tensor", 4.0 * count * level * n, (double)count * level * n * 8 * 7);
-    HE_TRY(launch_pdl(k_tensor, grid_for((size_t)count * level * n / 2), 256, 0, c->stream,
-                      A, B, D, d2, (size_t)level * n, level, count, c->log_n, c->d_primes));
+  size_t first = 0;
+  for (const MulPiece& p : pieces) {
+    ProfScope prof(c, "tensor", 4.0 * p.count * level * n, (double)p.count * level * n * 8 * 7);
+    const CtBatch Dp{d01 + first * D.stride, D.stride, level, 0};
+    HE_TRY(launch_pdl(k_tensor, grid_for((size_t)p.count * level * n / 2), 256, 0, c->stream,
+                      p.A, p.B, Dp, d2 + first * level * n, (size_t)level * n, level, p.count, c->log_n, c->d_primes));
+    first += p.count;
   }
   // with the rescale: the key switch's ModDown and the rescale as one division by P q_{level-1}
   return keyswitch_batch(c, d2, (size_t)level * n, level, count, c->d_rlk, D, 2, out, ar, 0, rescale);

@@ -1,5 +1,5 @@
 // params.cu -- host number theory and the constant tables the kernels read:
-// primes, roots, NTT twiddles with Shoup companions, basis-conversion,
+// primes, roots, NTT twiddles with their companions, basis-conversion,
 // ModDown and rescale constants, the Gaussian table.
 //
 // Conventions (free choices the paper leaves open; Sec. 3 names only N and

@@ -111,3 +111,28 @@ def test_gradient_sum_over_more_ciphertexts_than_a_split_sum_takes():
         he.he_lr_gradient_step(ctx, Z, W, cfg, out)
         res.append(out.residues())
     assert np.array_equal(res[0], res[1])
+
+
+@pytest.mark.parametrize("chunk", [0, 4, 1])
+def test_shards_in_pieces_give_the_residues_of_each_alone(chunk):
+    """Chunks that span shards (data in order, out of order and backwards, one
+    level above the weights) against each shard by itself."""
+    import torch
+    import paper_2006_10091_gb300 as he
+    g = 64
+    ctx = he.Context(12, 7, 40, 2, 59, 2.0 ** 40, seed=9, rot_steps=he.lr_rot_steps(1 << 11, g))
+    Z, W = uniform(ctx, torch, 7, 12, 7), uniform(ctx, torch, 6, 4, 8)
+    cfg = he.lr_config((0.5, -0.0843, 0.0, 0.0002), 1.0 / 16, g, 2.0 ** 27)
+    data = [Z[:3], [Z[5], Z[3], Z[9]], Z[8:5:-1], Z[10:11]]
+
+    def run(shards):
+        grads, sums = ctx.new_ct(1, len(shards)), [ctx.new_ct(3, len(z)) for z, _ in shards]
+        he.he_lr_gradient_step_workers(ctx, [(z, w, o) for (z, w), o in zip(shards, grads)], cfg)
+        he.he_lr_inference_workers(ctx, [(z, w, o) for (z, w), o in zip(shards, sums)], cfg)
+        return [[o.residues()] + [s.residues() for s in so] for o, so in zip(grads, sums)]
+
+    alone = [run([(z, w)])[0] for z, w in zip(data, W)]
+    he.he_set_tuning(ctx, "lr_chunk", chunk)
+    for a, b in zip(alone, run(list(zip(data, W)))):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
