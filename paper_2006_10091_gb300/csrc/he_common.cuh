@@ -17,13 +17,15 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fold_rules.h"
+
 #define HE_MAX_PRIMES 64
 
 struct PrimeDev {
   uint64_t q;
   uint64_t mu;        // Barrett constant floor(2^(2k)/q)
   uint32_t k;         // bit length of q
-  uint32_t delta;     // 2^k - q when 33 <= k <= 60 and it is below 2^28, 2^(k-11) and 2^((2k-4)/3), else 0
+  uint32_t delta;     // fold_delta(q): 2^k - q where folds apply, else 0
   uint64_t n_inv;     // N^-1 mod q
   uint64_t n_inv_sh;  // its Shoup companion
   uint64_t one_sh;    // Shoup companion of 1: floor(2^64 / q)
@@ -171,7 +173,7 @@ static __device__ __noinline__ uint32_t exact_lift_multiple(const uint64_t* u, s
 // q from two 23-bit halves of y < 2^46 and the pair (w, w2 = 2^23 w mod q),
 // S = y0 w + y1 w2 < 2^64 in one 64-bit sum without carries, minus its quotient
 // estimated from S's upper word (mu = floor(2^64 / q) < 2^32; it undershoots
-// floor(S / q) by less than 2.01), so the result is below 3q.  Nine instructions
+// S / q by less than 2 + 2^32 / q), so the result is below 3q.  Nine instructions
 // against the sixteen of a Shoup product (a 64-bit high product has four partial
 // products with carries): radix-8 butterfly chains in registers 4.09 per clock
 // and SM against 3.14.
@@ -180,7 +182,7 @@ struct SplitQ {
   uint64_t q3;            // 3q
 };
 constexpr uint32_t kSplitBits = 23;
-__host__ __device__ __forceinline__ bool split_prime(const PrimeDev& p) { return p.delta && p.k <= 40; }
+__host__ __device__ __forceinline__ bool split_prime(const PrimeDev& p) { return p.delta && p.k <= kSplitMaxBits; }
 __device__ __forceinline__ SplitQ split_q(const PrimeDev& p) {
   const uint64_t n = 0 - p.q;
   return SplitQ{(uint32_t)p.one_sh, lo32(n), hi32(n), 3 * p.q};
@@ -272,14 +274,6 @@ __device__ __forceinline__ void mac_split3(uint64_t& ll, uint64_t& hh, uint64_t&
   hh += (uint64_t)x.h * w.h;
   ss += (uint64_t)x.s * w.s;
 }
-// Whether nterms products of residues below 2^k (and part 0's term, below
-// 1.01 times as much) can be summed as split sums.
-__host__ __device__ __forceinline__ bool split3_fits(uint32_t k, uint32_t nterms) {
-  uint32_t bits = 0;
-  for (uint32_t x = nterms + 2; x; x >>= 1) ++bits;
-  return 2 * ((k + 1) / 2) + 2 + bits <= 64;
-}
-
 // The sum as a 128-bit value (hi:lo).
 __device__ __forceinline__ void split3_total(uint64_t ll, uint64_t hh, uint64_t ss, uint32_t sb, uint64_t& lo,
                                              uint64_t& hi) {

@@ -56,8 +56,8 @@ __host__ __device__ __forceinline__ uint32_t ks_prime(uint32_t t, uint32_t level
 
 // The basis conversion of one tile into shared memory, y = sum over u < CNT of
 // v_u c_u mod q for the T threads' elements of the tile (a few q, not reduced to
-// [0, q): the lazy transform that follows takes any 64-bit input, the corrected
-// one less than 2q).  Sources come as two 30-bit halves (split_source), v = v0
+// [0, q): the split transform that follows takes values below 2^(k+3), the lazy
+// one below 2^(k+5), the corrected one below 2q).  Sources come as two 30-bit halves (split_source), v = v0
 // + v1 2^30, constants as two half-width limbs at 2^e, e = ceil(k/2), of c and
 // c2 = 2^30 c mod q, so that the sum is A + B 2^e with two 64-bit sums of 32 x 32
 // -> 64-bit products, four multiply-adds per term and no carries, and one
@@ -120,29 +120,6 @@ __device__ __forceinline__ void conv_split(uint32_t cnt, uint64_t* sm, const uin
   else if (cnt == 3) conv_split_tile<TILE, T, 3>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
   else if (cnt == 4) conv_split_tile<TILE, T, 4>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
   else conv_split_tile<TILE, T, 5>(sm, wv, w, w2, stride, pr, tid, vv, vP, h);
-}
-
-// Whether the conversion of cnt sources below 2^src_bits to q runs as
-// conv_split_tile: the sum (plus 3q for ModDown's lift) stays below 2^64 and its
-// fold below 2^(k+5) (2^(k+3) for the split products' primes, 2q for the corrected
-// transforms'), so that the transform's values stay in range.
-inline bool conv_split_ok(uint64_t q, uint32_t cnt, uint32_t src_bits) {
-  const uint32_t k = 64 - __builtin_clzll(q), e = (k + 1) / 2;
-  if (k < 33 || k > 60 || cnt < 1 || cnt > 5 || src_bits > 60) return false;
-  const uint64_t delta = (1ull << k) - q;
-  if (delta >= (1ull << std::min({28u, k - 11, (2 * k - 4) / 3}))) return false;
-  typedef unsigned __int128 u128;
-  const u128 rho = (u128)delta << (2 * e - k);
-  u128 most = (u128)1 << src_bits;
-  if (cnt > 1) {
-    const u128 a = (u128)(2 * cnt) << (30 + e), b = (u128)(2 * cnt) << (30 + k - e);
-    if (b >> 64) return false;
-    most = a + ((u128)1 << (2 * e)) + ((b >> e) + 1) * rho;
-  }
-  most += 3 * (u128)q;
-  if (most >> 64) return false;
-  const u128 folded = ((u128)1 << k) + (most >> k) * delta;
-  return folded <= (k <= 40 ? (u128)1 << (k + 3) : q < (1ull << 58) ? (u128)1 << (k + 5) : 2 * (u128)q);
 }
 
 // The conversion of one tile for primes conv_split_ok turns down: Shoup

@@ -158,9 +158,7 @@ int build_tables(he_ctx* c) {
     p.q = q;
     p.k = (uint32_t)bitlen(q);
     p.mu = (uint64_t)(((u128)1 << (2 * p.k)) / q);
-    const uint64_t d = ((uint64_t)1 << p.k) - q;
-    // (the bounds the folds of he_common.cuh rely on)
-    if (p.k >= 33 && p.k <= 60 && d < (1ull << std::min({28u, p.k - 11, (2 * p.k - 4) / 3}))) p.delta = (uint32_t)d;
+    p.delta = fold_delta(q);
     p.n_inv = h_invmod((uint64_t)n % q, q);
     p.n_inv_sh = h_shoup(p.n_inv, q);
     p.one_sh = h_shoup(1, q);
