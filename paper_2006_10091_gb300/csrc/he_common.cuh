@@ -287,8 +287,8 @@ __device__ __forceinline__ void split3_total(uint64_t ll, uint64_t hh, uint64_t 
 }
 
 // The residue of the sum held by ll, hh, ss (2 sb = k or k + 1, prime with
-// delta != 0, at most 2^7 terms below 2^(k+1)): the sum is ll + mid 2^sb + hh 2^(2 sb) and 2^(2 sb)
-// = rho mod q (delta, or 2 delta for odd k), so with mid = mh 2^sb + ml it is
+// delta != 0, terms as split3_fits admits, so at most kSplit3Terms and part 0's):
+// the sum is ll + mid 2^sb + hh 2^(2 sb) and 2^(2 sb) = rho mod q (delta, or 2 delta for odd k), so with mid = mh 2^sb + ml it is
 // ll + ml 2^sb + (hh + mh) rho; hh + mh is folded below 1.25 2^k first, its
 // product by rho (up to 89 bits) folded like the value, which leaves it below
 // 1.3 rho delta + 2^k; the last fold leaves less than 2q because 3 delta^3 < 2^(2k-2).

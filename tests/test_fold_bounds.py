@@ -155,3 +155,38 @@ def test_low_word_of_a_128_bit_sum(rules, k):
     """reduce128_any: any 64-bit word folds below 2q, so that with the high part's [0, 2q) two corrections do."""
     for q in moduli(rules, k):
         assert fold_bound(M64, q) < 2 * q and 4 * q <= M64
+
+
+def split_sum_residue_holds(q, terms):
+    """split3_residue of `terms` products of residues below 2^k and of part 0's term (a folded sum below 1.01 times as
+    much), every intermediate at its largest."""
+    k = q.bit_length()
+    sb, d = (k + 1) // 2, (1 << k) - q
+    rho, low, high = d << (2 * sb - k), (1 << sb) - 1, (1 << (k - sb)) - 1  # the halves of a residue
+    part0 = (101 << k) // 100 >> sb                                         # the upper half of part 0's term
+    ll, hh = (terms + 1) * low * low, (terms * high + part0) * high
+    mid = terms * 2 * low * high + low * high + part0 * low
+    if (terms * (low + high) + low + part0) * (low + high) > M64:  # ss
+        return False
+    h = fold_bound(hh + (mid >> sb), q)
+    if h >= 5 << (k - 2) or h * rho >> 32 > M64 or h * rho >> k > M32:
+        return False
+    r = (h * rho >> k) * d + (1 << k) - 1 + (low << sb) + ll
+    return r <= M64 and fold_bound(r, q) < 2 * q
+
+
+@pytest.mark.parametrize("k", range(33, 61))
+def test_split_sums_the_rule_takes_reduce_to_residues(rules, k):
+    lo, hi = 0, 1 << 24  # the most terms the rule takes
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (mid, hi) if rules.split3(k, mid) else (lo, mid)
+    for q in moduli(rules, k):
+        for terms in {1, lo // 3, lo - 1, lo} - {0, -1}:
+            assert split_sum_residue_holds(q, terms), (q, terms)
+
+
+@pytest.mark.parametrize("k", range(33, 51))
+def test_every_stage_the_kernels_run_is_admitted(rules, k):
+    """16 rotations of the 21 digits whose tiles fit in shared memory, 50-bit limbs included."""
+    assert rules.split3(k, 16 * 21)
