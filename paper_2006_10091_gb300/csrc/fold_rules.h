@@ -31,14 +31,17 @@ constexpr uint32_t kSplitMaxBits = 40;
 
 // Products a split sum may hold.  split3_residue's last fold leaves less than
 // 2q up to 3470 of them (35 bits, delta at its bound: the narrowest prime for
-// its delta); the kernels ask for 16 rotations of 21 digits at most, whose tiles
-// then fill the shared memory.
+// its delta).  The callers' own limits keep below this (static assertions there):
+// a comparison in the kernels moved ks_row_rot's registers, a stage of seven
+// rotations at N = 2^14 1220 -> 1229 us.
 constexpr uint32_t kSplit3Terms = 1024;
 
 // Whether nterms products of residues below 2^k (and part 0's term, below
-// 1.01 times as much) can be summed as split sums.
+// 1.01 times as much) can be summed as split sums; nterms <= kSplit3Terms.
 HE_RULE bool split3_fits(uint32_t k, uint32_t nterms) {
-  return nterms <= kSplit3Terms && 2 * ((k + 1) / 2) + 2 + bit_length((uint64_t)nterms + 2) <= 64;
+  uint32_t bits = 0;
+  for (uint32_t x = nterms + 2; x; x >>= 1) ++bits;
+  return 2 * ((k + 1) / 2) + 2 + bits <= 64;
 }
 
 // Whether the conversion of cnt sources below 2^src_bits to q runs as

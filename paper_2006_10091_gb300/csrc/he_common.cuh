@@ -287,7 +287,7 @@ __device__ __forceinline__ void split3_total(uint64_t ll, uint64_t hh, uint64_t 
 }
 
 // The residue of the sum held by ll, hh, ss (2 sb = k or k + 1, prime with
-// delta != 0, terms as split3_fits admits, so at most kSplit3Terms and part 0's):
+// delta != 0, at most kSplit3Terms terms and part 0's, as split3_fits admits them):
 // the sum is ll + mid 2^sb + hh 2^(2 sb) and 2^(2 sb) = rho mod q (delta, or 2 delta for odd k), so with mid = mh 2^sb + ml it is
 // ll + ml 2^sb + (hh + mh) rho; hh + mh is folded below 1.25 2^k first, its
 // product by rho (up to 89 bits) folded like the value, which leaves it below

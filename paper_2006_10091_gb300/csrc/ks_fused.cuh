@@ -307,6 +307,7 @@ ks_modup_col_all(KsFusedArgs a) {
 // closed stage), ks_row_rot runs the row pass and sums all rotations for its
 // own positions from the tiles it holds in shared memory; otherwise the row
 // pass runs by itself and ks_gather_rot fetches the rows each rotation reads.
+static_assert(HE_MAX_ROT * HE_MAX_PRIMES <= kSplit3Terms, "products of a stage (rotations times digits)");
 struct KsRotArgs {
   KsFusedArgs k;           // k.acc: the accumulator (summed over the rotations)
   uint32_t nrot, count;

