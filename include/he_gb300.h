@@ -98,8 +98,9 @@ int he_sync(he_ctx* ctx);
  * of one batched operation (default 2^34), "lr_chunk" = data ciphertexts per
  * chunk of the logistic-regression step (0 = from the budget), "ntt_generic"
  * = 1 to run the runtime-shaped NTT kernel instead of the compile-time-shaped
- * one for N = 2^12 .. 2^16, "ntt_shape" = 0 (default), 1 or 2 for the three NTT tile-shape pairs compiled
- * per ring size (also used by the fused key switch), "ntt_pb_max" = at most this
+ * one for N = 2^12 .. 2^16, "ntt_shape" = 0, 1 or 2 for the three NTT tile-shape pairs compiled per ring
+ * size (also used by the fused key switch; a value means the same pair in every version of the library; the
+ * default is 2 for N = 2^14 and 2^16, 1 for N = 2^15, else 0), "ntt_pb_max" = at most this
  * many polynomials of one limb per NTT CTA (default 8), "ks_ct" = 1, 2 or 4
  * ciphertexts per CTA of the key switch's product kernel in stages whose
  * rotations keep each CTA's rows (0, the default: 2 when their tiles fit in

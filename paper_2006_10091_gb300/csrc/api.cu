@@ -242,6 +242,7 @@ int he_ctx_create(const he_params* p, const int32_t* rot_steps, size_t n_rot, vo
   c->alpha = (int)p->n_special;
   c->np = c->L + c->alpha;
   c->beta = (int)beta;
+  c->ntt_shape = default_pair(c->log_n);
   c->stream = (cudaStream_t)stream;
   cudaGetDevice(&c->device);
   {

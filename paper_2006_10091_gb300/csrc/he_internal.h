@@ -10,6 +10,7 @@
 
 #include "../../include/he_gb300.h"
 #include "he_common.cuh"
+#include "tile_pairs.h"
 
 namespace he {
 
@@ -138,7 +139,7 @@ struct he_ctx {
   size_t chunk_bytes = (size_t)1 << 34;  // scratch budget of one batched operation (16 GiB)
   uint32_t lr_chunk = 0;                 // data ciphertexts per chunk of the LR step (0: from the budget)
   bool ntt_generic = false;              // force the runtime-shaped NTT kernel (tuning)
-  int ntt_shape = 0;                     // NTT tile shapes: 0, 1 or 2 (ntt2.cu)
+  int ntt_shape = 0;                     // NTT tile shapes: 0, 1 or 2 (tile_pairs.h)
   uint32_t ntt_pb_max = 8;               // polynomials of one limb per NTT CTA, at most
   uint32_t ks_ct = 0;                    // ciphertexts per key-product CTA in closed stages (0: most that fit)
   std::map<std::string, cudaGraphExec_t> graphs;  // captured multi-worker steps

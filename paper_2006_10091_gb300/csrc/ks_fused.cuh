@@ -1384,5 +1384,26 @@ HE_KS_FUSED_DECL(14)
 HE_KS_FUSED_DECL(15)
 HE_KS_FUSED_DECL(16)
 #undef HE_KS_FUSED_DECL
+#define HE_KS_FUSED_DEFINE(NN)                                                                             \
+  int ks_rot_n##NN(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added,           \
+                 bool* pd_added) {                                                                         \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) {                                                       \
+      return ks_rot_run<NN, p.m1, p.k1, p.m2, p.k2>(c, a, count, handled, c0_added, pd_added);             \
+    });                                                                                                    \
+  }                                                                                                        \
+  size_t ks_rot_smem_n##NN(const he_ctx* c, uint32_t beta) {                                               \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return ks_rot_smem<NN, p.m2, p.k2>(beta); });         \
+  }                                                                                                        \
+  int md_fused_n##NN(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {                          \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) {                                                       \
+      return md_fused_run<NN, p.m1, p.k1, p.m2, p.k2>(c, a, count, handled);                               \
+    });                                                                                                    \
+  }                                                                                                        \
+  bool md_half_n##NN(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {                     \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return md_half<NN, p.m1, p.k1>(c, nd, targets, count); }); \
+  }                                                                                                        \
+  bool ks_half_n##NN(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint32_t count) {       \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return ks_half<NN, p.m1, p.k1>(c, level, beta, cnt, count); }); \
+  }
 
 }  // namespace he

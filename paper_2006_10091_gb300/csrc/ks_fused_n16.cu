@@ -1,36 +1,9 @@
 // ks_fused_n16.cu -- the fused key-switching kernels instantiated for N = 2^16
-// (the three tile shapes of ntt2.cu).
+// (the three tile shapes of tile_pairs.h).
 #include "ks_fused.cuh"
 
 namespace he {
 
-int ks_rot_n16(he_ctx* c, const KsRotArgs& a, uint32_t count, bool* handled, bool* c0_added, bool* pd_added) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_run<16, 8, 4, 8, 3>(c, a, count, handled, c0_added, pd_added)
-       : sh == 2 ? ks_rot_run<16, 7, 4, 9, 2>(c, a, count, handled, c0_added, pd_added) : ks_rot_run<16, 6, 5, 10, 1>(c, a, count, handled, c0_added, pd_added);
-}
-
-size_t ks_rot_smem_n16(const he_ctx* c, uint32_t beta) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? ks_rot_smem<16, 8, 3>(beta) : sh == 2 ? ks_rot_smem<16, 9, 2>(beta) : ks_rot_smem<16, 10, 1>(beta);
-}
-
-int md_fused_n16(he_ctx* c, const MdArgs& a, uint32_t count, bool* handled) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? md_fused_run<16, 8, 4, 8, 3>(c, a, count, handled)
-       : sh == 2 ? md_fused_run<16, 7, 4, 9, 2>(c, a, count, handled) : md_fused_run<16, 6, 5, 10, 1>(c, a, count, handled);
-}
-
-bool md_half_n16(const he_ctx* c, uint32_t nd, uint32_t targets, uint32_t count) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? md_half<16, 8, 4>(c, nd, targets, count)
-       : sh == 2 ? md_half<16, 7, 4>(c, nd, targets, count) : md_half<16, 6, 5>(c, nd, targets, count);
-}
-
-bool ks_half_n16(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint32_t count) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? ks_half<16, 8, 4>(c, level, beta, cnt, count)
-       : sh == 2 ? ks_half<16, 7, 4>(c, level, beta, cnt, count) : ks_half<16, 6, 5>(c, level, beta, cnt, count);
-}
+HE_KS_FUSED_DEFINE(16)
 
 }  // namespace he

@@ -1,13 +1,8 @@
 // ntt2.cu -- entry points of the two-pass NTT with compile-time tile shapes
 // (kernels in ntt2_impl.cuh, instantiated per ring size in ntt2_n12.cu ..
-// ntt2_n16.cu).  Three tile shapes per ring size (column pass bits, rows per
-// tile | row pass bits, rows per tile); c->ntt_shape picks one (the
-// autotuner times them); pair 0, the default, is the one that measured fastest
-// where the pairs differ: the gradient step at N = 2^14 63.2 ms against 66.0 and
-// 66.9, eight multiplications at N = 2^16 with 24 limbs 2.98 ms against 3.00 and
-// 3.94 (a 4096-word column tile, whose ModUp constants do not fit beside
-// it), a weighted sum at N = 2^15 106 us against 107 and 114.  The fused
-// key-switching kernels use the same pairs.  (Radix-16 rounds, Shape's LOG_V = 4 with 128-thread CTAs, measured
+// ntt2_n16.cu).  Three tile shapes per ring size (tile_pairs.h); c->ntt_shape
+// picks one (the autotuner times them).  The fused key-switching kernels use the
+// same pairs.  (Radix-16 rounds, Shape's LOG_V = 4 with 128-thread CTAs, measured
 // slower than these.)
 #include "ntt2_impl.cuh"
 

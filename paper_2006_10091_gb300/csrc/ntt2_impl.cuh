@@ -190,5 +190,15 @@ HE_NTT2_DECL(14)
 HE_NTT2_DECL(15)
 HE_NTT2_DECL(16)
 #undef HE_NTT2_DECL
+#define HE_NTT2_DEFINE(NN)                                                                                       \
+  int ntt2_n##NN(he_ctx* c, const PolyBatch& b, bool inv) {                                                      \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return run2_dir<NN, p.m1, p.k1, p.m2, p.k2>(c, b, inv); }); \
+  }                                                                                                              \
+  int ntt2_inv_rows_n##NN(he_ctx* c, const PolyBatch& b) {                                                       \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return run2_inv_rows<NN, p.m1, p.k1, p.m2, p.k2>(c, b); }); \
+  }                                                                                                              \
+  int ntt2_fwd_rows_n##NN(he_ctx* c, const PolyBatch& b) {                                                       \
+    return with_pair<NN>(c->ntt_shape, [&](auto p) { return run2_fwd_rows<NN, p.m1, p.k1, p.m2, p.k2>(c, b); }); \
+  }
 
 }  // namespace he

@@ -3,21 +3,6 @@
 
 namespace he {
 
-int ntt2_n15(he_ctx* c, const PolyBatch& b, bool inv) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? run2_dir<15, 8, 4, 7, 4>(c, b, inv) : sh == 2 ? run2_dir<15, 6, 5, 9, 2>(c, b, inv) : run2_dir<15, 7, 4, 8, 3>(c, b, inv);
-}
-
-int ntt2_inv_rows_n15(he_ctx* c, const PolyBatch& b) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? run2_inv_rows<15, 8, 4, 7, 4>(c, b)
-       : sh == 2 ? run2_inv_rows<15, 6, 5, 9, 2>(c, b) : run2_inv_rows<15, 7, 4, 8, 3>(c, b);
-}
-
-int ntt2_fwd_rows_n15(he_ctx* c, const PolyBatch& b) {
-  const int sh = c->ntt_shape;
-  return sh == 1 ? run2_fwd_rows<15, 8, 4, 7, 4>(c, b)
-       : sh == 2 ? run2_fwd_rows<15, 6, 5, 9, 2>(c, b) : run2_fwd_rows<15, 7, 4, 8, 3>(c, b);
-}
+HE_NTT2_DEFINE(15)
 
 }  // namespace he
