@@ -18,11 +18,15 @@ namespace he {
 void set_error(const std::string& msg);
 int fail(int code, const std::string& msg);
 
+// A failed call's error is taken off the runtime here, so that a later launch's
+// cudaGetLastError reports that launch and not this call again.
 #define HE_CUDA(call)                                                              \
   do {                                                                             \
     cudaError_t e_ = (call);                                                       \
-    if (e_ != cudaSuccess)                                                         \
+    if (e_ != cudaSuccess) {                                                       \
+      (void)cudaGetLastError();                                                    \
       return ::he::fail(HE_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+    }                                                                              \
   } while (0)
 
 #define HE_TRY(call)             \
