@@ -44,7 +44,6 @@ struct KsFusedArgs {
   const ulonglong2* itw;   // inverse twiddles
   int half;                // d2c holds the inverse transform's row pass only (ks_modup_col_all finishes it)
   uint32_t splits;         // CTAs of ks_modup_col_all that share one digit and tile's target limbs
-  int split_conv;          // the conversions run as conv_split_tile (every target allows it)
   const uint64_t* consts;  // ModUp constant tables
   uint32_t lo[HE_MAX_PRIMES], cnt[HE_MAX_PRIMES];
   uint64_t off[HE_MAX_PRIMES];
@@ -124,28 +123,53 @@ __device__ __forceinline__ void conv_split(uint32_t cnt, uint64_t* sm, const uin
 
 // The conversion of one tile for primes conv_split_ok turns down: Shoup
 // products by the constants (w[u * stride], companions wsh), kept in [0, 2q),
-// then to [0, q) and minus vP[vv[idx]] and h.
-template <int TILE, int T>
+// then to [0, q) and minus vP[vv[idx]] and h.  For the usual counts (CNT = 1 to
+// 5) the constants sit in registers for the whole tile; CNT = 0 takes any cnt.
+// (58-bit limbs, 61-bit special primes, N = 2^13, 64 rotations: ModUp 231 us with
+// a runtime count beside the folded sums in one kernel, 193 with these in a kernel
+// of their own; ModDown's conversion 190 and 159.)
+template <int TILE, int T, int CNT>
 __device__ __forceinline__ void conv_sum_tile(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
                                               const uint64_t* wsh, uint32_t stride, const PrimeDev& pr, uint32_t tid,
-                                              const uint32_t* vv = nullptr, const uint64_t* vP = nullptr,
-                                              uint64_t h = 0) {
+                                              const uint32_t* vv, const uint64_t* vP, uint64_t h) {
   const uint64_t q = pr.q, q2 = q + q;
+  uint64_t cw[CNT ? CNT : 1], cs[CNT ? CNT : 1];
+#pragma unroll
+  for (int u = 0; u < CNT; ++u) {
+    cw[u] = w[(size_t)u * stride];
+    cs[u] = wsh[(size_t)u * stride];
+  }
 #pragma unroll 2
   for (uint32_t idx = tid; idx < (uint32_t)TILE; idx += T) {
     uint64_t y = 0;
-    if (cnt == 1 && !vv) {
-      y = reduce64(wv[idx], pr);  // the constant is 1
+    if (CNT) {
+#pragma unroll
+      for (int u = 0; u < CNT; ++u) {
+        y += mul_shoup_lazy(wv[(size_t)u * TILE + idx], cw[u], cs[u], q);
+        if (CNT > 1) y = y >= q2 ? y - q2 : y;
+      }
     } else {
       for (uint32_t u = 0; u < cnt; ++u) {
         y += mul_shoup_lazy(wv[(size_t)u * TILE + idx], w[(size_t)u * stride], wsh[(size_t)u * stride], q);
         y = y >= q2 ? y - q2 : y;
       }
-      y = y >= q ? y - q : y;
     }
+    y = y >= q ? y - q : y;
     if (vv) y = sub_mod(sub_mod(y, vP[vv[idx]], q), h, q);
     sm[idx + (idx >> 3)] = y;
   }
+}
+
+template <int TILE, int T>
+__device__ __forceinline__ void conv_sum(uint32_t cnt, uint64_t* sm, const uint64_t* wv, const uint64_t* w,
+                                         const uint64_t* wsh, uint32_t stride, const PrimeDev& pr, uint32_t tid,
+                                         const uint32_t* vv = nullptr, const uint64_t* vP = nullptr, uint64_t h = 0) {
+  if (cnt == 1) conv_sum_tile<TILE, T, 1>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
+  else if (cnt == 2) conv_sum_tile<TILE, T, 2>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
+  else if (cnt == 3) conv_sum_tile<TILE, T, 3>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
+  else if (cnt == 4) conv_sum_tile<TILE, T, 4>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
+  else if (cnt == 5) conv_sum_tile<TILE, T, 5>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
+  else conv_sum_tile<TILE, T, 0>(cnt, sm, wv, w, wsh, stride, pr, tid, vv, vP, h);
 }
 
 // Column pass with the ModUp conversion in its load.  Grid: count * beta * nt * TILES.
@@ -212,9 +236,11 @@ __global__ void __launch_bounds__((1 << (LOG_M + LOG_K)) / 8) ks_modup_col(KsFus
 // in shared memory for those targets.  The nt targets are shared evenly by
 // a.splits CTAs, and by the G groups of T threads of a CTA, each with its own
 // tile and twiddles (the sources' tiles are what limits the CTAs of an SM, so
-// groups are how its warps are filled; conv_plan).  Grid: count * beta * splits
+// groups are how its warps are filled; conv_plan).  SPLIT: every target's
+// conversion runs as conv_split_tile (else all as conv_sum; an instance each, as
+// the two in one kernel cost both registers).  Grid: count * beta * splits
 // * TILES; dynamic shared memory: [G] twiddles, [G] tiles, cnt_max * TILE words.
-template <int LOG_N, int LOG_M, int LOG_K, int G>
+template <int LOG_N, int LOG_M, int LOG_K, int G, bool SPLIT>
 __global__ void __launch_bounds__(G * ((1 << (LOG_M + LOG_K)) / 8), 1024 / (G * ((1 << (LOG_M + LOG_K)) / 8)))
 ks_modup_col_all(KsFusedArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
@@ -238,7 +264,7 @@ ks_modup_col_all(KsFusedArgs a) {
   const uint64_t* mat_sh = mat + (size_t)cnt * a.np;
   const uint64_t* mat_2 = mat_sh + (size_t)cnt * a.np + 2 * cnt;
   const uint64_t* x = a.d2c + (size_t)i * a.level * N;
-  const bool halves = a.split_conv && cnt > 1;
+  const bool halves = SPLIT && cnt > 1;
   for (uint32_t u = grp; u < cnt; u += G) {
     const PrimeDev pa = a.primes[lo + u];
     if (a.half) {
@@ -282,8 +308,8 @@ ks_modup_col_all(KsFusedArgs a) {
     // the previous target's rounds ended with a barrier, and its write-out
     // reads only the words each thread rewrites below
     stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)prime * N, tile, tid, S::T);
-    if (a.split_conv) conv_split<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_2 + prime, a.np, pr, tid);
-    else conv_sum_tile<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr, tid);
+    if (SPLIT) conv_split<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_2 + prime, a.np, pr, tid);
+    else conv_sum<S::TILE, S::T>(cnt, sm, wv, mat + prime, mat_sh + prime, a.np, pr, tid);
     group_sync<G, S::T>(grp);
     uint64_t* out = a.ext + (((size_t)i * a.beta + j) * a.nt + t) * N;
     run_rounds<false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr, tid, grp);
@@ -844,7 +870,6 @@ struct MdArgs {
   int half;               // yP holds only the inverse transform's row pass: md_conv_col finishes it
   uint32_t splits;        // CTAs of md_conv_col that share one tile's target limbs
   int part_ctas;          // md_row_combine: a CTA per part instead of both parts in turn
-  int split_conv;         // the conversions run as conv_split_tile (every target allows it)
   const uint64_t* md;   // ModDown tables (params.cu)
 };
 
@@ -853,7 +878,7 @@ struct MdArgs {
 // memory ([alpha][TILE] words and [TILE] counts) for the CTA's share of the
 // level target limbs, which its G groups of T threads take in turn (as in
 // ks_modup_col_all).
-template <int LOG_N, int LOG_M, int LOG_K, int G>
+template <int LOG_N, int LOG_M, int LOG_K, int G, bool SPLIT>
 __global__ void __launch_bounds__(G * ((1 << (LOG_M + LOG_K)) / 8), 1024 / (G * ((1 << (LOG_M + LOG_K)) / 8)))
 md_conv_col(MdArgs a) {
   using S = Shape<LOG_N, LOG_M, LOG_K, true>;
@@ -879,7 +904,7 @@ md_conv_col(MdArgs a) {
   const uint64_t* phat = wlo + a.alpha + 9 * (size_t)a.L;         // [alpha][8] words of P/p_u, then [8] of P
   const uint64_t* mat_2 = phat + 8 * (size_t)a.alpha + 8;         // (alpha > 1)
   const uint64_t* yP = a.yP + (size_t)i * a.yp_stride + (size_t)p * a.yp_pstride;
-  const bool halves = a.split_conv && a.alpha > 1;
+  const bool halves = SPLIT && a.alpha > 1;
   // exact conversion: sum_u w_u (P/p_u) - v P, w_u = [y_u (P/p_u)^-1]_{p_u},
   // v = floor(sum_u w_u / p_u) (64.64 fixed point, resolved exactly near an
   // integer)
@@ -937,10 +962,10 @@ md_conv_col(MdArgs a) {
     const uint64_t hQ = hP[a.alpha + t];
     const uint64_t* vP = wlo + a.alpha + a.L + (size_t)t * 8;  // v P mod q_t, v < 8
     stage_twiddles<LOG_N, LOG_M, LOG_K, true>(stw, a.tw + (size_t)t * N, tile, tid, S::T);
-    if (a.split_conv)
+    if (SPLIT)
       conv_split<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_2 + t, a.L, pr, tid, vv, vP, hQ);
     else
-      conv_sum_tile<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, tid, vv, vP, hQ);
+      conv_sum<S::TILE, S::T>(a.alpha, sm, wv, mat + t, mat_sh + t, a.L, pr, tid, vv, vP, hQ);
     group_sync<G, S::T>(grp);
     run_rounds<false, LOG_N, LOG_M, LOG_K, true, 3, G>(sm, stw, pr, tid, grp);
     uint64_t* out = a.conv + (((size_t)i * 2 + p) * a.level + t) * N;
@@ -1107,8 +1132,8 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   uint32_t src_bits = 0;
   for (uint32_t u = 0; u < a.alpha; ++u)
     src_bits = std::max(src_bits, (uint32_t)(64 - __builtin_clzll(c->q[a.spr[u]])));
-  a.split_conv = 1;
-  for (uint32_t t = 0; t < a.level; ++t) a.split_conv &= conv_split_ok(c->q[t], a.alpha, src_bits) ? 1 : 0;
+  bool split = true;  // every target's conversion runs as conv_split_tile
+  for (uint32_t t = 0; t < a.level; ++t) split = split && conv_split_ok(c->q[t], a.alpha, src_bits);
   using SR = Shape<LOG_N, M2, K2, false>;
   const ConvPlan plan =
       conv_plan<LOG_N, M1, K1>(c, (size_t)count * 2 * SC::TILES, a.alpha, true, a.level, a.half != 0);
@@ -1122,11 +1147,12 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   static std::atomic<unsigned long long> attr_row{0};
   const auto conv_kernel = [&]() -> void (*)(MdArgs) {
     if constexpr (4 * SC::T <= 1024)
-      if (plan.groups == 4) return md_conv_col<LOG_N, M1, K1, 4>;
-    return plan.groups == 2 ? md_conv_col<LOG_N, M1, K1, 2> : md_conv_col<LOG_N, M1, K1, 1>;
+      if (plan.groups == 4) return split ? md_conv_col<LOG_N, M1, K1, 4, true> : md_conv_col<LOG_N, M1, K1, 4, false>;
+    if (plan.groups == 2) return split ? md_conv_col<LOG_N, M1, K1, 2, true> : md_conv_col<LOG_N, M1, K1, 2, false>;
+    return split ? md_conv_col<LOG_N, M1, K1, 1, true> : md_conv_col<LOG_N, M1, K1, 1, false>;
   }();
-  static std::atomic<unsigned long long> attr_g[3]{};
-  HE_TRY(set_smem_attr_once(attr_g[plan.groups >> 1], c->device, (const void*)conv_kernel, kConvSmemMax));
+  static std::atomic<unsigned long long> attr_g[2][3]{};
+  HE_TRY(set_smem_attr_once(attr_g[split][plan.groups >> 1], c->device, (const void*)conv_kernel, kConvSmemMax));
   HE_TRY(set_smem_attr_once(attr_row, c->device, (const void*)md_row_combine<LOG_N, M2, K2>, smr));
   const double n = (double)(1u << LOG_N);
   const double polys = 2.0 * count * a.level;  // transformed limbs
@@ -1173,13 +1199,13 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
   KsFusedArgs a = a0;
   uint32_t src_bits = 0;
   for (uint32_t t = 0; t < a.level; ++t) src_bits = std::max(src_bits, (uint32_t)(64 - __builtin_clzll(c->q[t])));
-  a.split_conv = 1;
+  bool split = true;  // every target's conversion runs as conv_split_tile
   for (uint32_t t = 0; t < a.nt; ++t)
     for (uint32_t j : {0u, a.beta - 1})  // (only the last digit may be shorter)
-      a.split_conv &= conv_split_ok(c->q[ks_prime(t, a.level, a.L)], a.cnt[j], src_bits) ? 1 : 0;
+      split = split && conv_split_ok(c->q[ks_prime(t, a.level, a.L)], a.cnt[j], src_bits);
   using SC = Shape<LOG_N, M1, K1, true>;
   const size_t smc = sizeof(ulonglong2) * SC::NTW + sizeof(uint64_t) * (SC::TILE + SC::TILE / 8);
-  static std::atomic<unsigned long long> attr_one{0}, attr_g[3]{};
+  static std::atomic<unsigned long long> attr_one{0}, attr_g[2][3]{};
   HE_TRY(set_smem_attr_once(attr_one, c->device, (const void*)ks_modup_col<LOG_N, M1, K1>, smc));
   const double n = (double)(1u << LOG_N);
   double own = 0;  // limbs each ciphertext takes as they are
@@ -1202,10 +1228,13 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
     if (plan.smem) {  // the targets of one digit and tile in `splits` CTAs
       const auto kernel = [&]() -> void (*)(KsFusedArgs) {
         if constexpr (4 * SC::T <= 1024)
-          if (plan.groups == 4) return ks_modup_col_all<LOG_N, M1, K1, 4>;
-        return plan.groups == 2 ? ks_modup_col_all<LOG_N, M1, K1, 2> : ks_modup_col_all<LOG_N, M1, K1, 1>;
+          if (plan.groups == 4)
+            return split ? ks_modup_col_all<LOG_N, M1, K1, 4, true> : ks_modup_col_all<LOG_N, M1, K1, 4, false>;
+        if (plan.groups == 2)
+          return split ? ks_modup_col_all<LOG_N, M1, K1, 2, true> : ks_modup_col_all<LOG_N, M1, K1, 2, false>;
+        return split ? ks_modup_col_all<LOG_N, M1, K1, 1, true> : ks_modup_col_all<LOG_N, M1, K1, 1, false>;
       }();
-      HE_TRY(set_smem_attr_once(attr_g[plan.groups >> 1], c->device, (const void*)kernel, kConvSmemMax));
+      HE_TRY(set_smem_attr_once(attr_g[split][plan.groups >> 1], c->device, (const void*)kernel, kConvSmemMax));
       a.splits = plan.splits;
       const size_t blocks = (size_t)count * a.beta * SC::TILES * a.splits;
       HE_TRY(launch_pdl(kernel, blocks, plan.groups * SC::T, plan.smem, c->stream,
