@@ -112,6 +112,7 @@ he_ctx* ctx_view(he_ctx* base, cudaStream_t stream) {
   v->d_primes = base->d_primes;
   v->d_tw = base->d_tw;
   v->d_itw = base->d_itw;
+  v->ntt_split = base->ntt_split;
   v->d_two64 = base->d_two64;
   v->d_gauss = base->d_gauss;
   v->d_fft = base->d_fft;

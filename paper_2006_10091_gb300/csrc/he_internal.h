@@ -120,6 +120,7 @@ struct he_ctx {
   PrimeDev* d_primes = nullptr;  // [np]
   uint64_t* d_tw = nullptr;      // [np][N] pairs (psi^brv(m), its companion, params.cu)
   uint64_t* d_itw = nullptr;     // [np][N] pairs (psi^-brv(m), its companion)
+  bool ntt_split = false;        // primes up to 40 bits have split companions in d_tw, d_itw (params.cu)
   uint64_t* d_two64 = nullptr;   // [np] 2^64 mod q
   uint64_t* d_gauss = nullptr;   // Gaussian CDT
   int gK = 0;

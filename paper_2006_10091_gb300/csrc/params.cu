@@ -173,7 +173,11 @@ int build_tables(he_ctx* c) {
 
   // twiddles: tw[m] = psi^brv(m), itw[m] = psi^-brv(m), each followed by its
   // companion: 2^23 times it mod q for the primes whose butterflies take split
-  // products (mul_split), else Shoup's
+  // products (mul_split), else Shoup's.  Rings below N = 2^11 keep Shoup's: their
+  // passes are a few CTAs long and pay for the second set of rounds in the kernel
+  // (eight rotations at N = 2^5 51.0 us with Shoup's alone, 54.4 with both; at 2^11
+  // 64 multiplications 208 and 200).
+  for (const PrimeDev& p : pd) c->ntt_split = c->ntt_split || (c->log_n >= 11 && split_prime(p));
   {
     std::vector<uint64_t> tw((size_t)np * n * 2), itw((size_t)np * n * 2), pw(n), ipw(n);
     for (int t = 0; t < np; ++t) {
@@ -189,7 +193,7 @@ int build_tables(he_ctx* c) {
         size_t o = ((size_t)t * n + m) * 2;
         tw[o] = pw[r];
         itw[o] = ipw[r];
-        if (split_prime(pd[t])) {
+        if (c->ntt_split && split_prime(pd[t])) {
           tw[o + 1] = h_mulmod(pw[r], 1ull << kSplitBits, q);
           itw[o + 1] = h_mulmod(ipw[r], 1ull << kSplitBits, q);
         } else {
