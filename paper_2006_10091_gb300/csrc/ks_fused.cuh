@@ -348,9 +348,10 @@ struct KsRotArgs {
   const uint64_t* c0;
   uint64_t c0_stride;
   // the merged ModDown's dropped limb (pd_limb: that limb, or beyond the targets):
-  // acc there also receives P d, both parts (pd_w: P mod q, Shoup pair).  In the
-  // kernels of small grids, whose launches count; the registers it takes cost
-  // ks_row_rot's others 3 %, more than the separate kernel.
+  // acc there also receives P d, both parts (pd_w: P mod q, Shoup pair).  Only in
+  // the key switch's kernel of small grids (ks_row_rot with digit groups), where
+  // launches count; the registers it takes cost ks_row_rot's others 3 %, more than
+  // the separate kernel.
   CtBatch pd;
   uint32_t pd_limb;
   uint64_t pd_w, pd_wsh;
@@ -826,8 +827,6 @@ __global__ void __launch_bounds__(kGatherThreads, 2) ks_gather_rot(KsRotArgs ra)
           if (p == 0 && add_c0) mac128(lo, hi, reduce64(s0[c][u], pr), pm);
           r2[u] = reduce128_any(hi, lo, pr);
         }
-        if (t == ra.pd_limb)
-          r2[u] = add_mod(r2[u], mul_shoup(cpoly(ra.pd, i0 + c, p, t, N)[eo + u], ra.pd_w, ra.pd_wsh, pr.q), pr.q);
       }
       *reinterpret_cast<ulonglong2*>(o + (size_t)p * a.nt * N) = make_ulonglong2(r2[0], r2[1]);
     }
@@ -1299,6 +1298,10 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   HE_TRY(set_smem_attr_once(attr4, c->device, (const void*)ks_row_rot<LOG_N, M2, K2 - 1, 4, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr_g1, c->device, (const void*)ks_gather_rot<LOG_N, 1>, kRotSmemMax));
   HE_TRY(set_smem_attr_once(attr_g2, c->device, (const void*)ks_gather_rot<LOG_N, 2>, kRotSmemMax));
+  bool closed = !ra.reduce_each;
+  for (uint32_t r = 0; r < ra.nrot && closed; ++r) closed = rot_closed<LOG_N, M2, K2 - 1>(ra.gal[r]);
+  // (a key switch, the only caller with a rotated input, rotates by the identity)
+  if (!closed && a.gal) return fail(HE_EINVAL, "ks_rot: a rotated input needs rotations that keep each tile's rows");
   HE_TRY((ks_modup_launch<LOG_N, M1, K1>(c, a, count)));
   const double n = (double)(1u << LOG_N);
   double own = 0;
@@ -1306,8 +1309,6 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   const double conv = (double)a.beta * a.nt - own;
   KsRotArgs rc = ra;
   rc.count = count;
-  bool closed = !ra.reduce_each;
-  for (uint32_t r = 0; r < ra.nrot && closed; ++r) closed = rot_closed<LOG_N, M2, K2 - 1>(ra.gal[r]);
   if (!closed) {  // the row pass by itself, in place (own limbs are read from the input)
     PolyBatch e;
     e.src = a.ext;
@@ -1354,7 +1355,7 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
                  count * n * 8 * (conv + own + 2.0 * a.nt + (c0 ? a.level : 0)) +
                      8.0 * n * ra.nrot * a.beta * 2.0 * a.nt,
                  macs + c0_work, bfly, mac3);
-  *pd_added = !closed;
+  *pd_added = false;
   if (!closed) {
     const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words
     const size_t blocks = (size_t)a.nt * ((count + ct - 1) / ct) * ((1u << LOG_N) / (2 * kGatherThreads));
