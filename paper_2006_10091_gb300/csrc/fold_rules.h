@@ -10,15 +10,11 @@
 #define HE_RULE inline
 #endif
 
-HE_RULE uint32_t bit_length(uint64_t x) {
-  uint32_t n = 0;
-  for (; x; x >>= 1) ++n;
-  return n;
-}
+inline uint32_t bit_length(uint64_t x) { return x ? 64 - __builtin_clzll(x) : 0; }
 
 // delta = 2^k - q of a prime q of k bits whose folds apply, else 0: 33 <= k <= 60
 // and delta below 2^28 and 2^((2k-4)/3) (both are below 2^(k-13) there).
-HE_RULE uint32_t fold_delta(uint64_t q) {
+inline uint32_t fold_delta(uint64_t q) {
   const uint32_t k = bit_length(q);
   if (k < 33 || k > 60) return 0;
   const uint64_t d = (1ull << k) - q;
