@@ -147,7 +147,11 @@ ALU_PEAK = {"per_second": ALU_MODMUL_PEAK, "note": "fallback: 152 SMs x 2070 MHz
             # split key products, three 32 x 32 -> 64-bit multiply-adds each (kind 4); fallback: the Shoup rate
             "mac3_per_second": ALU_MODMUL_PEAK, "mac3_note": "fallback: the Shoup-product rate",
             # radix-8 rounds of the lazy butterfly in registers (kind 2): the practical ceiling of a transform
-            "butterfly_per_second": None}
+            "butterfly_per_second": None,
+            # the same rounds as split products, on primes of up to 40 bits (kind 5); fallback: the lazy butterfly's
+            "split_butterfly_per_second": None,
+            # conversion products as folded sums, four 32 x 32 -> 64-bit multiply-adds each (kind 6); fallback: Shoup's
+            "folded_per_second": None}
 
 
 def measure_alu_peak(he) -> None:
@@ -166,6 +170,8 @@ def measure_alu_peak(he) -> None:
         ALU_PEAK["mac3_note"] = (f"measured: register-resident split key-product chain, three 32x32->64-bit "
                                  f"multiply-adds each ({m3['per_clock_per_sm']:.2f} per clock per SM)")
         ALU_PEAK["butterfly_per_second"] = he.he_probe_alu(2)["per_second"]
+        ALU_PEAK["split_butterfly_per_second"] = he.he_probe_alu(5)["per_second"]
+        ALU_PEAK["folded_per_second"] = he.he_probe_alu(6)["per_second"]
     except Exception:  # keep the fallbacks
         return
 
@@ -181,36 +187,49 @@ ALU_CLASSES = ("ntt", "intt", "ks_modup_ntt", "ks_ntt_rot_products", "moddown_nt
 KS_ROT_TRAFFIC_PER_ALG_BYTE = 555.7 / 577.8
 
 
+NARROW_KINDS = ("split_butterflies", "folded_products")
+
+
+def alu_time(p: dict) -> tuple:
+    """Seconds on the integer pipe of a class's work, each kind at its own
+    measured rate, and (amount, rate) of each kind.  Split butterflies and
+    folded products are parts of the butterflies and of the remaining
+    products."""
+    mac, mac3 = p.get("mac", 0.0), p.get("mac3", 0.0)
+    sbfly, folds = p.get("sbfly", 0.0), p.get("folds", 0.0)
+    shoup = ALU_PEAK["per_second"]
+    r_bfly = ALU_PEAK["butterfly_per_second"] or shoup
+    bfly = p.get("bfly", 0.0)
+    kinds = {"butterflies": (bfly - sbfly, r_bfly),
+             "shoup_products": (max(p["work"] - mac - mac3 - bfly - folds, 0.0), shoup),
+             "macs": (mac, ALU_PEAK["mac_per_second"]), "split_macs": (mac3, ALU_PEAK["mac3_per_second"]),
+             "split_butterflies": (sbfly, ALU_PEAK["split_butterfly_per_second"] or r_bfly),
+             "folded_products": (folds, ALU_PEAK["folded_per_second"] or shoup)}
+    return sum(n / r for n, r in kinds.values()), kinds
+
+
 def roof_time(p: dict, hbm_peak: float, name: str | None = None) -> float:
     """Seconds the class's work takes at its roof: max(weighted integer-pipe
     time, HBM time) for the integer classes (the transform and key-switching
     kernels and the tensor product's products), the HBM time for the rest."""
-    work, mac, bfly, by = p["work"], p.get("mac", 0.0), p.get("bfly", 0.0), p["bytes"]
-    mac3 = p.get("mac3", 0.0)
-    r_bfly = ALU_PEAK["butterfly_per_second"] or ALU_PEAK["per_second"]
-    other = max(work - mac - mac3 - bfly, 0.0)
-    t_alu = (bfly / r_bfly + other / ALU_PEAK["per_second"] + mac / ALU_PEAK["mac_per_second"]
-             + mac3 / ALU_PEAK["mac3_per_second"])
-    return max(t_alu, by / (hbm_peak * 1e9))
+    return max(alu_time(p)[0], p["bytes"] / (hbm_peak * 1e9))
 
 
 def class_roof(p: dict, hbm_peak: float, peak_kind: str, name: str, integer: bool | None = None) -> dict:
     """Roofline of one kernel class (or of several summed): the launch time
     against max(integer-pipe time, HBM time).  The integer-pipe time weighs
     each kind of work at its own measured register-resident rate: NTT
-    butterflies at the radix-8 lazy butterfly chain (he_probe_alu kind 2),
-    Shoup/Barrett products (conversions, scalings, reductions) at the Shoup
-    product chain (kind 1), the unreduced 128-bit key products at the
-    multiply-accumulate chain (kind 3) and the split key products at their own
-    chain (kind 4).  `frac_shoup_only` is the single-rate figure (every unit
-    of work at the Shoup rate)."""
+    butterflies at the radix-8 lazy butterfly chain (he_probe_alu kind 2) or,
+    on primes of up to 40 bits, the split one (kind 5), Shoup/Barrett products
+    (scalings, reductions, conversions that are not folded) at the Shoup
+    product chain (kind 1), conversion products as folded sums at theirs (kind
+    6), the unreduced 128-bit key products at the multiply-accumulate chain
+    (kind 3) and the split key products at their own chain (kind 4).
+    `frac_shoup_only` is the single-rate figure (every unit of work at the
+    Shoup rate)."""
     t = p["ms"] * 1e-3
-    work, mac, bfly, by = p["work"], p.get("mac", 0.0), p.get("bfly", 0.0), p["bytes"]
-    mac3 = p.get("mac3", 0.0)
-    r_bfly = ALU_PEAK["butterfly_per_second"] or ALU_PEAK["per_second"]
-    other = max(work - mac - mac3 - bfly, 0.0)
-    t_alu = (bfly / r_bfly + other / ALU_PEAK["per_second"] + mac / ALU_PEAK["mac_per_second"]
-             + mac3 / ALU_PEAK["mac3_per_second"])
+    work, by = p["work"], p["bytes"]
+    t_alu, kinds = alu_time(p)
     t_hbm = by / (hbm_peak * 1e9)
     gbs = by / t / 1e9 if t > 0 else 0.0
     base = {"kernel": name, "per_launch_ms": p["ms"] / max(1, p["launches"]), "launches": p["launches"],
@@ -224,17 +243,15 @@ def class_roof(p: dict, hbm_peak: float, peak_kind: str, name: str, integer: boo
             base.update({"bound": "alu", "achieved": rate / 1e9, "peak": peak / 1e9, "unit": "G modmul/s",
                          "frac": t_alu / t if t > 0 else 0.0,
                          "frac_shoup_only": rate / ALU_PEAK["per_second"],
-                         "work_mix": {"butterflies": bfly, "shoup_products": other, "macs": mac,
-                                      "split_macs": mac3},
-                         "peak_note": (f"weighted integer roof: {bfly:.3g} butterflies at the measured radix-8 "
-                                       f"lazy butterfly chain ({r_bfly / 1e9:.0f} G/s), {other:.3g} Shoup/Barrett "
-                                       f"products at {ALU_PEAK['note']} ({ALU_PEAK['per_second'] / 1e9:.0f} G/s), "
-                                       f"{mac:.3g} 128-bit key multiply-accumulates at {ALU_PEAK['mac_note']} "
-                                       f"({ALU_PEAK['mac_per_second'] / 1e9:.0f} G/s), {mac3:.3g} split key "
-                                       f"products at {ALU_PEAK['mac3_note']} "
-                                       f"({ALU_PEAK['mac3_per_second'] / 1e9:.0f} G/s)")})
-            if name in ("ntt", "intt"):  # butterflies alone against their chain
-                base["butterfly_chain_frac"] = (bfly / t) / r_bfly if t > 0 else 0.0
+                         # (the kinds of narrow primes only where there are any)
+                         "work_mix": {k: n for k, (n, _) in kinds.items() if n or k not in NARROW_KINDS},
+                         "peak_note": ("weighted integer roof: " + ", ".join(
+                             f"{n:.3g} {k} at {r / 1e9:.0f} G/s" for k, (n, r) in kinds.items() if n)
+                             + f"; Shoup chain {ALU_PEAK['note']}; 128-bit sums {ALU_PEAK['mac_note']}; "
+                               f"split key products {ALU_PEAK['mac3_note']}")})
+            if name in ("ntt", "intt"):  # butterflies alone against their chains
+                t_bfly = sum(n / r for n, r in (kinds["butterflies"], kinds["split_butterflies"]))
+                base["butterfly_chain_frac"] = t_bfly / t if t > 0 else 0.0
             return base
     base.update({"bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gbs / hbm_peak,
                  "peak_note": f"{peak_kind} HBM copy bandwidth"})
@@ -547,7 +564,8 @@ def large_rooflines(he, torch, stream, ctx, A, B, O, T):
 
     def summed(prof, names):
         keys = [k for k in names if k in prof]
-        return {f: sum(prof[k][f] for k in keys) for f in ("ms", "work", "mac", "mac3", "bfly", "bytes", "launches")}
+        return {f: sum(prof[k][f] for k in keys) for f in ("ms", "work", "mac", "mac3", "bfly", "sbfly", "folds",
+                                                         "bytes", "launches")}
 
     for key, fn in (("keyswitch_rotation", lambda: he.he_rotate_batch(ctx, A, 1, O)),
                     ("mul_relin_rescale", lambda: he.he_mul_relin_rescale_batch(ctx, A, B, O))):
@@ -1008,15 +1026,16 @@ def run_reference(args, rank: int):
 def run_micro(args):
     """One kernel class alone: forward/inverse NTT over `--polys` polynomials
     of 8 limbs at N = 2^log_n (more than L2), timed with CUDA events.  Each
-    rate is also given as a fraction of the register-resident radix-8 lazy
-    butterfly chain (he_probe_alu kind 2: the same butterflies with no memory
-    traffic), beside the fraction of the Shoup-product roof."""
+    rate is also given as a fraction of the register-resident radix-8 split
+    butterfly chain (he_probe_alu kind 5: the same butterflies, on 40-bit
+    primes, with no memory traffic), beside the fraction of the Shoup-product
+    roof."""
     import torch
     import __graft_entry__
     __graft_entry__.build()
     import paper_2006_10091_gb300 as he
     measure_alu_peak(he)
-    bfly_roof = he.he_probe_alu(2)["per_second"]
+    bfly_roof = he.he_probe_alu(5)["per_second"]
     from paper_2006_10091_gb300 import workloads
     stream = torch.cuda.Stream()
     torch.cuda.set_stream(stream)
@@ -1238,7 +1257,8 @@ def main():
         import __graft_entry__
         __graft_entry__.build()
         import paper_2006_10091_gb300 as he
-        names = ("imad_32", "shoup_product_64", "lazy_butterfly_radix8", "mac_128", "mac_split3")
+        names = ("imad_32", "shoup_product_64", "lazy_butterfly_radix8", "mac_128", "mac_split3",
+                 "split_butterfly_radix8", "folded_product")
         print(json.dumps({"micro": "alu", **{n: he.he_probe_alu(k) for k, n in enumerate(names)},
                           "fallback_roof": {"per_second": ALU_MODMUL_PEAK,
                                             "note": "152 SMs x 2070 MHz x 64 / 17.3 (Shoup product)"}}))

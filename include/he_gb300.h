@@ -115,7 +115,10 @@ int he_get_tuning(he_ctx* ctx, const char* key, double* value);
  * radix-8 rounds of the lazy forward butterfly, 3 = 64 x 64 -> 128-bit
  * multiply-accumulates (the key switch's unreduced key products on wide
  * primes), 4 = split key products of residues below 2^40 (three 32 x 32 ->
- * 64-bit multiply-adds each, the key products on narrower primes); per clock
+ * 64-bit multiply-adds each, the key products on narrower primes), 5 =
+ * radix-8 rounds of the split forward butterfly (primes of up to 40 bits), 6 =
+ * conversion products as folded sums (four 32 x 32 -> 64-bit multiply-adds
+ * each); per clock
  * per SM (at the device's maximum clock) and per second.  Runs two short
  * kernels on the default stream and synchronises. */
 int he_probe_alu(int kind, double* per_clock_per_sm, double* per_second);
@@ -525,6 +528,12 @@ int he_profile_names(he_ctx* ctx, char* buf, size_t cap);
  * 3, 4, 1).  Any output may be NULL. */
 int he_profile_read_kinds(he_ctx* ctx, const char* kernel_class, double* butterflies, double* macs,
                           double* split_macs);
+/* The parts of those kinds that run as cheaper instruction sequences: the
+ * butterflies on primes of up to 40 bits (split products, he_probe_alu kind 5)
+ * and the basis-conversion products summed with one folded reduction (kind 6).
+ * Any output may be NULL. */
+int he_profile_read_folded(he_ctx* ctx, const char* kernel_class, double* split_butterflies,
+                           double* folded_products);
 
 #ifdef __cplusplus
 }

@@ -131,6 +131,8 @@ def load():
         "he_profile_names": [VP, ctypes.c_char_p, ctypes.c_size_t],
         "he_profile_read_kinds": [VP, ctypes.c_char_p, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                                   ctypes.POINTER(ctypes.c_double)],
+        "he_profile_read_folded": [VP, ctypes.c_char_p, ctypes.POINTER(ctypes.c_double),
+                                   ctypes.POINTER(ctypes.c_double)],
         "he_set_tuning": [VP, ctypes.c_char_p, ctypes.c_double],
         "he_lr_train": [VP, VP, ctypes.c_size_t, ctypes.POINTER(he_lr_config), ctypes.c_uint32, ctypes.c_uint32,
                         ctypes.c_uint32, ctypes.c_uint32, CTP],
@@ -307,7 +309,7 @@ def he_get_tuning(ctx: Context, key: str) -> float:
 
 def he_probe_alu(kind: int) -> dict:
     """Register-resident integer throughput: kind 0 IMAD, 1 Shoup product, 2 lazy butterfly,
-    3 64 x 64 -> 128-bit multiply-accumulate."""
+    3 64 x 64 -> 128-bit multiply-accumulate, 4 split key product, 5 split butterfly, 6 folded conversion product."""
     pc, ps = ctypes.c_double(), ctypes.c_double()
     _check(load().he_probe_alu(kind, ctypes.byref(pc), ctypes.byref(ps)))
     return {"per_clock_per_sm": pc.value, "per_second": ps.value}
@@ -742,8 +744,10 @@ def he_profile_read(ctx, kernel_class: str) -> dict:
     bfly, mac, mac3 = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
     _check(load().he_profile_read_kinds(ctx.ptr, kernel_class.encode(), ctypes.byref(bfly), ctypes.byref(mac),
                                         ctypes.byref(mac3)))
+    sbfly, folds = ctypes.c_double(), ctypes.c_double()
+    _check(load().he_profile_read_folded(ctx.ptr, kernel_class.encode(), ctypes.byref(sbfly), ctypes.byref(folds)))
     return {"launches": n.value, "ms": ms.value, "work": work.value, "bytes": by.value, "mac": mac.value,
-            "mac3": mac3.value, "bfly": bfly.value}
+            "mac3": mac3.value, "bfly": bfly.value, "sbfly": sbfly.value, "folds": folds.value}
 
 
 def he_profile_names(ctx) -> list:

@@ -101,6 +101,8 @@ struct ProfClass {
   double mac = 0.0;   // the part of work that is unreduced 128-bit multiply-accumulates
   double mac3 = 0.0;  // ... that is split products summed as three 64-bit sums (mac_split3)
   double bfly = 0.0;  // the part of work that is NTT butterflies
+  double sbfly = 0.0; // the part of those butterflies that are split products (primes up to 40 bits)
+  double folds = 0.0; // the part of work that is conversion products as folded sums
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;
 };
 
@@ -188,7 +190,7 @@ namespace he {
 class ProfScope {
  public:
   ProfScope(he_ctx* c, const char* name, double work, double bytes, double mac = 0.0, double bfly = 0.0,
-            double mac3 = 0.0);
+            double mac3 = 0.0, double sbfly = 0.0, double folds = 0.0);
   ~ProfScope();
 
  private:
@@ -232,5 +234,27 @@ struct PolyBatch {
 };
 int ntt_forward(he_ctx* c, const PolyBatch& b);
 int ntt_inverse(he_ctx* c, const PolyBatch& b);
+
+// Whether the butterflies of prime `p` (its index) run as split products.
+inline bool split_limb(const he_ctx* c, uint32_t p) {
+  return c->ntt_split && bit_length(c->q[p]) <= kSplitMaxBits && fold_delta(c->q[p]);
+}
+// Transformed limbs of a batch, and how many of them have split butterflies
+// (for the kernel timing; nothing is counted while it is off).
+struct LimbCount {
+  double all = 0.0, split = 0.0;
+};
+inline LimbCount limb_count(const he_ctx* c, const PolyBatch& b) {
+  LimbCount n;
+  if (!c->prof_on) return n;
+  for (uint32_t t = b.limb0; t < b.limb0 + b.nl; ++t) {
+    double polys = b.npolys;
+    if (b.skip_alpha && t < b.level)  // digit t / skip_alpha takes the limb as it is
+      for (uint32_t j = t / b.skip_alpha; j < b.npolys; j += b.skip_beta ? b.skip_beta : 1) polys -= 1.0;
+    n.all += polys;
+    if (split_limb(c, t < b.level ? t : (uint32_t)c->L + t - b.level)) n.split += polys;
+  }
+  return n;
+}
 
 }  // namespace he

@@ -1155,6 +1155,9 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
   HE_TRY(set_smem_attr_once(attr_row, c->device, (const void*)md_row_combine<LOG_N, M2, K2>, smr));
   const double n = (double)(1u << LOG_N);
   const double polys = 2.0 * count * a.level;  // transformed limbs
+  double spolys = 0.0, sdrop = 0.0;            // those, and the dropped ones, with split butterflies
+  for (uint32_t t = 0; t < a.level && c->prof_on; ++t) spolys += split_limb(c, t) ? 2.0 * count : 0.0;
+  for (uint32_t u = 0; u < a.alpha && c->prof_on; ++u) sdrop += split_limb(c, a.spr[u]) ? 2.0 * count : 0.0;
   const char* nm_col = a.kind == 1 ? "rescale_ntt" : a.kind == 2 ? "moddown_rescale_ntt" : "moddown_ntt";
   const char* nm_row = a.kind == 1 ? "rescale_ntt_final" : a.kind == 2 ? "moddown_rescale_ntt_combine"
                                                                        : "moddown_ntt_combine";
@@ -1163,7 +1166,8 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
     const size_t blocks = (size_t)count * 2 * SC::TILES * a.splits;
     // with a half-transformed input, also the dropped limbs' inverse column pass
     const double bfly = polys * n / 2 * M1 + (a.half ? 2.0 * count * a.alpha * n / 2 * M1 : 0.0);
-    ProfScope prof(c, nm_col, bfly + polys * n * a.alpha, n * 8 * (2.0 * count * a.alpha + polys), 0.0, bfly);
+    ProfScope prof(c, nm_col, bfly + polys * n * a.alpha, n * 8 * (2.0 * count * a.alpha + polys), 0.0, bfly, 0.0,
+                   (spolys + (a.half ? sdrop : 0.0)) * n / 2 * M1, split ? polys * n * a.alpha : 0.0);
     HE_TRY(launch_pdl(conv_kernel, blocks, plan.groups * SC::T, plan.smem, c->stream,
                       a));
   }
@@ -1173,7 +1177,8 @@ int md_fused_run(he_ctx* c, const MdArgs& a0, uint32_t count, bool* handled) {
     a.part_ctas = (size_t)count * a.level * SR::TILES <= 304;
     const size_t blocks = (size_t)count * a.level * SR::TILES * (a.part_ctas ? 2 : 1);
     const double addw = a.has_add == 3 ? 1.5 * polys : a.has_add == 2 ? polys : a.has_add == 1 ? polys / 2 : 0.0;
-    ProfScope prof(c, nm_row, polys * (n / 2 * M2 + 2 * n), n * 8 * (3.0 * polys + addw), 0.0, polys * n / 2 * M2);
+    ProfScope prof(c, nm_row, polys * (n / 2 * M2 + 2 * n), n * 8 * (3.0 * polys + addw), 0.0, polys * n / 2 * M2,
+                   0.0, spolys * n / 2 * M2);
     HE_TRY(launch_pdl((md_row_combine<LOG_N, M2, K2>), blocks, SR::T, smr, c->stream,
                       a));
   }
@@ -1189,6 +1194,18 @@ bool ks_half(const he_ctx* c, uint32_t level, uint32_t beta, uint32_t cnt, uint3
   const ConvPlan half = conv_plan<LOG_N, M1, K1>(c, blocks, cnt, false, nt, true);
   const ConvPlan full = conv_plan<LOG_N, M1, K1>(c, blocks, cnt, false, nt, false);
   return half.smem && half.cost <= full.cost + col_pass_units((size_t)count * level, SC::TILES);
+}
+
+// Limbs per ciphertext with split butterflies: the converted ones (split) and
+// the input's own (all); nothing is counted while the timing is off.
+inline LimbCount ks_split_limbs(const he_ctx* c, const KsFusedArgs& a) {
+  LimbCount n;
+  for (uint32_t t = 0; t < a.nt && c->prof_on; ++t)
+    if (split_limb(c, ks_prime(t, a.level, a.L))) {
+      n.split += t < a.level ? a.beta - 1 : a.beta;
+      n.all += t < a.level ? 1 : 0;
+    }
+  return n;
 }
 
 // The ModUp + column-pass launch shared by the key switch and the hoisted
@@ -1210,6 +1227,7 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
   double own = 0;  // limbs each ciphertext takes as they are
   for (uint32_t j = 0; j < a.beta; ++j) own += a.cnt[j];
   const double conv = (double)a.beta * a.nt - own;  // converted limbs per ciphertext
+  const LimbCount sl = ks_split_limbs(c, a);
   double conv_products = 0;  // basis-conversion products (none when a digit is one limb)
   for (uint32_t j = 0; j < a.beta; ++j)
     if (a.cnt[j] > 1) conv_products += (double)(a.nt - a.cnt[j]) * a.cnt[j];
@@ -1218,11 +1236,13 @@ int ks_modup_launch(he_ctx* c, const KsFusedArgs& a0, uint32_t count) {
     // with a half-transformed input the kernel also runs the inverse column pass of the level input limbs
     const double inv_bfly = a.half ? (double)a.level * n / 2 * M1 + (double)a.level * n : 0.0;
     const double bfly = count * (conv * n / 2 * M1 + (a.half ? (double)a.level * n / 2 * M1 : 0.0));
-    ProfScope prof(c, "ks_modup_ntt", count * (conv * n / 2 * M1 + conv_products * n + inv_bfly),
-                   count * n * 8 * (a.level + conv), 0.0, bfly);
     // (the first digit has the most limbs)
     const ConvPlan plan =
         conv_plan<LOG_N, M1, K1>(c, (size_t)count * a.beta * SC::TILES, a.cnt[0], false, a.nt, a.half != 0);
+    ProfScope prof(c, "ks_modup_ntt", count * (conv * n / 2 * M1 + conv_products * n + inv_bfly),
+                   count * n * 8 * (a.level + conv), 0.0, bfly, 0.0,
+                   count * n / 2 * M1 * (sl.split + (a.half ? sl.all : 0.0)),
+                   split && plan.smem ? count * conv_products * n : 0.0);
     if (a.half && !plan.smem) return fail(HE_EINVAL, "ks_fused: half-transformed input needs the all-targets kernel");
     if (plan.smem) {  // the targets of one digit and tile in `splits` CTAs
       const auto kernel = [&]() -> void (*)(KsFusedArgs) {
@@ -1354,7 +1374,7 @@ int ks_rot_run(he_ctx* c, const KsRotArgs& ra, uint32_t count, bool* handled, bo
   ProfScope prof(c, "ks_ntt_rot_products", bfly + count * 2.0 * a.nt * n + macs + mac3 + c0_work,
                  count * n * 8 * (conv + own + 2.0 * a.nt + (c0 ? a.level : 0)) +
                      8.0 * n * ra.nrot * a.beta * 2.0 * a.nt,
-                 macs + c0_work, bfly, mac3);
+                 macs + c0_work, bfly, mac3, closed ? count * ks_split_limbs(c, a).split * n / 2 * M2 : 0.0);
   *pd_added = false;
   if (!closed) {
     const uint32_t ct = count >= 2 ? 2 : 1;  // two ciphertexts per CTA share its key words

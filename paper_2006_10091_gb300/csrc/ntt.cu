@@ -213,21 +213,12 @@ static int launch_pass(he_ctx* c, const PolyBatch& b, bool inv, bool col, int lo
   if (blocks > 0x7fffffffull) return fail(HE_EINVAL, "NTT batch too large");
   const size_t smem = sizeof(uint64_t) * (tilesz + tilesz / 8);
   // algorithmic work: (N/2) * log_m butterflies and 16 N bytes per transformed limb
-  double transforms = (double)b.npolys * b.nl;
-  if (b.skip_alpha && c->prof_on) {
-    transforms = 0;
-    for (uint32_t p = 0; p < b.npolys; ++p) {
-      const uint32_t j = p % a.skip_beta, lo = j * b.skip_alpha, hi = std::min(lo + b.skip_alpha, b.level);
-      uint32_t skipped = 0;
-      for (uint32_t t = b.limb0; t < b.limb0 + b.nl; ++t) skipped += (t >= lo && t < hi);
-      transforms += b.nl - skipped;
-    }
-  }
+  const LimbCount transforms = limb_count(c, b);
   const double nn = (double)(1u << c->log_n);
   // work: the butterflies, and the inverse's scaling by N^-1 in its last pass
-  const double scale = inv && last ? transforms * nn : 0.0;
-  ProfScope prof(c, inv ? "intt" : "ntt", transforms * nn / 2 * log_m + scale, transforms * nn * 16, 0.0,
-                 transforms * nn / 2 * log_m);
+  const double scale = inv && last ? transforms.all * nn : 0.0;
+  ProfScope prof(c, inv ? "intt" : "ntt", transforms.all * nn / 2 * log_m + scale, transforms.all * nn * 16,
+                 0.0, transforms.all * nn / 2 * log_m, 0.0, transforms.split * nn / 2 * log_m);
   const auto pick = [&](auto split) -> void (*)(NttPassArgs) {
     constexpr bool SPLIT = decltype(split)::value;
     if (inv) return col ? ntt_pass_kernel<true, true, SPLIT> : ntt_pass_kernel<true, false, SPLIT>;

@@ -126,21 +126,12 @@ int launch2(he_ctx* c, const PolyBatch& b, const uint64_t* src, uint64_t* dst, u
   const size_t blocks = (size_t)((b.npolys + pb - 1) / pb) * b.nl * S::TILES;
   if (blocks == 0) return HE_OK;
   if (blocks > 0x7fffffffull) return fail(HE_EINVAL, "NTT batch too large");
-  double transforms = (double)b.npolys * b.nl;
-  if (b.skip_alpha && c->prof_on) {
-    transforms = 0;
-    for (uint32_t p = 0; p < b.npolys; ++p) {
-      const uint32_t j = p % a.skip_beta, lo = j * b.skip_alpha, hi = min(lo + b.skip_alpha, b.level);
-      uint32_t skipped = 0;
-      for (uint32_t t = b.limb0; t < b.limb0 + b.nl; ++t) skipped += (t >= lo && t < hi);
-      transforms += b.nl - skipped;
-    }
-  }
+  const LimbCount transforms = limb_count(c, b);
   const double nn = (double)(1u << LOG_N);
   // work: the butterflies, and the inverse's scaling by N^-1 in its last pass
-  const double scale = INV && last ? transforms * nn : 0.0;
-  ProfScope prof(c, INV ? "intt" : "ntt", transforms * nn / 2 * LOG_M + scale, transforms * nn * 16, 0.0,
-                 transforms * nn / 2 * LOG_M);
+  const double scale = INV && last ? transforms.all * nn : 0.0;
+  ProfScope prof(c, INV ? "intt" : "ntt", transforms.all * nn / 2 * LOG_M + scale, transforms.all * nn * 16,
+                 0.0, transforms.all * nn / 2 * LOG_M, 0.0, transforms.split * nn / 2 * LOG_M);
   HE_TRY(launch_pdl((ntt2_kernel<INV, LOG_N, LOG_M, LOG_K, COL, LOG_V>), blocks, S::T, smem, c->stream,
                     a));
   return HE_OK;

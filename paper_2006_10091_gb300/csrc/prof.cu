@@ -13,7 +13,8 @@ static thread_local bool tl_prof_suppressed = false;
 ProfSuppress::ProfSuppress() : prev_(tl_prof_suppressed) { tl_prof_suppressed = true; }
 ProfSuppress::~ProfSuppress() { tl_prof_suppressed = prev_; }
 
-ProfScope::ProfScope(he_ctx* c, const char* name, double work, double bytes, double mac, double bfly, double mac3)
+ProfScope::ProfScope(he_ctx* c, const char* name, double work, double bytes, double mac, double bfly, double mac3,
+                     double sbfly, double folds)
     : c_(c) {
   if (!c->prof_on || tl_prof_suppressed) {
     c_ = nullptr;
@@ -25,6 +26,8 @@ ProfScope::ProfScope(he_ctx* c, const char* name, double work, double bytes, dou
   k.mac += mac;
   k.mac3 += mac3;
   k.bfly += bfly;
+  k.sbfly += sbfly;
+  k.folds += folds;
   k.launches += 1;
   cudaEvent_t a, b;
   cudaEventCreate(&a);
@@ -103,5 +106,13 @@ extern "C" int he_profile_read_kinds(he_ctx* c, const char* name, double* butter
   if (butterflies) *butterflies = it == c->prof.end() ? 0.0 : it->second.bfly;
   if (macs) *macs = it == c->prof.end() ? 0.0 : it->second.mac;
   if (split_macs) *split_macs = it == c->prof.end() ? 0.0 : it->second.mac3;
+  return HE_OK;
+}
+
+extern "C" int he_profile_read_folded(he_ctx* c, const char* name, double* split_butterflies, double* folded_products) {
+  if (!c || !name) return fail(HE_EINVAL, "null argument");
+  auto it = c->prof.find(name);
+  if (split_butterflies) *split_butterflies = it == c->prof.end() ? 0.0 : it->second.sbfly;
+  if (folded_products) *folded_products = it == c->prof.end() ? 0.0 : it->second.folds;
   return HE_OK;
 }
